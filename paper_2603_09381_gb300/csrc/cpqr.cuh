@@ -59,8 +59,16 @@ struct QrProb {
 };
 // Panels [j0, j0 + QR_NB) of every matrix with j0 < n; max_tiles = the most
 // 32-column tiles right of a panel in any matrix.
+// cluster: CTAs per matrix (1, 2, 4, 8), or 0 for as many as fill the SMs (the
+// partial sums of a reflector, hence the last bits, depend on it).
 template <typename C>
-void qr_panel(const QrProb<C>* d_prob, int nprob, int j0, cudaStream_t st);
+void qr_panel(const QrProb<C>* d_prob, int nprob, int j0, cudaStream_t st, int cluster = 0);
+// Trailing update of a complex128 panel (QR_NB reflectors, taus in T) on the
+// tensor cores at FP64 accuracy: V holds QR_NB x (n - QR_NB) entries of Y, Yp
+// ceil(n / 128) x mrb blocks of 128 x QR_NB partial sums, mrb = ceil(W / OZ_RB).
+// *err is set if a bounded wait runs out.
+constexpr int OZ_RB = 256;
+void qr_update_oz(const QrProb<double2>* d_prob, int nprob, int j0, int max_n, int max_w, int* err, cudaStream_t st);
 // max_rb: the most QR_RB-row blocks of rows j0..W-1 in any matrix.  With
 // tc_err (complex64 only) the last step, C -= V Y, runs on the tensor cores
 // (k_qr_apply_tc; max_w = the largest W), which set *tc_err if a bounded wait

@@ -5,7 +5,9 @@
 // the chip's FP64:HBM balance (~0.18).  The kernels therefore favour simple
 // shared-memory tiling with enough resident warps to keep the DFMA pipe busy.
 #include "dense_la.cuh"
+#include "oz_gemm.cuh"
 #include "prof.cuh"
+#include <type_traits>
 #include <algorithm>
 #include <vector>
 #include <cooperative_groups.h>
@@ -949,6 +951,37 @@ void launch_panel_cluster(const LuProb<C>* d_prob, int nprob, int p, cudaStream_
   cudaLaunchKernelEx(&cfg, k_lu_panel_cluster<C, 256>, d_prob, p, LU_NB);
 }
 
+// The trailing update of step p on trailing columns [lo, hi): complex128 on
+// the tensor cores where the caller gave them an error word, else on the FP64 pipe.
+template <typename C>
+void lu_update(const LuProb<C>* d_prob, int nprob, int maxm, int p, int lo, int hi, cudaStream_t st) {
+  if constexpr (std::is_same<C, double2>::value) {
+    if (g_oz_err) {
+      oz_lu_update(d_prob, nprob, maxm, p, LU_NB, lo, hi, g_oz_err, st);
+      return;
+    }
+  }
+  const int mt = maxm - p - LU_NB, n = std::min(hi, mt) - lo;
+  k_lu_update<C><<<dim3(((mt + TB - 1) / TB) * ((n + TB - 1) / TB), nprob), 256, 0, st>>>(d_prob, p, LU_NB, lo, hi);
+}
+
+// The off-diagonal update of a blocked triangular solve, by the same rule.
+template <typename C>
+void getrs_update(const SolveProb<C>* d_prob, int nprob, int maxm, int maxrhs, int p, int lower, cudaStream_t st) {
+  const int mt = lower ? maxm - p - RS_NB : p;
+  if constexpr (std::is_same<C, double2>::value) {
+    if (g_oz_err) {
+      oz_getrs_update(d_prob, nprob, maxm, maxrhs, p, RS_NB, lower, g_oz_err, st);
+      return;
+    }
+    if (maxrhs <= 8) {   // FP64: padding costs the bounding pipe
+      k_getrs_update_thin<C><<<dim3((mt + TH_ROWS - 1) / TH_ROWS, nprob), 128, 0, st>>>(d_prob, p, RS_NB, lower);
+      return;
+    }
+  }
+  k_getrs_update<C><<<dim3(((mt + TB - 1) / TB) * ((maxrhs + TB - 1) / TB), nprob), 256, 0, st>>>(d_prob, p, RS_NB, lower);
+}
+
 // A few large matrices (the top-level LU) with look-ahead, each panel on a
 // cluster of 8 CTAs: step p's update
 // of the next panel's LU_NB columns runs first, on a high-priority stream
@@ -990,17 +1023,15 @@ void la_getrf_lookahead(const LuProb<C>* d_prob, int nprob, int maxm, const int*
     if (mt <= 0) continue;
     const int nrest = mt - LU_NB;
     if (nrest > 0) cudaEventRecord(e_next, sp);   // interchanges and U12 of step p are done
-    const int tiles_m = (mt + TB - 1) / TB;
     const double fn = fu * std::min(1.0, (double)LU_NB / mt);
     KPROF_BEGIN(sp);
-    k_lu_update<C><<<dim3(tiles_m, nprob), 256, 0, sp>>>(d_prob, p, LU_NB, 0, LU_NB);
+    lu_update<C>(d_prob, nprob, maxm, p, 0, LU_NB, sp);
     pm_launch_count_add(1);
     KPROF_END(sp, kname<C>("lu_update", "lu_update32"), fn);
     if (nrest > 0) {
       cudaStreamWaitEvent(su, e_next, 0);
-      dim3 g2(tiles_m * ((nrest + TB - 1) / TB), nprob);
       KPROF_BEGIN(su);
-      k_lu_update<C><<<g2, 256, 0, su>>>(d_prob, p, LU_NB, LU_NB, 1 << 30);
+      lu_update<C>(d_prob, nprob, maxm, p, LU_NB, 1 << 30, su);
       pm_launch_count_add(1);
       KPROF_END(su, kname<C>("lu_update", "lu_update32"), fu - fn);
       cudaEventRecord(e_rest, su);
@@ -1046,10 +1077,8 @@ void la_getrf_batched(const LuProb<C>* d_prob, int nprob, int maxm, const int* h
     KPROF_END(st, kname<C>("lu_swap_trsm", "lu_swap_trsm32"), fs);
     int mt = maxm - p - LU_NB;
     if (mt > 0) {
-      int tiles = ((mt + TB - 1) / TB);
-      dim3 g2(tiles * tiles, nprob);
       KPROF_BEGIN(st);
-      k_lu_update<C><<<g2, 256, 0, st>>>(d_prob, p, LU_NB, 0, 1 << 30);
+      lu_update<C>(d_prob, nprob, maxm, p, 0, 1 << 30, st);
       pm_launch_count_add(1);
       KPROF_END(st, kname<C>("lu_update", "lu_update32"), fu);
     }
@@ -1118,32 +1147,19 @@ void la_getrs_batched(const SolveProb<C>* d_prob, int nprob, int maxm, int maxrh
     return;
   }
   dim3 gs((maxrhs + DG_RHS - 1) / DG_RHS, nprob);
-  const int tiles_n = (maxrhs + TB - 1) / TB;
   for (int p = 0; p < maxm; p += RS_NB) {
     k_getrs_diag<C><<<gs, 256, 0, st>>>(d_prob, p, RS_NB, 1);
     pm_launch_count_add(1);
-    int mt = maxm - p - RS_NB;
-    if (mt > 0) {
-      if (maxrhs <= 8 && sizeof(C) == sizeof(double2)) {   // FP64: padding costs the bounding pipe
-        k_getrs_update_thin<C><<<dim3((mt + TH_ROWS - 1) / TH_ROWS, nprob), 128, 0, st>>>(d_prob, p, RS_NB, 1);
-      } else {
-        dim3 g2(((mt + TB - 1) / TB) * tiles_n, nprob);
-        k_getrs_update<C><<<g2, 256, 0, st>>>(d_prob, p, RS_NB, 1);
-      }
+    if (maxm - p - RS_NB > 0) {
+      getrs_update<C>(d_prob, nprob, maxm, maxrhs, p, 1, st);
       pm_launch_count_add(1);
     }
   }
-  int last = ((maxm - 1) / RS_NB) * RS_NB;
-  for (int p = last; p >= 0; p -= RS_NB) {
+  for (int p = ((maxm - 1) / RS_NB) * RS_NB; p >= 0; p -= RS_NB) {
     k_getrs_diag<C><<<gs, 256, 0, st>>>(d_prob, p, RS_NB, 0);
     pm_launch_count_add(1);
     if (p > 0) {
-      if (maxrhs <= 8 && sizeof(C) == sizeof(double2)) {   // FP64: padding costs the bounding pipe
-        k_getrs_update_thin<C><<<dim3((p + TH_ROWS - 1) / TH_ROWS, nprob), 128, 0, st>>>(d_prob, p, RS_NB, 0);
-      } else {
-        dim3 g2(((p + TB - 1) / TB) * tiles_n, nprob);
-        k_getrs_update<C><<<g2, 256, 0, st>>>(d_prob, p, RS_NB, 0);
-      }
+      getrs_update<C>(d_prob, nprob, maxm, maxrhs, p, 0, st);
       pm_launch_count_add(1);
     }
   }
@@ -1156,14 +1172,12 @@ void la_trsm_upper_batched(const SolveProb<C>* d_prob, int nprob, int maxm, int 
   if (nprob <= 0 || maxm <= 0 || maxrhs <= 0) return;
   KPROF_BEGIN(st);
   dim3 gs((maxrhs + DG_RHS - 1) / DG_RHS, nprob);
-  const int tiles_n = (maxrhs + TB - 1) / TB;
   int last = ((maxm - 1) / RS_NB) * RS_NB;
   for (int p = last; p >= 0; p -= RS_NB) {
     k_getrs_diag<C><<<gs, 256, 0, st>>>(d_prob, p, RS_NB, 0);
     pm_launch_count_add(1);
     if (p > 0) {
-      dim3 g2(((p + TB - 1) / TB) * tiles_n, nprob);
-      k_getrs_update<C><<<g2, 256, 0, st>>>(d_prob, p, RS_NB, 0);
+      getrs_update<C>(d_prob, nprob, maxm, maxrhs, p, 0, st);
       pm_launch_count_add(1);
     }
   }

@@ -1,0 +1,294 @@
+// Complex128 products on the tensor cores, accurate to FP64 (the Ozaki
+// scheme: K. Ozaki, T. Ogita, S. Oishi, S. Rump, "Error-free transformations
+// of matrix multiplication by using fast routines of matrix multiplication",
+// Numer. Algorithms 59 (2012), with integer digits held in fp16).
+//
+// Why: GB300's FP64 pipe does 2 fused multiply-adds per clock and SM
+// (1.26 TFLOP/s measured for the chip), its tensor cores 4096 in fp16.  An
+// FP64 product as 36 exact fp16 products leaves the FP64 pipe one addition
+// per output and stage of 32 complex terms instead of 128 fused
+// multiply-adds.
+//
+// A stage multiplies a 128 x 32 by a 32 x 32 complex block.  Every row of A
+// and every column of B has, per stage, the exponent of its largest part;
+// relative to it each real is rounded to a 62-bit integer (nine bits more
+// than a double holds, for rows and columns of graded entries) and cut into
+// eight balanced base-256 digits, exact in fp16.  The products of digits i
+// and j of equal i + j = s <= 7 add up in one FP32 accumulator: at most
+// 64 x 8 products of at most 2^14, 2^23, hence exact.  What is left out
+// (s > 7) is below 2^-60 of the two maxima's product.  The eight sums are
+// joined in a 75-bit integer, rounded once to a double and added in FP64.  A
+// stage's result depends only on its row of A and its column of B, so the
+// tiling changes no bit.
+//
+// Layout: the real form [Ar | Ai] (128 x 64) times [[Br, Bi], [-Bi, Br]]
+// (64 x 64: real columns, then imaginary), A's digits as eight 128 x 64
+// operands, B's as eight 64 x 64 ones, one 64-column accumulator for each sum
+// (all 512 TMEM columns).  All MMAs have one shape and each sum its own
+// columns: MMAs of several widths on overlapping columns are not ordered among
+// themselves.  K-major, no swizzle: the core matrices are written by
+// conflict-free 16-byte stores.  195 KB of shared memory: one CTA per SM.
+#pragma once
+#include "pm_common.cuh"
+#include "tc_common.cuh"
+
+namespace oz {
+
+constexpr int T = 512;          // threads: (row, group of 8 k) for A; TMEM lane and 8 columns in the epilogue
+constexpr int TM = 128;         // complex rows of a tile
+constexpr int TN = 32;          // complex columns of a tile
+constexpr int TKC = 32;         // complex k of a stage
+constexpr int NS = 8;           // digits
+constexpr int KR = 2 * TKC;     // real k of a stage
+constexpr uint32_t SBO = (KR / 8) * 128;             // next 8 rows of an operand
+constexpr uint32_t A_BYTES = TM * KR * 2;            // one digit of A
+constexpr uint32_t B_BYTES = 2 * TN * KR * 2;        // one digit of B
+constexpr uint32_t OFF_B = NS * A_BYTES;
+constexpr uint32_t OFF_EXP = OFF_B + NS * B_BYTES;   // per k group: exponents of A's rows, then B's columns
+constexpr uint32_t OFF_BAR = OFF_EXP + 4 * (TM + TN) * 4;
+constexpr int SMEM = OFF_BAR + 32;
+constexpr int WAIT = 1 << 20;   // x ~1 us suspend hint: about a second
+
+// kind::f16 instruction descriptor: D f32 (bit 4), A and B fp16 (0), N >> 3 at bit 17, M >> 4 at bit 24
+__device__ __forceinline__ uint32_t idesc(int N) { return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(TM >> 4) << 24); }
+__device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
+  return (uint64_t)((saddr >> 4) & 0x3FFFu) | (uint64_t)(tcx::LBO >> 4) << 16 | (uint64_t)(SBO >> 4) << 32 |
+         (uint64_t)1 << 46;
+}
+__device__ __forceinline__ void mma(uint32_t tmem, uint64_t ad, uint64_t bd, uint32_t id, uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
+          tmem),
+      "l"(ad), "l"(bd), "r"(id), "r"(accumulate));
+}
+// four consecutive fp32 columns of this thread's TMEM lane, not waited for
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, float* d) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+               : "r"(taddr));
+}
+
+__device__ __forceinline__ int exponent(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
+
+// x relative to the exponent E >= exponent(x) as a 62-bit integer, plus the
+// bias that turns its lower seven base-256 digits into unsigned bytes; neg: of
+// -x.  Subnormal x counts as zero.
+__device__ __forceinline__ uint64_t digits(double x, int E, bool neg) {
+  const uint64_t b = (uint64_t)__double_as_longlong(x);
+  const int e = (int)(b >> 52) & 0x7FF;
+  uint64_t q = 0;
+  const int d = E - e;
+  if (e != 0 && d < 63) {
+    q = ((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 9;
+    if (d > 0) q = (q + (1ull << (d - 1))) >> d;
+    if (((b >> 63) != 0) != neg) q = 0 - q;
+  }
+  return q + 0x0080808080808080ull;
+}
+
+// Digit i (0: the largest) of two numbers as a pair of fp16: bytes go
+// through 1024 + byte (exact in fp16) to the signed digit.
+template <int I>
+__device__ __forceinline__ uint32_t digit_pair(uint64_t a, uint64_t b) {
+  uint32_t r;
+  if (I == 0) {   // the top digit is signed already, -64 .. 64: + 128 first
+    r = __byte_perm((uint32_t)(a >> 32), (uint32_t)(b >> 32), 0x0073) ^ 0x8080u;
+    r = __byte_perm(r, 0x64646464u, 0x4140);
+    asm("sub.f16x2 %0, %0, %1;" : "+r"(r) : "r"(0x64806480u));
+  } else {
+    constexpr int byte = 7 - I;
+    const uint32_t x = byte >= 4 ? (uint32_t)(a >> 32) : (uint32_t)a, y = byte >= 4 ? (uint32_t)(b >> 32) : (uint32_t)b;
+    constexpr uint32_t sel = (uint32_t)(byte & 3) | ((uint32_t)(4 + (byte & 3)) << 4);
+    r = __byte_perm(x, y, sel);                          // bytes 0 and 1
+    r = __byte_perm(r, 0x64646464u, 0x4140);             // 0x64 above each
+    asm("sub.f16x2 %0, %0, %1;" : "+r"(r) : "r"(0x64806480u));   // - 1152
+  }
+  return r;
+}
+template <int I>
+__device__ __forceinline__ uint4 digit8(const uint64_t* q) {
+  return make_uint4(digit_pair<I>(q[0], q[1]), digit_pair<I>(q[2], q[3]), digit_pair<I>(q[4], q[5]),
+                    digit_pair<I>(q[6], q[7]));
+}
+// the eight digits of eight numbers into eight operands `step` bytes apart
+__device__ __forceinline__ void put8(unsigned char* p, uint32_t step, const uint64_t* q) {
+  *reinterpret_cast<uint4*>(p) = digit8<0>(q);
+  *reinterpret_cast<uint4*>(p + step) = digit8<1>(q);
+  *reinterpret_cast<uint4*>(p + 2 * step) = digit8<2>(q);
+  *reinterpret_cast<uint4*>(p + 3 * step) = digit8<3>(q);
+  *reinterpret_cast<uint4*>(p + 4 * step) = digit8<4>(q);
+  *reinterpret_cast<uint4*>(p + 5 * step) = digit8<5>(q);
+  *reinterpret_cast<uint4*>(p + 6 * step) = digit8<6>(q);
+  *reinterpret_cast<uint4*>(p + 7 * step) = digit8<7>(q);
+}
+__device__ __forceinline__ uint32_t row_off(int row, int k) { return (uint32_t)(row >> 3) * SBO + (uint32_t)(k >> 3) * tcx::LBO + (uint32_t)(row & 7) * 16; }
+
+// The double nearest to V 2^(ex - 2112), V = sum_s v_s 2^(8 (7 - s)); ex: the
+// sum of the two exponents, or negative for a row or column that is not finite.
+__device__ __forceinline__ double join(const float* v, int ex) {
+  int64_t hi = ((int64_t)__float2int_rn(v[0]) << 24) + ((int64_t)__float2int_rn(v[1]) << 16) +
+               ((int64_t)__float2int_rn(v[2]) << 8) + __float2int_rn(v[3]);
+  const int64_t lo = ((int64_t)__float2int_rn(v[4]) << 24) + ((int64_t)__float2int_rn(v[5]) << 16) +
+                     ((int64_t)__float2int_rn(v[6]) << 8) + __float2int_rn(v[7]);
+  hi += lo >> 32;                       // V = hi 2^32 + l, 0 <= l < 2^32
+  uint32_t l = (uint32_t)lo;
+  const uint64_t sign = (uint64_t)hi & 0x8000000000000000ull;
+  if (sign) {                           // magnitude
+    hi = ~hi + (l == 0 ? 1 : 0);
+    l = 0u - l;
+  }
+  uint64_t mag = (uint64_t)hi, rest = (uint64_t)l << 32;
+  int e = 1023 + 95 + ex - 2112;
+  if (mag == 0) { mag = rest; rest = 0; e -= 64; }
+  const int lz = __clzll((long long)mag);   // V != 0: bit 63 of the shifted magnitude is set
+  mag = (mag << (lz & 63)) | ((rest >> 1) >> (63 - (lz & 63)));
+  e -= lz;
+  mag = (mag + 1024) >> 11;             // 53 bits (a carry goes on into the exponent)
+  uint64_t r = sign | (((uint64_t)(uint32_t)(e - 1) << 52) + mag);
+  if (lz == 64 || e <= 0) r = 0;
+  if (e >= 2047) r = sign | 0x7FF0000000000000ull;
+  if (ex < 0) r = 0x7FF8000000000000ull;
+  return __longlong_as_double((long long)r);
+}
+
+struct Cta {
+  unsigned char* sm;
+  uint32_t tmem;
+  uint32_t phase;
+  bool ok;
+};
+
+// All threads of the CTA; smem: oz::SMEM bytes of dynamic shared memory, 128-byte aligned.
+__device__ __forceinline__ Cta begin(unsigned char* sm) {
+  uint64_t* bar = reinterpret_cast<uint64_t*>(sm + OFF_BAR);
+  uint32_t* taddr = reinterpret_cast<uint32_t*>(sm + OFF_BAR + 16);
+  if (threadIdx.x == 0) {
+    tcx::mbar_init(bar);
+    asm volatile("fence.mbarrier_init.release.cluster;");
+  }
+  if (threadIdx.x < 32) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tcx::smem_u32(taddr)), "r"(512));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  return Cta{sm, *taddr, 0, true};
+}
+__device__ __forceinline__ void end(Cta& c, int* err) {
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  const int all_ok = __syncthreads_and(c.ok ? 1 : 0);
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  if (threadIdx.x < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(c.tmem), "r"(512));
+  if (!all_ok && threadIdx.x == 0) atomicExch(err, 1);
+}
+
+// One stage: acc[j] += (A B)(row, 8 cg + j) for this thread's row (32 (warp %
+// 4) + lane) and column group cg = warp / 4.  a(row, k) and b(k, col) return
+// the operands' entries, zero outside; new_a: A's digits are not in shared
+// memory yet.  All 512 threads call it.
+template <class FA, class FB>
+__device__ __forceinline__ void stage(Cta& c, bool new_a, const FA& a, const FB& b, double2* acc) {
+  const int tid = threadIdx.x, warp = tid >> 5;
+  int* ea = reinterpret_cast<int*>(c.sm + OFF_EXP);   // [k group][row]
+  int* eb = ea + 4 * TM;                              // [k group][column]
+  const int row = tid & (TM - 1), kg = tid >> 7;
+  const int bn = tid & 31, bg = (tid >> 5) & 3, bpart = tid >> 7;   // B: threads 0 .. 255
+  double2 va[8];
+  if (new_a) {
+    int e = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) va[i] = a(row, 8 * kg + i);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) e = max(e, max(exponent(va[i].x), exponent(va[i].y)));
+    ea[kg * TM + row] = e;
+  }
+  double vb[8];
+  if (tid < 256) {
+    int e = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const double2 v = b(8 * bg + i, bn);
+      e = max(e, max(exponent(v.x), exponent(v.y)));
+      vb[i] = bpart ? v.y : v.x;
+    }
+    if (bpart == 0) eb[bg * TN + bn] = e;
+  }
+  __syncthreads();
+  if (new_a) {
+    const int E = max(max(ea[row], ea[TM + row]), max(ea[2 * TM + row], ea[3 * TM + row]));
+    uint64_t q[8];
+    unsigned char* p = c.sm + row_off(row, 8 * kg);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) q[i] = digits(va[i].x, E, false);
+    put8(p, A_BYTES, q);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) q[i] = digits(va[i].y, E, false);
+    put8(p + (TKC / 8) * tcx::LBO, A_BYTES, q);
+  }
+  if (tid < 256) {
+    const int E = max(max(eb[bn], eb[TN + bn]), max(eb[2 * TN + bn], eb[3 * TN + bn]));
+    // real part: [row bn, k] and [row 32 + bn, 32 + k]; imaginary part: negated [row bn, 32 + k], [row 32 + bn, k]
+    uint64_t q[8];
+    unsigned char* B = c.sm + OFF_B;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) q[i] = digits(vb[i], E, false);
+    put8(B + row_off(TN + bn, (bpart ? 0 : TKC) + 8 * bg), B_BYTES, q);
+    if (bpart) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) q[i] = digits(vb[i], E, true);
+    }
+    put8(B + row_off(bn, (bpart ? TKC : 0) + 8 * bg), B_BYTES, q);
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  uint64_t* bar = reinterpret_cast<uint64_t*>(c.sm + OFF_BAR);
+  if (tid == 0) {
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    const uint32_t as = tcx::smem_u32(c.sm), bs = as + OFF_B;
+    for (int ks = 0; ks < KR / 16; ++ks) {
+      const uint32_t ko = ks * 2 * tcx::LBO;   // 16 fp16 along k = two core matrices
+#pragma unroll
+      for (int i = 0; i < NS; ++i) {
+        const uint64_t ad = sdesc(as + i * A_BYTES + ko);
+#pragma unroll
+        for (int j = 0; j < NS - i; ++j)
+          mma(c.tmem + (i + j) * 2 * TN, ad, sdesc(bs + j * B_BYTES + ko), idesc(2 * TN), ks + i > 0 ? 1u : 0u);
+      }
+    }
+    tcx::mma_commit(bar);
+  }
+  // the exponents of this thread's outputs, while the MMAs run
+  const int er = 32 * (warp & 3) + (tid & 31), cg = warp >> 2;
+  const int E = max(max(ea[er], ea[TM + er]), max(ea[2 * TM + er], ea[3 * TM + er]));
+  c.ok = c.ok && tcx::mbar_wait(bar, c.phase, WAIT);
+  c.phase ^= 1;
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  if (__all_sync(0xffffffffu, c.ok ? 1 : 0)) {
+    const uint32_t t0 = c.tmem + ((uint32_t)((warp & 3) * 32) << 16) + 8 * cg;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+      for (int part = 0; part < 2; ++part) {
+        float v[NS][4];
+#pragma unroll
+        for (int s = 0; s < NS; ++s) tmem_ld4(t0 + s * 2 * TN + part * TN + 4 * h, v[s]);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int n = 8 * cg + 4 * h + j;
+          const int F = max(max(eb[n], eb[TN + n]), max(eb[2 * TN + n], eb[3 * TN + n]));
+          const float w[NS] = {v[0][j], v[1][j], v[2][j], v[3][j], v[4][j], v[5][j], v[6][j], v[7][j]};
+          const double d = join(w, E == 0x7FF || F == 0x7FF ? -1 : E + F);
+          if (part == 0) acc[4 * h + j].x += d; else acc[4 * h + j].y += d;
+        }
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();   // the operands and accumulators may be overwritten
+  asm volatile("tcgen05.fence::after_thread_sync;");
+}
+
+}  // namespace oz

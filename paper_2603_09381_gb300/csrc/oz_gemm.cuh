@@ -1,0 +1,28 @@
+// Launchers of the FP64-accurate tensor-core products (oz.cuh): batched GEMM
+// and the trailing updates of the FP64 LU and LU solves.
+#pragma once
+#include "dense_la.cuh"
+
+// Error word of the bounded tensor-core waits of the running call (device
+// int, set to 1 when a wait runs out): thread-local, set by OzErrScope.
+extern thread_local int* g_oz_err;
+struct OzErrScope {
+  int* prev;
+  explicit OzErrScope(int* e) : prev(g_oz_err) { g_oz_err = e; }
+  ~OzErrScope() { g_oz_err = prev; }
+};
+
+// Tiles of an m x n product: rows in 128s, columns in groups of `per` tiles of 32.
+inline int oz_tiles(int m, int n, int per) { return ((m + 127) / 128) * ((n + 32 * per - 1) / (32 * per)); }
+// Column tiles per CTA for a batch of `tiles` single-tile products (A's digits are reused across them).
+int oz_per(long tiles);
+
+// d_off: prefix sums of oz_tiles(m, n, per).
+void oz_gemm_batched(const GemmDesc<double2>* d_desc, const int* d_off, int nprob, int total, int per, int* err,
+                     cudaStream_t st);
+// A22 -= L21 U12 on trailing columns [p + jb + lo, p + jb + hi) of every matrix (k_lu_update's contract).
+void oz_lu_update(const LuProb<double2>* d_prob, int nprob, int maxm, int p, int nb, int lo, int hi, int* err,
+                  cudaStream_t st);
+// The off-diagonal update of a blocked triangular solve (k_getrs_update's contract).
+void oz_getrs_update(const SolveProb<double2>* d_prob, int nprob, int maxm, int maxrhs, int p, int nb, int lower, int* err,
+                     cudaStream_t st);

@@ -17,6 +17,8 @@
 // (tile, block), so that the rows of a tall matrix spread over many CTAs.
 #include "cpqr.cuh"
 #include "prof.cuh"
+#include "oz.cuh"
+#include "oz_gemm.cuh"
 #include "tc_common.cuh"
 #include <cooperative_groups.h>
 #include <type_traits>
@@ -25,11 +27,20 @@ namespace cg = cooperative_groups;
 
 namespace {
 
-constexpr int PT = 512;      // panel CTA: two threads per row, 16 panel columns each
-constexpr int PR = PT / 2;   // rows per sweep of the panel CTA
+constexpr int PT = 512;      // panel CTA
 constexpr int UT = 256;      // update CTA
 constexpr int RC = 32;       // rows per staged chunk
-constexpr int HB = QR_NB / 2;
+// Q threads share a row of the panel, thread q holding columns q, q + Q, ..
+// Interleaved, the columns already factored drop out for all Q threads at
+// once: a warp's instructions shrink with the trailing block (a split in
+// halves kept every instruction alive until the last column).
+template <int Q_> struct PanelSplit {
+  static constexpr int Q = Q_;
+  static constexpr int HB = QR_NB / Q;      // columns per thread
+  static constexpr int RW = 32 / Q;         // rows per warp and sweep
+  static constexpr int PR = PT / Q;         // rows per sweep of the CTA
+  static_assert(RW == HB, "the reduction below leaves one column per lane");
+};
 
 // V entry (row r, panel column j) of a panel starting at j0: unit diagonal,
 // zero above, the stored reflector below.
@@ -47,71 +58,81 @@ __device__ __forceinline__ C v_entry(const QrProb<C>& p, int j0, int jb, int r, 
 // factors f_k in s_f, its column scaled by sc into v) and accumulates the
 // inputs of step jn = ja + 1: N = sum_{r >= c'} |a_jn[r]|^2 and
 // S_k = sum_{r > c'} conj(a_jn[r]) a_k[r] for k > jn (c' = j0 + jn), with row
-// c' itself stored to s_row.  Lanes 0-15 of a warp hold panel columns 0-15 of
-// 16 rows, lanes 16-31 columns 16-31 of the same rows; every entry a thread
-// needs is loaded before the pair stores anything.
+// c' itself stored to s_row.  Every entry a thread needs is loaded before the
+// threads of its row store anything.
 template <typename C>
 __device__ __forceinline__ void panel_pass(const QrProb<C>& p, int j0, int jb, int ja, const C* s_f, C sc,
                                            C* s_row, typename real_of<C>::type& N, C* S, int rank, int csize) {
   typedef typename real_of<C>::type R;
+  typedef PanelSplit<2> L;
+  constexpr int Q = L::Q, HB = L::HB, RW = L::RW;
   const int jn = ja + 1;
   const int ca = j0 + ja, cn = j0 + jn;
   C* Zp = p.Z + (size_t)j0 * p.ld;
   const size_t ld = p.ld;
-  const int lane = threadIdx.x & 31, half = lane >> 4;
-  const int kb = half * HB;
+  const int lane = threadIdx.x & 31, q = lane / RW;
   const int kmin = ja >= 0 ? ja : jn;
   const C fjn = (ja >= 0 && jn < jb) ? s_f[jn] : czero<C>();
   // warp-uniform sweep (the __syncwarp below needs every lane), rows guarded
-  for (int r0 = (ja >= 0 ? ca : cn) + (threadIdx.x >> 5) * 16 + rank * PR; r0 < p.W; r0 += PR * csize) {
-    const int r = r0 + (lane & 15);
+  for (int r0 = (ja >= 0 ? ca : cn) + (threadIdx.x >> 5) * RW + rank * L::PR; r0 < p.W; r0 += L::PR * csize) {
+    const int r = r0 + lane % RW;
     const bool act = r < p.W;
     C v[HB];
 #pragma unroll
     for (int k = 0; k < HB; ++k)
-      if (act && kb + k >= kmin && kb + k < jb) v[k] = Zp[r + (size_t)(kb + k) * ld];
+      if (Q * k + Q > kmin && act && Q * k + q >= kmin && Q * k + q < jb) v[k] = Zp[r + (size_t)(Q * k + q) * ld];
     const C x = (act && ja >= 0) ? Zp[r + (size_t)ja * ld] : czero<C>();
     const C yold = (act && jn < jb) ? Zp[r + (size_t)jn * ld] : czero<C>();
-    __syncwarp();   // both threads of the pair have read the row before either writes it
+    __syncwarp();   // the threads of the row have read it before any of them writes it
     if (!act) continue;
     C vr = czero<C>();
     if (ja >= 0) {
       vr = (r == ca) ? mk((R)1, (R)0) : x * sc;
-      if (r > ca && half == (ja >= HB)) Zp[r + (size_t)ja * ld] = vr;
+      if (r > ca && q == ja % Q) Zp[r + (size_t)ja * ld] = vr;
 #pragma unroll
       for (int k = 0; k < HB; ++k)
-        if (kb + k > ja && kb + k < jb) {
-          cfms(v[k], s_f[kb + k], vr);
-          Zp[r + (size_t)(kb + k) * ld] = v[k];
+        if (Q * k + Q - 1 > ja && Q * k + q > ja && Q * k + q < jb) {
+          cfms(v[k], s_f[Q * k + q], vr);
+          Zp[r + (size_t)(Q * k + q) * ld] = v[k];
         }
     }
     if (jn < jb && r >= cn) {
       C y = yold;
       if (ja >= 0) cfms(y, fjn, vr);
-      if (half == 0) N += abs2(y);
+      if (q == 0) N += abs2(y);
       if (r == cn) {
 #pragma unroll
-        for (int k = 0; k < HB; ++k) if (kb + k >= jn && kb + k < jb) s_row[kb + k] = v[k];
+        for (int k = 0; k < HB; ++k) if (Q * k + q >= jn && Q * k + q < jb) s_row[Q * k + q] = v[k];
       } else {
 #pragma unroll
-        for (int k = 0; k < HB; ++k) if (kb + k > jn && kb + k < jb) cfma_conj(S[k], y, v[k]);
+        for (int k = 0; k < HB; ++k)
+          if (Q * k + Q - 1 > jn && Q * k + q > jn && Q * k + q < jb) cfma_conj(S[k], y, v[k]);
       }
     }
   }
 }
 
-template <typename C>
+__device__ __forceinline__ float2 shfl_xor_c(float2 v, int o) {
+  return make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
+}
+__device__ __forceinline__ longlong2 shfl_xor_c(longlong2 v, int o) {
+  return make_longlong2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
+}
+
 // At most 112 registers: 512 x 112 leaves room on the SM for one CTA of the
 // operator assembly that may run beside the factorization.
+template <typename C>
 __global__ void __maxnreg__(112) k_qr_panel(const QrProb<C>* __restrict__ P, int j0) {
   typedef typename real_of<C>::type R;
+  typedef PanelSplit<2> L;
+  constexpr int Q = L::Q, HB = L::HB, RW = L::RW;
   cg::cluster_group cluster = cg::this_cluster();
   const int csize = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const QrProb<C> p = P[blockIdx.x / csize];
   if (j0 >= p.n) return;   // the whole cluster (same matrix) leaves
   const int jb = min(QR_NB, p.n - j0);
   const int W = p.W;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, half = lane >> 4;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q = lane / RW;
   constexpr int NV = 4 * QR_NB + 1;   // S (re, im), N, row c' (re, im)
   __shared__ R s_red[PT / 32][2 * QR_NB + 1];
   __shared__ R s_part[2][NV];         // this CTA's partial sums, by pass parity
@@ -135,22 +156,24 @@ __global__ void __maxnreg__(112) k_qr_panel(const QrProb<C>* __restrict__ P, int
     panel_pass(p, j0, jb, ja, s_f, sc, s_row, N, S, rank, csize);
     const int jn = ja + 1;
     if (jn >= jb) break;
-    // CTA sums: N over all lanes, S_k over the 16 lanes of each half
+    // CTA sums: N over all lanes; S over the RW lanes of each q, halving the
+    // columns with every exchange (lane i of a q ends with column slot i)
     N = warp_sum(N);
 #pragma unroll
-    for (int k = 0; k < HB; ++k)
+    for (int o = RW / 2, cnt = HB / 2; o > 0; o >>= 1, cnt >>= 1) {
+      const bool up = (lane & o) != 0;
 #pragma unroll
-      for (int o = 8; o > 0; o >>= 1) {
-        S[k].x += __shfl_xor_sync(0xffffffffu, S[k].x, o);
-        S[k].y += __shfl_xor_sync(0xffffffffu, S[k].y, o);
-      }
-    if ((lane & 15) == 0) {
-#pragma unroll
-      for (int k = 0; k < HB; ++k) {
-        s_red[warp][2 * (half * HB + k)] = S[k].x;
-        s_red[warp][2 * (half * HB + k) + 1] = S[k].y;
-      }
-      if (half == 0) s_red[warp][2 * QR_NB] = N;
+      for (int k = 0; k < HB / 2; ++k)
+        if (k < cnt) {
+          const C send = up ? S[k] : S[k + cnt], keep = up ? S[k + cnt] : S[k];
+          S[k] = keep + shfl_xor_c(send, o);
+        }
+    }
+    {
+      const int col = Q * (lane % RW) + q;
+      s_red[warp][2 * col] = S[0].x;
+      s_red[warp][2 * col + 1] = S[0].y;
+      if (lane == 0) s_red[warp][2 * QR_NB] = N;
     }
     __syncthreads();
     if (tid < 2 * QR_NB + 1) {
@@ -165,13 +188,14 @@ __global__ void __maxnreg__(112) k_qr_panel(const QrProb<C>* __restrict__ P, int
     cluster.sync();   // every CTA's partials of this pass are written
     if (tid < NV) {
       R t = 0;
-      for (int q = 0; q < csize; ++q) t += cluster.map_shared_rank(&s_part[par][0], q)[tid];   // rank order
+      for (int r = 0; r < csize; ++r) t += cluster.map_shared_rank(&s_part[par][0], r)[tid];   // rank order
       s_tot[tid] = t;
     }
     if (tid < QR_NB) s_row[tid] = czero<C>();
     __syncthreads();
-    if (tid == 0) {
-      // reflector of column jn (LAPACK zlarfg phase), factors of the next pass
+    if (warp == 0) {
+      // reflector of column jn (LAPACK zlarfg phase), factors of the next
+      // pass: lane k's column k (the scalars in every lane alike)
       const int c = j0 + jn;
       const C alpha = mk(s_tot[2 * QR_NB + 1 + 2 * jn], s_tot[2 * QR_NB + 2 + 2 * jn]);
       const R xnorm = sqrt(s_tot[2 * QR_NB]);
@@ -183,13 +207,15 @@ __global__ void __maxnreg__(112) k_qr_panel(const QrProb<C>* __restrict__ P, int
         tau = cdiv(bm - alpha, bm);
         scn = cdiv(mk((R)1, (R)0), alpha - bm);
       }
-      if (rank == 0) p.Z[c + (size_t)c * p.ld] = mk(beta, (R)0);
-      s_tau[jn] = tau;
-      s_sc = scn;
+      if (rank == 0 && lane == 0) p.Z[c + (size_t)c * p.ld] = mk(beta, (R)0);
+      if (lane == 0) {
+        s_tau[jn] = tau;
+        s_sc = scn;
+      }
       const C ctau = conj(tau), cscn = conj(scn);
-      for (int k = jn + 1; k < jb; ++k) {
-        const C rowk = mk(s_tot[2 * QR_NB + 1 + 2 * k], s_tot[2 * QR_NB + 2 + 2 * k]);
-        s_f[k] = ctau * (rowk + cscn * mk(s_tot[2 * k], s_tot[2 * k + 1]));
+      if (lane > jn && lane < jb) {
+        const C rowk = mk(s_tot[2 * QR_NB + 1 + 2 * lane], s_tot[2 * QR_NB + 2 + 2 * lane]);
+        s_f[lane] = ctau * (rowk + cscn * mk(s_tot[2 * lane], s_tot[2 * lane + 1]));
       }
     }
     __syncthreads();
@@ -248,6 +274,319 @@ __global__ void __maxnreg__(112) k_qr_panel(const QrProb<C>* __restrict__ P, int
   }
   if (rank == 0)
     for (int e = tid; e < QR_NB * QR_NB; e += PT) p.T[e] = s_t[e % QR_NB][e / QR_NB];
+}
+
+// ---- complex128 panel in 60-bit fixed point ----------------------------------------
+// The FP64 pipe does 2 fused multiply-adds per clock and SM, the integer
+// multipliers 64: a fixed-point complex multiply-add (12 wide multiplies,
+// ~10 other instructions) takes a quarter of the time of the 4 FP64 ones.
+// Fixed point suits a Householder panel: a reflection keeps the norm of
+// a column, so with a scale per column (its norm at most 1/4, a power of two)
+// nothing overflows, and every operation errs by ~2^-59 of the column's
+// scale, where FP64 errs by 2^-53 of the entry.
+//   entries   A = a 2^-60 scale_k, |a|_2 <= 1/4 per column (64-bit integers, in place of the doubles)
+//   v         |v| <= 1, 2^-60
+//   y         the column that defines the next reflector.  Its norm may be
+//             far below its scale, and the reflector must be orthogonal to
+//             working precision, so each warp shifts its rows of y up to use
+//             all bits before the dot products; the shifts are taken out when
+//             the warps' sums meet in FP64.
+// A number x is split as x = h 2^30 + l, 0 <= l < 2^30; a product keeps
+// h h' + (h l' + l h') / 2^30 and leaves out l l' / 2^60 (below one unit;
+// its mean is added).
+struct Fx { int h, l; };
+__device__ __forceinline__ Fx fx(long long v) { return Fx{(int)(v >> 30), (int)v & 0x3FFFFFFF}; }
+__device__ __forceinline__ void fx_mac(long long& hh, long long& cr, Fx a, Fx b) {
+  hh += (long long)a.h * b.h;
+  cr += (long long)a.h * b.l;
+  cr += (long long)a.l * b.h;
+}
+constexpr long long FX_HALF = 1ll << 30;   // rounding and the mean of two dropped l l', before >> 30
+// a + g v, g given as (re, im, -im)
+__device__ __forceinline__ longlong2 fx_cfma(longlong2 a, Fx gr, Fx gi, Fx ngi, Fx vr, Fx vi) {
+  long long cr = FX_HALF, ci = FX_HALF;
+  fx_mac(a.x, cr, gr, vr);
+  fx_mac(a.x, cr, ngi, vi);
+  fx_mac(a.y, ci, gr, vi);
+  fx_mac(a.y, ci, gi, vr);
+  a.x += cr >> 30;
+  a.y += ci >> 30;
+  return a;
+}
+constexpr double FX_ONE = 1152921504606846976.0;   // 2^60
+// x 2^60 / 2^e2 rounded, for |x| < 2^(e2 - 2); subnormal x counts as zero
+__device__ __forceinline__ long long fx_from(double x, int e2) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)(b >> 52) & 0x7FF, d = e2 + 1020 - ex;   // d >= 0
+  long long m = 0;
+  if (ex != 0 && d < 59) {
+    m = (long long)(((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 5);
+    if (d > 0) m = (m + (1ll << (d - 1))) >> d;
+  }
+  return (long long)b < 0 ? -m : m;
+}
+// the double nearest to a 2^(e2 - 60) (|e2| below 900)
+__device__ __forceinline__ double fx_to(long long a, int e2) {
+  const unsigned long long sign = (unsigned long long)a & 0x8000000000000000ull;
+  unsigned long long m = sign ? 0 - (unsigned long long)a : (unsigned long long)a;
+  const int lz = __clzll((long long)m);
+  m = ((m << (lz & 63)) + 1024) >> 11;   // 53 bits (a carry goes on into the exponent)
+  const unsigned long long r = ((unsigned long long)(unsigned)(1023 + 63 - lz - 60 + e2 - 1) << 52) + m;
+  return __longlong_as_double((long long)(a == 0 ? 0 : sign | r));
+}
+
+// A matrix's panel on a cluster; rows go to warps 8 at a time and stay there
+// for the whole panel.  T receives the taus.  Same reflectors and order as
+// k_qr_panel (LAPACK zlarfg phase convention).
+// Four threads per row: their 8 entries and 8 sums fit the registers.
+__global__ void __launch_bounds__(PT, 1) k_qr_panel_fx(const QrProb<double2>* __restrict__ P, int j0) {
+  typedef PanelSplit<4> L;
+  constexpr int Q = L::Q, HB = L::HB, RW = L::RW;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int csize = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const QrProb<double2> p = P[blockIdx.x / csize];
+  if (j0 >= p.n) return;   // the whole cluster (same matrix) leaves
+  const int jb = min(QR_NB, p.n - j0), W = p.W;
+  const size_t ld = p.ld;
+  longlong2* Zx = reinterpret_cast<longlong2*>(p.Z + (size_t)j0 * ld);   // the panel's columns as integers
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q = lane / RW;
+  const int rbeg = j0 + warp * RW + rank * L::PR, rstep = L::PR * csize;   // the warp's first row and stride
+  constexpr int NV = 4 * QR_NB + 1;   // S (re, im), N, row c' (re, im)
+  __shared__ double s_red[PT / 32][2 * QR_NB + 1];
+  __shared__ double s_part[2][NV];    // this CTA's partial sums, by pass parity
+  __shared__ double s_tot[NV];
+  __shared__ longlong2 s_row[QR_NB];  // row c' entries held by this CTA (zero elsewhere)
+  __shared__ int4 s_g[QR_NB];         // factors of the next pass: re, im as (h, l) ..
+  __shared__ int2 s_gn[QR_NB];        // .. and -im
+  __shared__ double s_beta[QR_NB];
+  __shared__ int s_exp[QR_NB];        // scale of column k: 2^s_exp
+  __shared__ int s_bad;               // columns from here on are not finite, or follow one that is not
+  __shared__ double2 s_tau[QR_NB];
+  __shared__ longlong2 s_sc;
+  __shared__ int s_ev;
+  // column norms: the scale of column k is the power of two that brings its norm into (1/8, 1/4]
+  {
+    double acc[HB];
+#pragma unroll
+    for (int k = 0; k < HB; ++k) acc[k] = 0.0;
+    for (int r = rbeg + lane % RW; r < W; r += rstep)
+#pragma unroll
+      for (int k = 0; k < HB; ++k)
+        if (Q * k + q < jb) acc[k] += abs2(p.Z[r + (size_t)(j0 + Q * k + q) * ld]);
+#pragma unroll
+    for (int k = 0; k < HB; ++k)
+#pragma unroll
+      for (int o = RW / 2; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+    if (lane % RW == 0)
+#pragma unroll
+      for (int k = 0; k < HB; ++k) s_red[warp][Q * k + q] = acc[k];
+    if (tid < QR_NB) s_row[tid] = make_longlong2(0, 0);
+    if (tid == 0) s_bad = QR_NB;
+    __syncthreads();
+    if (tid < QR_NB) {
+      double t = 0;
+#pragma unroll
+      for (int w = 0; w < PT / 32; ++w) t += s_red[w][tid];
+      s_part[1][tid] = t;
+    }
+    cluster.sync();
+    if (tid < jb) {
+      double t = 0;
+      for (int r = 0; r < csize; ++r) t += cluster.map_shared_rank(&s_part[1][0], r)[tid];
+      int e = 0;
+      if (!isfinite(t)) atomicMin(&s_bad, tid);
+      else if (t > 0) frexp(sqrt(t) * (1.0 + 1e-9), &e);
+      s_exp[tid] = e + 2;
+    }
+    __syncthreads();
+    for (int r = rbeg + lane % RW; r < W; r += rstep)
+#pragma unroll
+      for (int k = 0; k < HB; ++k)
+        if (Q * k + q < jb) {
+          const double2 z = p.Z[r + (size_t)(j0 + Q * k + q) * ld];
+          const int e2 = s_exp[Q * k + q];
+          const bool ok = Q * k + q < s_bad;
+          Zx[r + (size_t)(Q * k + q) * ld] = make_longlong2(ok ? fx_from(z.x, e2) : 0, ok ? fx_from(z.y, e2) : 0);
+        }
+    __syncwarp();
+  }
+  int par = 0;
+  for (int ja = -1; ja < jb; ++ja, par ^= 1) {
+    const int jn = ja + 1, ca = j0 + ja, cn = j0 + jn;
+    // column ja becomes v, column jn is brought up to date and measured
+    Fx scr = {0, 0}, sci = {0, 0}, nsci = {0, 0};
+    int ev = 0;
+    if (ja >= 0) {
+      const longlong2 sc = s_sc;
+      scr = fx(sc.x); sci = fx(sc.y); nsci = fx(-sc.y);
+      ev = s_ev;
+    }
+    unsigned long long any = 0;
+    for (int r0 = rbeg; r0 < W; r0 += rstep) {   // the same steps for the whole warp
+      const int r = r0 + lane % RW;
+      const bool act = r < W && r >= (ja >= 0 ? ca : cn);
+      const longlong2 x = act && ja >= 0 ? Zx[r + (size_t)ja * ld] : make_longlong2(0, 0);
+      longlong2 y = act && jn < jb ? Zx[r + (size_t)jn * ld] : make_longlong2(0, 0);
+      __syncwarp();   // the row's threads have read both before one of them writes
+      if (!act) continue;
+      if (ja >= 0) {
+        longlong2 v;
+        if (r == ca) {
+          v = make_longlong2(1ll << 60, 0);
+        } else {
+          v = fx_cfma(make_longlong2(0, 0), scr, sci, nsci, fx(x.x << ev), fx(x.y << ev));
+          v.x <<= 2; v.y <<= 2;
+          if (q == 0) Zx[r + (size_t)ja * ld] = v;
+        }
+        if (jn < jb) {
+          const int4 g = s_g[jn];
+          const int2 gn = s_gn[jn];
+          y = fx_cfma(y, Fx{g.x, g.y}, Fx{g.z, g.w}, Fx{gn.x, gn.y}, fx(v.x), fx(v.y));
+          if (q == 1) Zx[r + (size_t)jn * ld] = y;
+        }
+      }
+      if (jn < jb && r >= cn) any |= (unsigned long long)(y.x ^ (y.x >> 63)) | (unsigned long long)(y.y ^ (y.y >> 63));
+    }
+    __syncwarp();
+    if (jn >= jb) break;
+    // shift that brings this warp's rows of y just below 2^55
+    const unsigned ah = __reduce_or_sync(0xffffffffu, (unsigned)(any >> 32)), al = __reduce_or_sync(0xffffffffu, (unsigned)any);
+    const int top = ah ? 63 - __clz(ah) : (al ? 31 - __clz(al) : 0);
+    const int ew = 54 - top;   // top <= 58: may be negative
+    long long N = 0;
+    longlong2 S[HB];
+#pragma unroll
+    for (int k = 0; k < HB; ++k) S[k] = make_longlong2(0, 0);
+    for (int r = rbeg + lane % RW; r < W; r += rstep) {
+      if (r < (ja >= 0 ? ca : cn)) continue;
+      longlong2 a[HB];
+#pragma unroll
+      for (int k = 0; k < HB; ++k)
+        if (Q * k + Q - 1 > jn && Q * k + q > jn && Q * k + q < jb) a[k] = Zx[r + (size_t)(Q * k + q) * ld];
+      const longlong2 v = ja < 0 ? make_longlong2(0, 0) : r == ca ? make_longlong2(1ll << 60, 0) : Zx[r + (size_t)ja * ld];
+      const longlong2 y0 = Zx[r + (size_t)jn * ld];
+      const longlong2 y = ew >= 0 ? make_longlong2(y0.x << ew, y0.y << ew) : make_longlong2(y0.x >> -ew, y0.y >> -ew);
+      const Fx vr = fx(v.x), vi = fx(v.y), yr = fx(y.x), yi = fx(y.y), nyi = fx(-y.y);
+      if (r >= cn && q == 0) {
+        long long cr = FX_HALF;
+        fx_mac(N, cr, yr, yr);
+        fx_mac(N, cr, yi, yi);
+        N += cr >> 30;
+      }
+      if (r == cn && q == jn % Q) s_row[jn] = y0;
+#pragma unroll
+      for (int k = 0; k < HB; ++k)
+        if (Q * k + Q - 1 > jn && Q * k + q > jn && Q * k + q < jb) {
+          if (ja >= 0) {
+            const int4 g = s_g[Q * k + q];
+            const int2 gn = s_gn[Q * k + q];
+            a[k] = fx_cfma(a[k], Fx{g.x, g.y}, Fx{g.z, g.w}, Fx{gn.x, gn.y}, vr, vi);
+            Zx[r + (size_t)(Q * k + q) * ld] = a[k];
+          }
+          if (r == cn) {
+            s_row[Q * k + q] = a[k];
+          } else if (r > cn) {
+            const Fx ar = fx(a[k].x), ai = fx(a[k].y);
+            long long cr = FX_HALF, ci = FX_HALF;
+            fx_mac(S[k].x, cr, yr, ar);
+            fx_mac(S[k].x, cr, yi, ai);
+            fx_mac(S[k].y, ci, yr, ai);
+            fx_mac(S[k].y, ci, nyi, ar);
+            S[k].x += cr >> 30;
+            S[k].y += ci >> 30;
+          }
+        }
+    }
+    __syncwarp();
+    // warp sums as in k_qr_panel, in integers, then FP64 with the warp's shift taken out
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) N += __shfl_xor_sync(0xffffffffu, N, o);
+#pragma unroll
+    for (int o = RW / 2, cnt = HB / 2; o > 0; o >>= 1, cnt >>= 1) {
+      const bool up = (lane & o) != 0;
+#pragma unroll
+      for (int k = 0; k < HB / 2; ++k)
+        if (k < cnt) {
+          const longlong2 send = up ? S[k] : S[k + cnt], keep = up ? S[k + cnt] : S[k], got = shfl_xor_c(send, o);
+          S[k] = make_longlong2(keep.x + got.x, keep.y + got.y);
+        }
+    }
+    {
+      const int col = Q * (lane % RW) + q;
+      const double u = __longlong_as_double((long long)(1023 - 60 - ew) << 52);   // 2^(-60 - ew)
+      s_red[warp][2 * col] = (double)S[0].x * u;
+      s_red[warp][2 * col + 1] = (double)S[0].y * u;
+      if (lane == 0) s_red[warp][2 * QR_NB] = (double)N * u * __longlong_as_double((long long)(1023 - ew) << 52);
+    }
+    __syncthreads();
+    if (tid < 2 * QR_NB + 1) {
+      double t = 0;
+#pragma unroll
+      for (int w = 0; w < PT / 32; ++w) t += s_red[w][tid];
+      s_part[par][tid] = t;
+    } else if (tid < NV) {
+      const int k = (tid - 2 * QR_NB - 1) >> 1;
+      s_part[par][tid] = (double)(((tid - 2 * QR_NB - 1) & 1) ? s_row[k].y : s_row[k].x) * (1.0 / FX_ONE);
+    }
+    cluster.sync();   // every CTA's partials of this pass are written
+    if (tid < NV) {
+      double t = 0;
+      for (int r = 0; r < csize; ++r) t += cluster.map_shared_rank(&s_part[par][0], r)[tid];   // rank order
+      s_tot[tid] = t;
+    }
+    if (tid < QR_NB) s_row[tid] = make_longlong2(0, 0);
+    __syncthreads();
+    if (warp == 0) {
+      // reflector of column jn, in units of its scale; lane k: the factor of column k
+      const double2 alpha = make_double2(s_tot[2 * QR_NB + 1 + 2 * jn], s_tot[2 * QR_NB + 2 + 2 * jn]);
+      const double xnorm = sqrt(s_tot[2 * QR_NB]);
+      double2 tau = czero<double2>(), sc = czero<double2>();
+      double beta = 0;
+      int ex = 0;
+      if (xnorm > 0) {
+        beta = -copysign(xnorm, alpha.x);
+        const double2 bm = make_double2(beta, 0.0);
+        tau = cdiv(bm - alpha, bm);
+        sc = cdiv(make_double2(1.0, 0.0), alpha - bm);
+        ex = (int)((__double2hiint(xnorm) >> 20) & 0x7FF) - 1022;   // xnorm in [2^(ex - 1), 2^ex), ex <= -1
+        ex = max(ex, -60);
+      }
+      if (lane == 0) {
+        // v = x sc = 4 (x 2^ev) (sc 2^-ev / 4) with x 2^ev below 1/2 and |sc| 2^-ev <= 4
+        const int ev = -1 - ex;
+        const double u = 0.25 * FX_ONE * __longlong_as_double((long long)(1023 - ev) << 52);
+        s_sc = make_longlong2(__double2ll_rn(sc.x * u), __double2ll_rn(sc.y * u));
+        s_ev = ev;
+        s_beta[jn] = beta;
+        s_tau[jn] = jn < s_bad ? tau : make_double2(nan(""), 0.0);
+      }
+      if (lane > jn && lane < jb) {
+        const double2 ctau = conj(tau), csc = conj(sc);
+        const double2 rowk = make_double2(s_tot[2 * QR_NB + 1 + 2 * lane], s_tot[2 * QR_NB + 2 + 2 * lane]);
+        const double2 f = ctau * (rowk + csc * make_double2(s_tot[2 * lane], s_tot[2 * lane + 1]));
+        const Fx gr = fx(__double2ll_rn(-f.x * FX_ONE)), gi = fx(__double2ll_rn(-f.y * FX_ONE)),
+                 gn = fx(__double2ll_rn(f.y * FX_ONE));
+        s_g[lane] = make_int4(gr.h, gr.l, gi.h, gi.l);
+        s_gn[lane] = make_int2(gn.h, gn.l);
+      }
+    }
+    __syncthreads();
+  }
+  // back to doubles: v below the diagonal, the scaled R above it
+  for (int r = rbeg + lane % RW; r < W; r += rstep)
+#pragma unroll
+    for (int k = 0; k < HB; ++k) {
+      const int col = Q * k + q;
+      if (col >= jb) continue;
+      const longlong2 a = Zx[r + (size_t)col * ld];
+      const int e2 = r > j0 + col ? 0 : s_exp[col];
+      double2 z = make_double2(fx_to(a.x, e2), fx_to(a.y, e2));
+      if (r == j0 + col) z = make_double2(ldexp(s_beta[col], e2), 0.0);
+      if (col >= s_bad) z = make_double2(nan(""), nan(""));
+      p.Z[r + (size_t)(j0 + col) * ld] = z;
+    }
+  if (rank == 0 && tid < jb) p.T[tid] = s_tau[tid];
+  cluster.sync();   // no CTA leaves while another may still read its partial sums
 }
 
 // Trailing update Q^H C = C - V (T^H (V^H C)) for every 32-column tile of
@@ -523,6 +862,107 @@ __global__ void __maxnreg__(112) k_qr_apply_tc(const QrProb<float2>* __restrict_
   if (!all_ok && tid == 0) atomicExch(err, 1);
 }
 
+// ---- complex128 trailing update on the tensor cores (oz.cuh) -----------------------
+// Y^H = [V | C]^H V in partial sums over blocks of OZ_RB rows (one CTA per 128
+// columns from j0 on and row block), their sum with T^H applied, C -= V Y.
+
+// Partial (columns i, reflectors j): sum over the block's rows of conj(X_i) V_j, X the panel's V, then C.
+__global__ void __launch_bounds__(oz::T) k_qr_oz_ypart(const QrProb<double2>* __restrict__ P, int j0, int* err) {
+  extern __shared__ __align__(1024) unsigned char sm[];
+  const QrProb<double2> p = P[blockIdx.z];
+  const int c0 = j0 + (int)blockIdx.x * oz::TM, rbeg = j0 + (int)blockIdx.y * OZ_RB;
+  if (j0 + QR_NB >= p.n || c0 >= p.n || rbeg >= p.W) return;   // no trailing columns: no update
+  const int rend = min(p.W, rbeg + OZ_RB);
+  double2 acc[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) acc[j] = czero<double2>();
+  oz::Cta cta = oz::begin(sm);
+  for (int r0 = rbeg; r0 < rend; r0 += oz::TKC)
+    oz::stage(cta, true,
+              [&](int i, int l) {
+                const int c = c0 + i, r = r0 + l;
+                if (c >= p.n || r >= rend) return czero<double2>();
+                return conj(c < j0 + QR_NB ? v_entry(p, j0, QR_NB, r, c - j0) : p.Z[r + (size_t)c * p.ld]);
+              },
+              [&](int l, int j) { return r0 + l < rend ? v_entry(p, j0, QR_NB, r0 + l, j) : czero<double2>(); }, acc);
+  const int warp = threadIdx.x >> 5, i = 32 * (warp & 3) + (threadIdx.x & 31), cgp = 8 * (warp >> 2);
+  double2* yp = p.Yp + ((size_t)blockIdx.x * p.mrb + blockIdx.y) * (oz::TM * QR_NB);
+  if (cta.ok) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) yp[i + oz::TM * (cgp + j)] = acc[j];
+  }
+  oz::end(cta, err);
+}
+
+// Y = T^H (V^H C) for 32 columns: the partials summed in row-block order, then
+// T^{-H} x = y solved forward (T^{-1} = diag(1/tau) + the strict upper part of
+// V^H V), a warp per column and a lane per reflector.
+__global__ void __launch_bounds__(UT) k_qr_oz_yreduce(const QrProb<double2>* __restrict__ P, int j0) {
+  const QrProb<double2> p = P[blockIdx.y];
+  const int cbeg = QR_NB + 32 * (int)blockIdx.x;   // column offset from j0
+  if (j0 + cbeg >= p.n) return;
+  const int nrb = (p.W - j0 + OZ_RB - 1) / OZ_RB;
+  __shared__ double2 s_g[QR_NB][QR_NB + 1];        // G[l][j] = v_l^H v_j
+  const int tid = threadIdx.x, lane = tid & 31;
+  for (int e = tid; e < QR_NB * QR_NB; e += UT) {
+    const int l = e % QR_NB, j = e / QR_NB;
+    double2 a = czero<double2>();
+    if (l < j)
+      for (int b = 0; b < nrb; ++b) a = a + p.Yp[(size_t)b * (oz::TM * QR_NB) + l + oz::TM * j];
+    s_g[l][j] = a;
+  }
+  const double2 ctau = conj(p.T[lane]);
+  __syncthreads();
+  for (int w = tid >> 5; w < 32; w += UT / 32) {
+    const int o = cbeg + w;
+    if (j0 + o >= p.n) continue;
+    const double2* yp = p.Yp + (size_t)(o / oz::TM) * p.mrb * (oz::TM * QR_NB) + o % oz::TM + oz::TM * lane;
+    double2 x = czero<double2>();
+    for (int b = 0; b < nrb; ++b) x = x + yp[(size_t)b * (oz::TM * QR_NB)];
+    x = conj(x);
+    for (int l = 0; l < QR_NB; ++l) {
+      if (lane == l) x = ctau * x;
+      const double2 xl = make_double2(__shfl_sync(0xffffffffu, x.x, l), __shfl_sync(0xffffffffu, x.y, l));
+      if (lane > l) {
+        const double2 g = s_g[l][lane];
+        x.x = fma(-g.x, xl.x, x.x); x.x = fma(-g.y, xl.y, x.x);   // x -= conj(g) xl
+        x.y = fma(-g.x, xl.y, x.y); x.y = fma(g.y, xl.x, x.y);
+      }
+    }
+    p.V[lane + (size_t)QR_NB * (o - QR_NB)] = x;   // Y, QR_NB x trailing columns
+  }
+}
+
+__global__ void __launch_bounds__(oz::T) k_qr_oz_apply(const QrProb<double2>* __restrict__ P, int j0, int per, int* err) {
+  extern __shared__ __align__(1024) unsigned char sm[];
+  const QrProb<double2> p = P[blockIdx.z];
+  const int cfirst = j0 + QR_NB, r0 = j0 + (int)blockIdx.x * oz::TM, t0 = (int)blockIdx.y * per;
+  if (cfirst + t0 * oz::TN >= p.n || r0 >= p.W) return;
+  const int t1 = min(t0 + per, (p.n - cfirst + oz::TN - 1) / oz::TN);
+  const int warp = threadIdx.x >> 5, row = r0 + 32 * (warp & 3) + (threadIdx.x & 31), cgp = 8 * (warp >> 2);
+  oz::Cta cta = oz::begin(sm);
+  for (int t = t0; t < t1; ++t) {
+    const int c0 = t * oz::TN;   // trailing column
+    double2 acc[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[j] = czero<double2>();
+    oz::stage(cta, t == t0, [&](int i, int l) { return v_entry(p, j0, QR_NB, r0 + i, l); },
+              [&](int l, int j) {
+                return cfirst + c0 + j < p.n ? p.V[l + (size_t)QR_NB * (c0 + j)] : czero<double2>();
+              },
+              acc);
+    if (row < p.W && cta.ok) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (cfirst + c0 + cgp + j < p.n) {
+          double2* z = p.Z + row + (size_t)(cfirst + c0 + cgp + j) * p.ld;
+          *z = *z - acc[j];
+        }
+    }
+  }
+  oz::end(cta, err);
+}
+
 // Zeros below the diagonal of the top n x n block (the reflectors' storage).
 template <typename C>
 __global__ void k_qr_zero_lower(const QrProb<C>* __restrict__ P) {
@@ -536,14 +976,16 @@ __global__ void k_qr_zero_lower(const QrProb<C>* __restrict__ P) {
 }  // namespace
 
 template <typename C>
-void qr_panel(const QrProb<C>* d_prob, int nprob, int j0, cudaStream_t st) {
+void qr_panel(const QrProb<C>* d_prob, int nprob, int j0, cudaStream_t st, int cluster) {
   if (nprob <= 0) return;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   // cluster of up to 8 CTAs per matrix, enough to fill the SMs (one CTA per SM)
   int cs = 1;
-  while (cs < 8 && (long)nprob * cs * 2 <= sms) cs *= 2;
+  if (cluster > 0) cs = cluster;
+  else
+    while (cs < 8 && (long)nprob * cs * 2 <= sms) cs *= 2;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nprob * cs);
   cfg.blockDim = dim3(PT);
@@ -557,7 +999,8 @@ void qr_panel(const QrProb<C>* d_prob, int nprob, int j0, cudaStream_t st) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   KPROF_BEGIN(st);
-  cudaLaunchKernelEx(&cfg, k_qr_panel<C>, d_prob, j0);
+  if constexpr (std::is_same<C, double2>::value) cudaLaunchKernelEx(&cfg, k_qr_panel_fx, d_prob, j0);
+  else cudaLaunchKernelEx(&cfg, k_qr_panel<C>, d_prob, j0);
   pm_launch_count_add(1);
   KPROF_END(st, kname<C>("qr_panel", "qr_panel32"), 0.0);
 }
@@ -583,6 +1026,21 @@ void qr_update(const QrProb<C>* d_prob, int nprob, int j0, int max_tiles, int ma
   pm_launch_count_add(3);
   KPROF_END(st, on_tc ? "qr_update_tc32" : kname<C>("qr_update", "qr_update32"), 0.0);
 }
+void qr_update_oz(const QrProb<double2>* d_prob, int nprob, int j0, int max_n, int max_w, int* err, cudaStream_t st) {
+  const int nt = max_n - j0 - QR_NB;
+  if (nprob <= 0 || nt <= 0) return;
+  // the same value every time: idempotent across threads and devices
+  cudaFuncSetAttribute(k_qr_oz_ypart, cudaFuncAttributeMaxDynamicSharedMemorySize, oz::SMEM);
+  cudaFuncSetAttribute(k_qr_oz_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, oz::SMEM);
+  const int rbs = (max_w - j0 + OZ_RB - 1) / OZ_RB, mt = (max_w - j0 + oz::TM - 1) / oz::TM;
+  const int tiles = (nt + oz::TN - 1) / oz::TN, per = oz_per((long)mt * tiles * nprob);
+  KPROF_BEGIN(st);
+  k_qr_oz_ypart<<<dim3((max_n - j0 + oz::TM - 1) / oz::TM, rbs, nprob), oz::T, oz::SMEM, st>>>(d_prob, j0, err);
+  k_qr_oz_yreduce<<<dim3(tiles, nprob), UT, 0, st>>>(d_prob, j0);
+  k_qr_oz_apply<<<dim3(mt, (tiles + per - 1) / per, nprob), oz::T, oz::SMEM, st>>>(d_prob, j0, per, err);
+  pm_launch_count_add(3);
+  KPROF_END(st, "qr_update_oz", 0.0);
+}
 template <typename C>
 void qr_zero_lower(const QrProb<C>* d_prob, int nprob, int max_n, cudaStream_t st) {
   if (nprob <= 0 || max_n <= 0) return;
@@ -590,6 +1048,8 @@ void qr_zero_lower(const QrProb<C>* d_prob, int nprob, int max_n, cudaStream_t s
   pm_launch_count_add(1);
 }
 
-template void qr_panel<float2>(const QrProb<float2>*, int, int, cudaStream_t);
+template void qr_panel<float2>(const QrProb<float2>*, int, int, cudaStream_t, int);
+template void qr_panel<double2>(const QrProb<double2>*, int, int, cudaStream_t, int);
+template void qr_zero_lower<double2>(const QrProb<double2>*, int, int, cudaStream_t);
 template void qr_update<float2>(const QrProb<float2>*, int, int, int, int, cudaStream_t, int*, int, bool);
 template void qr_zero_lower<float2>(const QrProb<float2>*, int, int, cudaStream_t);

@@ -23,6 +23,7 @@
 #include "field.cuh"
 #include "mlp.cuh"
 #include "operator.cuh"
+#include "oz_gemm.cuh"
 #include "prof.cuh"
 
 typedef double2 Cd;
@@ -700,7 +701,36 @@ struct GemmBatch {
     for (auto& x : d) o.push_back(o.back() + gemm_tiles_shape(shape, x.m, x.n));
     return o;
   }
+  // complex128 products on the tensor cores (oz_gemm): all but those whose
+  // 128 x 32 tile would be mostly padding.  Per product, whatever the batch.
+  static bool on_tensor_cores(const GemmDesc<C>& x) { return x.m >= 32 && x.n >= 4 && x.k >= 16; }
   void run(Arena& scr, cudaStream_t st) {
+    if (std::is_same<C, double2>::value && g_oz_err) {
+      GemmBatch<C> rest;
+      std::vector<GemmDesc<double2>> t;
+      for (auto& x : d) {
+        if (on_tensor_cores(x)) t.push_back(*(const GemmDesc<double2>*)&x);
+        else { rest.d.push_back(x); rest.off.push_back(rest.off.back() + gemm_tiles(x.m, x.n)); }
+      }
+      if (!t.empty()) {
+        long tiles = 0;
+        for (auto& x : t) tiles += oz_tiles(x.m, x.n, 1);
+        const int per = oz_per(tiles);
+        std::vector<int> o{0};
+        double f = 0;
+        for (auto& x : t) { o.push_back(o.back() + oz_tiles(x.m, x.n, per)); f += 8.0 * x.m * x.n * x.k; }
+        auto* dt = upload(scr, t, st);
+        int* dof = upload(scr, o, st);
+        oz_gemm_batched(dt, dof, (int)t.size(), o.back(), per, g_oz_err, st);
+        if (g_kprof) g_kprof->add_flops("gemm_oz", f);
+        CK(cudaGetLastError());
+        rest.run_cuda_cores(scr, st);
+        return;
+      }
+    }
+    run_cuda_cores(scr, st);
+  }
+  void run_cuda_cores(Arena& scr, cudaStream_t st) {
     if (d.empty()) return;
     auto* dd = upload(scr, d, st);
     int dev = 0;
@@ -1018,6 +1048,12 @@ void sqnorm_batch(const std::vector<SqNormProb>& probs, Arena& scr, cudaStream_t
   CK(cudaGetLastError());
 }
 
+// complex128 ID inputs with at least this many candidates (and twice as many
+// rows) are reduced to their triangle first; a panel runs on a cluster of 8
+// CTAs above this many rows, else of 4.
+constexpr int QR_FIRST_MIN_N64 = 80;
+constexpr int QR_CLUSTER8_W64 = 2048;
+
 // Held-out proxy check bound: an ID passes while ||H_J - H_S T|| <= PROXY_CHECK_BOUND tol ||H||.
 constexpr double PROXY_CHECK_BOUND = 200.0;
 
@@ -1274,6 +1310,44 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
   // 3a. complex64: tall inputs reduced to their triangular factor first, so
   // that the pivoted steps stream n instead of W rows
   std::vector<int> We(W);   // rows the pivoted QR runs on (leading dimension stays W)
+  if constexpr (std::is_same<C, double2>::value) {
+    // complex128: the same reduction with the trailing updates on the tensor
+    // cores (FP64-accurate products).  Each rule looks at one matrix alone, so
+    // that a problem's bits do not depend on what shares its launches.
+    if (!(O.flags & PM_FLAG_NO_QR_FIRST) && g_oz_err) {
+      std::vector<QrProb<C>> qp[2];   // panels on 4 CTAs, on 8
+      int maxn = 0;
+      double fl = 0;
+      for (int i = 0; i < nid; ++i)
+        if (nn[i] >= QR_FIRST_MIN_N64 && W[i] >= 2 * nn[i]) {
+          const int mrb = (W[i] + OZ_RB - 1) / OZ_RB;
+          C* tau = scr.get<C>(QR_NB);
+          C* y = scr.get<C>((size_t)QR_NB * nn[i]);
+          C* yp = scr.get<C>((size_t)((nn[i] + 127) / 128) * mrb * 128 * QR_NB);
+          qp[W[i] > QR_CLUSTER8_W64].push_back(QrProb<C>{Z[i], W[i], W[i], nn[i], tau, y, yp, mrb});
+          We[i] = nn[i];
+          maxn = std::max(maxn, nn[i]);
+          for (int j0 = 0; j0 + QR_NB < nn[i]; j0 += QR_NB)
+            fl += 16.0 * (double)(W[i] - j0) * QR_NB * (nn[i] - j0 - QR_NB);
+        }
+      const int n4 = (int)qp[0].size();
+      std::vector<QrProb<C>> all(qp[0]);
+      all.insert(all.end(), qp[1].begin(), qp[1].end());
+      if (!all.empty()) {
+        int maxW = 0;
+        for (auto& x : all) maxW = std::max(maxW, x.W);
+        auto* dqp = upload(scr, all, st);
+        for (int j0 = 0; j0 < maxn; j0 += QR_NB) {
+          qr_panel<C>(dqp, n4, j0, st, 4);
+          qr_panel<C>(dqp + n4, (int)all.size() - n4, j0, st, 8);
+          qr_update_oz(dqp, (int)all.size(), j0, maxn, maxW, g_oz_err, st);
+        }
+        qr_zero_lower<C>(dqp, (int)all.size(), maxn, st);
+        CK(cudaGetLastError());
+        if (g_kprof) g_kprof->add_flops("qr_update_oz", fl);
+      }
+    }
+  }
   if constexpr (std::is_same<C, float2>::value) {
     if (!(O.flags & PM_FLAG_NO_QR_FIRST)) {
       std::vector<QrProb<C>> qp;
@@ -2493,8 +2567,14 @@ void factor_group_t(std::vector<pm_factor*>& Fs, double id_tol, Arena& scr, cuda
 
 void factor_group(std::vector<pm_factor*>& Fs, double id_tol, Arena& scr, cudaStream_t st) {
   if (Fs.empty()) return;
+  int* err = Fs[0]->d_wait_err;
+  OzErrScope oz(err);
   if (Fs[0]->precision == PM_FP64) factor_group_t<double2>(Fs, id_tol, scr, st);
   else factor_group_t<float2>(Fs, id_tol, scr, st);
+  int werr = 0;
+  CK(cudaMemcpyAsync(&werr, err, sizeof(int), cudaMemcpyDeviceToHost, st));
+  CK(cudaStreamSynchronize(st));
+  if (werr) fail(PM_ERR_TIMEOUT, "a wait on the tensor cores ran out");
 }
 
 // Mixed mode, after the complex64 levels: the FP64 self blocks, index maps and
@@ -2797,6 +2877,7 @@ pm_status solve_impl(const pm_factor* Fc, const pm_c64* rhs, int32_t nrhs, pm_c6
       ~ProfScope() { g_kprof = nullptr; }
     } scope(F->profiling ? &F->prof : nullptr);
     std::lock_guard<std::mutex> plan_lock(F->plan_mu);   // solves of one factor share its graphs
+    OzErrScope oz(F->d_wait_err);
     if (F->precision == PM_FP64 && F->opts.formulation >= PM_FORM_BM) {
       // Burton-Miller: its own right-hand side, then its [u; q] unknowns reordered
       const pm_geometry* g = F->g;
@@ -2824,7 +2905,7 @@ pm_status solve_impl(const pm_factor* Fc, const pm_c64* rhs, int32_t nrhs, pm_c6
     if (werr) {
       CK(cudaMemsetAsync(F->d_wait_err, 0, sizeof(int), st));
       CK(cudaStreamSynchronize(st));
-      fail(PM_ERR_TIMEOUT, "a bounded wait of the chained top-level solve ran out");
+      fail(PM_ERR_TIMEOUT, "a bounded wait of the solve (chained triangles, tensor cores) ran out");
     }
   });
 }
