@@ -16,7 +16,7 @@ namespace {
 
 constexpr int TB = 32;   // output tile
 constexpr int TK = 16;   // k step
-constexpr int MAXNB = 16;   // panel width bound of the LU kernels
+constexpr int MAXNB = 32;   // panel width of the LU kernels
 
 // One 32 x 32 output tile of  Cm = alpha * A * B + beta * Cm  (256 threads).
 // SUB: the caller's alpha = -1 and beta = 1, applied as Cm - A * B (the same
@@ -175,366 +175,200 @@ __device__ __forceinline__ float2 shfl_c(float2 v, int src) {
   return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
 }
 
-// Panel: columns [p, p+jb) of rows [p, m), one CTA per matrix, left-looking
-// (Crout): column c is brought up to date only when it is reached, from the
-// final L entries of the panel's earlier columns, so every entry is stored
-// once per column step and the update is fused with the pivot search.
-// Pivot = the largest |a|^2 in the column, lowest row index on ties (the
-// same choice as the right-looking order, up to rounding).
-template <typename C, int NT>
-__global__ void __launch_bounds__(NT) k_lu_panel(const LuProb<C>* __restrict__ P, int p, int nb) {
+// Panel: columns [p, p + jb) of rows [p, m) on a cluster of CTAs per matrix,
+// right-looking.  One FP64 pipe does 2 fused multiply-adds per clock, so a
+// panel on one SM is bound by it however small the matrix (512 rows: 15 us a
+// column); over 8 SMs the update of a column shrinks to the cost of its
+// barriers.  The rows go to the CTAs in cyclic chunks of 32 and stay there, in
+// shared memory when they fit (SM), else in place.  Per column: every CTA
+// proposes its largest |a|^2 (lowest row on ties) and a copy of that row, rank
+// 0, which owns the diagonal rows, a copy of the diagonal row; one cluster
+// barrier; every CTA reads the proposals, takes the winner's row as the row of
+// U, and the two owners swap; then l = a / pivot and a -= l u on each CTA's
+// rows.  An entry's operations do not depend on the number of CTAs, so neither
+// do the bits.  The comparisons run on the integer pipe (non-negative floats
+// order like their bit patterns).
+constexpr int LP_T = 256;
+template <typename C, bool SM>
+__global__ void __maxnreg__(128) k_lu_panel(const LuProb<C>* __restrict__ P, int p, int ldp) {
   typedef typename real_of<C>::type R;
-  const LuProb<C> pr = P[blockIdx.x];
-  const int m = pr.m;
-  if (p >= m) return;
-  const int jb = min(nb, m - p);
-  C* A = pr.A;
-  const size_t ld = pr.ld;
-  __shared__ R sval[NT / 32];
-  __shared__ int sidx[NT / 32];
-  __shared__ C s_l[MAXNB][MAXNB + 1];
-  __shared__ C s_u[MAXNB];
-  __shared__ int s_piv;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int jj = 0; jj < jb; ++jj) {
-    const int c = p + jj;
-    C* colc = A + (size_t)c * ld;
-    if (jj > 0) {
-      // U[0:jj, jj] = L11^{-1} A[p:c, c] (unit lower L11 of the current rows)
-      for (int e = tid; e < jj * jj; e += NT) s_l[e % jj][e / jj] = A[p + e % jj + (size_t)(p + e / jj) * ld];
-      __syncthreads();
-      if (warp == 0) {
-        C x = lane < jj ? colc[p + lane] : czero<C>();
-        for (int l = 0; l < jj - 1; ++l) {
-          const C xl = shfl_c(x, l);
-          if (lane > l && lane < jj) cfms(x, s_l[lane][l], xl);
-        }
-        if (lane < jj) {
-          s_u[lane] = x;
-          colc[p + lane] = x;
-        }
-      }
-      __syncthreads();
-    }
-    // rows c..m-1: a -= L[r, p:c] u, then the pivot search on the result
-    R best = -1;
-    int bi = m;
-    for (int r = c + tid; r < m; r += NT) {
-      C lr[MAXNB];   // the row's L entries, loaded together
-#pragma unroll
-      for (int l = 0; l < MAXNB; ++l) if (l < jj) lr[l] = A[r + (size_t)(p + l) * ld];
-      // four partial sums: short dependent chains (FP64 latency)
-      C a0 = colc[r], a1 = czero<C>(), a2 = czero<C>(), a3 = czero<C>();
-#pragma unroll
-      for (int l = 0; l < MAXNB; l += 4) {
-        if (l < jj) cfms(a0, lr[l], s_u[l]);
-        if (l + 1 < jj) cfms(a1, lr[l + 1], s_u[l + 1]);
-        if (l + 2 < jj) cfms(a2, lr[l + 2], s_u[l + 2]);
-        if (l + 3 < jj) cfms(a3, lr[l + 3], s_u[l + 3]);
-      }
-      const C a = (a0 + a1) + (a2 + a3);
-      if (jj > 0) colc[r] = a;
-      const R v = abs2(a);
-      if (v > best) { best = v; bi = r; }   // rows ascend: the first of equal values stays
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      const R v2 = __shfl_xor_sync(0xffffffffu, best, o);
-      const int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (v2 > best || (v2 == best && i2 < bi)) { best = v2; bi = i2; }
-    }
-    if (lane == 0) { sval[warp] = best; sidx[warp] = bi; }
-    __syncthreads();
-    if (tid == 0) {
-      R bv = sval[0];
-      int piv = sidx[0];
-      for (int w = 1; w < NT / 32; ++w)
-        if (sval[w] > bv || (sval[w] == bv && sidx[w] < piv)) { bv = sval[w]; piv = sidx[w]; }
-      if (!(bv > 0)) { piv = c; if (*pr.info == 0) *pr.info = c + 1; }
-      s_piv = piv;
-      pr.ipiv[c] = piv;
-    }
-    __syncthreads();
-    const int piv = s_piv;
-    if (piv != c && tid < jb) {
-      C* a = A + c + (size_t)(p + tid) * ld;
-      C* b = A + piv + (size_t)(p + tid) * ld;
-      const C t = *a; *a = *b; *b = t;
-    }
-    __syncthreads();
-    const C d = colc[c];
-    if (abs2(d) > 0) {
-      const C inv = cdiv(mk((R)1, (R)0), d);
-      int r = c + 1 + tid;
-      for (; r + NT < m; r += 2 * NT) {   // two rows per pass: both loads in flight
-        const C a0 = colc[r], a1 = colc[r + NT];
-        colc[r] = a0 * inv;
-        colc[r + NT] = a1 * inv;
-      }
-      if (r < m) colc[r] = colc[r] * inv;
-    }
-    __syncthreads();
-  }
-}
-
-// The same panel with its rows p..m-1 held in shared memory for the whole
-// panel (dynamic, (m - p) x jb, leading dimension m - p): loaded once,
-// factored there (the lazy updates read the L entries from shared memory
-// instead of L2), stored once; the same operations in the same order as
-// k_lu_panel, so the same bits.
-template <typename C, int NT>
-__global__ void __launch_bounds__(NT) k_lu_panel_smem(const LuProb<C>* __restrict__ P, int p, int nb) {
-  typedef typename real_of<C>::type R;
-  extern __shared__ __align__(16) unsigned char lu_sm[];
-  C* pan = reinterpret_cast<C*>(lu_sm);
-  const LuProb<C> pr = P[blockIdx.x];
-  const int m = pr.m;
-  if (p >= m) return;
-  const int jb = min(nb, m - p);
-  const int mr = m - p;
-  C* A = pr.A;
-  const size_t ld = pr.ld;
-  __shared__ R sval[NT / 32];
-  __shared__ int sidx[NT / 32];
-  __shared__ C s_l[MAXNB][MAXNB + 1];
-  __shared__ C s_u[MAXNB];
-  __shared__ int s_piv;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int e = tid; e < mr * jb; e += NT) pan[e] = A[p + e % mr + (size_t)(p + e / mr) * ld];
-  __syncthreads();
-  for (int jj = 0; jj < jb; ++jj) {
-    C* colc = pan + (size_t)jj * mr;   // local row i = global row p + i
-    if (jj > 0) {
-      for (int e = tid; e < jj * jj; e += NT) s_l[e % jj][e / jj] = pan[e % jj + (size_t)(e / jj) * mr];
-      __syncthreads();
-      if (warp == 0) {
-        C x = lane < jj ? colc[lane] : czero<C>();
-        for (int l = 0; l < jj - 1; ++l) {
-          const C xl = shfl_c(x, l);
-          if (lane > l && lane < jj) cfms(x, s_l[lane][l], xl);
-        }
-        if (lane < jj) {
-          s_u[lane] = x;
-          colc[lane] = x;
-        }
-      }
-      __syncthreads();
-    }
-    R best = -1;
-    int bi = m;
-    for (int r = jj + tid; r < mr; r += NT) {
-      C lr[MAXNB];
-#pragma unroll
-      for (int l = 0; l < MAXNB; ++l) if (l < jj) lr[l] = pan[r + (size_t)l * mr];
-      C a0 = colc[r], a1 = czero<C>(), a2 = czero<C>(), a3 = czero<C>();
-#pragma unroll
-      for (int l = 0; l < MAXNB; l += 4) {
-        if (l < jj) cfms(a0, lr[l], s_u[l]);
-        if (l + 1 < jj) cfms(a1, lr[l + 1], s_u[l + 1]);
-        if (l + 2 < jj) cfms(a2, lr[l + 2], s_u[l + 2]);
-        if (l + 3 < jj) cfms(a3, lr[l + 3], s_u[l + 3]);
-      }
-      const C a = (a0 + a1) + (a2 + a3);
-      if (jj > 0) colc[r] = a;
-      const R v = abs2(a);
-      if (v > best) { best = v; bi = p + r; }   // rows ascend: the first of equal values stays
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      const R v2 = __shfl_xor_sync(0xffffffffu, best, o);
-      const int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (v2 > best || (v2 == best && i2 < bi)) { best = v2; bi = i2; }
-    }
-    if (lane == 0) { sval[warp] = best; sidx[warp] = bi; }
-    __syncthreads();
-    const int c = p + jj;
-    if (tid == 0) {
-      R bv = sval[0];
-      int piv = sidx[0];
-      for (int w = 1; w < NT / 32; ++w)
-        if (sval[w] > bv || (sval[w] == bv && sidx[w] < piv)) { bv = sval[w]; piv = sidx[w]; }
-      if (!(bv > 0)) { piv = c; if (*pr.info == 0) *pr.info = c + 1; }
-      s_piv = piv;
-      pr.ipiv[c] = piv;
-    }
-    __syncthreads();
-    const int piv = s_piv - p;
-    if (piv != jj && tid < jb) {
-      C* a = pan + jj + (size_t)tid * mr;
-      C* b = pan + piv + (size_t)tid * mr;
-      const C t = *a; *a = *b; *b = t;
-    }
-    __syncthreads();
-    const C d = colc[jj];
-    if (abs2(d) > 0) {
-      const C inv = cdiv(mk((R)1, (R)0), d);
-      for (int r = jj + 1 + tid; r < mr; r += NT) colc[r] = colc[r] * inv;
-    }
-    __syncthreads();
-  }
-  for (int e = tid; e < mr * jb; e += NT) A[p + e % mr + (size_t)(p + e / mr) * ld] = pan[e];
-}
-
-// The same left-looking panel for one large matrix on a cluster of CTAs
-// (the top-level LU): the CTAs split the rows, so the lazy column updates
-// (FP64-bound on one SM) spread over the cluster's SMs.  Per column: every
-// CTA solves the small triangular system for U[0:jj] itself, updates its
-// rows and proposes a pivot; the proposals meet through distributed shared
-// memory (largest |a|^2, lowest row on ties, as in k_lu_panel); rank 0 swaps
-// the two rows; every CTA scales its rows.  Two cluster barriers per column
-// order these steps: a row's scaled L entry is next read by the thread that
-// wrote it (rows keep their thread from column to column), and the next
-// column's triangular solve reads only rows at or above the diagonal.
-template <typename C, int NT>
-__global__ void __launch_bounds__(NT) k_lu_panel_cluster(const LuProb<C>* __restrict__ P, int p, int nb) {
-  typedef typename real_of<C>::type R;
+  typedef unsigned long long u64;
   namespace cg = cooperative_groups;
+  constexpr int NW = LP_T / 32;
+  extern __shared__ __align__(16) unsigned char lu_sm[];
   cg::cluster_group cluster = cg::this_cluster();
-  const int csize = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
-  const LuProb<C> pr = P[blockIdx.x / csize];
+  const int cs = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const LuProb<C> pr = P[blockIdx.x / cs];
   const int m = pr.m;
   if (p >= m) return;   // the whole cluster leaves
-  const int jb = min(nb, m - p);
-  C* A = pr.A;
-  const size_t ld = pr.ld;
-  __shared__ R sval[NT / 32];
-  __shared__ int sidx[NT / 32];
-  __shared__ R c_val;   // this CTA's proposal, read by the cluster
-  __shared__ int c_idx;
-  __shared__ C s_l[MAXNB][MAXNB + 1];
-  __shared__ C s_u[MAXNB];
-  __shared__ int s_piv;
+  const int jb = min(MAXNB, m - p), mr = m - p;
+  C* pan = SM ? reinterpret_cast<C*>(lu_sm) : pr.A + p + (size_t)p * pr.ld;
+  const size_t ld = SM ? ldp : pr.ld;
+  __shared__ C s_slot[2][MAXNB], s_crow[2][MAXNB];   // by column parity: this CTA's proposal, the diagonal row
+  __shared__ u64 s_key[2];
+  __shared__ unsigned s_krow[2];
+  __shared__ u64 s_wk[NW];
+  __shared__ unsigned s_wr[NW];
+  __shared__ C s_u[MAXNB], s_inv;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int stride = NT * csize;
+  const int nch = ((mr + 31) / 32 - rank + cs - 1) / cs;   // this CTA's chunks of 32 rows
+  // chunk ch, lane i: row offset g from p, stored row
+  auto row_g = [&](int ch) { return (ch * cs + rank) * 32 + lane; };
+  auto row_s = [&](int ch) { return SM ? ch * 32 + lane : row_g(ch); };
+  // few chunks: several warps share one, each with its residue of the columns
+  const int q_n = nch <= 1 ? 8 : nch <= 2 ? 4 : nch <= 4 ? 2 : 1, slots = NW / q_n;
+  const int slot = warp % slots, q = warp / slots;
+  if (SM)
+    for (int ch = warp; ch < nch; ch += NW)
+      if (row_g(ch) < mr)
+        for (int k = 0; k < jb; ++k) pan[row_s(ch) + k * ld] = pr.A[p + row_g(ch) + (size_t)(p + k) * pr.ld];
+  __syncthreads();
+  u64 key = 0;
+  unsigned krow = 0xFFFFFFFFu;
+  auto propose = [&](C a, int g) {
+    const R v = abs2(a);
+    u64 k;
+    if (sizeof(R) == 8) k = (u64)__double_as_longlong((double)v); else k = (u64)__float_as_uint((float)v);
+    if (k > (sizeof(R) == 8 ? 0x7FF0000000000000ull : 0x7F800000ull)) k = 0;   // NaN
+    if (k > key || (k == key && (unsigned)g < krow)) { key = k; krow = (unsigned)g; }
+  };
+  for (int ch = warp; ch < nch; ch += NW)
+    if (row_g(ch) < mr) propose(pan[row_s(ch)], row_g(ch));
+  auto pick = [&](u64& k, unsigned& r) {   // the largest key of the warp, the lowest row among equals
+    const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(k >> 32));
+    const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(k >> 32) == hi ? (unsigned)k : 0u);
+    const u64 best = ((u64)hi << 32) | lo;
+    r = __reduce_min_sync(0xffffffffu, k == best ? r : 0xFFFFFFFFu);
+    k = best;
+  };
   for (int jj = 0; jj < jb; ++jj) {
-    const int c = p + jj;
-    C* colc = A + (size_t)c * ld;
-    if (jj > 0) {
-      for (int e = tid; e < jj * jj; e += NT) s_l[e % jj][e / jj] = A[p + e % jj + (size_t)(p + e / jj) * ld];
-      __syncthreads();
-      if (warp == 0) {
-        C x = lane < jj ? colc[p + lane] : czero<C>();
-        for (int l = 0; l < jj - 1; ++l) {
-          const C xl = shfl_c(x, l);
-          if (lane > l && lane < jj) cfms(x, s_l[lane][l], xl);
-        }
-        if (lane < jj) s_u[lane] = x;
-      }
-      __syncthreads();
-    }
-    R best = -1;
-    int bi = m;
-    for (int r = c + rank * NT + tid; r < m; r += stride) {
-      C lr[MAXNB];
-#pragma unroll
-      for (int l = 0; l < MAXNB; ++l) if (l < jj) lr[l] = A[r + (size_t)(p + l) * ld];
-      C a0 = colc[r], a1 = czero<C>(), a2 = czero<C>(), a3 = czero<C>();
-#pragma unroll
-      for (int l = 0; l < MAXNB; l += 4) {
-        if (l < jj) cfms(a0, lr[l], s_u[l]);
-        if (l + 1 < jj) cfms(a1, lr[l + 1], s_u[l + 1]);
-        if (l + 2 < jj) cfms(a2, lr[l + 2], s_u[l + 2]);
-        if (l + 3 < jj) cfms(a3, lr[l + 3], s_u[l + 3]);
-      }
-      const C a = (a0 + a1) + (a2 + a3);
-      if (jj > 0) colc[r] = a;
-      const R v = abs2(a);
-      if (v > best || (v == best && r < bi)) { best = v; bi = r; }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      const R v2 = __shfl_xor_sync(0xffffffffu, best, o);
-      const int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (v2 > best || (v2 == best && i2 < bi)) { best = v2; bi = i2; }
-    }
-    if (lane == 0) { sval[warp] = best; sidx[warp] = bi; }
+    const int par = jj & 1;
+    pick(key, krow);
+    if (lane == 0) { s_wk[warp] = key; s_wr[warp] = krow; }
     __syncthreads();
-    if (tid == 0) {
-      R bv = sval[0];
-      int bix = sidx[0];
-      for (int w = 1; w < NT / 32; ++w)
-        if (sval[w] > bv || (sval[w] == bv && sidx[w] < bix)) { bv = sval[w]; bix = sidx[w]; }
-      c_val = bv;
-      c_idx = bix;
+    u64 ck = lane < NW ? s_wk[lane] : 0;
+    unsigned cr = lane < NW ? s_wr[lane] : 0xFFFFFFFFu;
+    pick(ck, cr);
+    if (warp == 0 && ck > 0 && lane < jb) {
+      const int g = (int)cr, ch = (g / 32 - rank) / cs;
+      s_slot[par][lane] = pan[(SM ? ch * 32 + g % 32 : g) + lane * ld];
     }
-    cluster.sync();   // proposals and updated column entries are visible
-    if (tid == 0) {
-      R bv = -1;
-      int piv = m;
-      for (int q = 0; q < csize; ++q) {
-        const R v = *cluster.map_shared_rank(&c_val, q);
-        const int i = *cluster.map_shared_rank(&c_idx, q);
-        if (v > bv || (v == bv && i < piv)) { bv = v; piv = i; }
+    if (warp == 1 && rank == 0 && lane < jb) s_crow[par][lane] = pan[jj + lane * ld];
+    if (tid == 64) { s_key[par] = ck; s_krow[par] = cr; }
+    cluster.sync();   // the proposals are visible
+    u64 wk = lane < cs ? *cluster.map_shared_rank(&s_key[par], lane) : 0;
+    unsigned wr = lane < cs ? *cluster.map_shared_rank(&s_krow[par], lane) : 0xFFFFFFFFu;
+    pick(wk, wr);
+    const int piv = wk > 0 ? (int)wr : jj;                   // offset from p
+    const int owner = (piv / 32) % cs;
+    const C* urow = wk > 0 ? cluster.map_shared_rank(&s_slot[par][0], owner) : cluster.map_shared_rank(&s_crow[par][0], 0);
+    if (warp == 0) {
+      if (lane < jb) s_u[lane] = urow[lane];
+    } else if (warp == 1) {
+      const C d = urow[jj];
+      const R d2 = abs2(d), ri = d2 > 0 ? (R)1 / d2 : (R)0;
+      if (lane == 0) s_inv = mk(d.x * ri, -d.y * ri);
+    } else if (warp == 2) {
+      if (piv != jj && rank == owner && lane < jb) {
+        const int ch = (piv / 32 - rank) / cs;
+        pan[(SM ? ch * 32 + piv % 32 : piv) + lane * ld] = cluster.map_shared_rank(&s_crow[par][0], 0)[lane];
       }
-      if (!(bv > 0)) { piv = c; if (rank == 0 && *pr.info == 0) *pr.info = c + 1; }
-      s_piv = piv;
-      if (rank == 0) pr.ipiv[c] = piv;
+    } else if (warp == 3) {
+      if (piv != jj && rank == 0 && lane < jb) pan[jj + lane * ld] = urow[lane];
+      if (rank == 0 && lane == 0) {
+        pr.ipiv[p + jj] = p + piv;
+        if (wk == 0 && *pr.info == 0) *pr.info = p + jj + 1;
+      }
     }
     __syncthreads();
-    const int piv = s_piv;
-    if (rank == 0) {
-      if (jj > 0 && tid < jj) colc[p + tid] = s_u[tid];   // U entries of this column
-      if (piv != c && tid < jb) {
-        C* a = A + c + (size_t)(p + tid) * ld;
-        C* b = A + piv + (size_t)(p + tid) * ld;
-        const C t = *a; *a = *b; *b = t;
-      }
-    }
-    cluster.sync();   // the swap is visible; every CTA has read its proposal slots
-    const C d = colc[c];
-    if (abs2(d) > 0) {
-      const C inv = cdiv(mk((R)1, (R)0), d);
-      for (int r = c + 1 + rank * NT + tid; r < m; r += stride) colc[r] = colc[r] * inv;
+    const C inv = s_inv;
+    for (int ch = warp; ch < nch; ch += NW) {
+      const int g = row_g(ch);
+      if (g > jj && g < mr) pan[row_s(ch) + jj * ld] = pan[row_s(ch) + jj * ld] * inv;
     }
     __syncthreads();
+    key = 0;
+    krow = 0xFFFFFFFFu;
+    for (int ch = slot; ch < nch; ch += slots) {
+      const int g = row_g(ch);
+      if (g <= jj || g >= mr) continue;
+      C* row = pan + row_s(ch);
+      const C l = row[jj * ld];
+      int k = jj + 1 + (q - (jj + 1) % q_n + q_n) % q_n;   // the first column after jj of this residue
+      if (k == jj + 1 && k < jb) {
+        C a = row[k * ld];
+        cfms(a, l, s_u[k]);
+        row[k * ld] = a;
+        propose(a, g);
+        k += q_n;
+      }
+      for (; k + 3 * q_n < jb; k += 4 * q_n) {   // four columns in flight
+        C a0 = row[k * ld], a1 = row[(k + q_n) * ld], a2 = row[(k + 2 * q_n) * ld], a3 = row[(k + 3 * q_n) * ld];
+        cfms(a0, l, s_u[k]); cfms(a1, l, s_u[k + q_n]); cfms(a2, l, s_u[k + 2 * q_n]); cfms(a3, l, s_u[k + 3 * q_n]);
+        row[k * ld] = a0; row[(k + q_n) * ld] = a1; row[(k + 2 * q_n) * ld] = a2; row[(k + 3 * q_n) * ld] = a3;
+      }
+      for (; k < jb; k += q_n) {
+        C a = row[k * ld];
+        cfms(a, l, s_u[k]);
+        row[k * ld] = a;
+      }
+    }
   }
-  cluster.sync();   // no CTA leaves while another may still read its proposal slots
+  __syncthreads();
+  if (SM)
+    for (int ch = warp; ch < nch; ch += NW)
+      if (row_g(ch) < mr)
+        for (int k = 0; k < jb; ++k) pr.A[p + row_g(ch) + (size_t)(p + k) * pr.ld] = pan[row_s(ch) + k * ld];
+  cluster.sync();   // no CTA leaves while another may still read its proposal
 }
 
 // Row interchanges of the panel applied to every other column, then the unit
 // lower triangular solve U12 = L11^{-1} A12 on the columns right of the panel.
-// Thread 0 of each CTA composes the panel's jb interchanges into one map over
-// the rows they touch (the jb panel rows first, then at most jb rows below).
-// One warp per column: lane i gathers the column's entry for position i (the
-// panel rows are contiguous, so the first half of the warp reads one
-// coalesced segment), the swapped-in rows below are written back, and the
-// triangular solve runs across the lanes, each lane's row taking its
-// subtractions in the same (ascending) order as a row-by-row substitution.
+// A warp per column.  The warp composes the panel's jb interchanges into a map
+// over the rows they touch: lane i holds the panel row p + i and the i-th of
+// the at most jb rows below the panel (row, and whose entry comes there).  The
+// column's entries are gathered through it (the panel rows are contiguous:
+// coalesced), the rows below written back, and the solve runs across the
+// lanes, each lane's row taking its subtractions in ascending order.
 template <typename C>
-__global__ void __launch_bounds__(256) k_lu_swap_trsm(const LuProb<C>* __restrict__ P, int p, int nb) {
-  constexpr int MB = MAXNB;
-  static_assert(2 * MB <= 32, "one lane per touched row");
+__global__ void __launch_bounds__(256) k_lu_swap_trsm(const LuProb<C>* __restrict__ P, int p) {
+  static_assert(MAXNB == 32, "a lane per panel row");
   const LuProb<C> pr = P[blockIdx.y];
   const int m = pr.m;
   if (p >= m) return;
-  const int jb = min(nb, m - p);
-  __shared__ int s_row[2 * MB], s_org[2 * MB];
-  __shared__ int s_cnt;
-  __shared__ C s_l[MB][MB + 1];
+  const int jb = min(MAXNB, m - p);
+  __shared__ C s_l[MAXNB][MAXNB + 1];
   C* A = pr.A;
   const size_t ld = pr.ld;
-  if (threadIdx.x == 0) {
-    int cnt = jb;
-    for (int i = 0; i < jb; ++i) { s_row[i] = p + i; s_org[i] = p + i; }
-    for (int c = 0; c < jb; ++c) {
-      const int r = pr.ipiv[p + c];
-      int ir = r - p;
-      if (ir >= jb) {
-        ir = -1;
-        for (int i = jb; i < cnt; ++i) if (s_row[i] == r) ir = i;
-        if (ir < 0) { ir = cnt++; s_row[ir] = r; s_org[ir] = r; }
-      }
-      const int t = s_org[c]; s_org[c] = s_org[ir]; s_org[ir] = t;
-    }
-    s_cnt = cnt;
-  }
-  for (int e = threadIdx.x; e < jb * jb; e += blockDim.x) s_l[e % jb][e / jb] = A[p + e % jb + (size_t)(p + e / jb) * ld];
-  __syncthreads();
   const int lane = threadIdx.x & 31;
-  const int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int j0 = blockIdx.x * (blockDim.x >> 5);
+  if (j0 + (int)(blockDim.x >> 5) > p + jb)   // some column right of the panel
+    for (int e = threadIdx.x; e < jb * jb; e += blockDim.x) s_l[e % jb][e / jb] = A[p + e % jb + (size_t)(p + e / jb) * ld];
+  __syncthreads();
+  const int j = j0 + (threadIdx.x >> 5);
   if (j >= m || (j >= p && j < p + jb)) return;   // whole warps leave together
+  const int piv = lane < jb ? pr.ipiv[p + lane] : 0;
+  int org = p + lane, row = -1, orow = -1, cnt = 0;
+  for (int c = 0; c < jb; ++c) {
+    const int r = __shfl_sync(0xffffffffu, piv, c), oc = __shfl_sync(0xffffffffu, org, c);
+    if (r < p + jb) {
+      const int o = __shfl_sync(0xffffffffu, org, r - p);
+      if (lane == r - p) org = oc;
+      if (lane == c) org = o;
+    } else {
+      const unsigned hit = __ballot_sync(0xffffffffu, row == r);
+      const int s = hit ? __ffs(hit) - 1 : cnt++;
+      if (!hit && lane == s) { row = r; orow = r; }
+      const int o = __shfl_sync(0xffffffffu, orow, s);
+      if (lane == s) orow = oc;
+      if (lane == c) org = o;
+    }
+  }
   C* col = A + (size_t)j * ld;
-  const int cnt = s_cnt;
-  C v = lane < cnt ? col[s_org[lane]] : czero<C>();
+  C v = lane < jb ? col[org] : czero<C>();
+  const C below = lane < cnt ? col[orow] : czero<C>();
   __syncwarp();                                    // every read before any write
-  if (lane >= jb && lane < cnt) col[s_row[lane]] = v;   // rows below the panel
+  if (lane < cnt) col[row] = below;
   if (j >= p + jb) {
     for (int q = 0; q < jb - 1; ++q) {
       const C vq = shfl_c(v, q);
@@ -671,38 +505,6 @@ __global__ void __launch_bounds__(256) k_getrs_update(const SolveProb<C>* __rest
                mk((R)-1, (R)0), mk((R)1, (R)0), 0, t % tiles_m, t / tiles_m);
 }
 
-// The same update for at most 8 right-hand sides: one thread per (row,
-// right-hand side), the block's B rows staged in shared memory (the 32 x 32
-// tile of the general kernel would spend 3/4 of its FP64 work on padding).
-constexpr int TH_ROWS = 16;
-template <typename C>
-__global__ void __launch_bounds__(128) k_getrs_update_thin(const SolveProb<C>* __restrict__ P, int p, int nb, int lower) {
-  __shared__ C sb[32][8];
-  const SolveProb<C> pr = P[blockIdx.y];
-  if (p >= pr.m) return;
-  const int jb = min(nb, pr.m - p);
-  const int r0 = lower ? p + jb : 0;
-  const int mt = lower ? pr.m - p - jb : p;
-  if (mt <= 0 || blockIdx.x * TH_ROWS >= mt) return;
-  for (int e = threadIdx.x; e < jb * pr.nrhs; e += blockDim.x) {
-    const int l = e % jb, q = e / jb;
-    sb[l][q] = pr.B[p + l + (size_t)q * pr.ldb];
-  }
-  __syncthreads();
-  const int i = blockIdx.x * TH_ROWS + (threadIdx.x & (TH_ROWS - 1)), q = threadIdx.x / TH_ROWS;
-  if (i >= mt || q >= pr.nrhs) return;
-  const C* a = pr.A + r0 + i + (size_t)p * pr.ld;
-  C acc0 = czero<C>(), acc1 = czero<C>();   // two chains (FP64 latency)
-  int l = 0;
-  for (; l + 1 < jb; l += 2) {
-    cfma(acc0, a[(size_t)l * pr.ld], sb[l][q]);
-    cfma(acc1, a[(size_t)(l + 1) * pr.ld], sb[l + 1][q]);
-  }
-  if (l < jb) cfma(acc0, a[(size_t)l * pr.ld], sb[l][q]);
-  C* out = pr.B + r0 + i + (size_t)q * pr.ldb;
-  *out = *out - (acc0 + acc1);
-}
-
 // One triangle of the LU solves of a batch of matrices, each with at most 8
 // right-hand sides, as ONE launch: every matrix is a chain of RS_NB-row
 // blocks, one CTA per block and group of rg right-hand sides (the columns
@@ -714,13 +516,12 @@ __global__ void __launch_bounds__(128) k_getrs_update_thin(const SolveProb<C>* _
 // from the top, upper: by distance from the bottom), hence a CTA only ever
 // waits on CTAs that took a smaller ticket and are already running: no
 // co-residency is assumed.  A CTA subtracts the products of the blocks it
-// depends on in the same order and with the same two-chain sums as
-// k_getrs_update_thin, each as soon as that block's flag is up, then solves
-// its diagonal block as k_getrs_diag does, stores the result and raises its
-// own flag.  In FP64 the results are bit-identical to the launch-per-block
-// sequence, without ~4 launches per block on the critical path.  With rg <= 4
-// the two sums of a product (even and odd terms) are taken by two threads
-// and joined in the same order, so the bits do not depend on rg.  Every wait
+// depends on in their order, each as two interleaved sums and as soon as
+// that block's flag is up, then solves its diagonal block as k_getrs_diag
+// does, stores the result and raises its own flag: ~4 launches per block less
+// on the critical path than the blocked solve.  With rg <= 4 the two sums of a
+// product (even and odd terms) are taken by two threads and joined in the same
+// order, so the bits do not depend on rg.  Every wait
 // is bounded (TS_WAIT_NS); a wait that runs out sets *err and the shared
 // abort word, and every CTA then leaves without writing.
 // items[t] = (matrix, block, flag base of the matrix and group, group);
@@ -916,9 +717,8 @@ void la_gemm_batched_shape(int shape, const GemmDesc<C>* d_desc, const int* d_ti
   KPROF_END(st, kname<C>("gemm_batched", "gemm_batched32"), 0.0);
 }
 
-constexpr int LU_NB = 16;
-constexpr size_t LU_PANEL_SMEM = 216 * 1024;   // panels up to this size stay in shared memory
-static_assert(LU_NB <= MAXNB, "LU panel wider than the kernels' shared tiles");
+constexpr int LU_NB = MAXNB;
+constexpr size_t LU_PANEL_SMEM = 216 * 1024;   // a CTA's rows of a panel up to this size stay in shared memory
 constexpr int RS_NB = 32;
 
 // Flop counts of step p (panel, unit-lower solve of U12, trailing GEMM) for the profiler.
@@ -934,56 +734,60 @@ inline void lu_step_flops(const int* h_m, int nprob, int p, double& fp, double& 
   }
 }
 
+// Panel of step p: as many CTAs per matrix (up to 8) as fill the SMs, but no
+// more than chunks of 32 rows, and as many as keep the rows in shared memory.
 template <typename C>
-void launch_panel_cluster(const LuProb<C>* d_prob, int nprob, int p, cudaStream_t st) {
+void lu_panel(const LuProb<C>* d_prob, int nprob, int maxm, int p, cudaStream_t st) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int nch = (maxm - p + 31) / 32;
+  auto bytes = [&](int cs) { return (size_t)((nch + cs - 1) / cs) * 32 * LU_NB * sizeof(C); };
+  int cs = 1;
+  while (cs < 8 && cs < nch && ((long)nprob * cs * 2 <= sms || bytes(cs) > LU_PANEL_SMEM)) cs *= 2;
+  const bool smem = bytes(cs) <= LU_PANEL_SMEM;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(nprob * 8);
-  cfg.blockDim = dim3(256);
-  cfg.dynamicSmemBytes = 0;
+  cfg.gridDim = dim3(nprob * cs);
+  cfg.blockDim = dim3(LP_T);
+  cfg.dynamicSmemBytes = smem ? bytes(cs) : 0;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 8;
+  attr[0].val.clusterDim.x = cs;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, k_lu_panel_cluster<C, 256>, d_prob, p, LU_NB);
+  const int ldp = ((nch + cs - 1) / cs) * 32;
+  if (smem) {
+    // the same value every time: idempotent across threads and devices
+    cudaFuncSetAttribute(k_lu_panel<C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LU_PANEL_SMEM);
+    cudaLaunchKernelEx(&cfg, k_lu_panel<C, true>, d_prob, p, ldp);
+  } else {
+    cudaLaunchKernelEx(&cfg, k_lu_panel<C, false>, d_prob, p, ldp);
+  }
 }
 
 // The trailing update of step p on trailing columns [lo, hi): complex128 on
-// the tensor cores where the caller gave them an error word, else on the FP64 pipe.
+// the tensor cores (g_oz_err: their error word), complex64 on the FP32 pipe.
 template <typename C>
 void lu_update(const LuProb<C>* d_prob, int nprob, int maxm, int p, int lo, int hi, cudaStream_t st) {
-  if constexpr (std::is_same<C, double2>::value) {
-    if (g_oz_err) {
-      oz_lu_update(d_prob, nprob, maxm, p, LU_NB, lo, hi, g_oz_err, st);
-      return;
-    }
-  }
   const int mt = maxm - p - LU_NB, n = std::min(hi, mt) - lo;
-  k_lu_update<C><<<dim3(((mt + TB - 1) / TB) * ((n + TB - 1) / TB), nprob), 256, 0, st>>>(d_prob, p, LU_NB, lo, hi);
+  if constexpr (std::is_same<C, double2>::value) oz_lu_update(d_prob, nprob, maxm, p, LU_NB, lo, hi, g_oz_err, st);
+  else k_lu_update<C><<<dim3(((mt + TB - 1) / TB) * ((n + TB - 1) / TB), nprob), 256, 0, st>>>(d_prob, p, LU_NB, lo, hi);
 }
 
 // The off-diagonal update of a blocked triangular solve, by the same rule.
 template <typename C>
 void getrs_update(const SolveProb<C>* d_prob, int nprob, int maxm, int maxrhs, int p, int lower, cudaStream_t st) {
   const int mt = lower ? maxm - p - RS_NB : p;
-  if constexpr (std::is_same<C, double2>::value) {
-    if (g_oz_err) {
-      oz_getrs_update(d_prob, nprob, maxm, maxrhs, p, RS_NB, lower, g_oz_err, st);
-      return;
-    }
-    if (maxrhs <= 8) {   // FP64: padding costs the bounding pipe
-      k_getrs_update_thin<C><<<dim3((mt + TH_ROWS - 1) / TH_ROWS, nprob), 128, 0, st>>>(d_prob, p, RS_NB, lower);
-      return;
-    }
-  }
-  k_getrs_update<C><<<dim3(((mt + TB - 1) / TB) * ((maxrhs + TB - 1) / TB), nprob), 256, 0, st>>>(d_prob, p, RS_NB, lower);
+  if constexpr (std::is_same<C, double2>::value)
+    oz_getrs_update(d_prob, nprob, maxm, maxrhs, p, RS_NB, lower, g_oz_err, st);
+  else
+    k_getrs_update<C><<<dim3(((mt + TB - 1) / TB) * ((maxrhs + TB - 1) / TB), nprob), 256, 0, st>>>(d_prob, p, RS_NB, lower);
 }
 
-// A few large matrices (the top-level LU) with look-ahead, each panel on a
-// cluster of 8 CTAs: step p's update
+// A few large matrices (the top-level LU) with look-ahead: step p's update
 // of the next panel's LU_NB columns runs first, on a high-priority stream
 // with the panels, and the rest of the trailing update on a low-priority
 // stream, so that panel p+1 (latency-bound, on one 8-CTA cluster) overlaps
@@ -1009,13 +813,13 @@ void la_getrf_lookahead(const LuProb<C>* d_prob, int nprob, int maxm, const int*
     double fp, fs, fu;
     lu_step_flops(h_m, nprob, p, fp, fs, fu);
     KPROF_BEGIN(sp);
-    launch_panel_cluster<C>(d_prob, nprob, p, sp);
+    lu_panel<C>(d_prob, nprob, maxm, p, sp);
     pm_launch_count_add(1);
     KPROF_END(sp, kname<C>("lu_panel", "lu_panel32"), fp);
     if (rest_pending) cudaStreamWaitEvent(sp, e_rest, 0);
     dim3 g1((maxm + 7) / 8, nprob);   // a warp per column
     KPROF_BEGIN(sp);
-    k_lu_swap_trsm<C><<<g1, 256, 0, sp>>>(d_prob, p, LU_NB);
+    k_lu_swap_trsm<C><<<g1, 256, 0, sp>>>(d_prob, p);
     pm_launch_count_add(1);
     KPROF_END(sp, kname<C>("lu_swap_trsm", "lu_swap_trsm32"), fs);
     rest_pending = false;
@@ -1052,7 +856,7 @@ void la_getrf_lookahead(const LuProb<C>* d_prob, int nprob, int maxm, const int*
 template <typename C>
 void la_getrf_batched(const LuProb<C>* d_prob, int nprob, int maxm, const int* h_m, cudaStream_t st) {
   if (nprob <= 0 || maxm <= 0) return;
-  if (nprob <= 8 && maxm >= 2048) {
+  if (nprob <= 8 && maxm >= 512) {
     la_getrf_lookahead<C>(d_prob, nprob, maxm, h_m, st);
     return;
   }
@@ -1060,19 +864,12 @@ void la_getrf_batched(const LuProb<C>* d_prob, int nprob, int maxm, const int* h
     double fp = 0, fs = 0, fu = 0;
     if (g_kprof) lu_step_flops(h_m, nprob, p, fp, fs, fu);
     KPROF_BEGIN(st);
-    const size_t pan_bytes = (size_t)(maxm - p) * std::min(LU_NB, maxm - p) * sizeof(C);
-    if (pan_bytes <= LU_PANEL_SMEM) {
-      // the same value every time: idempotent across threads and devices
-      cudaFuncSetAttribute(k_lu_panel_smem<C, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LU_PANEL_SMEM);
-      k_lu_panel_smem<C, 256><<<nprob, 256, pan_bytes, st>>>(d_prob, p, LU_NB);
-    } else {
-      k_lu_panel<C, 256><<<nprob, 256, 0, st>>>(d_prob, p, LU_NB);
-    }
+    lu_panel<C>(d_prob, nprob, maxm, p, st);
     pm_launch_count_add(1);
     KPROF_END(st, kname<C>("lu_panel", "lu_panel32"), fp);
     dim3 g1((maxm + 7) / 8, nprob);   // a warp per column
     KPROF_BEGIN(st);
-    k_lu_swap_trsm<C><<<g1, 256, 0, st>>>(d_prob, p, LU_NB);
+    k_lu_swap_trsm<C><<<g1, 256, 0, st>>>(d_prob, p);
     pm_launch_count_add(1);
     KPROF_END(st, kname<C>("lu_swap_trsm", "lu_swap_trsm32"), fs);
     int mt = maxm - p - LU_NB;
