@@ -1,11 +1,15 @@
 // Off-boundary fields from a boundary solution (see field.cuh).  One CTA per
-// (evaluation point or direction, right-hand side) sums the trapezoid rule
-// over every node in a fixed order (block-wide reduction), so results are
-// reproducible; the far field needs one sincos per term, the near field one
-// Hankel pair.
+// evaluation point or direction sums the trapezoid rule over every node in a
+// fixed order (block-wide reduction), so results are reproducible.  The near
+// field's Hankel pair and the far field's sincos, which bound these kernels on
+// the FP64 pipe (about 100 of its instructions a node against 8 a right-hand
+// side), are formed once for up to NR right-hand sides: 8 x 8 stars, 4,096
+// points and 720 directions, 8 right-hand sides: 65 ms with one CTA per
+// right-hand side.
 #include "field.cuh"
 #include "hankel.cuh"
 #include "prof.cuh"
+#include <type_traits>
 
 namespace {
 
@@ -33,62 +37,93 @@ __device__ __forceinline__ void qu_of(const InclDev* inc, const int* incl, const
   u = phi[d.row_off + d.n + l];
 }
 
+template <int NR>
 __global__ void __launch_bounds__(FT) k_far_field(const InclDev* __restrict__ inc, NodesDev nd, int total, double k,
                                                   const double2* __restrict__ phi, int ldphi,
                                                   const double* __restrict__ ang, int ndir, double2* out) {
   __shared__ double2 sh[FT / 32];
-  const int dir = blockIdx.x, c = blockIdx.y;
+  const int dir = blockIdx.x;
   double sa, ca;
   sincos(ang[dir], &sa, &ca);
-  const double2* ph = phi + (size_t)c * ldphi;
-  double2 acc = make_double2(0, 0);
+  double2 acc[NR];
+#pragma unroll
+  for (int c = 0; c < NR; ++c) acc[c] = make_double2(0, 0);
   for (int i = threadIdx.x; i < total; i += FT) {
-    double2 q, u;
-    qu_of(inc, nd.incl, ph, i, q, u);
     double s, co;
     sincos(-k * (ca * nd.x[i] + sa * nd.y[i]), &s, &co);      // e^{-i k xhat.y}
     const double kn = k * (ca * nd.nx[i] + sa * nd.ny[i]);
-    // -i k (xhat.n) u - q  (eps+ = 1)
-    const double tx = kn * u.y - q.x, ty = -kn * u.x - q.y;
     const double w = nd.w[i];
-    acc.x += w * (co * tx - s * ty);
-    acc.y += w * (co * ty + s * tx);
+    s *= w;
+    co *= w;
+#pragma unroll
+    for (int c = 0; c < NR; ++c) {
+      double2 q, u;
+      qu_of(inc, nd.incl, phi + (size_t)c * ldphi, i, q, u);
+      // -i k (xhat.n) u - q  (eps+ = 1)
+      const double tx = kn * u.y - q.x, ty = -kn * u.x - q.y;
+      acc[c].x += co * tx - s * ty;
+      acc[c].y += co * ty + s * tx;
+    }
   }
-  const double2 t = block_sum2(acc, sh);
-  if (threadIdx.x == 0) {
-    // gamma = (i/4) sqrt(2/(pi k)) e^{-i pi/4} = (sqrt(2/(pi k)) / 4) e^{i pi/4}
-    const double gm = 0.25 * sqrt(2.0 / (3.141592653589793 * k)) * 0.7071067811865476;
-    out[dir + (size_t)c * ndir] = make_double2(gm * (t.x - t.y), gm * (t.x + t.y));
+#pragma unroll
+  for (int c = 0; c < NR; ++c) {
+    const double2 t = block_sum2(acc[c], sh);
+    if (threadIdx.x == 0) {
+      // gamma = (i/4) sqrt(2/(pi k)) e^{-i pi/4} = (sqrt(2/(pi k)) / 4) e^{i pi/4}
+      const double gm = 0.25 * sqrt(2.0 / (3.141592653589793 * k)) * 0.7071067811865476;
+      out[dir + (size_t)c * ndir] = make_double2(gm * (t.x - t.y), gm * (t.x + t.y));
+    }
+    __syncthreads();
   }
 }
 
+template <int NR>
 __global__ void __launch_bounds__(FT) k_scattered(const InclDev* __restrict__ inc, NodesDev nd, int total, double k,
                                                   const double2* __restrict__ phi, int ldphi,
                                                   const double* __restrict__ xy, int npts, double2* out) {
   __shared__ double2 sh[FT / 32];
-  const int p = blockIdx.x, c = blockIdx.y;
+  const int p = blockIdx.x;
   const double px = xy[2 * p], py = xy[2 * p + 1];
-  const double2* ph = phi + (size_t)c * ldphi;
-  double2 acc = make_double2(0, 0);
+  double2 acc[NR];
+#pragma unroll
+  for (int c = 0; c < NR; ++c) acc[c] = make_double2(0, 0);
   for (int i = threadIdx.x; i < total; i += FT) {
-    double2 q, u;
-    qu_of(inc, nd.incl, ph, i, q, u);
     const double dx = px - nd.x[i], dy = py - nd.y[i];
     const double r = sqrt(dx * dx + dy * dy);
     const double z = k * r;
     double J0, Y0, J1, Y1;
     if (z < HK_ZA) { J0 = j0(z); Y0 = y0(z); J1 = j1(z); Y1 = y1(z); }
     else hankel01(z, J0, Y0, J1, Y1);
-    const double b = (nd.nx[i] * dx + nd.ny[i] * dy) / r;
+    const double w = 0.25 * nd.w[i], b = k * w * ((nd.nx[i] * dx + nd.ny[i] * dy) / r);
     // G = (i/4) H0 = (-Y0 + i J0)/4;  dG/dn_y = (i k/4) H1 b = k b (-Y1 + i J1)/4
-    const double gx = -0.25 * Y0, gy = 0.25 * J0;
-    const double dx2 = -0.25 * k * b * Y1, dy2 = 0.25 * k * b * J1;
-    const double w = nd.w[i];
-    acc.x += w * ((dx2 * u.x - dy2 * u.y) - (gx * q.x - gy * q.y));
-    acc.y += w * ((dx2 * u.y + dy2 * u.x) - (gx * q.y + gy * q.x));
+    const double gx = -w * Y0, gy = w * J0, ex = -b * Y1, ey = b * J1;
+#pragma unroll
+    for (int c = 0; c < NR; ++c) {
+      double2 q, u;
+      qu_of(inc, nd.incl, phi + (size_t)c * ldphi, i, q, u);
+      acc[c].x += (ex * u.x - ey * u.y) - (gx * q.x - gy * q.y);
+      acc[c].y += (ex * u.y + ey * u.x) - (gx * q.y + gy * q.x);
+    }
   }
-  const double2 t = block_sum2(acc, sh);
-  if (threadIdx.x == 0) out[p + (size_t)c * npts] = t;
+#pragma unroll
+  for (int c = 0; c < NR; ++c) {
+    const double2 t = block_sum2(acc[c], sh);
+    if (threadIdx.x == 0) out[p + (size_t)c * npts] = t;
+    __syncthreads();
+  }
+}
+
+// f(first right-hand side, group size as a constant) over groups of 8, 4, 2, 1
+template <class F>
+void rhs_groups(int nrhs, F f) {
+  for (int c = 0; c < nrhs;) {
+    const int left = nrhs - c;
+    if (left >= 8) { f(c, std::integral_constant<int, 8>()); c += 8; }
+    else if (left >= 4) { f(c, std::integral_constant<int, 4>()); c += 4; }
+    else if (left >= 2) { f(c, std::integral_constant<int, 2>()); c += 2; }
+    else { f(c, std::integral_constant<int, 1>()); c += 1; }
+    pm_launch_count_add(1);
+  }
 }
 
 }  // namespace
@@ -96,13 +131,17 @@ __global__ void __launch_bounds__(FT) k_scattered(const InclDev* __restrict__ in
 void far_field(const InclDev* d_inc, NodesDev nodes, int total, double k0, const double2* phi, int ldphi, int nrhs,
                const double* d_angles, int ndir, double2* out, cudaStream_t st) {
   if (ndir <= 0 || nrhs <= 0) return;
-  k_far_field<<<dim3(ndir, nrhs), FT, 0, st>>>(d_inc, nodes, total, k0, phi, ldphi, d_angles, ndir, out);
-  pm_launch_count_add(1);
+  rhs_groups(nrhs, [&](int c, auto nr) {
+    k_far_field<decltype(nr)::value><<<ndir, FT, 0, st>>>(d_inc, nodes, total, k0, phi + (size_t)c * ldphi, ldphi,
+                                                          d_angles, ndir, out + (size_t)c * ndir);
+  });
 }
 
 void scattered_field(const InclDev* d_inc, NodesDev nodes, int total, double k0, const double2* phi, int ldphi,
                      int nrhs, const double* d_xy, int npts, double2* out, cudaStream_t st) {
   if (npts <= 0 || nrhs <= 0) return;
-  k_scattered<<<dim3(npts, nrhs), FT, 0, st>>>(d_inc, nodes, total, k0, phi, ldphi, d_xy, npts, out);
-  pm_launch_count_add(1);
+  rhs_groups(nrhs, [&](int c, auto nr) {
+    k_scattered<decltype(nr)::value><<<npts, FT, 0, st>>>(d_inc, nodes, total, k0, phi + (size_t)c * ldphi, ldphi, d_xy,
+                                                          npts, out + (size_t)c * npts);
+  });
 }
