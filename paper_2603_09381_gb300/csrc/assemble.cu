@@ -270,31 +270,29 @@ __device__ __forceinline__ C omit_entry(const PointsDev& P, int t, int s, double
   const double dx = P.x[pt] - P.x[ps], dy = P.y[pt] - P.y[ps];
   const double r2 = dx * dx + dy * dy;
   if (!(r2 > 0)) return czero<C>();
-  const double r = sqrt(r2);
-  const double z = k * r;
+  const double z = k * sqrt(r2);
   const double w = P.w[ps];
+  // only the orders the entry needs (a warp's entries are mostly of one kind)
+  const bool near = z < HK_ZA;
+  const double iz = 1.0 / z;
   double J0, Y0, J1, Y1;
-  if (z < HK_ZA) {                  // near entries: only the Bessel pair the entry needs
-    if (rg == 0 && cg == 0) return mk((R)(0.25 * y0(z) * w), (R)(-0.25 * j0(z) * w));
-    J1 = j1(z); Y1 = y1(z);
-    if (rg == 1 && cg == 1) { J0 = j0(z); Y0 = y0(z); } else { J0 = 0; Y0 = 0; }
-  } else {
-    hankel01(z, J0, Y0, J1, Y1);
-  }
-  if (rg == 0 && cg == 0)           // -eps+ S = -(i/4) H0 w
+  if (rg == 0 && cg == 0) {         // -eps+ S = -(i/4) H0 w
+    if (near) { J0 = j0(z); Y0 = y0(z); } else hankel_asym(z, iz, J0, Y0, J1, Y1);
     return mk((R)(0.25 * Y0 * w), (R)(-0.25 * J0 * w));
-  if (rg == 0) {                    // D = (ik/4) H1 (n_y.d)/r w
-    double g = (P.nx[ps] * dx + P.ny[ps] * dy) / r * 0.25 * k * w;
-    return mk((R)(-Y1 * g), (R)(J1 * g));
   }
-  if (cg == 0) {                    // -D* = (ik/4) H1 (n_x.d)/r w
-    double g = (P.nx[pt] * dx + P.ny[pt] * dy) / r * 0.25 * k * w;
+  const double ir = k * iz;
+  if (rg != cg) {
+    // D = (ik/4) H1 (n_y.d)/r w;  -D* = (ik/4) H1 (n_x.d)/r w
+    if (near) { J1 = j1(z); Y1 = y1(z); } else hankel_asym(z, iz, J0, Y0, J1, Y1);
+    const int pn = rg == 0 ? ps : pt;
+    const double g = (P.nx[pn] * dx + P.ny[pn] * dy) * ir * 0.25 * k * w;
     return mk((R)(-Y1 * g), (R)(J1 * g));
   }
   // N/eps+ = (ik/4) [k H0 a b + H1/r (nn - 2 a b)] w,  a = n_x.d/r, b = n_y.d/r
-  const double a = (P.nx[pt] * dx + P.ny[pt] * dy) / r, b = (P.nx[ps] * dx + P.ny[ps] * dy) / r;
+  if (near) { J0 = j0(z); Y0 = y0(z); J1 = j1(z); Y1 = y1(z); } else hankel_asym(z, iz, J0, Y0, J1, Y1);
+  const double a = (P.nx[pt] * dx + P.ny[pt] * dy) * ir, b = (P.nx[ps] * dx + P.ny[ps] * dy) * ir;
   const double nn = P.nx[pt] * P.nx[ps] + P.ny[pt] * P.ny[ps];
-  const double c0 = k * a * b, c1 = (nn - 2 * a * b) / r;
+  const double c0 = k * a * b, c1 = (nn - 2 * a * b) * ir;
   const double Hre = c0 * J0 + c1 * J1, Him = c0 * Y0 + c1 * Y1;   // k H0 ab + H1/r (...)
   const double f = 0.25 * k * w;
   return mk((R)(-Him * f), (R)(Hre * f));

@@ -13,8 +13,9 @@
 //   - 8 <= z < 60: polynomial fits of P_nu - 1 and z Q_nu in 1/z^2 on
 //     [8, 12), [12, 20), [20, 30), [30, 60) (hankel_fit.h, written by
 //     gen_hankel_fit.py from 40-digit values; within 2e-17 of P_nu and Q_nu).
-//   One sincos of w_0 = z - pi/4 serves both orders (w_1 = w_0 - pi/2); the
-//   subtraction adds at most half an ulp of z to the phase.
+//   One sine and cosine of w_0 = z - pi/4 serve both orders (w_1 = w_0 - pi/2).
+//   A caller that uses one order pays for one: what it leaves unused is
+//   compiled away.
 // The interval of z is chosen on z rounded to FP32 (comparisons on the FP32
 // pipes): next to a boundary either neighbouring form is within its bound.
 // z < 8: CUDA's j0 / y0 / j1 / y1.
@@ -47,11 +48,48 @@ static __constant__ double c_hk_a0[HK_TERMS] = HK_ROW(0);
 static __constant__ double c_hk_a1[HK_TERMS] = HK_ROW(1);
 #undef HK_ROW
 
+// sin and cos of z - pi/4 for z >= 8 (up to ~1e9): with c = n + 1/2 the nearest
+// half-integer to z 2/pi, z - pi/4 = n pi/2 + y, y = z - c pi/2 in [-pi/4,
+// pi/4] by two fused multiply-adds with pi/2 in two parts (Cody and Waite),
+// then the Taylor sums to y^17 and y^16 (remainders below 1e-19 and 2e-18) and
+// the quadrant: 24 FP64 operations and no slow path.
+__device__ __forceinline__ void hk_sincos_shifted(double z, double& sn, double& cs) {
+  const double magic = 6755399441055744.0;                       // 1.5 2^52: rounds to an integer
+  const double t = fma(z, 0.63661977236758134308, -0.5) + magic;
+  const int n = __double2loint(t);
+  const double c = (t - magic) + 0.5;
+  double y = fma(-c, 1.57079632679489661923, z);
+  y = fma(-c, 6.123233995736766e-17, y);
+  const double x = y * y;
+  double a = 1.0 / 355687428096000.0;                            // 17!
+  a = fma(a, x, -1.0 / 1307674368000.0);
+  a = fma(a, x, 1.0 / 6227020800.0);
+  a = fma(a, x, -1.0 / 39916800.0);
+  a = fma(a, x, 1.0 / 362880.0);
+  a = fma(a, x, -1.0 / 5040.0);
+  a = fma(a, x, 1.0 / 120.0);
+  a = fma(a, x, -1.0 / 6.0);
+  const double s0 = fma(y * x, a, y);
+  double b = 1.0 / 20922789888000.0;                             // 16!
+  b = fma(b, x, -1.0 / 87178291200.0);
+  b = fma(b, x, 1.0 / 479001600.0);
+  b = fma(b, x, -1.0 / 3628800.0);
+  b = fma(b, x, 1.0 / 40320.0);
+  b = fma(b, x, -1.0 / 720.0);
+  b = fma(b, x, 1.0 / 24.0);
+  b = fma(b, x, -0.5);
+  const double c0 = fma(x, b, 1.0);
+  // quadrant: signs by flipping the top bit
+  const double u = (n & 1) ? c0 : s0, v = (n & 1) ? s0 : c0;
+  sn = __hiloint2double(__double2hiint(u) ^ ((n & 2) << 30), __double2loint(u));
+  cs = __hiloint2double(__double2hiint(v) ^ (((n + 1) & 2) << 30), __double2loint(v));
+}
+
 // J and Y of orders 0 and 1 from P_nu, Q_nu (iz = 1/z).
 __device__ __forceinline__ void hankel_combine(double z, double iz, double P0, double Q0, double P1, double Q1,
                                                double& J0, double& Y0, double& J1, double& Y1) {
   double c, d;
-  sincos(z - 0.78539816339744830962, &d, &c);                  // sin, cos of z - pi/4
+  hk_sincos_shifted(z, d, c);                                  // sin, cos of z - pi/4
   const double s = sqrt(0.63661977236758134308 * iz);          // sqrt(2/(pi z))
   J0 = s * (P0 * c - Q0 * d);
   Y0 = s * (P0 * d + Q0 * c);
