@@ -505,7 +505,7 @@ __global__ void __launch_bounds__(256) k_getrs_update(const SolveProb<C>* __rest
                mk((R)-1, (R)0), mk((R)1, (R)0), 0, t % tiles_m, t / tiles_m);
 }
 
-// One triangle of the LU solves of a batch of matrices, each with at most 8
+// One triangle of the LU solves of a batch of matrices, each with at most CHAIN_MAX_RHS
 // right-hand sides, as ONE launch: every matrix is a chain of RS_NB-row
 // blocks, one CTA per block and group of rg right-hand sides (the columns
 // are independent chains; in FP64 a CTA's products and diagonal solve are
@@ -925,7 +925,7 @@ void la_getrs_batched(const SolveProb<C>* d_prob, int nprob, int maxm, int maxrh
     k_getrs_swap<C><<<gsw, 128, 0, st>>>(d_prob);
   }
   pm_launch_count_add(1);
-  if (chain && maxrhs <= 8) {
+  if (chain && maxrhs <= CHAIN_MAX_RHS) {
     // few right-hand sides: each triangle of every matrix in one chained launch
     const int T = chain->total_blocks;
     cudaMemsetAsync(chain->sync, 0, sizeof(int) * la_chain_sync_ints(T), st);

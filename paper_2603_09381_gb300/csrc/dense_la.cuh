@@ -37,7 +37,7 @@ void la_gemm_batched(const GemmDesc<C>* d_desc, const int* d_tile_off, int nprob
 // h_m: host copy of the matrix sizes (flop accounting for the optional profiler)
 template <typename C>
 void la_getrf_batched(const LuProb<C>* d_prob, int nprob, int maxm, const int* h_m, cudaStream_t st);
-// Chained triangular solves (k_trsv_chain): with at most 8 right-hand sides
+// Chained triangular solves (k_trsv_chain): with at most CHAIN_MAX_RHS right-hand sides
 // per matrix, each triangle of every matrix of the batch runs in ONE launch
 // whose blocks wait on one another through flags (bounded waits).
 // la_chain_items fills the 2 x total ticket items (lower, then upper) for the
@@ -48,6 +48,7 @@ void la_getrf_batched(const LuProb<C>* d_prob, int nprob, int maxm, const int* h
 // *err is set to 1 if a wait runs out (the results are then invalid).
 // no_flag (failure-path tests): every block first waits, with a 1 ms bound,
 // on a flag that nothing sets.
+constexpr int CHAIN_MAX_RHS = 64;
 struct ChainArgs {
   const int4* items;
   int total_blocks;   // items per triangle

@@ -821,7 +821,7 @@ void lu_batch(std::vector<LuProb<C>>& probs, Arena& scr, cudaStream_t st, const 
     if (h[i] != 0) fail(PM_ERR_SINGULAR, std::string(what) + ": exactly singular pivot in LU");
 }
 
-// wait_err (optional): lets batches with at most 8 right-hand sides take the
+// wait_err (optional): lets batches with at most CHAIN_MAX_RHS right-hand sides take the
 // chained triangular solves (one launch per triangle for all matrices),
 // whose bounded waits report there.
 template <class C>
@@ -835,7 +835,7 @@ void solve_batch(std::vector<SolveProb<C>>& probs, Arena& scr, cudaStream_t st, 
     hm.push_back(p.m); hr.push_back(p.nrhs);
   }
   auto* dp = upload(scr, probs, st);
-  if (wait_err && maxr <= 8) {
+  if (wait_err && maxr <= CHAIN_MAX_RHS) {
     std::vector<int4> items;
     ChainArgs ch;
     // FP64: two columns per CTA (the links of the chain are bound by one SM's
