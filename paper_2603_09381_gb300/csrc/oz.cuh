@@ -123,14 +123,9 @@ __device__ __forceinline__ void put8(unsigned char* p, uint32_t step, const uint
 }
 __device__ __forceinline__ uint32_t row_off(int row, int k) { return (uint32_t)(row >> 3) * SBO + (uint32_t)(k >> 3) * tcx::LBO + (uint32_t)(row & 7) * 16; }
 
-// The double nearest to V 2^(ex - 2112), V = sum_s v_s 2^(8 (7 - s)); ex: the
-// sum of the two exponents, or negative for a row or column that is not finite.
-__device__ __forceinline__ double join(const float* v, int ex) {
-  int64_t hi = ((int64_t)__float2int_rn(v[0]) << 24) + ((int64_t)__float2int_rn(v[1]) << 16) +
-               ((int64_t)__float2int_rn(v[2]) << 8) + __float2int_rn(v[3]);
-  const int64_t lo = ((int64_t)__float2int_rn(v[4]) << 24) + ((int64_t)__float2int_rn(v[5]) << 16) +
-                     ((int64_t)__float2int_rn(v[6]) << 8) + __float2int_rn(v[7]);
-  hi += lo >> 32;                       // V = hi 2^32 + l, 0 <= l < 2^32
+// The double nearest to (hi 2^32 + lo) 2^p2.
+__device__ __forceinline__ double join(int64_t hi, int64_t lo, int p2) {
+  hi += lo >> 32;                       // = hi 2^32 + l, 0 <= l < 2^32
   uint32_t l = (uint32_t)lo;
   const uint64_t sign = (uint64_t)hi & 0x8000000000000000ull;
   if (sign) {                           // magnitude
@@ -138,17 +133,26 @@ __device__ __forceinline__ double join(const float* v, int ex) {
     l = 0u - l;
   }
   uint64_t mag = (uint64_t)hi, rest = (uint64_t)l << 32;
-  int e = 1023 + 95 + ex - 2112;
+  int e = 1023 + 95 + p2;
   if (mag == 0) { mag = rest; rest = 0; e -= 64; }
-  const int lz = __clzll((long long)mag);   // V != 0: bit 63 of the shifted magnitude is set
+  const int lz = __clzll((long long)mag);   // not zero: bit 63 of the shifted magnitude is set
   mag = (mag << (lz & 63)) | ((rest >> 1) >> (63 - (lz & 63)));
   e -= lz;
   mag = (mag + 1024) >> 11;             // 53 bits (a carry goes on into the exponent)
   uint64_t r = sign | (((uint64_t)(uint32_t)(e - 1) << 52) + mag);
   if (lz == 64 || e <= 0) r = 0;
   if (e >= 2047) r = sign | 0x7FF0000000000000ull;
-  if (ex < 0) r = 0x7FF8000000000000ull;
   return __longlong_as_double((long long)r);
+}
+// The double nearest to V 2^(ex - 2112), V = sum_s v_s 2^(8 (7 - s)); ex: the
+// sum of the two exponents, or negative for a row or column that is not finite.
+__device__ __forceinline__ double join(const float* v, int ex) {
+  const int64_t hi = ((int64_t)__float2int_rn(v[0]) << 24) + ((int64_t)__float2int_rn(v[1]) << 16) +
+                     ((int64_t)__float2int_rn(v[2]) << 8) + __float2int_rn(v[3]);
+  const int64_t lo = ((int64_t)__float2int_rn(v[4]) << 24) + ((int64_t)__float2int_rn(v[5]) << 16) +
+                     ((int64_t)__float2int_rn(v[6]) << 8) + __float2int_rn(v[7]);
+  const double r = join(hi, lo, ex - 2112);
+  return ex < 0 ? __longlong_as_double(0x7FF8000000000000ll) : r;
 }
 
 struct Cta {
@@ -183,12 +187,13 @@ __device__ __forceinline__ void end(Cta& c, int* err) {
   if (!all_ok && threadIdx.x == 0) atomicExch(err, 1);
 }
 
-// One stage: acc[j] += (A B)(row, 8 cg + j) for this thread's row (32 (warp %
-// 4) + lane) and column group cg = warp / 4.  a(row, k) and b(k, col) return
-// the operands' entries, zero outside; new_a: A's digits are not in shared
-// memory yet.  All 512 threads call it.
-template <class FA, class FB>
-__device__ __forceinline__ void stage(Cta& c, bool new_a, const FA& a, const FB& b, double2* acc) {
+// One stage: emit(j, part, d) receives the real (part 0) and imaginary parts
+// of (A B)(row, 8 cg + j), j = 0 .. 7, for this thread's row (32 (warp % 4) +
+// lane) and column group cg = warp / 4.  a(row, k) and b(k, col) return the
+// operands' entries, zero outside; new_a: A's digits are not in shared memory
+// yet; during() runs while the MMAs do (loads for emit).  All 512 threads call it.
+template <class FA, class FB, class FE, class FD>
+__device__ __forceinline__ void stage(Cta& c, bool new_a, const FA& a, const FB& b, const FE& emit, const FD& during) {
   const int tid = threadIdx.x, warp = tid >> 5;
   int* ea = reinterpret_cast<int*>(c.sm + OFF_EXP);   // [k group][row]
   int* eb = ea + 4 * TM;                              // [k group][column]
@@ -262,6 +267,7 @@ __device__ __forceinline__ void stage(Cta& c, bool new_a, const FA& a, const FB&
   // the exponents of this thread's outputs, while the MMAs run
   const int er = 32 * (warp & 3) + (tid & 31), cg = warp >> 2;
   const int E = max(max(ea[er], ea[TM + er]), max(ea[2 * TM + er], ea[3 * TM + er]));
+  during();
   c.ok = c.ok && tcx::mbar_wait(bar, c.phase, WAIT);
   c.phase ^= 1;
   asm volatile("tcgen05.fence::after_thread_sync;");
@@ -281,7 +287,7 @@ __device__ __forceinline__ void stage(Cta& c, bool new_a, const FA& a, const FB&
           const int F = max(max(eb[n], eb[TN + n]), max(eb[2 * TN + n], eb[3 * TN + n]));
           const float w[NS] = {v[0][j], v[1][j], v[2][j], v[3][j], v[4][j], v[5][j], v[6][j], v[7][j]};
           const double d = join(w, E == 0x7FF || F == 0x7FF ? -1 : E + F);
-          if (part == 0) acc[4 * h + j].x += d; else acc[4 * h + j].y += d;
+          emit(4 * h + j, part, d);
         }
       }
     }

@@ -18,9 +18,9 @@ __device__ __forceinline__ void oz_tiles_of(oz::Cta& cta, int m, int n, int k, c
   const int warp = threadIdx.x >> 5, row = r0 + 32 * (warp & 3) + (threadIdx.x & 31), cg = 8 * (warp >> 2);
   for (int t = t0; t < t1; ++t) {
     const int c0 = t * oz::TN;
-    double2 acc[8];
+    double2 v[8];   // MODE 0: the sums; 1: C, loaded during the first stage's MMAs, minus them
 #pragma unroll
-    for (int j = 0; j < 8; ++j) acc[j] = make_double2(0.0, 0.0);
+    for (int j = 0; j < 8; ++j) v[j] = make_double2(0.0, 0.0);
     for (int l0 = 0; l0 < k; l0 += oz::TKC)
       oz::stage(cta, k > oz::TKC || t == t0,
                 [&](int i, int l) {
@@ -29,19 +29,26 @@ __device__ __forceinline__ void oz_tiles_of(oz::Cta& cta, int m, int n, int k, c
                 [&](int l, int j) {
                   return l0 + l < k && c0 + j < n ? B[l0 + l + (c0 + j) * ldb] : make_double2(0.0, 0.0);
                 },
-                acc);
+                [&](int j, int part, double d) {
+                  double& o = part == 0 ? v[j].x : v[j].y;
+                  o = MODE == 1 ? o - d : o + d;
+                },
+                [&] {
+                  if (MODE != 1 || l0 > 0 || row >= m) return;
+#pragma unroll
+                  for (int j = 0; j < 8; ++j)
+                    if (c0 + cg + j < n) v[j] = C[row + (c0 + cg + j) * ldc];
+                });
     if (row < m && cta.ok) {
 #pragma unroll
       for (int j = 0; j < 8; ++j)
         if (c0 + cg + j < n) {
           double2* p = C + row + (c0 + cg + j) * ldc;
-          if (MODE == 1) {
-            *p = *p - acc[j];
-          } else {
-            double2 v = alpha.y == 0.0 && alpha.x == 1.0 ? acc[j] : alpha * acc[j];
-            if (!beta_zero) v = v + beta * (*p);
-            *p = v;
+          if (MODE == 0) {
+            if (!(alpha.y == 0.0 && alpha.x == 1.0)) v[j] = alpha * v[j];
+            if (!beta_zero) v[j] = v[j] + beta * (*p);
           }
+          *p = v[j];
         }
     }
   }

@@ -879,12 +879,13 @@ __global__ void __launch_bounds__(oz::T) k_qr_oz_ypart(const QrProb<double2>* __
   oz::Cta cta = oz::begin(sm);
   for (int r0 = rbeg; r0 < rend; r0 += oz::TKC)
     oz::stage(cta, true,
-              [&](int i, int l) {
-                const int c = c0 + i, r = r0 + l;
-                if (c >= p.n || r >= rend) return czero<double2>();
-                return conj(c < j0 + QR_NB ? v_entry(p, j0, QR_NB, r, c - j0) : p.Z[r + (size_t)c * p.ld]);
-              },
-              [&](int l, int j) { return r0 + l < rend ? v_entry(p, j0, QR_NB, r0 + l, j) : czero<double2>(); }, acc);
+                    [&](int i, int l) {
+                      const int c = c0 + i, r = r0 + l;
+                      if (c >= p.n || r >= rend) return czero<double2>();
+                      return conj(c < j0 + QR_NB ? v_entry(p, j0, QR_NB, r, c - j0) : p.Z[r + (size_t)c * p.ld]);
+                    },
+                    [&](int l, int j) { return r0 + l < rend ? v_entry(p, j0, QR_NB, r0 + l, j) : czero<double2>(); },
+                    [&](int j, int part, double d) { if (part == 0) acc[j].x += d; else acc[j].y += d; }, [] {});
   const int warp = threadIdx.x >> 5, i = 32 * (warp & 3) + (threadIdx.x & 31), cgp = 8 * (warp >> 2);
   double2* yp = p.Yp + ((size_t)blockIdx.x * p.mrb + blockIdx.y) * (oz::TM * QR_NB);
   if (cta.ok) {
@@ -943,21 +944,22 @@ __global__ void __launch_bounds__(oz::T) k_qr_oz_apply(const QrProb<double2>* __
   oz::Cta cta = oz::begin(sm);
   for (int t = t0; t < t1; ++t) {
     const int c0 = t * oz::TN;   // trailing column
-    double2 acc[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) acc[j] = czero<double2>();
+    double2 z[8];   // C, minus the products
     oz::stage(cta, t == t0, [&](int i, int l) { return v_entry(p, j0, QR_NB, r0 + i, l); },
-              [&](int l, int j) {
-                return cfirst + c0 + j < p.n ? p.V[l + (size_t)QR_NB * (c0 + j)] : czero<double2>();
-              },
-              acc);
+                     [&](int l, int j) {
+                       return cfirst + c0 + j < p.n ? p.V[l + (size_t)QR_NB * (c0 + j)] : czero<double2>();
+                     },
+                     [&](int j, int part, double d) { if (part == 0) z[j].x -= d; else z[j].y -= d; },
+                     [&] {
+#pragma unroll
+                       for (int j = 0; j < 8; ++j)
+                         z[j] = row < p.W && cfirst + c0 + cgp + j < p.n ? p.Z[row + (size_t)(cfirst + c0 + cgp + j) * p.ld]
+                                                                         : czero<double2>();
+                     });
     if (row < p.W && cta.ok) {
 #pragma unroll
       for (int j = 0; j < 8; ++j)
-        if (cfirst + c0 + cgp + j < p.n) {
-          double2* z = p.Z + row + (size_t)(cfirst + c0 + cgp + j) * p.ld;
-          *z = *z - acc[j];
-        }
+        if (cfirst + c0 + cgp + j < p.n) p.Z[row + (size_t)(cfirst + c0 + cgp + j) * p.ld] = z[j];
     }
   }
   oz::end(cta, err);
