@@ -12,8 +12,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libpmchwt.so")
-SOURCES = ["assemble.cu", "cpqr.cu", "dense_la.cu", "field.cu", "mlp.cu", "operator.cu", "oz_gemm.cu", "peaks.cu", "qr.cu",
-           "runtime.cu", "tc_gemm.cu"]
+SOURCES = ["assemble.cu", "cpqr.cu", "dense_la.cu", "field.cu", "mlp.cu", "operator.cu", "oz_gemm.cu", "oz_matvec.cu",
+           "peaks.cu", "qr.cu", "runtime.cu", "tc_gemm.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]
 

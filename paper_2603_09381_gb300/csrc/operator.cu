@@ -302,7 +302,8 @@ static_assert(MV32_KT % MV32_G == 0, "runs hold whole load groups");
 template <int NR>
 __global__ void __launch_bounds__(MV_ROWS) k_dense_matvec32(const float2* __restrict__ Ah, size_t lda, int N,
                                                             const double2* __restrict__ X, int ldx,
-                                                            double2* __restrict__ Y, int ldy, int seg) {
+                                                            double2* __restrict__ Y, int ldy, int seg,
+                                                            unsigned char* __restrict__ rexp) {
   __shared__ float2 xs[MV32_KT][NR];
   __shared__ double2 accd[NR][MV_ROWS];   // this thread's FP64 sums: accd[q][threadIdx.x]
   const int row = blockIdx.x * MV_ROWS + threadIdx.x;
@@ -329,6 +330,7 @@ __global__ void __launch_bounds__(MV_ROWS) k_dense_matvec32(const float2* __rest
       // columns at or past cnt load as zero and meet zero X entries: they add 0
       const int cnt = min(MV32_KT, k1 - kb);
       const float2* col = Ah + row + (size_t)kb * lda;
+      unsigned int top = 0;   // the run's largest |part|, as bits
       float2 acc[NR];
 #pragma unroll
       for (int q = 0; q < NR; ++q) acc[q] = make_float2(0.f, 0.f);
@@ -346,9 +348,13 @@ __global__ void __launch_bounds__(MV_ROWS) k_dense_matvec32(const float2* __rest
         }
 #pragma unroll
         for (int g = 0; g < MV32_G; ++g)
+          top = max(top, max(__float_as_uint(cur[g].x) & 0x7FFFFFFFu, __float_as_uint(cur[g].y) & 0x7FFFFFFFu));
+#pragma unroll
+        for (int g = 0; g < MV32_G; ++g)
 #pragma unroll
           for (int q = 0; q < NR; ++q) cfma(acc[q], cur[g], xs[kk + g][q]);
       }
+      if (rexp) rexp[row + (size_t)(kb / MV32_KT) * N] = (unsigned char)(top >> 23);
 #pragma unroll
       for (int q = 0; q < NR; ++q) {
         double2 d = accd[q][threadIdx.x];
@@ -363,137 +369,6 @@ __global__ void __launch_bounds__(MV_ROWS) k_dense_matvec32(const float2* __rest
   for (int q = 0; q < NR; ++q) {
     atomicAdd(&Y[row + (size_t)q * ldy].x, accd[q][threadIdx.x].x);
     atomicAdd(&Y[row + (size_t)q * ldy].y, accd[q][threadIdx.x].y);
-  }
-}
-
-// Float-float building blocks (Dekker / Knuth): exact FP32 product error via
-// FMA, exact sum error via TwoSum.
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = a + b;
-  const float bb = s - a;
-  e = (a - (s - bb)) + (b - bb);
-}
-
-// acc (hi, lo) += a * x for split a = (ah, al), x = (xh, xl): the hi products
-// are split exactly (fmaf); their error and the cross terms are gathered in
-// one FMA chain, which goes to lo with the TwoSum error (12 FP32 operations).
-__device__ __forceinline__ void ff_mac(float& hi, float& lo, float ah, float al, float xh, float xl, float sgn) {
-  const float p = ah * xh;
-  float t = fmaf(ah, xh, -p);   // the exact error of ah xh
-  t = fmaf(ah, xl, t);
-  t = fmaf(al, xh, t);
-  float s, e;
-  two_sum(hi, sgn * p, s, e);
-  hi = s;
-  lo += e + sgn * t;
-}
-
-template <int NR>
-__global__ void __launch_bounds__(MV_ROWS) k_dense_matvec_ff(const float2* __restrict__ Ah,
-                                                             const float2* __restrict__ Al, size_t lda, int N,
-                                                             const double2* __restrict__ X, int ldx,
-                                                             double2* __restrict__ Y, int ldy, int seg) {
-  __shared__ float4 xs[NR][MV_KT];   // {hi(re), hi(im), lo(re), lo(im)} of x
-  const int row = blockIdx.x * MV_ROWS + threadIdx.x;
-  const int k0 = blockIdx.y * seg, k1 = min(N, k0 + seg);
-  float rh[NR], rl[NR], ih[NR], il[NR];
-#pragma unroll
-  for (int q = 0; q < NR; ++q) { rh[q] = rl[q] = ih[q] = il[q] = 0.f; }
-  for (int kb = k0; kb < k1; kb += MV_KT) {
-    __syncthreads();
-    for (int e = threadIdx.x; e < NR * MV_KT; e += MV_ROWS) {
-      const int q = e / MV_KT, kk = e % MV_KT;
-      const double2 v = (kb + kk < k1) ? X[kb + kk + (size_t)q * ldx] : make_double2(0, 0);
-      xs[q][kk] = split4(v.x, v.y);
-    }
-    __syncthreads();
-    if (row < N) {
-      const int cnt = min(MV_KT, k1 - kb);
-      const float2* colh = Ah + row + (size_t)kb * lda;
-      const float2* coll = Al + row + (size_t)kb * lda;
-      for (int kk = 0; kk < cnt; ++kk) {
-        const float2 h = __ldg(colh + (size_t)kk * lda), l = __ldg(coll + (size_t)kk * lda);
-        const float4 a = make_float4(h.x, h.y, l.x, l.y);
-#pragma unroll
-        for (int q = 0; q < NR; ++q) {
-          const float4 x = xs[q][kk];
-          // re += a.re x.re - a.im x.im ;  im += a.re x.im + a.im x.re
-          ff_mac(rh[q], rl[q], a.x, a.z, x.x, x.z, 1.f);
-          ff_mac(rh[q], rl[q], a.y, a.w, x.y, x.w, -1.f);
-          ff_mac(ih[q], il[q], a.x, a.z, x.y, x.w, 1.f);
-          ff_mac(ih[q], il[q], a.y, a.w, x.x, x.z, 1.f);
-        }
-      }
-    }
-  }
-  if (row >= N) return;
-#pragma unroll
-  for (int q = 0; q < NR; ++q) {
-    atomicAdd(&Y[row + (size_t)q * ldy].x, (double)rh[q] + (double)rl[q]);
-    atomicAdd(&Y[row + (size_t)q * ldy].y, (double)ih[q] + (double)il[q]);
-  }
-}
-
-// The float-float product with its (hi, lo) sums restarted every FFC_FOLD
-// columns and folded into FP64.  Within a group of m terms lo's own rounding
-// is at most ~(m^2/2 + 7m) u^2 sum |a||x| (u = 2^-24): with m = 16 about 9e-13
-// of sum_j |a_ij||x_j| per row, below the n 2^-53 worst case of a sequential
-// FP64 sum over a ~20,000-term segment, so this product can end the
-// refinement in place of the FP64 one.
-constexpr int FFC_FOLD = 16;
-template <int NR>
-__global__ void __launch_bounds__(MV_ROWS) k_dense_matvec_ffc(const float2* __restrict__ Ah,
-                                                              const float2* __restrict__ Al, size_t lda, int N,
-                                                              const double2* __restrict__ X, int ldx,
-                                                              double2* __restrict__ Y, int ldy, int seg) {
-  __shared__ float4 xs[NR][MV_KT];   // {hi(re), hi(im), lo(re), lo(im)} of x
-  const int row = blockIdx.x * MV_ROWS + threadIdx.x;
-  const int k0 = blockIdx.y * seg, k1 = min(N, k0 + seg);
-  double2 accd[NR];
-#pragma unroll
-  for (int q = 0; q < NR; ++q) accd[q] = make_double2(0.0, 0.0);
-  for (int kb = k0; kb < k1; kb += MV_KT) {
-    __syncthreads();
-    for (int e = threadIdx.x; e < NR * MV_KT; e += MV_ROWS) {
-      const int q = e / MV_KT, kk = e % MV_KT;
-      const double2 v = (kb + kk < k1) ? X[kb + kk + (size_t)q * ldx] : make_double2(0, 0);
-      xs[q][kk] = split4(v.x, v.y);
-    }
-    __syncthreads();
-    if (row < N) {
-      const int cnt = min(MV_KT, k1 - kb);
-      const float2* colh = Ah + row + (size_t)kb * lda;
-      const float2* coll = Al + row + (size_t)kb * lda;
-      for (int kf = 0; kf < cnt; kf += FFC_FOLD) {
-        const int kend = min(cnt, kf + FFC_FOLD);
-        float rh[NR], rl[NR], ih[NR], il[NR];
-#pragma unroll
-        for (int q = 0; q < NR; ++q) { rh[q] = rl[q] = ih[q] = il[q] = 0.f; }
-        for (int kk = kf; kk < kend; ++kk) {
-          const float2 h = __ldg(colh + (size_t)kk * lda), l = __ldg(coll + (size_t)kk * lda);
-          const float4 a = make_float4(h.x, h.y, l.x, l.y);
-#pragma unroll
-          for (int q = 0; q < NR; ++q) {
-            const float4 x = xs[q][kk];
-            ff_mac(rh[q], rl[q], a.x, a.z, x.x, x.z, 1.f);
-            ff_mac(rh[q], rl[q], a.y, a.w, x.y, x.w, -1.f);
-            ff_mac(ih[q], il[q], a.x, a.z, x.y, x.w, 1.f);
-            ff_mac(ih[q], il[q], a.y, a.w, x.x, x.z, 1.f);
-          }
-        }
-#pragma unroll
-        for (int q = 0; q < NR; ++q) {
-          accd[q].x += (double)rh[q] + (double)rl[q];
-          accd[q].y += (double)ih[q] + (double)il[q];
-        }
-      }
-    }
-  }
-  if (row >= N) return;
-#pragma unroll
-  for (int q = 0; q < NR; ++q) {
-    atomicAdd(&Y[row + (size_t)q * ldy].x, accd[q].x);
-    atomicAdd(&Y[row + (size_t)q * ldy].y, accd[q].y);
   }
 }
 
@@ -667,23 +542,7 @@ void dense_matvec64(SplitOp A, int N, const double2* X, int ldx, double2* Y, int
 }
 
 template <int NR>
-void launch_matvec_ff(SplitOp A, int N, const double2* X, int ldx, double2* Y, int ldy,
-                      cudaStream_t st) {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int rb = (N + MV_ROWS - 1) / MV_ROWS;
-  int segs = std::max(1, (sms * 12 + rb - 1) / rb);
-  int seg = (N + segs - 1) / segs;
-  seg = ((seg + MV_KT - 1) / MV_KT) * MV_KT;
-  segs = (N + seg - 1) / seg;
-  dim3 g(rb, segs);
-  k_dense_matvec_ff<NR><<<g, MV_ROWS, 0, st>>>(A.hi, A.lo, A.ld, N, X, ldx, Y, ldy, seg);
-  pm_launch_count_add(1);
-}
-
-template <int NR>
-void launch_matvec32(SplitOp A, int N, const double2* X, int ldx, double2* Y, int ldy,
+void launch_matvec32(SplitOp A, int N, const double2* X, int ldx, double2* Y, int ldy, unsigned char* rexp,
                      cudaStream_t st) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
@@ -693,11 +552,11 @@ void launch_matvec32(SplitOp A, int N, const double2* X, int ldx, double2* Y, in
   int seg = (N + segs - 1) / segs;
   seg = ((seg + MV32_KT - 1) / MV32_KT) * MV32_KT;
   segs = (N + seg - 1) / seg;
-  k_dense_matvec32<NR><<<dim3(rb, segs), MV_ROWS, 0, st>>>(A.hi, A.ld, N, X, ldx, Y, ldy, seg);
+  k_dense_matvec32<NR><<<dim3(rb, segs), MV_ROWS, 0, st>>>(A.hi, A.ld, N, X, ldx, Y, ldy, seg, rexp);
   pm_launch_count_add(1);
 }
 
-void dense_matvec32(SplitOp A, int N, const double2* X, int ldx, double2* Y, int ldy, int nrhs,
+void dense_matvec32(SplitOp A, int N, const double2* X, int ldx, double2* Y, int ldy, int nrhs, unsigned char* rexp,
                     cudaStream_t st) {
   if (N <= 0 || nrhs <= 0) return;
   for (int q = 0; q < nrhs; ++q) cudaMemsetAsync(Y + (size_t)q * ldy, 0, sizeof(double2) * N, st);
@@ -706,61 +565,12 @@ void dense_matvec32(SplitOp A, int N, const double2* X, int ldx, double2* Y, int
     const int left = nrhs - r0;
     const double2* Xr = X + (size_t)r0 * ldx;
     double2* Yr = Y + (size_t)r0 * ldy;
-    if (left >= 8) { launch_matvec32<8>(A, N, Xr, ldx, Yr, ldy, st); r0 += 8; }
-    else if (left >= 4) { launch_matvec32<4>(A, N, Xr, ldx, Yr, ldy, st); r0 += 4; }
-    else if (left >= 2) { launch_matvec32<2>(A, N, Xr, ldx, Yr, ldy, st); r0 += 2; }
-    else { launch_matvec32<1>(A, N, Xr, ldx, Yr, ldy, st); r0 += 1; }
+    if (left >= 8) { launch_matvec32<8>(A, N, Xr, ldx, Yr, ldy, rexp, st); r0 += 8; }
+    else if (left >= 4) { launch_matvec32<4>(A, N, Xr, ldx, Yr, ldy, rexp, st); r0 += 4; }
+    else if (left >= 2) { launch_matvec32<2>(A, N, Xr, ldx, Yr, ldy, rexp, st); r0 += 2; }
+    else { launch_matvec32<1>(A, N, Xr, ldx, Yr, ldy, rexp, st); r0 += 1; }
   }
   KPROF_END(st, "dense_matvec32", 0.0);
-}
-
-void dense_matvec_ff(SplitOp A, int N, const double2* X, int ldx, double2* Y, int ldy, int nrhs,
-                     cudaStream_t st) {
-  if (N <= 0 || nrhs <= 0) return;
-  for (int q = 0; q < nrhs; ++q) cudaMemsetAsync(Y + (size_t)q * ldy, 0, sizeof(double2) * N, st);
-  KPROF_BEGIN(st);
-  for (int r0 = 0; r0 < nrhs;) {
-    const int left = nrhs - r0;
-    const double2* Xr = X + (size_t)r0 * ldx;
-    double2* Yr = Y + (size_t)r0 * ldy;
-    if (left >= 8) { launch_matvec_ff<8>(A, N, Xr, ldx, Yr, ldy, st); r0 += 8; }
-    else if (left >= 4) { launch_matvec_ff<4>(A, N, Xr, ldx, Yr, ldy, st); r0 += 4; }
-    else if (left >= 2) { launch_matvec_ff<2>(A, N, Xr, ldx, Yr, ldy, st); r0 += 2; }
-    else { launch_matvec_ff<1>(A, N, Xr, ldx, Yr, ldy, st); r0 += 1; }
-  }
-  KPROF_END(st, "dense_matvec_ff", 0.0);
-}
-
-template <int NR>
-void launch_matvec_ffc(SplitOp A, int N, const double2* X, int ldx, double2* Y, int ldy,
-                       cudaStream_t st) {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int rb = (N + MV_ROWS - 1) / MV_ROWS;
-  int segs = std::max(1, (sms * 12 + rb - 1) / rb);
-  int seg = (N + segs - 1) / segs;
-  seg = ((seg + MV_KT - 1) / MV_KT) * MV_KT;
-  segs = (N + seg - 1) / seg;
-  k_dense_matvec_ffc<NR><<<dim3(rb, segs), MV_ROWS, 0, st>>>(A.hi, A.lo, A.ld, N, X, ldx, Y, ldy, seg);
-  pm_launch_count_add(1);
-}
-
-void dense_matvec_ffc(SplitOp A, int N, const double2* X, int ldx, double2* Y, int ldy, int nrhs,
-                      cudaStream_t st) {
-  if (N <= 0 || nrhs <= 0) return;
-  for (int q = 0; q < nrhs; ++q) cudaMemsetAsync(Y + (size_t)q * ldy, 0, sizeof(double2) * N, st);
-  KPROF_BEGIN(st);
-  for (int r0 = 0; r0 < nrhs;) {
-    const int left = nrhs - r0;
-    const double2* Xr = X + (size_t)r0 * ldx;
-    double2* Yr = Y + (size_t)r0 * ldy;
-    if (left >= 8) { launch_matvec_ffc<8>(A, N, Xr, ldx, Yr, ldy, st); r0 += 8; }
-    else if (left >= 4) { launch_matvec_ffc<4>(A, N, Xr, ldx, Yr, ldy, st); r0 += 4; }
-    else if (left >= 2) { launch_matvec_ffc<2>(A, N, Xr, ldx, Yr, ldy, st); r0 += 2; }
-    else { launch_matvec_ffc<1>(A, N, Xr, ldx, Yr, ldy, st); r0 += 1; }
-  }
-  KPROF_END(st, "dense_matvec_ffc", 0.0);
 }
 
 void residual64(const double2* B, const double2* Y, double2* R, int N, int nrhs, double* norms2, cudaStream_t st) {

@@ -52,20 +52,21 @@ void split_copy(const double2* src, int lds, SplitOp dst, int m, int n, const do
 // Y (N x nrhs) = A X in FP64 arithmetic (entries hi + lo); Y overwritten.
 void dense_matvec64(SplitOp A, int N, const double2* X, int ldx, double2* Y, int ldy, int nrhs,
                     cudaStream_t st);
-// The same product in float-float arithmetic on the FP32 pipes: error-free
-// FP32 products of the hi parts (FMA), first-order cross terms, compensated
-// sums; ~1e-13 relative, for refinement residuals.
-void dense_matvec_ff(SplitOp A, int N, const double2* X, int ldx, double2* Y, int ldy, int nrhs,
-                     cudaStream_t st);
-// The float-float product with its sums folded into FP64 every 16 columns:
-// worst-case error ~9e-13 of sum_j |a_ij||x_j| per row, so it may decide the
-// convergence of the refinement (PM_FLAG_FF_CONFIRM).
-void dense_matvec_ffc(SplitOp A, int N, const double2* X, int ldx, double2* Y, int ldy, int nrhs,
-                      cudaStream_t st);
 // The same product with the hi parts in FP32 arithmetic (~1e-7 relative to
-// |A| |X|): the first refinement residual only.
-void dense_matvec32(SplitOp A, int N, const double2* X, int ldx, double2* Y, int ldy, int nrhs,
+// |A| |X|): the first refinement residual only.  rexp (optional): receives the
+// row exponents of dense_row_exponents on the way.
+void dense_matvec32(SplitOp A, int N, const double2* X, int ldx, double2* Y, int ldy, int nrhs, unsigned char* rexp,
                     cudaStream_t st);
+// The product on the tensor cores at FP64 accuracy (oz_matvec.cu): the parts
+// of a row as 54-bit integers relative to the largest of 128 or 512 columns,
+// exact products and sums.  rexp: the exponents of every row's largest part in
+// every 128 columns (ceil(N / 128) x N); xdig, xexp: workspace of
+// dense_matvec_oz_bytes(N) bytes and 8 ceil(N / 128) entries; *err is set if a
+// bounded wait runs out.
+void dense_row_exponents(SplitOp A, int N, unsigned char* rexp, cudaStream_t st);
+size_t dense_matvec_oz_bytes(int N);
+void dense_matvec_oz(SplitOp A, int N, const unsigned char* rexp, const double2* X, int ldx, double2* Y, int ldy, int nrhs,
+                     unsigned char* xdig, unsigned short* xexp, int* err, cudaStream_t st);
 // R = B - Y, and norms2[2 r] += |R[:, r]|^2, norms2[2 r + 1] += |B[:, r]|^2 (norms2 zeroed by caller)
 void residual64(const double2* B, const double2* Y, double2* R, int N, int nrhs, double* norms2, cudaStream_t st);
 // dst[:, r] = scale[r] * src[:, r] (FP64 -> FP32)

@@ -346,6 +346,8 @@ struct pm_factor {
   cudaEvent_t op_done = nullptr;
   double* d_colscale = nullptr; // its column scales: A = dense64 diag(d_colscale)
   size_t dense_bytes = 0;
+  unsigned char* row_exp = nullptr;   // exponents of its rows per 128 columns (once row_exp_ready; under plan_mu)
+  bool row_exp_ready = false;
   // CUDA graphs of the compressed inverse (FP64) or the mixed preconditioner,
   // one per right-hand-side count; solves of one factor are serialised by plan_mu
   std::mutex plan_mu;
@@ -2166,10 +2168,10 @@ void apply_operator64(pm_factor* F, const double2* X, int nrhs, double2* Y, Aren
 
 // Iterative refinement (mixed mode): x <- x + M^{-1} (b - A x) until the
 // relative residual of every column is below refine_tol.  With the dense
-// operator the first residual is an FP32 product, the later intermediate ones
-// float-float (~1e-13 relative) on the FP32 pipes, or, once the residual is
-// small, the update r <- r - A dx with an FP32 product; only FP64 residuals
-// decide convergence.
+// operator the first residual is an FP32 product, the later ones FP64-accurate
+// products on the tensor cores, or, once the residual is small, the update
+// r <- r - A dx with an FP32 product; only FP64-accurate residuals decide
+// convergence.
 void solve_refined(pm_factor* F, const double2* B, int nrhs, double2* X, Arena& ws, cudaStream_t st,
                    pm_solve_info* info) {
   const pm_geometry* g = F->g;
@@ -2189,34 +2191,39 @@ void solve_refined(pm_factor* F, const double2* B, int nrhs, double2* X, Arena& 
     for (int r = 0; r < nrhs; ++r) worst = std::max(worst, std::sqrt(hn[2 * r]) / std::max(std::sqrt(hn[2 * r + 1]), 1e-300));
     return worst;
   };
-  // The residual that can end the refinement: the float-float product folded
-  // into FP64 every 16 columns (a smaller worst-case error bound than a
-  // sequential FP64 sum, on the FP32 pipes), or with PM_FLAG_FP64_CONFIRM the
-  // FP64 product.
-  const bool ff_confirm = F->dense64 && !(F->opts.flags & PM_FLAG_FP64_CONFIRM);
+  // The residuals from the stored operator: the tensor-core product (FP64
+  // accuracy), which may also end the refinement; with
+  // PM_FLAG_FP64_CONFIRM that is left to the FP64 product.
+  const bool oz_confirm = F->dense64 && !(F->opts.flags & PM_FLAG_FP64_CONFIRM);
   // the stored operator is column-scaled: its products take diag(cs) x
   double2* Xs = F->dense64 ? ws.get<double2>((size_t)N * nrhs) : nullptr;
+  unsigned char* xdig = F->dense64 ? ws.get<unsigned char>(dense_matvec_oz_bytes(N)) : nullptr;
+  unsigned short* xexp = F->dense64 ? ws.get<unsigned short>(8 * (size_t)((N + 127) / 128)) : nullptr;
   auto scaled = [&](const double2* x) -> const double2* {
     scale_rows(F->d_colscale, x, N, Xs, N, N, nrhs, st);
     return Xs;
   };
-  auto residual = [&](const double2* x) {
-    if (ff_confirm) {
-      dense_matvec_ffc(F->dense_op, N, scaled(x), N, Y, N, nrhs, st);
-      CK(cudaGetLastError());
-    } else {
-      apply_operator64(F, x, nrhs, Y, ws, st);
+  auto residual_oz = [&](const double2* x) {
+    if (!F->row_exp_ready) {
+      dense_row_exponents(F->dense_op, N, F->row_exp, st);
+      F->row_exp_ready = true;
     }
-    return finish();
-  };
-  auto residual_low = [&](const double2* x) {
-    dense_matvec_ff(F->dense_op, N, scaled(x), N, Y, N, nrhs, st);
+    dense_matvec_oz(F->dense_op, N, F->row_exp, scaled(x), N, Y, N, nrhs, xdig, xexp, g_oz_err, st);
     CK(cudaGetLastError());
     return finish();
+  };
+  auto residual = [&](const double2* x) {
+    if (oz_confirm) return residual_oz(x);
+    apply_operator64(F, x, nrhs, Y, ws, st);
+    return finish();
+  };
+  auto product32 = [&](const double2* x) {
+    dense_matvec32(F->dense_op, N, scaled(x), N, Y, N, nrhs, F->row_exp_ready ? nullptr : F->row_exp, st);
+    F->row_exp_ready = true;
+    CK(cudaGetLastError());
   };
   auto residual_f32 = [&](const double2* x) {
-    dense_matvec32(F->dense_op, N, scaled(x), N, Y, N, nrhs, st);
-    CK(cudaGetLastError());
+    product32(x);
     return finish();
   };
   std::vector<double> bnorm(nrhs, 1.0);
@@ -2225,8 +2232,7 @@ void solve_refined(pm_factor* F, const double2* B, int nrhs, double2* X, Arena& 
   // so it is used only while 1e-6 |r| is far below refine_tol; the new
   // residual goes to dx's buffer and the two buffers swap.
   auto residual_update32 = [&]() {
-    dense_matvec32(F->dense_op, N, scaled(dX), N, Y, N, nrhs, st);
-    CK(cudaGetLastError());
+    product32(dX);
     CK(cudaMemsetAsync(norms, 0, 2 * nrhs * sizeof(double), st));
     residual64(R, Y, dX, N, nrhs, norms, st);
     std::swap(R, dX);
@@ -2266,10 +2272,9 @@ void solve_refined(pm_factor* F, const double2* B, int nrhs, double2* X, Arena& 
     if (F->dense64) {
       // Refinement contracts the residual by a nearly constant factor; when
       // that trend says this step meets the tolerance, the residual is formed
-      // in FP64 straight away (a wrong guess costs nothing: that residual
-      // drives the next step).  Otherwise float-float or the FP32 update,
-      // confirmed in FP64 once it meets the tolerance.
-      // (factor 2 of margin: a wrong guess costs a second FP64 product)
+      // by the confirming product straight away.  Otherwise the tensor-core
+      // product or the cheaper FP32 update, confirmed once it meets the tolerance
+      // (factor 2 of margin: a wrong guess costs a second product).
       const double rate = prev > 0 ? res / prev : 1.0;
       exact = res * rate <= 0.5 * tolr;
     }
@@ -2277,11 +2282,15 @@ void solve_refined(pm_factor* F, const double2* B, int nrhs, double2* X, Arena& 
     if (exact) r_new = residual(X);
     else if (prev < 0) {
       // first step (x0 = 0): its residual is ~1e-3 of b, far above the ~1e-6
-      // error of an FP32 product; a smaller one is formed again in float-float
+      // error of an FP32 product; a smaller one is formed again at FP64 accuracy
       r_new = residual_f32(X);
-      if (r_new < 1e-4) r_new = residual_low(X);
-    } else if (1e-6 * res <= 0.05 * tolr) r_new = residual_update32();
-    else r_new = residual_low(X);
+      if (r_new < 1e-4) { r_new = residual_oz(X); exact = oz_confirm; }
+    } else if (1e-6 * res <= 0.05 * tolr) {
+      r_new = residual_update32();
+    } else {
+      r_new = residual_oz(X);
+      exact = oz_confirm;
+    }
     if (!exact && r_new <= tolr) { r_new = residual(X); exact = true; }
     prev = res;
     res = r_new;
@@ -2653,6 +2662,7 @@ void start_mixed_operator(pm_factor* F, bool beside) {
   if (!F->dense64) return;
   OpNodes nd{g->nodes.x, g->nodes.y, g->nodes.nx, g->nodes.ny, g->nodes.w, g->nodes.incl, F->d_iu, F->d_iq};
   F->d_colscale = F->arena.get<double>((size_t)g->N);
+  F->row_exp = F->arena.get<unsigned char>((size_t)((g->N + 127) / 128) * g->N);
   dense_colscale(g->nodes.w, F->d_iu, F->d_iq, g->total_nodes, g->k0, F->d_colscale, F->st);
   if (beside) {
     int pr_lo = 0, pr_hi = 0;
