@@ -181,12 +181,13 @@ __device__ __forceinline__ float2 shfl_c(float2 v, int src) {
 // column); over 8 SMs the update of a column shrinks to the cost of its
 // barriers.  The rows go to the CTAs in cyclic chunks of 32 and stay there, in
 // shared memory when they fit (SM), else in place.  Per column: every CTA
-// proposes its largest |a|^2 (lowest row on ties) and a copy of that row, rank
-// 0, which owns the diagonal rows, a copy of the diagonal row; one cluster
-// barrier; every CTA reads the proposals, takes the winner's row as the row of
-// U, and the two owners swap; then l = a / pivot and a -= l u on each CTA's
-// rows.  An entry's operations do not depend on the number of CTAs, so neither
-// do the bits.  The comparisons run on the integer pipe (non-negative floats
+// writes its largest |a|^2 (lowest row on ties) and a copy of that row to every
+// CTA's shared memory, rank 0, which owns the diagonal rows, a copy of the
+// diagonal row; one cluster barrier; every CTA takes the winner's row as the
+// row of U, the two owners swap, and a -= (a_jj / pivot) u on each CTA's rows.
+// The column itself is divided by its pivot when the panel is written back.
+// An entry's operations do not depend on the number of CTAs, so neither do the
+// bits.  The comparisons run on the integer pipe (non-negative floats
 // order like their bit patterns).
 constexpr int LP_T = 256;
 template <typename C, bool SM>
@@ -204,12 +205,14 @@ __global__ void __maxnreg__(128) k_lu_panel(const LuProb<C>* __restrict__ P, int
   const int jb = min(MAXNB, m - p), mr = m - p;
   C* pan = SM ? reinterpret_cast<C*>(lu_sm) : pr.A + p + (size_t)p * pr.ld;
   const size_t ld = SM ? ldp : pr.ld;
-  __shared__ C s_slot[2][MAXNB], s_crow[2][MAXNB];   // by column parity: this CTA's proposal, the diagonal row
-  __shared__ u64 s_key[2];
-  __shared__ unsigned s_krow[2];
+  // by column parity: the CTAs' proposals (their rows in slots 0 .. 7) and the diagonal row (slot 8)
+  __shared__ C s_slot[2][9][MAXNB];
+  __shared__ u64 s_key[2][8];
+  __shared__ unsigned s_krow[2][8];
   __shared__ u64 s_wk[NW];
   __shared__ unsigned s_wr[NW];
-  __shared__ C s_u[MAXNB], s_inv;
+  __shared__ C s_inv[MAXNB];
+  static_assert(NW == 8, "a warp writes to each CTA of the cluster");
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nch = ((mr + 31) / 32 - rank + cs - 1) / cs;   // this CTA's chunks of 32 rows
   // chunk ch, lane i: row offset g from p, stored row
@@ -222,7 +225,7 @@ __global__ void __maxnreg__(128) k_lu_panel(const LuProb<C>* __restrict__ P, int
     for (int ch = warp; ch < nch; ch += NW)
       if (row_g(ch) < mr)
         for (int k = 0; k < jb; ++k) pan[row_s(ch) + k * ld] = pr.A[p + row_g(ch) + (size_t)(p + k) * pr.ld];
-  __syncthreads();
+  cluster.sync();   // every CTA of the cluster runs before one writes to another
   u64 key = 0;
   unsigned krow = 0xFFFFFFFFu;
   auto propose = [&](C a, int g) {
@@ -249,76 +252,76 @@ __global__ void __maxnreg__(128) k_lu_panel(const LuProb<C>* __restrict__ P, int
     u64 ck = lane < NW ? s_wk[lane] : 0;
     unsigned cr = lane < NW ? s_wr[lane] : 0xFFFFFFFFu;
     pick(ck, cr);
-    if (warp == 0 && ck > 0 && lane < jb) {
-      const int g = (int)cr, ch = (g / 32 - rank) / cs;
-      s_slot[par][lane] = pan[(SM ? ch * 32 + g % 32 : g) + lane * ld];
+    if (warp < cs) {   // this CTA's proposal to CTA `warp`
+      if (ck > 0 && lane < jb) {
+        const int g = (int)cr, ch = (g / 32 - rank) / cs;
+        cluster.map_shared_rank(&s_slot[par][rank][0], warp)[lane] = pan[(SM ? ch * 32 + g % 32 : g) + lane * ld];
+      }
+      if (rank == 0 && lane < jb) cluster.map_shared_rank(&s_slot[par][8][0], warp)[lane] = pan[jj + lane * ld];
+      if (lane == 0) {
+        *cluster.map_shared_rank(&s_key[par][rank], warp) = ck;
+        *cluster.map_shared_rank(&s_krow[par][rank], warp) = cr;
+      }
     }
-    if (warp == 1 && rank == 0 && lane < jb) s_crow[par][lane] = pan[jj + lane * ld];
-    if (tid == 64) { s_key[par] = ck; s_krow[par] = cr; }
-    cluster.sync();   // the proposals are visible
-    u64 wk = lane < cs ? *cluster.map_shared_rank(&s_key[par], lane) : 0;
-    unsigned wr = lane < cs ? *cluster.map_shared_rank(&s_krow[par], lane) : 0xFFFFFFFFu;
+    cluster.sync();   // the proposals have arrived
+    u64 wk = lane < cs ? s_key[par][lane] : 0;
+    unsigned wr = lane < cs ? s_krow[par][lane] : 0xFFFFFFFFu;
     pick(wk, wr);
     const int piv = wk > 0 ? (int)wr : jj;                   // offset from p
     const int owner = (piv / 32) % cs;
-    const C* urow = wk > 0 ? cluster.map_shared_rank(&s_slot[par][0], owner) : cluster.map_shared_rank(&s_crow[par][0], 0);
-    if (warp == 0) {
-      if (lane < jb) s_u[lane] = urow[lane];
-    } else if (warp == 1) {
-      const C d = urow[jj];
+    const C* u = wk > 0 ? s_slot[par][owner] : s_slot[par][8];   // the row of U
+    if (warp == 1) {
+      const C d = u[jj];
       const R d2 = abs2(d), ri = d2 > 0 ? (R)1 / d2 : (R)0;
-      if (lane == 0) s_inv = mk(d.x * ri, -d.y * ri);
+      if (lane == 0) s_inv[jj] = mk(d.x * ri, -d.y * ri);
     } else if (warp == 2) {
       if (piv != jj && rank == owner && lane < jb) {
         const int ch = (piv / 32 - rank) / cs;
-        pan[(SM ? ch * 32 + piv % 32 : piv) + lane * ld] = cluster.map_shared_rank(&s_crow[par][0], 0)[lane];
+        pan[(SM ? ch * 32 + piv % 32 : piv) + lane * ld] = s_slot[par][8][lane];
       }
     } else if (warp == 3) {
-      if (piv != jj && rank == 0 && lane < jb) pan[jj + lane * ld] = urow[lane];
+      if (piv != jj && rank == 0 && lane < jb) pan[jj + lane * ld] = u[lane];
       if (rank == 0 && lane == 0) {
         pr.ipiv[p + jj] = p + piv;
         if (wk == 0 && *pr.info == 0) *pr.info = p + jj + 1;
       }
     }
     __syncthreads();
-    const C inv = s_inv;
-    for (int ch = warp; ch < nch; ch += NW) {
-      const int g = row_g(ch);
-      if (g > jj && g < mr) pan[row_s(ch) + jj * ld] = pan[row_s(ch) + jj * ld] * inv;
-    }
-    __syncthreads();
+    const C inv = s_inv[jj];
     key = 0;
     krow = 0xFFFFFFFFu;
     for (int ch = slot; ch < nch; ch += slots) {
       const int g = row_g(ch);
       if (g <= jj || g >= mr) continue;
       C* row = pan + row_s(ch);
-      const C l = row[jj * ld];
+      const C l = row[jj * ld] * inv;
       int k = jj + 1 + (q - (jj + 1) % q_n + q_n) % q_n;   // the first column after jj of this residue
       if (k == jj + 1 && k < jb) {
         C a = row[k * ld];
-        cfms(a, l, s_u[k]);
+        cfms(a, l, u[k]);
         row[k * ld] = a;
         propose(a, g);
         k += q_n;
       }
       for (; k + 3 * q_n < jb; k += 4 * q_n) {   // four columns in flight
         C a0 = row[k * ld], a1 = row[(k + q_n) * ld], a2 = row[(k + 2 * q_n) * ld], a3 = row[(k + 3 * q_n) * ld];
-        cfms(a0, l, s_u[k]); cfms(a1, l, s_u[k + q_n]); cfms(a2, l, s_u[k + 2 * q_n]); cfms(a3, l, s_u[k + 3 * q_n]);
+        cfms(a0, l, u[k]); cfms(a1, l, u[k + q_n]); cfms(a2, l, u[k + 2 * q_n]); cfms(a3, l, u[k + 3 * q_n]);
         row[k * ld] = a0; row[(k + q_n) * ld] = a1; row[(k + 2 * q_n) * ld] = a2; row[(k + 3 * q_n) * ld] = a3;
       }
       for (; k < jb; k += q_n) {
         C a = row[k * ld];
-        cfms(a, l, s_u[k]);
+        cfms(a, l, u[k]);
         row[k * ld] = a;
       }
     }
   }
   __syncthreads();
-  if (SM)
-    for (int ch = warp; ch < nch; ch += NW)
-      if (row_g(ch) < mr)
-        for (int k = 0; k < jb; ++k) pr.A[p + row_g(ch) + (size_t)(p + k) * pr.ld] = pan[row_s(ch) + k * ld];
+  for (int ch = warp; ch < nch; ch += NW)
+    if (row_g(ch) < mr)
+      for (int k = 0; k < jb; ++k) {
+        const C a = pan[row_s(ch) + k * ld];
+        pr.A[p + row_g(ch) + (size_t)(p + k) * pr.ld] = row_g(ch) > k ? a * s_inv[k] : a;
+      }
   cluster.sync();   // no CTA leaves while another may still read its proposal
 }
 
@@ -449,9 +452,15 @@ __global__ void __launch_bounds__(256) k_getrs_swap_smem(const SolveProb<C>* __r
 // Diagonal block solve on rows [p, p+jb), jb <= 32: unit lower (lower=1) or
 // upper.  The block is staged in shared memory; one warp per right-hand side,
 // lane r holding row p+r, each solved entry broadcast by a shuffle.
-constexpr int DG_RHS = 32;   // right-hand sides per CTA (8 warps)
+// per: right-hand sides per CTA.  A warp's column is a chain of up to 31
+// dependent multiply-adds, in FP64 2 us of its SM quarter: with few columns in
+// the batch each warp takes one and each SM quarter one warp.
+constexpr int DG_RHS = 32;   // the most right-hand sides per CTA (8 warps)
+inline int diag_per(int nprob, int maxrhs, int sms) {
+  return (long)nprob * ((maxrhs + 3) / 4) <= sms ? 4 : (long)nprob * ((maxrhs + 7) / 8) <= 2 * sms ? 8 : DG_RHS;
+}
 template <typename C>
-__global__ void __launch_bounds__(256) k_getrs_diag(const SolveProb<C>* __restrict__ P, int p, int nb, int lower) {
+__global__ void __launch_bounds__(256) k_getrs_diag(const SolveProb<C>* __restrict__ P, int p, int nb, int lower, int per) {
   typedef typename real_of<C>::type R;
   __shared__ C sa[32][33];
   const SolveProb<C> pr = P[blockIdx.y];
@@ -466,8 +475,8 @@ __global__ void __launch_bounds__(256) k_getrs_diag(const SolveProb<C>* __restri
   // reciprocals of the diagonal, all lanes at once (the solve chain below
   // then multiplies instead of dividing: FP64 division is a long sequence)
   const C dinv = (!lower && lane < jb) ? cdiv(mk((R)1, (R)0), sa[lane][lane]) : czero<C>();
-  const int j1 = min(pr.nrhs, (int)(blockIdx.x + 1) * DG_RHS);
-  for (int j = blockIdx.x * DG_RHS + (threadIdx.x >> 5); j < j1; j += blockDim.x >> 5) {
+  const int j1 = min(pr.nrhs, (int)(blockIdx.x + 1) * per);
+  for (int j = blockIdx.x * per + (threadIdx.x >> 5); j < j1; j += blockDim.x >> 5) {
     C* col = pr.B + (size_t)j * pr.ldb + p;
     C x = lane < jb ? col[lane] : czero<C>();
     if (lower) {
@@ -734,14 +743,18 @@ inline void lu_step_flops(const int* h_m, int nprob, int p, double& fp, double& 
   }
 }
 
+int sm_count() {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
+}
+
 // Panel of step p: as many CTAs per matrix (up to 8) as fill the SMs, but no
 // more than chunks of 32 rows, and as many as keep the rows in shared memory.
 template <typename C>
 void lu_panel(const LuProb<C>* d_prob, int nprob, int maxm, int p, cudaStream_t st) {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int nch = (maxm - p + 31) / 32;
+  const int sms = sm_count(), nch = (maxm - p + 31) / 32;
   auto bytes = [&](int cs) { return (size_t)((nch + cs - 1) / cs) * 32 * LU_NB * sizeof(C); };
   int cs = 1;
   while (cs < 8 && cs < nch && ((long)nprob * cs * 2 <= sms || bytes(cs) > LU_PANEL_SMEM)) cs *= 2;
@@ -943,9 +956,11 @@ void la_getrs_batched(const SolveProb<C>* d_prob, int nprob, int maxm, int maxrh
     KPROF_END(st, kname<C>("getrs", "getrs32"), fl);
     return;
   }
-  dim3 gs((maxrhs + DG_RHS - 1) / DG_RHS, nprob);
+  const int per = diag_per(nprob, maxrhs, sm_count());
+  const dim3 gs((maxrhs + per - 1) / per, nprob);
+  const int dt = std::min(256, 32 * per);
   for (int p = 0; p < maxm; p += RS_NB) {
-    k_getrs_diag<C><<<gs, 256, 0, st>>>(d_prob, p, RS_NB, 1);
+    k_getrs_diag<C><<<gs, dt, 0, st>>>(d_prob, p, RS_NB, 1, per);
     pm_launch_count_add(1);
     if (maxm - p - RS_NB > 0) {
       getrs_update<C>(d_prob, nprob, maxm, maxrhs, p, 1, st);
@@ -953,7 +968,7 @@ void la_getrs_batched(const SolveProb<C>* d_prob, int nprob, int maxm, int maxrh
     }
   }
   for (int p = ((maxm - 1) / RS_NB) * RS_NB; p >= 0; p -= RS_NB) {
-    k_getrs_diag<C><<<gs, 256, 0, st>>>(d_prob, p, RS_NB, 0);
+    k_getrs_diag<C><<<gs, dt, 0, st>>>(d_prob, p, RS_NB, 0, per);
     pm_launch_count_add(1);
     if (p > 0) {
       getrs_update<C>(d_prob, nprob, maxm, maxrhs, p, 0, st);
@@ -968,10 +983,12 @@ void la_trsm_upper_batched(const SolveProb<C>* d_prob, int nprob, int maxm, int 
                            double flops, cudaStream_t st) {
   if (nprob <= 0 || maxm <= 0 || maxrhs <= 0) return;
   KPROF_BEGIN(st);
-  dim3 gs((maxrhs + DG_RHS - 1) / DG_RHS, nprob);
+  const int per = diag_per(nprob, maxrhs, sm_count());
+  const dim3 gs((maxrhs + per - 1) / per, nprob);
+  const int dt = std::min(256, 32 * per);
   int last = ((maxm - 1) / RS_NB) * RS_NB;
   for (int p = last; p >= 0; p -= RS_NB) {
-    k_getrs_diag<C><<<gs, 256, 0, st>>>(d_prob, p, RS_NB, 0);
+    k_getrs_diag<C><<<gs, dt, 0, st>>>(d_prob, p, RS_NB, 0, per);
     pm_launch_count_add(1);
     if (p > 0) {
       getrs_update<C>(d_prob, nprob, maxm, maxrhs, p, 0, st);
