@@ -598,18 +598,31 @@ void assemble_self(const pm_geometry* g, const std::vector<int>& incl, const std
   // Maue: N-block += diag(1/|x'|) Dt (S0+/e+ + S0-/e-) Dt
   std::vector<GemmDesc<C>> d1(m), d2(m);
   std::vector<int> off1(m + 1, 0), off2(m + 1, 0);
+  const bool oz = std::is_same<C, double2>::value && g_oz_err;   // on the tensor cores (oz_gemm)
+  long tiles = 0;
+  for (int i = 0; i < m; ++i) tiles += oz_tiles(sub[i].n, sub[i].n, 1);
+  const int per = oz_per(tiles);
   for (int i = 0; i < m; ++i) {
     int n = sub[i].n;
     d1[i] = GemmDesc<C>{n, n, n, Cm[i], n, dts[n], n, E[i], n, cone<C>(), czero_h<C>(), 1};
     C* tgt = bm ? A[i] : A[i] + n + (size_t)n * lda[i];
     d2[i] = GemmDesc<C>{n, n, n, DtS[i], n, E[i], n, tgt, lda[i], cone<C>(), cone<C>(), 0};
-    off1[i + 1] = off1[i] + gemm_tiles(n, n);
-    off2[i + 1] = off2[i] + gemm_tiles(n, n);
+    off1[i + 1] = off1[i] + (oz ? oz_tiles(n, n, per) : gemm_tiles(n, n));
+    off2[i + 1] = off2[i] + (oz ? oz_tiles(n, n, per) : gemm_tiles(n, n));
   }
-  auto* dd1 = upload(scr, d1, st); auto* do1 = upload(scr, off1, st);
-  la_gemm_batched<C>(dd1, do1, m, off1[m], st);
-  auto* dd2 = upload(scr, d2, st); auto* do2 = upload(scr, off2, st);
-  la_gemm_batched<C>(dd2, do2, m, off2[m], st);
+  auto run = [&](const std::vector<GemmDesc<C>>& d, const std::vector<int>& off) {
+    auto* dd = upload(scr, d, st);
+    auto* dof = upload(scr, off, st);
+    if constexpr (std::is_same<C, double2>::value) {
+      if (oz) {
+        oz_gemm_batched(dd, dof, m, off[m], per, g_oz_err, st);
+        return;
+      }
+    }
+    la_gemm_batched<C>(dd, dof, m, off[m], st);
+  };
+  run(d1, off1);
+  run(d2, off2);
   CK(cudaGetLastError());
 }
 
