@@ -1,18 +1,27 @@
 // Column-pivoted Householder QR, one launch per elimination step.
 //
-// Each CTA owns up to 32 columns of one matrix.  At step s every CTA of the
-// matrix reads the same squared trailing norms, picks the same pivot
-// (largest norm; norms within a factor 1 - 1e-12 of the largest count as
-// tied and the lowest column index wins), forms the Householder reflector of
-// the pivot column (LAPACK zlarfg phase convention) and applies H^H to its
-// own columns, recomputing their trailing norms from scratch for step s+1.
-// The pivot column itself is left in place; R_ss goes to rdiag[s].  Because
+// Each CTA owns up to 16 columns of one matrix.  The step's pivot (largest
+// trailing norm; norms within a factor 1 - 1e-12 of the largest count as tied
+// and the lowest column index wins) and its Householder reflector (LAPACK
+// zlarfg phase convention) are read from the matrix's CpqrPick, written at
+// the end of the previous step by the matrix's last CTA to finish: choosing
+// them anew in every CTA cost more than the columns (square roots, divisions
+// and comparisons on the FP64 pipe, 10 us of an SM per step).  The CTA applies
+// H^H to its columns, recomputing their trailing norms from scratch.  The
+// pivot column itself is left in place; R_ss goes to rdiag[s].  Because
 // consecutive steps are consecutive launches no grid-wide barrier is needed.
-// Work per entry and step: ~10 real FMAs on 48 bytes, so the FP64 pipe, not
-// HBM, bounds it on GB300.
+//
+// complex128 columns are held in 60-bit fixed point (fx.cuh, one power-of-two
+// scale per column from its initial norm): a reflection keeps a column's
+// norm, and the integer multipliers do a complex multiply-add in a quarter of
+// the FP64 pipe's time.  The pivot column enters the dot products shifted up
+// to its norm, and the trailing norms are sums of exact 120-bit squares, so
+// both keep a double's relative accuracy however far a column has decayed.
 #include "cpqr.cuh"
+#include "fx.cuh"
 #include "prof.cuh"
 #include <algorithm>
+#include <cooperative_groups.h>
 #include <atomic>
 #include <mutex>
 
@@ -27,12 +36,128 @@ __global__ void __launch_bounds__(256) k_init_norms(const CpqrProb<C>* __restric
   const CpqrProb<C> p = P[ch.id];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int c = ch.c0 + warp; c < ch.c1; c += 8) {
-    const C* col = p.Z + (size_t)c * p.ld;
+    C* col = p.Z + (size_t)c * p.ld;
     R acc = 0;
     for (int r = lane; r < p.W; r += 32) acc += abs2(col[r]);
     acc = warp_sum(acc);
     if (lane == 0) p.norm2[c] = (double)acc;
+    if constexpr (sizeof(C) == 16) {
+      // to fixed point, the norm brought into (1/8, 1/4] (a column that is not finite: zeros)
+      int e = 0;
+      const bool ok = isfinite(acc);
+      if (ok && acc > 0) frexp(sqrt(acc) * (1.0 + 1e-9), &e);
+      e += 2;
+      longlong2* f = reinterpret_cast<longlong2*>(col);
+      for (int r = lane; r < p.W; r += 32) {
+        const double2 z = col[r];
+        f[r] = make_longlong2(ok ? fx_from(z.x, e) : 0, ok ? fx_from(z.y, e) : 0);
+      }
+      if (lane == 0) p.cexp[c] = e;
+    }
   }
+}
+
+__device__ __forceinline__ double ld_norm(const double* p) { return __ldcg(p); }
+
+// Pivot and reflector of step s (the matrix's norms of step s are complete),
+// or the end of the phase.  All 256 threads of one CTA.  Norms are compared
+// as integers (non-negative doubles order like their bit patterns).
+template <typename C>
+__device__ void cpqr_pick(const CpqrProb<C>& p, int s) {
+  typedef typename real_of<C>::type R;
+  typedef unsigned long long u64;
+  __shared__ u64 s_k[8];
+  __shared__ int s_i[8];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int n = p.n;
+  const double* cur = p.norm2 + (s & 1) * n;
+  auto key_of = [&](int c) -> u64 {   // 0: pivoted (negative) or not a number
+    const u64 b = (u64)__double_as_longlong(ld_norm(cur + c));
+    return b <= 0x7FF0000000000000ull ? b + 1 : 0;
+  };
+  u64 k = 0;
+  if (s < p.target)
+    for (int c = tid; c < n; c += 256) { const u64 x = key_of(c); k = x > k ? x : k; }
+  const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(k >> 32));
+  const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(k >> 32) == hi ? (unsigned)k : 0u);
+  if (lane == 0) s_k[warp] = ((u64)hi << 32) | lo;
+  __syncthreads();
+  k = s_k[0];
+#pragma unroll
+  for (int w = 1; w < 8; ++w) k = s_k[w] > k ? s_k[w] : k;
+  const double mx = k ? __longlong_as_double((long long)(k - 1)) : 0.0;
+  // lowest index within the tie band
+  const u64 band = k ? (u64)__double_as_longlong((1.0 - TIE) * mx) + 1 : ~0ull;
+  int qi = n;
+  if (k)
+    for (int c = tid; c < n; c += 256) if (key_of(c) >= band) { qi = c; break; }
+  qi = __reduce_min_sync(0xffffffffu, qi);
+  if (lane == 0) s_i[warp] = qi;
+  __syncthreads();
+  if (warp != 0) return;
+  qi = s_i[0];
+#pragma unroll
+  for (int w = 1; w < 8; ++w) qi = min(qi, s_i[w]);
+  CpqrPick<C> pk{};
+  pk.q = -1;
+  bool go = k != 0 && qi < n;
+  if (go && p.mode == CPQR_FIND_RANK) {
+    const double ref = s == 0 ? sqrt(mx) : *p.ref;
+    if (s == 0 && lane == 0) *p.ref = ref;
+    if (!(sqrt(mx) > p.tol * ref)) {
+      if (lane == 0) *p.rank = s;
+      go = false;
+    }
+  }
+  if (go) {
+    pk.q = qi;
+    const double nq = ld_norm(cur + qi);
+    C tau = czero<C>();
+    if constexpr (sizeof(C) == 16) {
+      const int eq = p.cexp[qi];
+      const longlong2 a = __ldcg(reinterpret_cast<const longlong2*>(p.Z + s + (size_t)qi * p.ld));
+      const double2 alpha = make_double2(fx_to(a.x, 0), fx_to(a.y, 0));   // in units of the column's scale
+      double beta;
+      double2 sc;
+      const double nn = ldexp(nq, -2 * eq);
+      fx_reflector(alpha, nn, beta, tau, sc);
+      pk.ev = fx_shift(nq, eq);   // x 2^ev below 1, sc 2^-ev at most 2
+      pk.sc = __longlong_as_double((long long)(1023 - pk.ev) << 52) * sc;
+      pk.csc = __longlong_as_double((long long)(1023 - 60 - pk.ev) << 52) * conj(sc);   // applied to the shifted sums
+      // A factorization continued past its rank can meet a column whose integers
+      // are all zero: R_ss is then the unit of its scale, not zero, so that
+      // the interpolation matrix stays finite.
+      pk.beta = make_double2(ldexp(beta != 0 ? beta : 0x1p-58, eq), 0.0);
+    } else {
+      const C alpha = __ldcg(p.Z + s + (size_t)qi * p.ld);
+      const R xnorm = (R)sqrt(nq);
+      const R beta = -copysign(xnorm, alpha.x);
+      C sc = czero<C>();
+      pk.reflect = xnorm > 0;
+      if (pk.reflect) {
+        const C bm = mk(beta, (R)0);
+        tau = cdiv(bm - alpha, bm);
+        sc = cdiv(mk((R)1, (R)0), alpha - bm);
+      }
+      pk.sc = sc;
+      pk.csc = conj(sc);
+      pk.beta = mk(beta, (R)0);
+    }
+    pk.ctau = conj(tau);
+    if (lane == 0) {
+      p.rdiag[s] = pk.beta;
+      p.perm[s] = qi;
+    }
+  }
+  if (lane == 0) *p.pick = pk;
+}
+
+// First pivot of a phase (step `base` of every matrix).
+template <typename C>
+__global__ void __launch_bounds__(256) k_cpqr_start(const CpqrProb<C>* __restrict__ P) {
+  const CpqrProb<C> p = P[blockIdx.x];
+  cpqr_pick<C>(p, p.base);
+  if (threadIdx.x == 0) *p.done = 0;
 }
 
 // Sum of one value over the 256 threads of the CTA (every thread gets it).
@@ -97,82 +222,21 @@ __device__ void cta_columns(const CpqrProb<C>& p, const CpqrChunk& ch, int s, in
   }
 }
 
-// One elimination step of the chunk's matrix on the chunk's columns (all 256
-// threads of the CTA take the same path through the barriers).
+// One elimination step of a complex64 chunk's columns (all 256 threads of
+// the CTA take the same path through the barriers).
 template <typename C, bool TALL>
-__device__ void cpqr_chunk_step(const CpqrProb<C>& p, const CpqrChunk& ch, int t) {
+__device__ void cpqr_columns(const CpqrProb<C>& p, const CpqrChunk& ch, int s, const CpqrPick<C>& pk) {
   typedef typename real_of<C>::type R;
-  const int s = p.base + t;
-  if (s >= p.target) return;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  __shared__ double red[8];
-  __shared__ int redi[8];
-  __shared__ double s_mx;
-  __shared__ int s_q;
-  __shared__ int s_done;
-  // Another CTA may set the rank during this launch: read it once so that the
-  // whole CTA takes the same path through the barriers below.
-  if (tid == 0) s_done = (p.mode == CPQR_FIND_RANK) && (*(volatile int*)p.rank >= 0);
-  __syncthreads();
-  if (s_done) return;
-  const int n = p.n;
+  const int n = p.n, q = pk.q;
   const double* cur = p.norm2 + (s & 1) * n;
   double* nxt = p.norm2 + ((s + 1) & 1) * n;
-  // pass 1: largest squared norm among unpivoted columns
-  double mx = -1.0;
-  for (int c = tid; c < n; c += 256) mx = fmax(mx, cur[c]);
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if (lane == 0) red[warp] = mx;
-  __syncthreads();
-  if (tid == 0) {
-    double m2 = red[0];
-    for (int w = 1; w < 8; ++w) m2 = fmax(m2, red[w]);
-    s_mx = m2;
-  }
-  __syncthreads();
-  mx = s_mx;
-  // pass 2: lowest index within the tie band
-  const double band = (1.0 - TIE) * mx;
-  int qi = n;
-  for (int c = tid; c < n; c += 256) if (cur[c] >= 0 && cur[c] >= band) { qi = c; break; }
-  for (int o = 16; o > 0; o >>= 1) qi = min(qi, __shfl_xor_sync(0xffffffffu, qi, o));
-  if (lane == 0) redi[warp] = qi;
-  __syncthreads();
-  if (tid == 0) {
-    int q2 = redi[0];
-    for (int w = 1; w < 8; ++w) q2 = min(q2, redi[w]);
-    s_q = q2;
-  }
-  __syncthreads();
-  const int q = s_q;
-  if (mx < 0 || q >= n) return;  // no unpivoted column left
-  if (p.mode == CPQR_FIND_RANK) {
-    double ref = (s == 0) ? sqrt(mx) : *p.ref;
-    if (s == 0 && ch.first && tid == 0) *p.ref = ref;
-    if (!(sqrt(mx) > p.tol * ref)) {
-      if (ch.first && tid == 0) *p.rank = s;
-      return;
-    }
-  }
   const C* xq = p.Z + (size_t)q * p.ld;
-  const C alpha = xq[s];
-  const R xnorm = (R)sqrt(cur[q]);
-  const R beta = -copysign(xnorm, alpha.x);
-  C tau = czero<C>(), sc = czero<C>();
-  const bool reflect = xnorm > 0;
-  if (reflect) {
-    C bm = mk(beta, (R)0);
-    tau = cdiv(bm - alpha, bm);
-    sc = cdiv(mk((R)1, (R)0), alpha - bm);
-  }
-  const C ctau = conj(tau), csc = conj(sc);
+  const C ctau = pk.ctau, sc = pk.sc, csc = pk.csc;
+  const bool reflect = pk.reflect;
   // complex64 tall enough to fill the CTA (short columns are barrier-bound) and fitting in registers
   if (TALL && sizeof(C) == 8 && reflect && p.W >= 2048 && p.W <= 256 * 32) {
     cta_columns<C, 32>(p, ch, s, q, xq, ctau, csc, sc, cur, nxt);
-    if (tid == 0 && q >= ch.c0 && q < ch.c1) {
-      p.rdiag[s] = mk(beta, (R)0);
-      p.perm[s] = q;
-    }
     return;
   }
   for (int c = ch.c0 + warp; c < ch.c1; c += 8) {
@@ -221,21 +285,158 @@ __device__ void cpqr_chunk_step(const CpqrProb<C>& p, const CpqrChunk& ch, int t
     acc = warp_sum(acc);
     if (lane == 0) nxt[c] = (double)acc;
   }
-  if (tid == 0 && q >= ch.c0 && q < ch.c1) {
-    p.rdiag[s] = mk(beta, (R)0);
-    p.perm[s] = q;
+}
+
+// Sums over the warp of a 59-bit signed integer, 24 bits at a time, as two
+// words whose value is hi 2^24 + lo.
+__device__ __forceinline__ void warp_sum_parts(long long x, long long& hi, unsigned& lo) {
+  lo = __reduce_add_sync(0xffffffffu, (unsigned)x & 0xFFFFFFu);
+  const unsigned mid = __reduce_add_sync(0xffffffffu, (unsigned)(x >> 24) & 0xFFFFFFu);
+  const int top = __reduce_add_sync(0xffffffffu, (int)(x >> 48));
+  hi = ((long long)top << 24) + mid;
+}
+
+// d += conj(x) (a 2^ea).  Both are shifted up to their norms, so that the sum
+// has a double's accuracy relative to them: a factorization continued far past
+// its rank works on columns of a few units, and row entries that are off by as
+// much as the pivot make the interpolation matrix grow with every step.
+__device__ __forceinline__ void fx_dot(longlong2& d, longlong2 x, longlong2 a, int ea) {
+  const Fx xr = fx(x.x), xi = fx(x.y), nxi = fx(-x.y), ar = fx(a.x << ea), ai = fx(a.y << ea);
+  long long cr = FX_HALF, ci = FX_HALF;
+  fx_mac(d.x, cr, xr, ar); fx_mac(d.x, cr, xi, ai);
+  fx_mac(d.y, ci, xr, ai); fx_mac(d.y, ci, nxi, ar);
+  d.x += cr >> 30;
+  d.y += ci >> 30;
+}
+// From the sum x^H a (parts of warp_sum_parts) over the rows below s: the entry
+// a_s is updated and the factor of the rows below formed, a += g (x 2^ev): |f| is
+// at most 1/2 (a reflection moves a by at most twice its norm of 1/4), so |g| at most 1.
+__device__ __forceinline__ void fx_factor(double2 ctau, double2 csc, double2 sc, longlong2 h, uint2 l, int ea,
+                                          longlong2* a_s, int4& g, int2& gn) {
+  const longlong2 as = *a_s;
+  const double u = __longlong_as_double((long long)(1023 - ea) << 52);
+  const double2 dot = make_double2(u * ((double)h.x * 16777216.0 + (double)l.x), u * ((double)h.y * 16777216.0 + (double)l.y));
+  const double2 f = ctau * (make_double2(fx_to(as.x, 0), fx_to(as.y, 0)) + csc * dot);   // conj(tau) v^H a
+  *a_s = make_longlong2(as.x - __double2ll_rn(f.x * FX_ONE), as.y - __double2ll_rn(f.y * FX_ONE));
+  const double2 t = -(f * sc);
+  const long long ti = __double2ll_rn(t.y * FX_ONE);
+  const Fx r = fx(__double2ll_rn(t.x * FX_ONE)), i = fx(ti), ni = fx(-ti);
+  g = make_int4(r.h, r.l, i.h, i.l);
+  gn = make_int2(ni.h, ni.l);
+}
+__device__ __forceinline__ longlong2 fx_update(longlong2 a, longlong2 x, int4 g, int2 gn) {
+  return fx_cfma(a, Fx{g.x, g.y}, Fx{g.z, g.w}, Fx{gn.x, gn.y}, fx(x.x), fx(x.y));
+}
+// Exact sum of squares of integers below 2^58: a = h 2^29 + l, 0 <= l < 2^29,
+// sums of h^2, h l and l^2, folded before they can overflow (every 8 entries).
+struct FxSquares {
+  long long A = 0, B = 0, D = 0;
+  __device__ __forceinline__ void part(long long v) {
+    const int h = (int)(v >> 29), l = (int)v & 0x1FFFFFFF;
+    A += (long long)h * h;
+    B += (long long)h * l;
+    D += (long long)l * l;
   }
+  __device__ __forceinline__ void add(longlong2 a) { part(a.x); part(a.y); }
+  // the sum is A 2^58 + B 2^30 + D
+  __device__ __forceinline__ void fold() {
+    B += D >> 30; D &= 0x3FFFFFFF;
+    A += B >> 28; B &= 0xFFFFFFF;
+  }
+  // over the warp: x 2^58 + y
+  __device__ __forceinline__ longlong2 warp_total() {
+    fold();
+    longlong2 t;
+    long long h;
+    unsigned l;
+    warp_sum_parts(A, h, l);
+    t.x = (h << 24) + l;
+    warp_sum_parts((B << 30) + D, h, l);
+    t.y = (h << 24) + l;
+    return t;
+  }
+};
+// (x 2^58 + y) 2^-120 scale^2
+__device__ __forceinline__ double fx_norm2(longlong2 w, int e) {
+  return ldexp(fma((double)w.x, 0x1p58, (double)w.y), 2 * e - 120);
+}
+
+// One elimination step of a complex128 chunk's columns in fixed point, two
+// columns per warp: dot products with the shifted pivot column; the chunk's
+// factors at once, a thread per column (a warp's FP64 instruction costs the
+// same for one lane as for 32); the update and the exact squares of the new
+// entries; the chunk's norms at once.
+__device__ void cpqr_columns_fx(const CpqrProb<double2>& p, const CpqrChunk& ch, int s, const CpqrPick<double2>& pk) {
+  static_assert(CPQR_CB == 16, "two columns per warp");
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int n = p.n, q = pk.q, W = p.W, ev = pk.ev;
+  const double* cur = p.norm2 + (s & 1) * n;
+  double* nxt = p.norm2 + ((s + 1) & 1) * n;
+  __shared__ longlong2 s_dot[CPQR_CB], s_nrm[CPQR_CB];
+  __shared__ uint2 s_dlo[CPQR_CB];
+  __shared__ int4 s_g[CPQR_CB];
+  __shared__ int2 s_gn[CPQR_CB];
+  const longlong2* xq = reinterpret_cast<const longlong2*>(p.Z + (size_t)q * p.ld);
+  const int c0 = ch.c0 + warp, c1 = c0 + 8;
+  const bool on0 = c0 < ch.c1 && c0 != q && !(cur[c0] < 0), on1 = c1 < ch.c1 && c1 != q && !(cur[c1] < 0);
+  longlong2* a0 = reinterpret_cast<longlong2*>(p.Z + (size_t)c0 * p.ld);
+  longlong2* a1 = reinterpret_cast<longlong2*>(p.Z + (size_t)c1 * p.ld);
+  const longlong2 zero = make_longlong2(0, 0);
+  if (on0 || on1) {
+    const int e0 = on0 ? fx_shift(cur[c0], p.cexp[c0]) : 0, e1 = on1 ? fx_shift(cur[c1], p.cexp[c1]) : 0;
+    longlong2 d0 = zero, d1 = zero;
+#pragma unroll 2
+    for (int r = s + 1 + lane; r < W; r += 32) {
+      const longlong2 x = xq[r], y0 = on0 ? a0[r] : zero, y1 = on1 ? a1[r] : zero;
+      const longlong2 xs = make_longlong2(x.x << ev, x.y << ev);
+      fx_dot(d0, xs, y0, e0);
+      fx_dot(d1, xs, y1, e1);
+    }
+    longlong2 h;
+    uint2 l;
+    warp_sum_parts(d0.x, h.x, l.x); warp_sum_parts(d0.y, h.y, l.y);
+    if (lane == 0) { s_dot[warp] = h; s_dlo[warp] = l; }
+    warp_sum_parts(d1.x, h.x, l.x); warp_sum_parts(d1.y, h.y, l.y);
+    if (lane == 0) { s_dot[warp + 8] = h; s_dlo[warp + 8] = l; }
+  }
+  __syncthreads();
+  const int c = ch.c0 + tid;
+  const bool mine = tid < CPQR_CB && c < ch.c1 && c != q && !(cur[c] < 0);
+  if (mine)
+    fx_factor(pk.ctau, pk.csc, pk.sc, s_dot[tid], s_dlo[tid], fx_shift(cur[c], p.cexp[c]),
+              reinterpret_cast<longlong2*>(p.Z + s + (size_t)c * p.ld), s_g[tid], s_gn[tid]);
+  __syncthreads();
+  if (on0 || on1) {
+    const int4 g0 = s_g[warp], g1 = s_g[warp + 8];
+    const int2 n0 = s_gn[warp], n1 = s_gn[warp + 8];
+    FxSquares q0, q1;
+    int it = 0;
+#pragma unroll 2
+    for (int r = s + 1 + lane; r < W; r += 32) {
+      const longlong2 x = xq[r], xs = make_longlong2(x.x << ev, x.y << ev);
+      if (on0) { const longlong2 v = fx_update(a0[r], xs, g0, n0); a0[r] = v; q0.add(v); }
+      if (on1) { const longlong2 v = fx_update(a1[r], xs, g1, n1); a1[r] = v; q1.add(v); }
+      if ((++it & 7) == 0) { q0.fold(); q1.fold(); }
+    }
+    longlong2 w = q0.warp_total();
+    if (lane == 0) s_nrm[warp] = w;
+    w = q1.warp_total();
+    if (lane == 0) s_nrm[warp + 8] = w;
+  }
+  __syncthreads();
+  if (tid < CPQR_CB && c < ch.c1) nxt[c] = mine ? fx_norm2(s_nrm[tid], p.cexp[c]) : -1.0;
 }
 
 // Persistent grid (a multiple of the SM count): CTAs take chunks from a
 // per-launch counter, largest matrices first, until none is left.  TALL
 // compiles in the register-resident path for tall complex64 columns; without
 // it the kernel needs far fewer registers (more resident CTAs), which is what
-// the n x n triangles of the QR-first path want.
+// the n x n triangles of the QR-first path want.  The CTA that finishes a
+// matrix's last chunk picks the next step's pivot.
 template <typename C, bool TALL>
 __global__ void __launch_bounds__(256) k_cpqr_step(const CpqrProb<C>* __restrict__ P, const CpqrChunk* __restrict__ chunks,
                                                    int nchunk, int t, int* __restrict__ counter) {
-  __shared__ int s_ci;
+  __shared__ int s_ci, s_last;
   for (;;) {
     if (threadIdx.x == 0) s_ci = atomicAdd(counter, 1);
     __syncthreads();
@@ -243,7 +444,24 @@ __global__ void __launch_bounds__(256) k_cpqr_step(const CpqrProb<C>* __restrict
     if (ci >= nchunk) break;
     const CpqrChunk ch = chunks[ci];
     const CpqrProb<C> p = P[ch.id];
-    cpqr_chunk_step<C, TALL>(p, ch, t);
+    const int s = p.base + t;
+    // the matrix's pick is rewritten only after all of its chunks are done
+    const CpqrPick<C> pk = *p.pick;
+    if (s < p.target && pk.q >= 0) {
+      if constexpr (sizeof(C) == 16) cpqr_columns_fx(p, ch, s, pk);
+      else cpqr_columns<C, TALL>(p, ch, s, pk);
+      __threadfence();
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        s_last = atomicAdd(p.done, 1) == (p.n + CPQR_CB - 1) / CPQR_CB - 1;
+        if (s_last) *p.done = 0;
+      }
+      __syncthreads();
+      if (s_last) {
+        __threadfence();
+        cpqr_pick<C>(p, s + 1);
+      }
+    }
     __syncthreads();
   }
 }
@@ -257,7 +475,11 @@ __global__ void k_interp_gather(const InterpProb<C>* __restrict__ P) {
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k <= 0 || e >= (size_t)k * p.n) return;
   const int i = (int)(e % k), j = (int)(e / k);
-  const C v = p.Z[i + (size_t)p.perm[j] * p.ld];
+  C v = p.Z[i + (size_t)p.perm[j] * p.ld];
+  if constexpr (sizeof(C) == 16) {   // complex128 columns are in fixed point
+    const int e = p.cexp[p.perm[j]];
+    v = make_double2(fx_to(__double_as_longlong(v.x), e), fx_to(__double_as_longlong(v.y), e));
+  }
   if (j < k) p.R11[i + (size_t)j * k] = i < j ? v : (i == j ? p.rdiag[i] : czero<C>());
   else p.T[i + (size_t)(j - k) * p.ldt] = v;
 }
@@ -326,6 +548,12 @@ void cpqr_init_norms(const CpqrProb<C>* d_prob, const CpqrChunk* d_chunk, int nc
   k_init_norms<C><<<nchunk, 256, 0, st>>>(d_prob, d_chunk);
   pm_launch_count_add(1);
 }
+template <typename C>
+void cpqr_start(const CpqrProb<C>* d_prob, int nprob, cudaStream_t st) {
+  if (nprob <= 0) return;
+  k_cpqr_start<C><<<nprob, 256, 0, st>>>(d_prob);
+  pm_launch_count_add(1);
+}
 template <typename C, bool TALL>
 int cpqr_grid() {   // SMs x resident CTAs, once per instance
   static std::atomic<int> grid_cache{0};
@@ -346,7 +574,7 @@ void cpqr_step(const CpqrProb<C>* d_prob, const CpqrChunk* d_chunk, int nchunk, 
                cudaStream_t st, bool tall) {
   if (nchunk <= 0) return;
   KPROF_BEGIN(st);
-  if (tall) k_cpqr_step<C, true><<<std::min(cpqr_grid<C, true>(), nchunk), 256, 0, st>>>(d_prob, d_chunk, nchunk, t, d_counter);
+  if (tall && sizeof(C) == 8) k_cpqr_step<C, true><<<std::min(cpqr_grid<C, true>(), nchunk), 256, 0, st>>>(d_prob, d_chunk, nchunk, t, d_counter);
   else k_cpqr_step<C, false><<<std::min(cpqr_grid<C, false>(), nchunk), 256, 0, st>>>(d_prob, d_chunk, nchunk, t, d_counter);
   pm_launch_count_add(1);
   KPROF_END(st, kname<C>("cpqr_step", "cpqr_step32"), 0.0);   // work is added per level from the steps performed
@@ -374,6 +602,8 @@ void copy_batched(const CopyProb<S, D>* d_prob, int nprob, int max_elems, cudaSt
 }
 
 template void cpqr_init_norms<double2>(const CpqrProb<double2>*, const CpqrChunk*, int, cudaStream_t);
+template void cpqr_start<double2>(const CpqrProb<double2>*, int, cudaStream_t);
+template void cpqr_start<float2>(const CpqrProb<float2>*, int, cudaStream_t);
 template void cpqr_step<double2>(const CpqrProb<double2>*, const CpqrChunk*, int, int, int*, cudaStream_t, bool);
 template void interp_gather<double2>(const InterpProb<double2>*, int, size_t, cudaStream_t);
 template void scatter_interp<double2>(const ScatterProb<double2>*, int, int, cudaStream_t);

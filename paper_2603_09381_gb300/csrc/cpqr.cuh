@@ -6,6 +6,15 @@
 
 enum { CPQR_FIND_RANK = 0, CPQR_EXTEND = 1 };
 
+// Pivot and reflector of a matrix's next step (q < 0: none, the phase is over).
+template <typename C>
+struct CpqrPick {
+  int q;
+  int ev;                        // complex128: shift of the pivot column's integers
+  int reflect;                   // complex64: the pivot column is not zero
+  C ctau, csc, sc, beta;         // conj(tau), conj(1 / (alpha - beta)), 1 / (alpha - beta) (complex128: scaled), R_ss
+};
+
 template <typename C>
 struct CpqrProb {
   C* Z; int ld; int W; int n;    // W x n, factored in place (columns never move)
@@ -18,6 +27,9 @@ struct CpqrProb {
   C* rdiag;                      // rdiag[s] = R_ss
   int* rank;                     // -1 until the rank criterion stops the factorization
   double* ref;                   // |R_11|
+  CpqrPick<C>* pick;
+  int* done;                     // chunks finished in the running step
+  int* cexp;                     // complex128: column c holds integers of 2^(cexp[c] - 60)
 };
 
 struct CpqrChunk { int id; int c0; int c1; int first; };
@@ -28,6 +40,7 @@ struct InterpProb {              // T (k x (n-k)) = R11^{-1} R12 in pivot order
   const int* perm; const C* rdiag;
   C* T; int ldt;
   C* R11;                        // k x k workspace (leading dimension k): R11 in pivot order
+  const int* cexp;               // complex128: the columns' scales
 };
 
 template <typename C>
@@ -60,9 +73,10 @@ struct QrProb {
 // Panels [j0, j0 + QR_NB) of every matrix with j0 < n; max_tiles = the most
 // 32-column tiles right of a panel in any matrix.
 // cluster: CTAs per matrix (1, 2, 4, 8), or 0 for as many as fill the SMs (the
-// partial sums of a reflector, hence the last bits, depend on it).
+// partial sums of a reflector, hence the last bits, depend on it).  max_w
+// (complex128): the most rows of a matrix.
 template <typename C>
-void qr_panel(const QrProb<C>* d_prob, int nprob, int j0, cudaStream_t st, int cluster = 0);
+void qr_panel(const QrProb<C>* d_prob, int nprob, int j0, cudaStream_t st, int cluster = 0, int max_w = 0);
 // Trailing update of a complex128 panel (QR_NB reflectors, taus in T) on the
 // tensor cores at FP64 accuracy: V holds QR_NB x (n - QR_NB) entries of Y, Yp
 // ceil(n / 128) x mrb blocks of 128 x QR_NB partial sums, mrb = ceil(W / OZ_RB).
@@ -81,8 +95,12 @@ template <typename C>
 void qr_zero_lower(const QrProb<C>* d_prob, int nprob, int max_n, cudaStream_t st);
 
 void complete_perm(const PermFill* d_prob, int nprob, cudaStream_t st);
+// Initial norms; complex128 columns go to fixed point (cexp) here.
 template <typename C>
 void cpqr_init_norms(const CpqrProb<C>* d_prob, const CpqrChunk* d_chunk, int nchunk, cudaStream_t st);
+// Before the first step of a phase (mode, base, target set): its first pivot.
+template <typename C>
+void cpqr_start(const CpqrProb<C>* d_prob, int nprob, cudaStream_t st);
 // One elimination step (launch index t) of every active matrix; d_counter:
 // a zeroed int, distinct for every launch (chunk dispenser).  tall: some
 // complex64 matrix has W >= 2048 rows (selects the kernel instance with the

@@ -16,6 +16,7 @@
 // QR_RB-row block), their sum in block order times T^H, and C_b -= V_b Y per
 // (tile, block), so that the rows of a tall matrix spread over many CTAs.
 #include "cpqr.cuh"
+#include "fx.cuh"
 #include "prof.cuh"
 #include "oz.cuh"
 #include "oz_gemm.cuh"
@@ -291,55 +292,16 @@ __global__ void __maxnreg__(112) k_qr_panel(const QrProb<C>* __restrict__ P, int
 //             working precision, so each warp shifts its rows of y up to use
 //             all bits before the dot products; the shifts are taken out when
 //             the warps' sums meet in FP64.
-// A number x is split as x = h 2^30 + l, 0 <= l < 2^30; a product keeps
-// h h' + (h l' + l h') / 2^30 and leaves out l l' / 2^60 (below one unit;
-// its mean is added).
-struct Fx { int h, l; };
-__device__ __forceinline__ Fx fx(long long v) { return Fx{(int)(v >> 30), (int)v & 0x3FFFFFFF}; }
-__device__ __forceinline__ void fx_mac(long long& hh, long long& cr, Fx a, Fx b) {
-  hh += (long long)a.h * b.h;
-  cr += (long long)a.h * b.l;
-  cr += (long long)a.l * b.h;
-}
-constexpr long long FX_HALF = 1ll << 30;   // rounding and the mean of two dropped l l', before >> 30
-// a + g v, g given as (re, im, -im)
-__device__ __forceinline__ longlong2 fx_cfma(longlong2 a, Fx gr, Fx gi, Fx ngi, Fx vr, Fx vi) {
-  long long cr = FX_HALF, ci = FX_HALF;
-  fx_mac(a.x, cr, gr, vr);
-  fx_mac(a.x, cr, ngi, vi);
-  fx_mac(a.y, ci, gr, vi);
-  fx_mac(a.y, ci, gi, vr);
-  a.x += cr >> 30;
-  a.y += ci >> 30;
-  return a;
-}
-constexpr double FX_ONE = 1152921504606846976.0;   // 2^60
-// x 2^60 / 2^e2 rounded, for |x| < 2^(e2 - 2); subnormal x counts as zero
-__device__ __forceinline__ long long fx_from(double x, int e2) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const int ex = (int)(b >> 52) & 0x7FF, d = e2 + 1020 - ex;   // d >= 0
-  long long m = 0;
-  if (ex != 0 && d < 59) {
-    m = (long long)(((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 5);
-    if (d > 0) m = (m + (1ll << (d - 1))) >> d;
-  }
-  return (long long)b < 0 ? -m : m;
-}
-// the double nearest to a 2^(e2 - 60) (|e2| below 900)
-__device__ __forceinline__ double fx_to(long long a, int e2) {
-  const unsigned long long sign = (unsigned long long)a & 0x8000000000000000ull;
-  unsigned long long m = sign ? 0 - (unsigned long long)a : (unsigned long long)a;
-  const int lz = __clzll((long long)m);
-  m = ((m << (lz & 63)) + 1024) >> 11;   // 53 bits (a carry goes on into the exponent)
-  const unsigned long long r = ((unsigned long long)(unsigned)(1023 + 63 - lz - 60 + e2 - 1) << 52) + m;
-  return __longlong_as_double((long long)(a == 0 ? 0 : sign | r));
-}
-
+// (fx.cuh holds the arithmetic.)
 // A matrix's panel on a cluster; rows go to warps 8 at a time and stay there
 // for the whole panel.  T receives the taus.  Same reflectors and order as
 // k_qr_panel (LAPACK zlarfg phase convention).
 // Four threads per row: their 8 entries and 8 sums fit the registers.
-__global__ void __launch_bounds__(PT, 1) k_qr_panel_fx(const QrProb<double2>* __restrict__ P, int j0) {
+// SM: a CTA's rows (at most FX_SWEEPS per warp and thread) stay in dynamic
+// shared memory, leading dimension ldp; else in place, in L2.
+constexpr int FX_SWEEPS = 3;   // 3 x 128 rows x 32 columns: 192 KB
+template <bool SM>
+__global__ void __launch_bounds__(PT, 1) k_qr_panel_fx(const QrProb<double2>* __restrict__ P, int j0, int ldp) {
   typedef PanelSplit<4> L;
   constexpr int Q = L::Q, HB = L::HB, RW = L::RW;
   cg::cluster_group cluster = cg::this_cluster();
@@ -347,10 +309,14 @@ __global__ void __launch_bounds__(PT, 1) k_qr_panel_fx(const QrProb<double2>* __
   const QrProb<double2> p = P[blockIdx.x / csize];
   if (j0 >= p.n) return;   // the whole cluster (same matrix) leaves
   const int jb = min(QR_NB, p.n - j0), W = p.W;
+  extern __shared__ __align__(16) unsigned char fx_sm[];
   const size_t ld = p.ld;
-  longlong2* Zx = reinterpret_cast<longlong2*>(p.Z + (size_t)j0 * ld);   // the panel's columns as integers
+  // the panel's columns as integers: row r, sweep by sweep, at stored row x
+  longlong2* Zx = SM ? reinterpret_cast<longlong2*>(fx_sm) : reinterpret_cast<longlong2*>(p.Z + (size_t)j0 * ld);
+  const size_t ldx = SM ? ldp : ld;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q = lane / RW;
   const int rbeg = j0 + warp * RW + rank * L::PR, rstep = L::PR * csize;   // the warp's first row and stride
+  const int xbeg = SM ? warp * RW + lane % RW : rbeg + lane % RW, xstep = SM ? L::PR : rstep;
   constexpr int NV = 4 * QR_NB + 1;   // S (re, im), N, row c' (re, im)
   __shared__ double s_red[PT / 32][2 * QR_NB + 1];
   __shared__ double s_part[2][NV];    // this CTA's partial sums, by pass parity
@@ -399,14 +365,14 @@ __global__ void __launch_bounds__(PT, 1) k_qr_panel_fx(const QrProb<double2>* __
       s_exp[tid] = e + 2;
     }
     __syncthreads();
-    for (int r = rbeg + lane % RW; r < W; r += rstep)
+    for (int r = rbeg + lane % RW, x = xbeg; r < W; r += rstep, x += xstep)
 #pragma unroll
       for (int k = 0; k < HB; ++k)
         if (Q * k + q < jb) {
           const double2 z = p.Z[r + (size_t)(j0 + Q * k + q) * ld];
           const int e2 = s_exp[Q * k + q];
           const bool ok = Q * k + q < s_bad;
-          Zx[r + (size_t)(Q * k + q) * ld] = make_longlong2(ok ? fx_from(z.x, e2) : 0, ok ? fx_from(z.y, e2) : 0);
+          Zx[x + (size_t)(Q * k + q) * ldx] = make_longlong2(ok ? fx_from(z.x, e2) : 0, ok ? fx_from(z.y, e2) : 0);
         }
     __syncwarp();
   }
@@ -422,11 +388,11 @@ __global__ void __launch_bounds__(PT, 1) k_qr_panel_fx(const QrProb<double2>* __
       ev = s_ev;
     }
     unsigned long long any = 0;
-    for (int r0 = rbeg; r0 < W; r0 += rstep) {   // the same steps for the whole warp
+    for (int r0 = rbeg, xr = xbeg; r0 < W; r0 += rstep, xr += xstep) {   // the same steps for the whole warp
       const int r = r0 + lane % RW;
       const bool act = r < W && r >= (ja >= 0 ? ca : cn);
-      const longlong2 x = act && ja >= 0 ? Zx[r + (size_t)ja * ld] : make_longlong2(0, 0);
-      longlong2 y = act && jn < jb ? Zx[r + (size_t)jn * ld] : make_longlong2(0, 0);
+      const longlong2 x = act && ja >= 0 ? Zx[xr + (size_t)ja * ldx] : make_longlong2(0, 0);
+      longlong2 y = act && jn < jb ? Zx[xr + (size_t)jn * ldx] : make_longlong2(0, 0);
       __syncwarp();   // the row's threads have read both before one of them writes
       if (!act) continue;
       if (ja >= 0) {
@@ -435,14 +401,14 @@ __global__ void __launch_bounds__(PT, 1) k_qr_panel_fx(const QrProb<double2>* __
           v = make_longlong2(1ll << 60, 0);
         } else {
           v = fx_cfma(make_longlong2(0, 0), scr, sci, nsci, fx(x.x << ev), fx(x.y << ev));
-          v.x <<= 2; v.y <<= 2;
-          if (q == 0) Zx[r + (size_t)ja * ld] = v;
+          v.x <<= 1; v.y <<= 1;
+          if (q == 0) Zx[xr + (size_t)ja * ldx] = v;
         }
         if (jn < jb) {
           const int4 g = s_g[jn];
           const int2 gn = s_gn[jn];
           y = fx_cfma(y, Fx{g.x, g.y}, Fx{g.z, g.w}, Fx{gn.x, gn.y}, fx(v.x), fx(v.y));
-          if (q == 1) Zx[r + (size_t)jn * ld] = y;
+          if (q == 1) Zx[xr + (size_t)jn * ldx] = y;
         }
       }
       if (jn < jb && r >= cn) any |= (unsigned long long)(y.x ^ (y.x >> 63)) | (unsigned long long)(y.y ^ (y.y >> 63));
@@ -457,14 +423,14 @@ __global__ void __launch_bounds__(PT, 1) k_qr_panel_fx(const QrProb<double2>* __
     longlong2 S[HB];
 #pragma unroll
     for (int k = 0; k < HB; ++k) S[k] = make_longlong2(0, 0);
-    for (int r = rbeg + lane % RW; r < W; r += rstep) {
+    for (int r = rbeg + lane % RW, xr = xbeg; r < W; r += rstep, xr += xstep) {
       if (r < (ja >= 0 ? ca : cn)) continue;
       longlong2 a[HB];
 #pragma unroll
       for (int k = 0; k < HB; ++k)
-        if (Q * k + Q - 1 > jn && Q * k + q > jn && Q * k + q < jb) a[k] = Zx[r + (size_t)(Q * k + q) * ld];
-      const longlong2 v = ja < 0 ? make_longlong2(0, 0) : r == ca ? make_longlong2(1ll << 60, 0) : Zx[r + (size_t)ja * ld];
-      const longlong2 y0 = Zx[r + (size_t)jn * ld];
+        if (Q * k + Q - 1 > jn && Q * k + q > jn && Q * k + q < jb) a[k] = Zx[xr + (size_t)(Q * k + q) * ldx];
+      const longlong2 v = ja < 0 ? make_longlong2(0, 0) : r == ca ? make_longlong2(1ll << 60, 0) : Zx[xr + (size_t)ja * ldx];
+      const longlong2 y0 = Zx[xr + (size_t)jn * ldx];
       const longlong2 y = ew >= 0 ? make_longlong2(y0.x << ew, y0.y << ew) : make_longlong2(y0.x >> -ew, y0.y >> -ew);
       const Fx vr = fx(v.x), vi = fx(v.y), yr = fx(y.x), yi = fx(y.y), nyi = fx(-y.y);
       if (r >= cn && q == 0) {
@@ -481,7 +447,7 @@ __global__ void __launch_bounds__(PT, 1) k_qr_panel_fx(const QrProb<double2>* __
             const int4 g = s_g[Q * k + q];
             const int2 gn = s_gn[Q * k + q];
             a[k] = fx_cfma(a[k], Fx{g.x, g.y}, Fx{g.z, g.w}, Fx{gn.x, gn.y}, vr, vi);
-            Zx[r + (size_t)(Q * k + q) * ld] = a[k];
+            Zx[xr + (size_t)(Q * k + q) * ldx] = a[k];
           }
           if (r == cn) {
             s_row[Q * k + q] = a[k];
@@ -539,22 +505,13 @@ __global__ void __launch_bounds__(PT, 1) k_qr_panel_fx(const QrProb<double2>* __
     if (warp == 0) {
       // reflector of column jn, in units of its scale; lane k: the factor of column k
       const double2 alpha = make_double2(s_tot[2 * QR_NB + 1 + 2 * jn], s_tot[2 * QR_NB + 2 + 2 * jn]);
-      const double xnorm = sqrt(s_tot[2 * QR_NB]);
-      double2 tau = czero<double2>(), sc = czero<double2>();
-      double beta = 0;
-      int ex = 0;
-      if (xnorm > 0) {
-        beta = -copysign(xnorm, alpha.x);
-        const double2 bm = make_double2(beta, 0.0);
-        tau = cdiv(bm - alpha, bm);
-        sc = cdiv(make_double2(1.0, 0.0), alpha - bm);
-        ex = (int)((__double2hiint(xnorm) >> 20) & 0x7FF) - 1022;   // xnorm in [2^(ex - 1), 2^ex), ex <= -1
-        ex = max(ex, -60);
-      }
+      double beta;
+      double2 tau, sc;
+      fx_reflector(alpha, s_tot[2 * QR_NB], beta, tau, sc);
       if (lane == 0) {
-        // v = x sc = 4 (x 2^ev) (sc 2^-ev / 4) with x 2^ev below 1/2 and |sc| 2^-ev <= 4
-        const int ev = -1 - ex;
-        const double u = 0.25 * FX_ONE * __longlong_as_double((long long)(1023 - ev) << 52);
+        // v = x sc = 2 (x 2^ev) (sc 2^-ev / 2) with x 2^ev below 1 and |sc| 2^-ev at most 2
+        const int ev = fx_shift(s_tot[2 * QR_NB], 0);
+        const double u = 0.5 * FX_ONE * __longlong_as_double((long long)(1023 - ev) << 52);
         s_sc = make_longlong2(__double2ll_rn(sc.x * u), __double2ll_rn(sc.y * u));
         s_ev = ev;
         s_beta[jn] = beta;
@@ -573,12 +530,12 @@ __global__ void __launch_bounds__(PT, 1) k_qr_panel_fx(const QrProb<double2>* __
     __syncthreads();
   }
   // back to doubles: v below the diagonal, the scaled R above it
-  for (int r = rbeg + lane % RW; r < W; r += rstep)
+  for (int r = rbeg + lane % RW, x = xbeg; r < W; r += rstep, x += xstep)
 #pragma unroll
     for (int k = 0; k < HB; ++k) {
       const int col = Q * k + q;
       if (col >= jb) continue;
-      const longlong2 a = Zx[r + (size_t)col * ld];
+      const longlong2 a = Zx[x + (size_t)col * ldx];
       const int e2 = r > j0 + col ? 0 : s_exp[col];
       double2 z = make_double2(fx_to(a.x, e2), fx_to(a.y, e2));
       if (r == j0 + col) z = make_double2(ldexp(s_beta[col], e2), 0.0);
@@ -978,7 +935,7 @@ __global__ void k_qr_zero_lower(const QrProb<C>* __restrict__ P) {
 }  // namespace
 
 template <typename C>
-void qr_panel(const QrProb<C>* d_prob, int nprob, int j0, cudaStream_t st, int cluster) {
+void qr_panel(const QrProb<C>* d_prob, int nprob, int j0, cudaStream_t st, int cluster, int max_w) {
   if (nprob <= 0) return;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
@@ -1001,8 +958,20 @@ void qr_panel(const QrProb<C>* d_prob, int nprob, int j0, cudaStream_t st, int c
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   KPROF_BEGIN(st);
-  if constexpr (std::is_same<C, double2>::value) cudaLaunchKernelEx(&cfg, k_qr_panel_fx, d_prob, j0);
-  else cudaLaunchKernelEx(&cfg, k_qr_panel<C>, d_prob, j0);
+  if constexpr (std::is_same<C, double2>::value) {
+    const int sweeps = (max_w - j0 + PanelSplit<4>::PR * cs - 1) / (PanelSplit<4>::PR * cs), ldp = sweeps * PanelSplit<4>::PR;
+    if (sweeps <= FX_SWEEPS) {
+      cfg.dynamicSmemBytes = (size_t)ldp * QR_NB * sizeof(double2);
+      // the same value every time: idempotent across threads and devices
+      cudaFuncSetAttribute(k_qr_panel_fx<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)(FX_SWEEPS * PanelSplit<4>::PR * QR_NB * sizeof(double2)));
+      cudaLaunchKernelEx(&cfg, k_qr_panel_fx<true>, d_prob, j0, ldp);
+    } else {
+      cudaLaunchKernelEx(&cfg, k_qr_panel_fx<false>, d_prob, j0, 0);
+    }
+  } else {
+    cudaLaunchKernelEx(&cfg, k_qr_panel<C>, d_prob, j0);
+  }
   pm_launch_count_add(1);
   KPROF_END(st, kname<C>("qr_panel", "qr_panel32"), 0.0);
 }
@@ -1050,8 +1019,8 @@ void qr_zero_lower(const QrProb<C>* d_prob, int nprob, int max_n, cudaStream_t s
   pm_launch_count_add(1);
 }
 
-template void qr_panel<float2>(const QrProb<float2>*, int, int, cudaStream_t, int);
-template void qr_panel<double2>(const QrProb<double2>*, int, int, cudaStream_t, int);
+template void qr_panel<float2>(const QrProb<float2>*, int, int, cudaStream_t, int, int);
+template void qr_panel<double2>(const QrProb<double2>*, int, int, cudaStream_t, int, int);
 template void qr_zero_lower<double2>(const QrProb<double2>*, int, int, cudaStream_t);
 template void qr_update<float2>(const QrProb<float2>*, int, int, int, int, cudaStream_t, int*, int, bool);
 template void qr_zero_lower<float2>(const QrProb<float2>*, int, int, cudaStream_t);

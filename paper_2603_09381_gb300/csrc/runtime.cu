@@ -1067,7 +1067,7 @@ void sqnorm_batch(const std::vector<SqNormProb>& probs, Arena& scr, cudaStream_t
 // rows) are reduced to their triangle first; a panel runs on a cluster of 8
 // CTAs above this many rows, else of 4.
 constexpr int QR_FIRST_MIN_N64 = 80;
-constexpr int QR_CLUSTER8_W64 = 2048;
+constexpr int QR_CLUSTER8_W64 = 1536;
 
 // Held-out proxy check bound: an ID passes while ||H_J - H_S T|| <= PROXY_CHECK_BOUND tol ||H||.
 constexpr double PROXY_CHECK_BOUND = 200.0;
@@ -1353,8 +1353,8 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
         for (auto& x : all) maxW = std::max(maxW, x.W);
         auto* dqp = upload(scr, all, st);
         for (int j0 = 0; j0 < maxn; j0 += QR_NB) {
-          qr_panel<C>(dqp, n4, j0, st, 4);
-          qr_panel<C>(dqp + n4, (int)all.size() - n4, j0, st, 8);
+          qr_panel<C>(dqp, n4, j0, st, 4, std::min(maxW, QR_CLUSTER8_W64));
+          qr_panel<C>(dqp + n4, (int)all.size() - n4, j0, st, 8, maxW);
           qr_update_oz(dqp, (int)all.size(), j0, maxn, maxW, g_oz_err, st);
         }
         qr_zero_lower<C>(dqp, (int)all.size(), maxn, st);
@@ -1487,6 +1487,10 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
   C* rdiag = scr.get<C>(std::max(total_n, 1));
   int* rank = scr.get<int>(nid);
   double* ref = scr.get<double>(nid);
+  CpqrPick<C>* pick = scr.get<CpqrPick<C>>(nid);
+  int* done = scr.get<int>(nid);
+  int* cexp = scr.get<int>(std::max(total_n, 1));
+  CK(cudaMemsetAsync(ref, 0, nid * sizeof(double), st));
   CK(cudaMemsetAsync(rank, 0xff, nid * sizeof(int), st));
   CK(cudaMemsetAsync(perm, 0, std::max(total_n, 1) * sizeof(int), st));
   std::vector<CpqrProb<C>> cp(nid);
@@ -1495,7 +1499,8 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
   for (int i = 0; i < nid; ++i) {
     int tgt = std::min(We[i], nn[i]);
     cp[i] = CpqrProb<C>{Z[i], W[i], We[i], nn[i], tol, CPQR_FIND_RANK, 0, tgt,
-                        norm2 + 2 * (size_t)noff[i], perm + noff[i], rdiag + noff[i], rank + i, ref + i};
+                        norm2 + 2 * (size_t)noff[i], perm + noff[i], rdiag + noff[i], rank + i, ref + i, pick + i,
+                        done + i, cexp + noff[i]};
     maxT = std::max(maxT, tgt);
     for (int c0 = 0; c0 < nn[i]; c0 += CPQR_CB) chunks.push_back(CpqrChunk{i, c0, std::min(c0 + CPQR_CB, nn[i]), c0 == 0});
   }
@@ -1509,6 +1514,7 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
   auto* dch = upload(scr, chunks, st);
   const int nch = (int)chunks.size();
   cpqr_init_norms<C>(dcp, dch, nch, st);
+  cpqr_start<C>(dcp, nid, st);
   std::vector<int> hr(nid);
   // With predicted ranks, run the predicted number of steps (+1, where the stop
   // test of the last rank happens) before the first check; otherwise check
@@ -1572,6 +1578,7 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
   }
   if (maxExt > 0) {
     dcp = upload(scr, cp, st);
+    cpqr_start<C>(dcp, nid, st);
     for (int t = 0; t < maxExt; ++t) cpqr_step<C>(dcp, dch, nch, t, ctr + maxT + t, st, tall);
     for (const auto& J : jobs) J.F->stats.cpqr_launches += maxExt;
     CK(cudaGetLastError());
@@ -1630,7 +1637,7 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
     if (k <= 0 || n - k <= 0 || zero_in[i]) continue;
     T[i] = scr.get<C>((size_t)k * (n - k));
     C* r11 = scr.get<C>((size_t)k * k);
-    ip.push_back(InterpProb<C>{Z[i], W[i], n, k, perm + noff[i], rdiag + noff[i], T[i], k, r11});
+    ip.push_back(InterpProb<C>{Z[i], W[i], n, k, perm + noff[i], rdiag + noff[i], T[i], k, r11, cexp + noff[i]});
     ts.push_back(SolveProb<C>{r11, k, k, nullptr, T[i], k, n - k});
     maxcols = std::max(maxcols, n - k);
     maxk = std::max(maxk, k);
