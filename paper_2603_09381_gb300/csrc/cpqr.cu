@@ -466,6 +466,213 @@ __global__ void __launch_bounds__(256) k_cpqr_step(const CpqrProb<C>* __restrict
   }
 }
 
+// ---- all steps of a small matrix in one launch ------------------------------------------
+// A matrix whose columns fit the shared memory of a cluster (up to 8 CTAs) runs
+// its whole phase there: column c in CTA c % cs, a warp per column.  Per step
+// one cluster barrier, after which every CTA reads all norms and the pivot
+// column from the others' shared memory and forms the same reflector: a few
+// microseconds, against a launch, a chunk's descriptors and the L2 round trips
+// of k_cpqr_step (20 us and more however small the matrix).  Per column the
+// arithmetic is that of k_cpqr_step; in complex128 the sums are exact, so the
+// bits are the same too.
+constexpr int RT = 512;
+constexpr int RES_MAX_N = 512;      // a thread per column when the norms are compared
+constexpr int RES_MAX_COLS = 192;   // local columns
+constexpr size_t RES_SMEM = 200 * 1024;
+
+template <typename C>
+__global__ void __launch_bounds__(RT, 1) k_cpqr_resident(const CpqrProb<C>* __restrict__ P, const int* __restrict__ list) {
+  namespace cg = cooperative_groups;
+  typedef typename real_of<C>::type R;
+  typedef unsigned long long u64;
+  constexpr bool FX = sizeof(C) == 16;
+  constexpr int NW = RT / 32;
+  extern __shared__ __align__(16) unsigned char rs_sm[];
+  cg::cluster_group cluster = cg::this_cluster();
+  const int cs = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const CpqrProb<C> p = P[list[blockIdx.x / cs]];
+  const int n = p.n, W = p.W, ncl = n > rank ? (n - rank + cs - 1) / cs : 0;   // this CTA's columns rank, rank + cs, ..
+  C* s_x = reinterpret_cast<C*>(rs_sm);                  // the pivot column (complex128: shifted integers)
+  C* s_c = s_x + W;                                      // columns, leading dimension W
+  __shared__ double s_norm[2][RES_MAX_COLS];             // trailing norms by step parity (-1: pivoted)
+  __shared__ u64 s_k[NW];
+  __shared__ int s_i[NW];
+  __shared__ C s_ctau, s_csc, s_sc;
+  __shared__ int s_ev;
+  __shared__ longlong2 s_dot[FX ? RES_MAX_COLS : 1], s_nrm[FX ? RES_MAX_COLS : 1];
+  __shared__ uint2 s_dlo[FX ? RES_MAX_COLS : 1];
+  __shared__ int4 s_g[FX ? RES_MAX_COLS : 1];
+  __shared__ int2 s_gn[FX ? RES_MAX_COLS : 1];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  for (int l = warp; l < ncl; l += NW) {
+    const C* src = p.Z + (size_t)(rank + cs * l) * p.ld;
+    for (int r = lane; r < W; r += 32) s_c[(size_t)l * W + r] = src[r];
+  }
+  for (int l = tid; l < ncl; l += RT) s_norm[p.base & 1][l] = p.norm2[(p.base & 1) * n + rank + cs * l];
+  double ref = p.mode == CPQR_FIND_RANK && p.base > 0 ? *p.ref : 0.0;
+  int s = p.base;
+  for (; s < p.target; ++s) {
+    const int par = s & 1;
+    cluster.sync();   // the norms of step s are complete everywhere
+    // the largest norm, then the lowest column within the tie band
+    u64 key = 0;
+    if (tid < n) {
+      const u64 b = (u64)__double_as_longlong(cluster.map_shared_rank(&s_norm[par][0], tid % cs)[tid / cs]);
+      key = b <= 0x7FF0000000000000ull ? b + 1 : 0;   // 0: pivoted or not a number
+    }
+    const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(key >> 32));
+    const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(key >> 32) == hi ? (unsigned)key : 0u);
+    if (lane == 0) s_k[warp] = ((u64)hi << 32) | lo;
+    __syncthreads();
+    u64 k = s_k[0];
+#pragma unroll
+    for (int w = 1; w < NW; ++w) k = s_k[w] > k ? s_k[w] : k;
+    const double mx = k ? __longlong_as_double((long long)(k - 1)) : 0.0;
+    const u64 band = k ? (u64)__double_as_longlong((1.0 - TIE) * mx) + 1 : ~0ull;
+    const int qw = __reduce_min_sync(0xffffffffu, key >= band ? tid : RES_MAX_N);
+    if (lane == 0) s_i[warp] = qw;
+    __syncthreads();
+    int q = s_i[0];
+#pragma unroll
+    for (int w = 1; w < NW; ++w) q = min(q, s_i[w]);
+    if (!k || q >= n) break;   // no unpivoted column left (the same in every CTA)
+    if (p.mode == CPQR_FIND_RANK) {
+      if (s == 0) {
+        ref = sqrt(mx);
+        if (rank == 0 && tid == 0) *p.ref = ref;
+      }
+      if (!(sqrt(mx) > p.tol * ref)) {
+        if (rank == 0 && tid == 0) *p.rank = s;
+        break;
+      }
+    }
+    const int qr = q % cs, ql = q / cs;
+    const double nq = cluster.map_shared_rank(&s_norm[par][0], qr)[ql];
+    const C* xq = cluster.map_shared_rank(s_c, qr) + (size_t)ql * W;
+    int ev = 0;
+    if constexpr (FX) {
+      const int eq = p.cexp[q];
+      const double nn = ldexp(nq, -2 * eq);   // in units of the column's scale
+      ev = fx_shift(nq, eq);
+      for (int r = s + 1 + tid; r < W; r += RT) {
+        const longlong2 v = *reinterpret_cast<const longlong2*>(xq + r);
+        *reinterpret_cast<longlong2*>(s_x + r) = make_longlong2(v.x << ev, v.y << ev);
+      }
+      if (warp == NW - 1) {
+        const longlong2 a = *reinterpret_cast<const longlong2*>(xq + s);
+        double beta;
+        double2 tau, sc;
+        fx_reflector(make_double2(fx_to(a.x, 0), fx_to(a.y, 0)), nn, beta, tau, sc);
+        if (lane == 0) {
+          s_ctau = conj(tau);
+          s_sc = __longlong_as_double((long long)(1023 - ev) << 52) * sc;
+          s_csc = __longlong_as_double((long long)(1023 - 60 - ev) << 52) * conj(sc);
+          if (rank == 0) {
+            p.rdiag[s] = make_double2(ldexp(beta != 0 ? beta : 0x1p-58, eq), 0.0);
+            p.perm[s] = q;
+          }
+        }
+      }
+    } else {
+      for (int r = s + 1 + tid; r < W; r += RT) s_x[r] = xq[r];
+      if (warp == NW - 1) {
+        const C alpha = xq[s];
+        const R xnorm = (R)sqrt(nq);
+        const R beta = -copysign(xnorm, alpha.x);
+        C tau = czero<C>(), sc = czero<C>();
+        if (xnorm > 0) {
+          const C bm = mk(beta, (R)0);
+          tau = cdiv(bm - alpha, bm);
+          sc = cdiv(mk((R)1, (R)0), alpha - bm);
+        }
+        if (lane == 0) {
+          s_ctau = conj(tau);
+          s_sc = sc;
+          s_csc = conj(sc);
+          if (rank == 0) {
+            p.rdiag[s] = mk(beta, (R)0);
+            p.perm[s] = q;
+          }
+        }
+      }
+    }
+    __syncthreads();
+    auto active = [&](int l) { return !(s_norm[par][l] < 0) && rank + cs * l != q; };
+    if constexpr (FX) {
+      const longlong2* x = reinterpret_cast<const longlong2*>(s_x);
+      for (int l = warp; l < ncl; l += NW) {
+        if (!active(l)) continue;
+        const longlong2* a = reinterpret_cast<const longlong2*>(s_c + (size_t)l * W);
+        const int ea = fx_shift(s_norm[par][l], p.cexp[rank + cs * l]);
+        longlong2 d = make_longlong2(0, 0);
+        for (int r = s + 1 + lane; r < W; r += 32) fx_dot(d, x[r], a[r], ea);
+        longlong2 h;
+        uint2 lw;
+        warp_sum_parts(d.x, h.x, lw.x);
+        warp_sum_parts(d.y, h.y, lw.y);
+        if (lane == 0) { s_dot[l] = h; s_dlo[l] = lw; }
+      }
+      __syncthreads();
+      for (int l = tid; l < ncl; l += RT)
+        if (active(l))
+          fx_factor(s_ctau, s_csc, s_sc, s_dot[l], s_dlo[l], fx_shift(s_norm[par][l], p.cexp[rank + cs * l]),
+                    reinterpret_cast<longlong2*>(s_c + (size_t)l * W + s), s_g[l], s_gn[l]);
+      __syncthreads();
+      for (int l = warp; l < ncl; l += NW) {
+        if (!active(l)) continue;
+        longlong2* a = reinterpret_cast<longlong2*>(s_c + (size_t)l * W);
+        const int4 g = s_g[l];
+        const int2 gn = s_gn[l];
+        FxSquares sq;
+        int it = 0;
+        for (int r = s + 1 + lane; r < W; r += 32) {
+          a[r] = fx_update(a[r], x[r], g, gn);
+          sq.add(a[r]);
+          if ((++it & 7) == 0) sq.fold();
+        }
+        const longlong2 w = sq.warp_total();
+        if (lane == 0) s_nrm[l] = w;
+      }
+      __syncthreads();
+      for (int l = tid; l < ncl; l += RT)
+        s_norm[par ^ 1][l] = active(l) ? fx_norm2(s_nrm[l], p.cexp[rank + cs * l]) : -1.0;
+    } else {
+      const C ctau = s_ctau, sc = s_sc, csc = s_csc;
+      for (int l = warp; l < ncl; l += NW) {
+        if (!active(l)) {
+          if (lane == 0) s_norm[par ^ 1][l] = -1.0;
+          continue;
+        }
+        C* a = s_c + (size_t)l * W;
+        C dot = czero<C>();
+        for (int r = s + 1 + lane; r < W; r += 32) cfma_conj(dot, s_x[r], a[r]);
+        dot.x = warp_sum(dot.x);
+        dot.y = warp_sum(dot.y);
+        const C a_s = a[s];
+        __syncwarp();
+        const C f = ctau * (a_s + csc * dot), fs = f * sc;   // as in cpqr_columns
+        if (lane == 0) a[s] = a_s - f;
+        R e = 0;
+        for (int r = s + 1 + lane; r < W; r += 32) {
+          C v = a[r];
+          cfms(v, fs, s_x[r]);
+          a[r] = v;
+          e += abs2(v);
+        }
+        e = warp_sum(e);
+        if (lane == 0) s_norm[par ^ 1][l] = (double)e;
+      }
+    }
+  }
+  cluster.sync();   // no CTA leaves while another may still read its norms or columns
+  // the norms of step s and the columns, for a later phase
+  for (int l = tid; l < ncl; l += RT) p.norm2[(s & 1) * n + rank + cs * l] = s_norm[s & 1][l];
+  for (int l = warp; l < ncl; l += NW) {
+    C* dst = p.Z + (size_t)(rank + cs * l) * p.ld;
+    for (int r = lane; r < W; r += 32) dst[r] = s_c[(size_t)l * W + r];
+  }
+}
+
 // R11 (k x k, upper, diagonal from rdiag, zero below) and R12 (into T) in
 // pivot order, both with leading dimension k.
 template <typename C>
@@ -554,6 +761,44 @@ void cpqr_start(const CpqrProb<C>* d_prob, int nprob, cudaStream_t st) {
   k_cpqr_start<C><<<nprob, 256, 0, st>>>(d_prob);
   pm_launch_count_add(1);
 }
+template <typename C>
+int cpqr_resident_ctas(int n, int W) {
+  for (int cs = 1; cs <= 8; cs *= 2) {
+    const size_t cols = (n + cs - 1) / cs;
+    if (n <= RES_MAX_N && cols <= RES_MAX_COLS && (cols + 1) * W * sizeof(C) <= RES_SMEM) return cs;
+  }
+  return 0;
+}
+template <typename C>
+void cpqr_resident(const CpqrProb<C>* d_prob, const int* d_list, const int* h_n, const int* h_w, int count, int cs,
+                   cudaStream_t st) {
+  if (count <= 0) return;
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int max_n = *std::max_element(h_n, h_n + count);
+  while (cs < 8 && (long)count * cs * 2 <= sms && cs * 32 <= max_n) cs *= 2;   // spread a few matrices wider
+  size_t bytes = 0;
+  for (int i = 0; i < count; ++i) bytes = std::max(bytes, ((size_t)(h_n[i] + cs - 1) / cs + 1) * h_w[i] * sizeof(C));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(count * cs);
+  cfg.blockDim = dim3(RT);
+  cfg.dynamicSmemBytes = bytes;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cs;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  // the same value every time: idempotent across threads and devices
+  cudaFuncSetAttribute(k_cpqr_resident<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RES_SMEM);
+  KPROF_BEGIN(st);
+  cudaLaunchKernelEx(&cfg, k_cpqr_resident<C>, d_prob, d_list);
+  pm_launch_count_add(1);
+  KPROF_END(st, kname<C>("cpqr_resident", "cpqr_resident32"), 0.0);
+}
 template <typename C, bool TALL>
 int cpqr_grid() {   // SMs x resident CTAs, once per instance
   static std::atomic<int> grid_cache{0};
@@ -602,6 +847,10 @@ void copy_batched(const CopyProb<S, D>* d_prob, int nprob, int max_elems, cudaSt
 }
 
 template void cpqr_init_norms<double2>(const CpqrProb<double2>*, const CpqrChunk*, int, cudaStream_t);
+template int cpqr_resident_ctas<double2>(int, int);
+template int cpqr_resident_ctas<float2>(int, int);
+template void cpqr_resident<double2>(const CpqrProb<double2>*, const int*, const int*, const int*, int, int, cudaStream_t);
+template void cpqr_resident<float2>(const CpqrProb<float2>*, const int*, const int*, const int*, int, int, cudaStream_t);
 template void cpqr_start<double2>(const CpqrProb<double2>*, int, cudaStream_t);
 template void cpqr_start<float2>(const CpqrProb<float2>*, int, cudaStream_t);
 template void cpqr_step<double2>(const CpqrProb<double2>*, const CpqrChunk*, int, int, int*, cudaStream_t, bool);

@@ -1066,6 +1066,7 @@ void sqnorm_batch(const std::vector<SqNormProb>& probs, Arena& scr, cudaStream_t
 // complex128 ID inputs with at least this many candidates (and twice as many
 // rows) are reduced to their triangle first; a panel runs on a cluster of 8
 // CTAs above this many rows, else of 4.
+constexpr int RESIDENT_WAVES_64 = 4, RESIDENT_WAVES_32 = 8;
 constexpr int QR_FIRST_MIN_N64 = 80;
 constexpr int QR_CLUSTER8_W64 = 1536;
 
@@ -1494,27 +1495,55 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
   CK(cudaMemsetAsync(rank, 0xff, nid * sizeof(int), st));
   CK(cudaMemsetAsync(perm, 0, std::max(total_n, 1) * sizeof(int), st));
   std::vector<CpqrProb<C>> cp(nid);
-  std::vector<CpqrChunk> chunks;
+  std::vector<CpqrChunk> chunks, init;
   int maxT = 0;
+  // matrices small enough run all their steps in one launch (k_cpqr_resident)
+  // while their CTAs take few enough waves of the SMs; with more of them the
+  // step kernel's fuller use of the SMs wins
+  std::vector<int> rcs(nid, 0);
+  long rctas = 0;
+  for (int i = 0; i < nid; ++i) {
+    if (nn[i] > 0) rcs[i] = cpqr_resident_ctas<C>(nn[i], We[i]);
+    rctas += rcs[i];
+  }
+  int sms = 0;
+  CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, current_device()));
+  if (rctas > (long)sms * (sizeof(C) == sizeof(double2) ? RESIDENT_WAVES_64 : RESIDENT_WAVES_32)) std::fill(rcs.begin(), rcs.end(), 0);
   for (int i = 0; i < nid; ++i) {
     int tgt = std::min(We[i], nn[i]);
     cp[i] = CpqrProb<C>{Z[i], W[i], We[i], nn[i], tol, CPQR_FIND_RANK, 0, tgt,
                         norm2 + 2 * (size_t)noff[i], perm + noff[i], rdiag + noff[i], rank + i, ref + i, pick + i,
                         done + i, cexp + noff[i]};
-    maxT = std::max(maxT, tgt);
-    for (int c0 = 0; c0 < nn[i]; c0 += CPQR_CB) chunks.push_back(CpqrChunk{i, c0, std::min(c0 + CPQR_CB, nn[i]), c0 == 0});
+    if (!rcs[i]) maxT = std::max(maxT, tgt);
+    for (int c0 = 0; c0 < nn[i]; c0 += CPQR_CB) {
+      const CpqrChunk ch{i, c0, std::min(c0 + CPQR_CB, nn[i]), c0 == 0};
+      init.push_back(ch);
+      if (!rcs[i]) chunks.push_back(ch);
+    }
   }
+  auto run_resident = [&](const CpqrProb<C>* d) {   // the phase of the resident matrices that have steps to do
+    for (int cs = 1; cs <= 8; cs *= 2) {
+      std::vector<int> list, hn, hw;
+      for (int i = 0; i < nid; ++i)
+        if (rcs[i] == cs && cp[i].target > cp[i].base) { list.push_back(i); hn.push_back(nn[i]); hw.push_back(We[i]); }
+      if (list.empty()) continue;
+      const int* dl = upload(scr, list, st);
+      cpqr_resident<C>(d, dl, hn.data(), hw.data(), (int)list.size(), cs, st);
+    }
+    CK(cudaGetLastError());
+  };
   // tallest matrices first: their chunks carry the most work per step
   std::stable_sort(chunks.begin(), chunks.end(), [&](const CpqrChunk& a, const CpqrChunk& b) { return We[a.id] > We[b.id]; });
   bool tall = false;   // any complex64 input pivoted on >= 2048 rows
-  for (int i = 0; i < nid; ++i) tall = tall || We[i] >= 2048;
+  for (int i = 0; i < nid; ++i) tall = tall || (!rcs[i] && We[i] >= 2048);
   int* ctr = scr.get<int>(2 * (size_t)maxT + 2);
   CK(cudaMemsetAsync(ctr, 0, (2 * (size_t)maxT + 2) * sizeof(int), st));
   auto* dcp = upload(scr, cp, st);
   auto* dch = upload(scr, chunks, st);
   const int nch = (int)chunks.size();
-  cpqr_init_norms<C>(dcp, dch, nch, st);
-  cpqr_start<C>(dcp, nid, st);
+  cpqr_init_norms<C>(dcp, upload(scr, init, st), (int)init.size(), st);
+  if (nch > 0) cpqr_start<C>(dcp, nid, st);   // (also picks for the resident ones, before they move on)
+  run_resident(dcp);
   std::vector<int> hr(nid);
   // With predicted ranks, run the predicted number of steps (+1, where the stop
   // test of the last rank happens) before the first check; otherwise check
@@ -1525,7 +1554,7 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
     // (over- or under-predicted bounds) finish under the regular 16-step checks
     std::vector<int> due;
     for (int i = 0; i < nid; ++i)
-      if (cp[i].target > 0) due.push_back(std::min(cp[i].target, khat[i] + 1) - 1);
+      if (cp[i].target > 0 && !rcs[i]) due.push_back(std::min(cp[i].target, khat[i] + 1) - 1);
     if (!due.empty()) {
       std::sort(due.begin(), due.end());
       first_check = std::max(0, due[(due.size() - 1) / 2]);
@@ -1542,7 +1571,7 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
       CK(cudaStreamSynchronize(st));
       for (const auto& J : jobs) J.F->stats.rank_checks++;
       int pending = 0;
-      for (int i = 0; i < nid; ++i) if (hr[i] < 0 && t + 1 < cp[i].target) ++pending;
+      for (int i = 0; i < nid; ++i) if (!rcs[i] && hr[i] < 0 && t + 1 < cp[i].target) ++pending;
       if (pending == 0) break;
     }
   }
@@ -1562,7 +1591,7 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
     for (int i = 0; i < nid; ++i) jobs[job_of[i / 4]].F->stats.predictor_fallbacks += r[i] > khat[i];   // above the bound
   // 4. pair ranks k_g = max(row rank, column rank); extend the shorter factorization
   std::vector<int> kk(nid);
-  int maxExt = 0;
+  int maxExt = 0, resExt = 0;
   for (int b = 0; b < nb; ++b)
     for (int grp = 0; grp < 2; ++grp) {
       int ir = 4 * b + grp, ic = 4 * b + 2 + grp;
@@ -1574,11 +1603,12 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
     cp[i].mode = CPQR_EXTEND;
     cp[i].base = r[i];
     cp[i].target = std::max(kk[i], r[i]);
-    maxExt = std::max(maxExt, cp[i].target - cp[i].base);
+    (rcs[i] ? resExt : maxExt) = std::max(rcs[i] ? resExt : maxExt, cp[i].target - cp[i].base);
   }
-  if (maxExt > 0) {
+  if (maxExt > 0 || resExt > 0) {
     dcp = upload(scr, cp, st);
-    cpqr_start<C>(dcp, nid, st);
+    if (maxExt > 0) cpqr_start<C>(dcp, nid, st);
+    if (resExt > 0) run_resident(dcp);
     for (int t = 0; t < maxExt; ++t) cpqr_step<C>(dcp, dch, nch, t, ctr + maxT + t, st, tall);
     for (const auto& J : jobs) J.F->stats.cpqr_launches += maxExt;
     CK(cudaGetLastError());
