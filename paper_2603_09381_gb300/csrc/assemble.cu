@@ -270,26 +270,27 @@ __device__ __forceinline__ C omit_entry(const PointsDev& P, int t, int s, double
   const double dx = P.x[pt] - P.x[ps], dy = P.y[pt] - P.y[ps];
   const double r2 = dx * dx + dy * dy;
   if (!(r2 > 0)) return czero<C>();
-  const double z = k * sqrt(r2);
+  double r, ir;
+  hk_distance(r2, r, ir);
+  const double z = k * r;
   const double w = P.w[ps];
   // only the orders the entry needs (a warp's entries are mostly of one kind)
-  const bool near = z < HK_ZA;
-  const double iz = 1.0 / z;
+  const bool near = (float)z < (float)HK_ZA;
+  const double q = hk_rsqrt(z), iz = q * q;
   double J0, Y0, J1, Y1;
   if (rg == 0 && cg == 0) {         // -eps+ S = -(i/4) H0 w
-    if (near) { J0 = j0(z); Y0 = y0(z); } else hankel_asym(z, iz, J0, Y0, J1, Y1);
+    if (near) { J0 = j0(z); Y0 = y0(z); } else hankel_asym(z, iz, q, J0, Y0, J1, Y1);
     return mk((R)(0.25 * Y0 * w), (R)(-0.25 * J0 * w));
   }
-  const double ir = k * iz;
   if (rg != cg) {
     // D = (ik/4) H1 (n_y.d)/r w;  -D* = (ik/4) H1 (n_x.d)/r w
-    if (near) { J1 = j1(z); Y1 = y1(z); } else hankel_asym(z, iz, J0, Y0, J1, Y1);
+    if (near) { J1 = j1(z); Y1 = y1(z); } else hankel_asym(z, iz, q, J0, Y0, J1, Y1);
     const int pn = rg == 0 ? ps : pt;
     const double g = (P.nx[pn] * dx + P.ny[pn] * dy) * ir * 0.25 * k * w;
     return mk((R)(-Y1 * g), (R)(J1 * g));
   }
   // N/eps+ = (ik/4) [k H0 a b + H1/r (nn - 2 a b)] w,  a = n_x.d/r, b = n_y.d/r
-  if (near) { J0 = j0(z); Y0 = y0(z); J1 = j1(z); Y1 = y1(z); } else hankel_asym(z, iz, J0, Y0, J1, Y1);
+  if (near) { J0 = j0(z); Y0 = y0(z); J1 = j1(z); Y1 = y1(z); } else hankel_asym(z, iz, q, J0, Y0, J1, Y1);
   const double a = (P.nx[pt] * dx + P.ny[pt] * dy) * ir, b = (P.nx[ps] * dx + P.ny[ps] * dy) * ir;
   const double nn = P.nx[pt] * P.nx[ps] + P.ny[pt] * P.ny[ps];
   const double c0 = k * a * b, c1 = (nn - 2 * a * b) * ir;
@@ -334,18 +335,18 @@ __device__ __forceinline__ float2 omit_entry<float2>(const PointsDev& P, int t, 
 __device__ __forceinline__ void kernels4(const PointsDev& P, int pt, int ps, double k, double2& S, double2& D,
                                          double2& Ds, double2& N) {
   const double dx = P.x[pt] - P.x[ps], dy = P.y[pt] - P.y[ps];
-  const double r = sqrt(dx * dx + dy * dy);
+  double r, ir;
+  hk_distance(dx * dx + dy * dy, r, ir);
   const double z = k * r, w = P.w[ps];
   double J0, Y0, J1, Y1;
-  if (z < HK_ZA) { J0 = j0(z); Y0 = y0(z); J1 = j1(z); Y1 = y1(z); }
-  else hankel01(z, J0, Y0, J1, Y1);
-  const double a = (P.nx[pt] * dx + P.ny[pt] * dy) / r, b = (P.nx[ps] * dx + P.ny[ps] * dy) / r;
+  hankel01(z, J0, Y0, J1, Y1);
+  const double a = (P.nx[pt] * dx + P.ny[pt] * dy) * ir, b = (P.nx[ps] * dx + P.ny[ps] * dy) * ir;
   const double nn = P.nx[pt] * P.nx[ps] + P.ny[pt] * P.ny[ps];
   const double f = 0.25 * k * w;
   S = make_double2(-0.25 * Y0 * w, 0.25 * J0 * w);       // (i/4) H0 w
   D = make_double2(-Y1 * b * f, J1 * b * f);               // (ik/4) H1 b w
   Ds = make_double2(Y1 * a * f, -J1 * a * f);              // -(ik/4) H1 a w
-  const double c0 = k * a * b, c1 = (nn - 2 * a * b) / r;
+  const double c0 = k * a * b, c1 = (nn - 2 * a * b) * ir;
   N = make_double2(-(c0 * Y0 + c1 * Y1) * f, (c0 * J0 + c1 * J1) * f);
 }
 

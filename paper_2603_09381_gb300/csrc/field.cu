@@ -89,12 +89,10 @@ __global__ void __launch_bounds__(FT) k_scattered(const InclDev* __restrict__ in
   for (int c = 0; c < NR; ++c) acc[c] = make_double2(0, 0);
   for (int i = threadIdx.x; i < total; i += FT) {
     const double dx = px - nd.x[i], dy = py - nd.y[i];
-    const double r = sqrt(dx * dx + dy * dy);
-    const double z = k * r;
-    double J0, Y0, J1, Y1;
-    if (z < HK_ZA) { J0 = j0(z); Y0 = y0(z); J1 = j1(z); Y1 = y1(z); }
-    else hankel01(z, J0, Y0, J1, Y1);
-    const double w = 0.25 * nd.w[i], b = k * w * ((nd.nx[i] * dx + nd.ny[i] * dy) / r);
+    double r, ir, J0, Y0, J1, Y1;
+    hk_distance(dx * dx + dy * dy, r, ir);
+    hankel01(k * r, J0, Y0, J1, Y1);
+    const double w = 0.25 * nd.w[i], b = k * w * ((nd.nx[i] * dx + nd.ny[i] * dy) * ir);
     // G = (i/4) H0 = (-Y0 + i J0)/4;  dG/dn_y = (i k/4) H1 b = k b (-Y1 + i J1)/4
     const double gx = -w * Y0, gy = w * J0, ex = -b * Y1, ey = b * J1;
 #pragma unroll

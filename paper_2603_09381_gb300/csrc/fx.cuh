@@ -18,6 +18,11 @@ __device__ __forceinline__ void fx_mac(long long& hh, long long& cr, Fx a, Fx b)
   cr += (long long)a.l * b.h;
 }
 constexpr long long FX_HALF = 1ll << 29;   // rounds the cross terms' >> 30
+__device__ __forceinline__ long long fx_mul(Fx a, Fx b) {
+  long long hh = 0, cr = FX_HALF;
+  fx_mac(hh, cr, a, b);
+  return hh + (cr >> 30);
+}
 // a + g v, g given as (re, im, -im)
 __device__ __forceinline__ longlong2 fx_cfma(longlong2 a, Fx gr, Fx gi, Fx ngi, Fx vr, Fx vi) {
   long long cr = FX_HALF, ci = FX_HALF;

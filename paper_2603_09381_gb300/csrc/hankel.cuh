@@ -1,23 +1,23 @@
-// Bessel functions J0, J1, Y0, Y1 of a positive real argument in FP64, for the
-// Hankel functions H_nu = J_nu + i Y_nu of the Helmholtz kernels.
+// Bessel functions J0, J1, Y0, Y1 of a positive real argument to FP64 accuracy,
+// for the Hankel functions H_nu = J_nu + i Y_nu of the Helmholtz kernels.
 //
 // z >= 8: Hankel's modulus-phase form (DLMF 10.17.3-10.17.4; Abramowitz &
 //   Stegun 9.2.5-9.2.10)
-//     H_nu(z) = sqrt(2/(pi z)) e^{i w} (P_nu(z) + i Q_nu(z)),  w = z - nu pi/2 - pi/4,
-//   with P_nu and Q_nu from
-//   - z >= 60: the asymptotic expansion in 1/z^2,
-//       P = sum_k (-1)^k a_{2k}(nu) z^{-2k},  Q = sum_k (-1)^k a_{2k+1}(nu) z^{-2k-1},
-//       a_k(nu) = prod_{j=1..k} (4 nu^2 - (2j-1)^2) / (k! 8^k),
-//     12 terms (remainder below 1e-17: for real z it is bounded by the first
-//     omitted term, DLMF 10.17(iii));
-//   - 8 <= z < 60: polynomial fits of P_nu - 1 and z Q_nu in 1/z^2 on
-//     [8, 12), [12, 20), [20, 30), [30, 60) (hankel_fit.h, written by
-//     gen_hankel_fit.py from 40-digit values; within 2e-17 of P_nu and Q_nu).
-//   One sine and cosine of w_0 = z - pi/4 serve both orders (w_1 = w_0 - pi/2).
+//     H_nu(z) = sqrt(2/(pi z)) e^{i w} (P_nu(z) + i Q_nu(z)),  w = z - nu pi/2 - pi/4.
+//   What bounds it is the FP64 pipe (2 fused multiply-adds per clock and SM), so
+//   P_nu, Q_nu, the reduction of z by pi/2, sine, cosine and their products are
+//   computed in 60-bit fixed point on the integer multipliers: every value is
+//   below 1.01 and within about 1e-17, a tenth of what the FP64 forms give.
+//   FP64 does 1/sqrt(z) from an FP32 estimate (6 operations) and the scaling:
+//   14 FP64 operations for one order of about 70 before.
+//   - P_nu and z Q_nu: polynomials in 1/z^2 on [8, 12), [12, 20), [20, 30),
+//     [30, 60), [60, inf) (hankel_fit.h, written by gen_hankel_fit.py from
+//     40-digit values).
+//   - sine and cosine of w_0 = z - pi/4 serve both orders (w_1 = w_0 - pi/2).
 //   A caller that uses one order pays for one: what it leaves unused is
 //   compiled away.
 // The interval of z is chosen on z rounded to FP32 (comparisons on the FP32
-// pipes): next to a boundary either neighbouring form is within its bound.
+// pipes): the fits hold a little beyond their ends.
 // z < 8: CUDA's j0 / y0 / j1 / y1.
 // Complex z (lossy interiors, self blocks): Miller's backward recurrence
 //   J_{n-1} = (2n/z) J_n - J_{n+1} from an even start M > |z| + 25 + 3 sqrt|z|,
@@ -28,121 +28,121 @@
 //     (pi/2) Y1 = -J0/z + (ln(z/2) + gamma) J1 + sum_{k>=1} (-1)^k (J_{2k-1} - J_{2k+1})/k.
 #pragma once
 #include <cuda_runtime.h>
+#include "fx.cuh"
 #include "hankel_fit.h"
 
 constexpr double HK_ZA = 8.0;    // modulus-phase form from here up
-constexpr double HK_ZS = 60.0;   // asymptotic series from here up
-constexpr int HK_TERMS = 12;     // a_0 .. a_11
 
-// a_k(nu) = prod_{j=1..k} (4 nu^2 - (2j-1)^2) / (8 j), with the (-1)^floor(k/2)
-// sign of the series folded in (evaluated at compile time).
-constexpr double hk_coef(int nu, int k) {
-  double a = 1.0;
-  for (int j = 1; j <= k; ++j) a *= (4.0 * nu * nu - (2.0 * j - 1) * (2.0 * j - 1)) / (8.0 * j);
-  return ((k / 2) & 1) ? -a : a;
+// 1/sqrt(z): Newton's iteration of third order on an FP32 estimate q (relative
+// error d below 2^-21): 1/sqrt(z) = q (1 - e)^(-1/2), e = 1 - z q^2, taken to
+// q (1 + e/2 + 3 e^2/8); q^2 is exact.
+__device__ __forceinline__ double hk_rsqrt(double z) {
+  const double q = (double)rsqrtf((float)z);
+  const double e = fma(-z, q * q, 1.0);
+  return fma(q * e, fma(0.375, e, 0.5), q);
 }
-#define HK_ROW(nu) \
-  {hk_coef(nu, 0), hk_coef(nu, 1), hk_coef(nu, 2), hk_coef(nu, 3), hk_coef(nu, 4), hk_coef(nu, 5), hk_coef(nu, 6), \
-   hk_coef(nu, 7), hk_coef(nu, 8), hk_coef(nu, 9), hk_coef(nu, 10), hk_coef(nu, 11)}
-static __constant__ double c_hk_a0[HK_TERMS] = HK_ROW(0);
-static __constant__ double c_hk_a1[HK_TERMS] = HK_ROW(1);
-#undef HK_ROW
-
-// sin and cos of z - pi/4 for z >= 8 (up to ~1e9): with c = n + 1/2 the nearest
-// half-integer to z 2/pi, z - pi/4 = n pi/2 + y, y = z - c pi/2 in [-pi/4,
-// pi/4] by two fused multiply-adds with pi/2 in two parts (Cody and Waite),
-// then the Taylor sums to y^17 and y^16 (remainders below 1e-19 and 2e-18) and
-// the quadrant: 24 FP64 operations and no slow path.
-__device__ __forceinline__ void hk_sincos_shifted(double z, double& sn, double& cs) {
-  const double magic = 6755399441055744.0;                       // 1.5 2^52: rounds to an integer
-  const double t = fma(z, 0.63661977236758134308, -0.5) + magic;
-  const int n = __double2loint(t);
-  const double c = (t - magic) + 0.5;
-  double y = fma(-c, 1.57079632679489661923, z);
-  y = fma(-c, 6.123233995736766e-17, y);
-  const double x = y * y;
-  double a = 1.0 / 355687428096000.0;                            // 17!
-  a = fma(a, x, -1.0 / 1307674368000.0);
-  a = fma(a, x, 1.0 / 6227020800.0);
-  a = fma(a, x, -1.0 / 39916800.0);
-  a = fma(a, x, 1.0 / 362880.0);
-  a = fma(a, x, -1.0 / 5040.0);
-  a = fma(a, x, 1.0 / 120.0);
-  a = fma(a, x, -1.0 / 6.0);
-  const double s0 = fma(y * x, a, y);
-  double b = 1.0 / 20922789888000.0;                             // 16!
-  b = fma(b, x, -1.0 / 87178291200.0);
-  b = fma(b, x, 1.0 / 479001600.0);
-  b = fma(b, x, -1.0 / 3628800.0);
-  b = fma(b, x, 1.0 / 40320.0);
-  b = fma(b, x, -1.0 / 720.0);
-  b = fma(b, x, 1.0 / 24.0);
-  b = fma(b, x, -0.5);
-  const double c0 = fma(x, b, 1.0);
-  // quadrant: signs by flipping the top bit
-  const double u = (n & 1) ? c0 : s0, v = (n & 1) ? s0 : c0;
-  sn = __hiloint2double(__double2hiint(u) ^ ((n & 2) << 30), __double2loint(u));
-  cs = __hiloint2double(__double2hiint(v) ^ (((n + 1) & 2) << 30), __double2loint(v));
-}
-
-// J and Y of orders 0 and 1 from P_nu, Q_nu (iz = 1/z).
-__device__ __forceinline__ void hankel_combine(double z, double iz, double P0, double Q0, double P1, double Q1,
-                                               double& J0, double& Y0, double& J1, double& Y1) {
-  double c, d;
-  hk_sincos_shifted(z, d, c);                                  // sin, cos of z - pi/4
-  const double s = sqrt(0.63661977236758134308 * iz);          // sqrt(2/(pi z))
-  J0 = s * (P0 * c - Q0 * d);
-  Y0 = s * (P0 * d + Q0 * c);
-  J1 = s * (P1 * d + Q1 * c);
-  Y1 = s * (Q1 * d - P1 * c);
-}
-
-// z >= 60: the expansion's 12 terms (P from the even, Q from the odd indices).
-__device__ __forceinline__ void hankel_series(double z, double iz, double& J0, double& Y0, double& J1, double& Y1) {
-  constexpr int PE = 10, QO = 11;
-  const double u = iz * iz;
-  double P0 = c_hk_a0[PE], P1 = c_hk_a1[PE];
-  double Q0 = c_hk_a0[QO], Q1 = c_hk_a1[QO];
-#pragma unroll
-  for (int k = PE - 2; k >= 0; k -= 2) {
-    P0 = fma(P0, u, c_hk_a0[k]);
-    P1 = fma(P1, u, c_hk_a1[k]);
-  }
-#pragma unroll
-  for (int k = QO - 2; k >= 1; k -= 2) {
-    Q0 = fma(Q0, u, c_hk_a0[k]);
-    Q1 = fma(Q1, u, c_hk_a1[k]);
-  }
-  hankel_combine(z, iz, P0, Q0 * iz, P1, Q1 * iz, J0, Y0, J1, Y1);
-}
-
-// z >= 8 (iz = 1/z)
-__device__ __forceinline__ void hankel_asym(double z, double iz, double& J0, double& Y0, double& J1, double& Y1) {
-  const float zf = (float)z;
-  if (zf >= (float)HK_ZS) {
-    hankel_series(z, iz, J0, Y0, J1, Y1);
+// r = sqrt(r2) and ir = 1/r: one FP64 iteration on the estimate gives ir, and
+// a last one on r itself its rounding (z = k r is a phase, so that its error
+// counts as z times r's); FP32's range is left to sqrt and the division.
+__device__ __forceinline__ void hk_distance(double r2, double& r, double& ir) {
+  const float f = (float)r2;
+  if (!(f > 1e-30f && f < 1e30f)) {
+    r = sqrt(r2);
+    ir = 1.0 / r;
     return;
   }
+  ir = hk_rsqrt(r2);
+  r = r2 * ir;
+  r = fma(fma(-r, r, r2), 0.5 * ir, r);
+}
+
+// sin and cos of z - pi/4 in 60-bit fixed point for z >= 8.  With f = z 2/pi =
+// n + 1/2 + g/2, |g| <= 1: z - pi/4 = n pi/2 + g pi/4.  z is an integer of 2^-50,
+// 2/pi has 96 bits, and f mod 4 is kept to 62 bits: five 32-bit products in
+// place of Cody and Waite's FP64 steps.  From z = 8192 up (to about 1e9) whole
+// turns are taken off in FP64 first.
+__device__ __forceinline__ void hk_sincos_shifted(double z, long long& sn, long long& cs) {
+  if (z >= 8192.0) {
+    const double n = rint(z * 0.15915494309189533577) - 4.0;   // leaves z in about [22, 29]
+    z = fma(-n, 2.4492935982947064e-16, fma(-n, 6.2831853071795864769, z));
+  }
+  const unsigned long long b = (unsigned long long)__double_as_longlong(z);
+  const int e = (int)(b >> 52) - 1023;                             // 2 .. 12
+  const unsigned long long Z = ((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << (e - 2);
+  const unsigned z0 = (unsigned)Z, z1 = (unsigned)(Z >> 32);
+  const unsigned k2 = 0xA2F9836Eu, k1 = 0x4E441529u, k0 = 0xFC2757D1u;   // 2/pi 2^96
+  const unsigned long long lo = (unsigned long long)__umulhi(z0, k1) + __umulhi(z1, k0);
+  const unsigned long long m0 = (unsigned long long)z0 * k2 + lo, m = m0 + (unsigned long long)z1 * k1;
+  const unsigned long long hi = (unsigned long long)z1 * k2 + (m >> 32) + ((unsigned long long)(m < m0) << 32);
+  const unsigned long long f = (hi << 12) | ((unsigned)m >> 20);          // 2^62 to a quadrant, mod 4
+  const int n = (int)(f >> 62);
+  const long long g = (long long)(f & 0x3FFFFFFFFFFFFFFFull) - (1ll << 61);
+  const Fx gf = fx(g >> 1);
+  const long long x = fx_mul(gf, gf);
+  const int x31 = (int)min(x >> 29, 0x7FFFFFFFll);
+  long long s, c;
+  hankel_sincos_fit(fx(x), x31, s, c);
+  s = fx_mul(fx(s), gf);
+  const long long u = (n & 1) ? c : s, v = (n & 1) ? s : c;
+  sn = (n & 2) ? -u : u;
+  cs = ((n + 1) & 2) ? -v : v;
+}
+
+// z >= 8, with iz = 1/z and q = 1/sqrt(z)
+__device__ __forceinline__ void hankel_asym(double z, double iz, double q, double& J0, double& Y0, double& J1,
+                                            double& Y1) {
+  const float zf = (float)z;
   const double v = iz * iz;
-  double P0, zQ0, P1, zQ1;
-  if (zf >= 30.f) hankel_fit3(v, P0, zQ0, P1, zQ1);
-  else if (zf >= 20.f) hankel_fit2(v, P0, zQ0, P1, zQ1);
-  else if (zf >= 12.f) hankel_fit1(v, P0, zQ0, P1, zQ1);
-  else hankel_fit0(v, P0, zQ0, P1, zQ1);
-  hankel_combine(z, iz, P0, zQ0 * iz, P1, zQ1 * iz, J0, Y0, J1, Y1);
+  const long long three = 0x4008000000000000ll;   // 3.0: 3 + x lies in [2, 4)
+  long long P0, Q0, P1, Q1;
+  auto mapped = [&](double ivh, double sh, int& x31) {
+    const long long X = __double_as_longlong(fma(v, ivh, sh)) - three;   // x 2^51
+    x31 = (int)(X >> 20);
+    return fx(X << 9);
+  };
+  int x31;
+  if (zf >= 60.f) {
+    const Fx x = mapped(HK_IVH4, HK_SH4, x31);
+    hankel_fit4(x, x31, P0, Q0, P1, Q1);
+  } else if (zf >= 30.f) {
+    const Fx x = mapped(HK_IVH3, HK_SH3, x31);
+    hankel_fit3(x, x31, P0, Q0, P1, Q1);
+  } else if (zf >= 20.f) {
+    const Fx x = mapped(HK_IVH2, HK_SH2, x31);
+    hankel_fit2(x, x31, P0, Q0, P1, Q1);
+  } else if (zf >= 12.f) {
+    const Fx x = mapped(HK_IVH1, HK_SH1, x31);
+    hankel_fit1(x, x31, P0, Q0, P1, Q1);
+  } else {
+    const Fx x = mapped(HK_IVH0, HK_SH0, x31);
+    hankel_fit0(x, x31, P0, Q0, P1, Q1);
+  }
+  // 1/z in 2^-60 (0.375 + 1/z lies in [0.375, 0.5], whose last place is 2^-54)
+  const Fx izf = fx((__double_as_longlong(0.375 + iz) - 0x3FD8000000000000ll) << 6);
+  long long sn, cs;
+  hk_sincos_shifted(z, sn, cs);
+  const Fx s = fx(sn), c = fx(cs), ns = fx(-sn), nc = fx(-cs);
+  const Fx p0 = fx(P0), q0 = fx(fx_mul(fx(Q0), izf)), p1 = fx(P1), q1 = fx(fx_mul(fx(Q1), izf));
+  const double amp = 6.9205453937208734e-19 * q;     // sqrt(2/pi) 2^-60 / sqrt(z)
+  auto two = [&](Fx a0, Fx b0, Fx a1, Fx b1) {
+    long long hh = 0, cr = FX_HALF;
+    fx_mac(hh, cr, a0, b0);
+    fx_mac(hh, cr, a1, b1);
+    return amp * (double)(hh + (cr >> 30));
+  };
+  J0 = two(p0, c, q0, ns);
+  Y0 = two(p0, s, q0, c);
+  J1 = two(p1, s, q1, c);
+  Y1 = two(q1, s, p1, nc);
 }
 
-// Below z = 8 CUDA's j0/y0/j1/y1 (~1e-15 absolute, measured against scipy
-// on GB300).
+// The pair of orders at z (below 8 CUDA's j0/y0/j1/y1: ~1e-15 absolute,
+// measured against scipy on GB300).
 __device__ __forceinline__ void hankel01(double z, double& J0, double& Y0, double& J1, double& Y1) {
-  if ((float)z >= (float)HK_ZA) hankel_asym(z, 1.0 / z, J0, Y0, J1, Y1);
-  else { J0 = j0(z); Y0 = y0(z); J1 = j1(z); Y1 = y1(z); }
-}
-
-// Same, with 1/z supplied by the caller.
-__device__ __forceinline__ void hankel01_inv(double z, double iz, double& J0, double& Y0, double& J1, double& Y1) {
-  if ((float)z >= (float)HK_ZA) hankel_asym(z, iz, J0, Y0, J1, Y1);
-  else { J0 = j0(z); Y0 = y0(z); J1 = j1(z); Y1 = y1(z); }
+  if ((float)z >= (float)HK_ZA) {
+    const double q = hk_rsqrt(z);
+    hankel_asym(z, q * q, q, J0, Y0, J1, Y1);
+  } else { J0 = j0(z); Y0 = y0(z); J1 = j1(z); Y1 = y1(z); }
 }
 
 // ---- complex argument (lossy interior wavenumbers, self blocks only) ---------------

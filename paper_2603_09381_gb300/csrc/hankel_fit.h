@@ -1,42 +1,115 @@
-// Generated by gen_hankel_fit.py (do not edit): polynomial fits of P_nu - 1
-// and z Q_nu (nu = 0, 1; Hankel's modulus-phase functions) in
-// x = (1/z^2 - vm) * ivh on [za, zb), as Horner's rule with FMAs; each
-// fit's FP64 Horner evaluation is within 2e-17 of 40-digit values of
-// P_nu and Q_nu on its interval.
+// Generated by gen_hankel_fit.py (do not edit): polynomials in 60-bit fixed
+// point (value 2^60) for P_nu and z Q_nu (nu = 0, 1; Hankel's modulus-phase
+// functions) in x = (1/z^2 - vm) ivh on [za, zb), and for sin(pi/4 g) / g and
+// cos(pi/4 g) in x = g^2; x31 is x 2^31.  The worst errors are those of the
+// integer evaluation against 40-digit values.
 #pragma once
+#include "fx.cuh"
 
-// [8, 12): degree 8; worst errors P0 8.5e-18, P1 9.1e-18, Q0 6.6e-18, Q1 1.1e-17
-__device__ __forceinline__ void hankel_fit0(double v, double& P0, double& zQ0, double& P1, double& zQ1) {
-  const double x = (v - 0.011284722222222222) * 230.4;
-  P0 = 1.0 + fma(fma(fma(fma(fma(fma(fma(fma(2.0003243220372645e-14, x, -2.2273219801295706e-13), x, 2.877808512281104e-12), x, -4.6714710774619215e-11), x, 1.0006172374860289e-09), x, -3.166397818736442e-08), x, 1.814169765268025e-06), x, -0.0002950162265086234), x, -0.0007799148995263191);
-  zQ0 = fma(fma(fma(fma(fma(fma(fma(fma(-1.1330329239856097e-13, x, 1.1531804867167383e-12), x, -1.3329499126387227e-11), x, 1.8929620132985877e-10), x, -3.4108456414084695e-09), x, 8.519763513764875e-08), x, -3.428624550961081e-06), x, 0.00029803873518218676), x, -0.12420024064419449);
-  P1 = 1.0 + fma(fma(fma(fma(fma(fma(fma(fma(-2.1795300816051397e-14, x, 2.4465717039320324e-13), x, -3.1962670879571853e-12), x, 5.2678138178408974e-11), x, -1.1547070558568262e-09), x, 3.800380466014811e-08), x, -2.3607614958476865e-06), x, 0.0004954834135131119), x, 0.0013049438453204222);
-  zQ1 = fma(fma(fma(fma(fma(fma(fma(fma(1.2290877706937287e-13, x, -1.2597549881006295e-12), x, 1.4699877795874322e-11), x, -2.1139745593807694e-10), x, 3.879730420729237e-09), x, -9.980539419896165e-08), x, 4.241181347684872e-06), x, -0.0004206344655296184), x, 0.37387571752819715);
+// [8, 12): degree 9; worst errors P0 3.1e-18, zQ0 4.0e-18, P1 1.7e-18, zQ1 4.6e-18
+constexpr double HK_IVH0 = 230.39880192553878, HK_SH0 = 0.4000115199400963;   // 3 + x = v ivh + sh
+__device__ __forceinline__ void hankel_fit0(Fx x, int x31, long long& P0, long long& zQ0, long long& P1, long long& zQ1) {
+  P0 = (((long long)(__mulhi(__mulhi(__mulhi(__mulhi(__mulhi(-75497, x31) + 369009, x31) + -2011947, x31) + 13271949, x31) + -107727473, x31) + 1153656588) * x31) >> 31) + -36506640537ll;
+  P0 = fx_mul(fx(P0), x) + 2091616869006ll;
+  P0 = fx_mul(fx(P0), x) + -340132312063272ll;
+  P0 = fx_mul(fx(P0), x) + 1152022323267156046ll;
+  zQ0 = (((long long)(__mulhi(__mulhi(__mulhi(__mulhi(1846158, x31) + -8360641, x31) + 41507879, x31) + -245893239, x31) + 1746187918) * x31) >> 34) + -3932516902ll;
+  zQ0 = fx_mul(fx(zQ0), x) + 98227679808ll;
+  zQ0 = fx_mul(fx(zQ0), x) + -3952975497315ll;
+  zQ0 = fx_mul(fx(zQ0), x) + 343617037986412ll;
+  zQ0 = fx_mul(fx(zQ0), x) + -143193127628803991ll;
+  P1 = (((long long)(__mulhi(__mulhi(__mulhi(__mulhi(__mulhi(81744, x31) + -402068, x31) + 2210662, x31) + -14740625, x31) + 121479208, x31) + -1331313680) * x31) >> 31) + 43816075326ll;
+  P1 = fx_mul(fx(P1), x) + -2721800739440ll;
+  P1 = fx_mul(fx(P1), x) + 571256442247997ll;
+  P1 = fx_mul(fx(P1), x) + 1154426003570932652ll;
+  zQ1 = (((long long)(__mulhi(__mulhi(__mulhi(__mulhi(-995790, x31) + 4534715, x31) + -22679061, x31) + 135586513, x31) + -975028249) * x31) >> 33) + 4473115236ll;
+  zQ1 = fx_mul(fx(zQ1), x) + -115069537238ll;
+  zQ1 = fx_mul(fx(zQ1), x) + 4889799343820ll;
+  zQ1 = fx_mul(fx(zQ1), x) + -484961023115042ll;
+  zQ1 = fx_mul(fx(zQ1), x) + 431049353818652747ll;
 }
 
-// [12, 20): degree 7; worst errors P0 4.1e-18, P1 4.4e-18, Q0 2.7e-18, Q1 3.9e-18
-__device__ __forceinline__ void hankel_fit1(double v, double& P0, double& zQ0, double& P1, double& zQ1) {
-  const double x = (v - 0.004722222222222222) * 450.0;
-  P0 = 1.0 + fma(fma(fma(fma(fma(fma(fma(-7.428492863313096e-15, x, 1.3452274639023845e-13), x, -3.1325911207970516e-12), x, 1.0230676675301092e-10), x, -5.239038684952377e-09), x, 5.173170077780672e-07), x, -0.0001539761434764863), x, -0.00032958782261562015);
-  zQ0 = fma(fma(fma(fma(fma(fma(fma(4.368762522231656e-14, x, -6.999155641418278e-13), x, 1.3999316764738929e-11), x, -3.774539069741578e-10), x, 1.4944731756585217e-08), x, -1.0144160023851982e-06), x, 0.00015823056460246331), x, -0.12465902754552165);
-  P1 = 1.0 + fma(fma(fma(fma(fma(fma(fma(8.07619305224235e-15, x, -1.4787089761202547e-13), x, 3.4979590984203945e-12), x, -1.169829262713386e-10), x, 6.236953997484424e-09), x, -6.687571300365866e-07), x, 0.00025748506648688734), x, 0.0005502380229727974);
-  zQ1 = fma(fma(fma(fma(fma(fma(fma(-4.725841352980723e-14, x, 7.642666250359328e-13), x, -1.54877106323279e-11), x, 4.255814922070184e-10), x, -1.7369794181361695e-08), x, 1.2467127907500323e-06), x, -0.00022231259952368683), x, 0.3745217799333954);
+// [12, 20): degree 8; worst errors P0 1.2e-18, zQ0 1.8e-18, P1 1.5e-18, zQ1 2.5e-18
+constexpr double HK_IVH1 = 449.9980875067781, HK_SH1 = 0.8750070312201174;   // 3 + x = v ivh + sh
+__device__ __forceinline__ void hankel_fit1(Fx x, int x31, long long& P0, long long& zQ0, long long& P1, long long& zQ1) {
+  P0 = (((long long)(__mulhi(__mulhi(__mulhi(__mulhi(148362, x31) + -1096284, x31) + 9852092, x31) + -115574610, x31) + 1887269839) * x31) >> 35) + -6040276433ll;
+  P0 = fx_mul(fx(P0), x) + 596430936214ll;
+  P0 = fx_mul(fx(P0), x) + -177523159095511ll;
+  P0 = fx_mul(fx(P0), x) + 1152541515363450942ll;
+  zQ0 = (((long long)(__mulhi(__mulhi(__mulhi(__mulhi(-241604, x31) + 1611835, x31) + -12790680, x31) + 129123574, x31) + -1740746727) * x31) >> 33) + 17230318826ll;
+  zQ0 = fx_mul(fx(zQ0), x) + -1169551860577ll;
+  zQ0 = fx_mul(fx(zQ0), x) + 182428191255145ll;
+  zQ0 = fx_mul(fx(zQ0), x) + -143722073235753236ll;
+  P1 = (((long long)(__mulhi(__mulhi(__mulhi(__mulhi(-79992, x31) + 595935, x31) + -5415613, x31) + 64527295, x31) + -1079001320) * x31) >> 34) + 7190808990ll;
+  P1 = fx_mul(fx(P1), x) + -771030987004ll;
+  P1 = fx_mul(fx(P1), x) + 296861328839925ll;
+  P1 = fx_mul(fx(P1), x) + 1153555886449906696ll;
+  zQ1 = (((long long)(__mulhi(__mulhi(__mulhi(__mulhi(129749, x31) + -871789, x31) + 6984415, x31) + -71425934, x31) + 981350571) * x31) >> 32) + -20026260650ll;
+  zQ1 = fx_mul(fx(zQ1), x) + 1437374082965ll;
+  zQ1 = fx_mul(fx(zQ1), x) + -256310060300338ll;
+  zQ1 = fx_mul(fx(zQ1), x) + 431794213516225119ll;
 }
 
-// [20, 30): degree 5; worst errors P0 6.9e-18, P1 7.6e-18, Q0 2.7e-18, Q1 3.5e-18
-__device__ __forceinline__ void hankel_fit2(double v, double& P0, double& zQ0, double& P1, double& zQ1) {
-  const double x = (v - 0.0018055555555555555) * 1440.0;
-  P0 = 1.0 + fma(fma(fma(fma(fma(-1.3513107726086284e-14, x, 1.2117156812560966e-12), x, -1.7813249243609856e-10), x, 5.264459166519726e-08), x, -4.8550672177118736e-05), x, -0.000126590812991621);
-  zQ0 = fma(fma(fma(fma(fma(6.43182961026453e-14, x, -4.689118667172334e-12), x, 5.250313440377417e-10), x, -1.0522594898999896e-07), x, 5.0304462465742396e-05), x, -0.12486848761997836);
-  P1 = 1.0 + fma(fma(fma(fma(fma(1.5001912782507538e-14, x, -1.3784231930794933e-12), x, 2.111505611891377e-10), x, -6.783306984418302e-08), x, 8.102309374398434e-05), x, 0.00021112237130376652);
-  zQ1 = fma(fma(fma(fma(fma(-7.0755138413687e-14, x, 5.260397014146786e-12), x, -6.076329848233797e-10), x, 1.2889584566649194e-07), x, -7.052471422245871e-05), x, 0.3748157534782049);
+// [20, 30): degree 6; worst errors P0 1.2e-18, zQ0 1.8e-18, P1 1.6e-18, zQ1 1.9e-18
+constexpr double HK_IVH2 = 1439.9925120346174, HK_SH2 = 0.4000115199400963;   // 3 + x = v ivh + sh
+__device__ __forceinline__ void hankel_fit2(Fx x, int x31, long long& P0, long long& zQ0, long long& P1, long long& zQ1) {
+  P0 = (((long long)(__mulhi(__mulhi(__mulhi(16192, x31) + -498559, x31) + 22346600, x31) + -1643007791) * x31) >> 34) + 60695711973ll;
+  P0 = fx_mul(fx(P0), x) + -55975404844096ll;
+  P0 = fx_mul(fx(P0), x) + 1152775555224312600ll;
+  zQ0 = (((long long)(__mulhi(__mulhi(__mulhi(-22727, x31) + 593247, x31) + -21616667, x31) + 1210658654) * x31) >> 32) + -121318518304ll;
+  zQ0 = fx_mul(fx(zQ0), x) + 57997397654245ll;
+  zQ0 = fx_mul(fx(zQ0), x) + -143963564508812217ll;
+  P1 = (((long long)(__mulhi(__mulhi(__mulhi(-17689, x31) + 553487, x31) + -25421313, x31) + 1947550461) * x31) >> 34) + -78207016989ll;
+  P1 = fx_mul(fx(P1), x) + 93413752583658ll;
+  P1 = fx_mul(fx(P1), x) + 1153164912315653951ll;
+  zQ1 = (((long long)(__mulhi(__mulhi(__mulhi(24669, x31) + -652618, x31) + 24250550, x31) + -1401128031) * x31) >> 32) + 148608334503ll;
+  zQ1 = fx_mul(fx(zQ1), x) + -81309881848326ll;
+  zQ1 = fx_mul(fx(zQ1), x) + 432133142287821409ll;
 }
 
-// [30, 60): degree 5; worst errors P0 4.2e-19, P1 4.7e-19, Q0 4.2e-19, Q1 1.9e-18
-__device__ __forceinline__ void hankel_fit3(double v, double& P0, double& zQ0, double& P1, double& zQ1) {
-  const double x = (v - 0.0006944444444444445) * 2400.0;
-  P0 = 1.0 + fma(fma(fma(fma(fma(-1.236819519863229e-15, x, 1.7220582968230657e-13), x, -4.023004964022949e-11), x, 1.926677176986748e-08), x, -2.9232313939608e-05), x, -4.8774229638190575e-05);
-  zQ0 = fma(fma(fma(fma(fma(6.0663698458852235e-15, x, -6.809738540378647e-13), x, 1.2026524140297202e-10), x, -3.8815508555123996e-08), x, 3.0387178037374223e-05), x, -0.12494924632029707);
-  P1 = 1.0 + fma(fma(fma(fma(fma(1.3694934530572003e-15, x, -1.9546050214033642e-13), x, 4.7600974796015765e-11), x, -2.4792623491778678e-08), x, 4.874508257366922e-05), x, 8.131089458888334e-05);
-  zQ1 = fma(fma(fma(fma(fma(-6.656197229655161e-15, x, 7.622405152537548e-13), x, -1.3893426756730535e-10), x, 4.748266385402064e-08), x, -4.2565161666463816e-05), x, 0.37492892551841844);
+// [30, 60): degree 6; worst errors P0 8.1e-19, zQ0 1.1e-18, P1 2.1e-18, zQ1 1.7e-18
+constexpr double HK_IVH3 = 2399.9920000194666, HK_SH3 = 1.3333368888770372;   // 3 + x = v ivh + sh
+__device__ __forceinline__ void hankel_fit3(Fx x, int x31, long long& P0, long long& zQ0, long long& P1, long long& zQ1) {
+  P0 = (((long long)(__mulhi(__mulhi(__mulhi(3917, x31) + -182525, x31) + 12705247, x31) + -1484241651) * x31) >> 36) + 22213223316ll;
+  P0 = fx_mul(fx(P0), x) + -33702675623519ll;
+  P0 = fx_mul(fx(P0), x) + 1152865271681221178ll;
+  zQ0 = (((long long)(__mulhi(__mulhi(__mulhi(-5716, x31) + 223813, x31) + -12559773, x31) + 1109262107) * x31) >> 34) + -44751532086ll;
+  zQ0 = fx_mul(fx(zQ0), x) + 35034147624808ll;
+  zQ0 = fx_mul(fx(zQ0), x) + -144056672997020199ll;
+  P1 = (((long long)(__mulhi(__mulhi(__mulhi(-4266, x31) + 202105, x31) + -14421031, x31) + 1756183503) * x31) >> 36) + -28584139020ll;
+  P1 = fx_mul(fx(P1), x) + 56199441159698ll;
+  P1 = fx_mul(fx(P1), x) + 1153015249798176109ll;
+  zQ1 = (((long long)(__mulhi(__mulhi(__mulhi(6186, x31) + -245574, x31) + 14058722, x31) + -1281455197) * x31) >> 34) + 54744148306ll;
+  zQ1 = fx_mul(fx(zQ1), x) + -49074453594471ll;
+  zQ1 = fx_mul(fx(zQ1), x) + 432263620831174666ll;
+}
+
+// [60, inf): degree 5; worst errors P0 3.8e-18, zQ0 1.5e-18, P1 2.3e-18, zQ1 1.6e-18
+constexpr double HK_IVH4 = 7199.9784000288, HK_SH4 = 2.000001999998;   // 3 + x = v ivh + sh
+__device__ __forceinline__ void hankel_fit4(Fx x, int x31, long long& P0, long long& zQ0, long long& P1, long long& zQ1) {
+  P0 = (((long long)(__mulhi(__mulhi(__mulhi(-26, x31) + 5147, x31) + -1758051, x31) + 1244493904) * x31) >> 30) + -11254049595363ll;
+  P0 = fx_mul(fx(P0), x) + 1152910248089021218ll;
+  zQ0 = (((long long)(__mulhi(__mulhi(32734, x31) + -5272507, x31) + 1355594956) * x31) >> 39) + -5034963891ll;
+  zQ0 = fx_mul(fx(zQ0), x) + 11718073379233ll;
+  zQ0 = fx_mul(fx(zQ0), x) + -144103464985663420ll;
+  P1 = (((long long)(__mulhi(__mulhi(__mulhi(28, x31) + -5835, x31) + 2078197, x31) + -1600338001) * x31) >> 30) + 18758647156994ll;
+  P1 = fx_mul(fx(P1), x) + 1152940266419231021ll;
+  zQ1 = (((long long)(__mulhi(__mulhi(-35865, x31) + 5894639, x31) + -1564530870) * x31) >> 39) + 6154932962ll;
+  zQ1 = fx_mul(fx(zQ1), x) + -16407094677854ll;
+  zQ1 = fx_mul(fx(zQ1), x) + 432329151004672616ll;
+}
+
+// sin(pi/4 g) / g and cos(pi/4 g), x = g^2 in [0, 1]: degree 7; worst errors 2.7e-18, 1.9e-18
+__device__ __forceinline__ void hankel_sincos_fit(Fx x, int x31, long long& s, long long& c) {
+  s = (((long long)(__mulhi(__mulhi(-46638, x31) + 8010676, x31) + -1012984170) * x31) >> 30) + 361281429875ll;
+  s = fx_mul(fx(s), x) + -42169492358488ll;
+  s = fx_mul(fx(s), x) + 2871229454931309ll;
+  s = fx_mul(fx(s), x) + -93093237402363180ll;
+  s = fx_mul(fx(s), x) + 905502432259640355ll;
+  c = (((long long)(__mulhi(-7117105, x31) + 1060735015) * x31) >> 34) + -28374970853ll;
+  c = fx_mul(fx(c), x) + 4139980228268ll;
+  c = fx_mul(fx(c), x) + -375843056765200ll;
+  c = fx_mul(fx(c), x) + 18278814420134577ll;
+  c = fx_mul(fx(c), x) + -355589973624321938ll;
+  c = fx_mul(fx(c), x) + 1152921504606846976ll;
 }

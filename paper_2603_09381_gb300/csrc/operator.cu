@@ -28,7 +28,6 @@ __global__ void __launch_bounds__(OP_T) k_apply_offdiag(OpNodes nd, int total, d
   __shared__ double2 sxq[NR][OP_S], sxu[NR][OP_S];
   const int t = blockIdx.x * OP_T + threadIdx.x;
   const bool active = t < total;
-  const double ik = 1.0 / k;
   double tx = 0, ty = 0, tnx = 0, tny = 0;
   int tinc = -1;
   if (active) { tx = nd.x[t]; ty = nd.y[t]; tnx = nd.nx[t]; tny = nd.ny[t]; tinc = nd.incl[t]; }
@@ -58,11 +57,9 @@ __global__ void __launch_bounds__(OP_T) k_apply_offdiag(OpNodes nd, int total, d
     for (int j = 0; j < cnt; ++j) {
       if (sinc[j] == tinc) continue;
       const double dx = tx - sx[j], dy = ty - sy[j];
-      const double ir = rsqrt(dx * dx + dy * dy);       // one reciprocal square root per pair
-      const double r = (dx * dx + dy * dy) * ir;
-      const double z = k * r;
-      double J0, Y0, J1, Y1;
-      hankel01_inv(z, ir * ik, J0, Y0, J1, Y1);
+      double r, ir, J0, Y0, J1, Y1;
+      hk_distance(dx * dx + dy * dy, r, ir);
+      hankel01(k * r, J0, Y0, J1, Y1);
       const double w = sw[j];
       const double a = (tnx * dx + tny * dy) * ir, b = (snx[j] * dx + sny[j] * dy) * ir;
       const double nn = tnx * snx[j] + tny * sny[j];
@@ -165,15 +162,13 @@ __device__ __forceinline__ float4 split4(double re, double im) {
 // with N = -(c0 Y0 + c1 Y1) + i (c0 J0 + c1 J1), c0 = k a b,
 // c1 = (n_t.n_s - 2 a b)/r, symmetric in the pair.
 // The pair (t, s), t < s, of different inclusions: both 2 x 2 entry blocks.
-__device__ __forceinline__ void offdiag_pair(const OpNodes& nd, int t, int s, double k, double ik, const SplitOp& A) {
+__device__ __forceinline__ void offdiag_pair(const OpNodes& nd, int t, int s, double k, const SplitOp& A) {
   const int ti = nd.incl[t], si = nd.incl[s];
   if (ti == si) return;
   const double dx = nd.x[t] - nd.x[s], dy = nd.y[t] - nd.y[s];
-  const double ir = rsqrt(dx * dx + dy * dy);
-  const double r = (dx * dx + dy * dy) * ir;
-  const double z = k * r;
-  double J0, Y0, J1, Y1;
-  hankel01_inv(z, ir * ik, J0, Y0, J1, Y1);
+  double r, ir, J0, Y0, J1, Y1;
+  hk_distance(dx * dx + dy * dy, r, ir);
+  hankel01(k * r, J0, Y0, J1, Y1);
   const double tnx = nd.nx[t], tny = nd.ny[t], snx = nd.nx[s], sny = nd.ny[s];
   const double a = (tnx * dx + tny * dy) * ir, b = (snx * dx + sny * dy) * ir;
   const double ab = a * b;
@@ -194,12 +189,12 @@ __device__ __forceinline__ void offdiag_pair(const OpNodes& nd, int t, int s, do
   store_split(A, qs + qt * lda, Nre, Nim);
 }
 
-__global__ void __launch_bounds__(256) k_dense_offdiag(OpNodes nd, int total, double k, double ik, SplitOp A) {
+__global__ void __launch_bounds__(256) k_dense_offdiag(OpNodes nd, int total, double k, SplitOp A) {
   if (blockIdx.x * 64 >= blockIdx.y * 4 + 3) return;   // whole block on or below the diagonal
   const int s = blockIdx.y * 4 + (threadIdx.x & 3);
   const int t = blockIdx.x * 64 + (threadIdx.x >> 2);
   if (s >= total || t >= s) return;
-  offdiag_pair(nd, t, s, k, ik, A);
+  offdiag_pair(nd, t, s, k, A);
 }
 
 // Persistent form, for a run beside other kernels with a small footprint
@@ -208,7 +203,7 @@ __global__ void __launch_bounds__(256) k_dense_offdiag(OpNodes nd, int total, do
 // passes of 32 t x 4 s (s fastest: whole-sector writes in both halves).
 // At most 64 registers: 128 x 64 = 8,192 of the SM's 65,536 (a 512-thread
 // CTA of 112 registers still fits beside it).
-__global__ void __maxnreg__(64) k_dense_offdiag_rows(OpNodes nd, int total, double k, double ik, SplitOp A,
+__global__ void __maxnreg__(64) k_dense_offdiag_rows(OpNodes nd, int total, double k, SplitOp A,
                                                            int* __restrict__ counter) {
   __shared__ int s_item;
   const int rows = (total + 3) / 4;
@@ -221,7 +216,7 @@ __global__ void __maxnreg__(64) k_dense_offdiag_rows(OpNodes nd, int total, doub
     const int s0 = (rows - 1 - item) * 4;
     const int s = s0 + (threadIdx.x & 3);
     for (int t = threadIdx.x >> 2; t < s0 + 3; t += 32)
-      if (s < total && t < s) offdiag_pair(nd, t, s, k, ik, A);
+      if (s < total && t < s) offdiag_pair(nd, t, s, k, A);
   }
 }
 
@@ -487,7 +482,7 @@ void assemble_dense_offdiag64(OpNodes nd, int total, double k0, SplitOp A, cudaS
   if (total <= 0) return;
   dim3 g((total + 63) / 64, (total + 3) / 4);
   KPROF_BEGIN(st);
-  k_dense_offdiag<<<g, 256, 0, st>>>(nd, total, k0, 1.0 / k0, A);
+  k_dense_offdiag<<<g, 256, 0, st>>>(nd, total, k0, A);
   pm_launch_count_add(1);
   KPROF_END(st, "dense_offdiag64", 0.0);
 }
@@ -504,7 +499,7 @@ void assemble_dense_offdiag64_rows(OpNodes nd, int total, double k0, SplitOp A, 
   cudaFuncSetAttribute(k_dense_offdiag_rows, cudaFuncAttributePreferredSharedMemoryCarveout,
                        cudaSharedmemCarveoutMaxShared);
   KPROF_BEGIN(st);
-  k_dense_offdiag_rows<<<sms, 128, 0, st>>>(nd, total, k0, 1.0 / k0, A, counter);
+  k_dense_offdiag_rows<<<sms, 128, 0, st>>>(nd, total, k0, A, counter);
   pm_launch_count_add(1);
   KPROF_END(st, "dense_offdiag64", 0.0);
 }
