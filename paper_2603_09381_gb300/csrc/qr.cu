@@ -55,64 +55,6 @@ __device__ __forceinline__ C v_entry(const QrProb<C>& p, int j0, int jb, int r, 
   return p.Z[r + (size_t)d * p.ld];
 }
 
-// One pass over the panel rows: applies reflector `ja` (if ja >= 0; its
-// factors f_k in s_f, its column scaled by sc into v) and accumulates the
-// inputs of step jn = ja + 1: N = sum_{r >= c'} |a_jn[r]|^2 and
-// S_k = sum_{r > c'} conj(a_jn[r]) a_k[r] for k > jn (c' = j0 + jn), with row
-// c' itself stored to s_row.  Every entry a thread needs is loaded before the
-// threads of its row store anything.
-template <typename C>
-__device__ __forceinline__ void panel_pass(const QrProb<C>& p, int j0, int jb, int ja, const C* s_f, C sc,
-                                           C* s_row, typename real_of<C>::type& N, C* S, int rank, int csize) {
-  typedef typename real_of<C>::type R;
-  typedef PanelSplit<2> L;
-  constexpr int Q = L::Q, HB = L::HB, RW = L::RW;
-  const int jn = ja + 1;
-  const int ca = j0 + ja, cn = j0 + jn;
-  C* Zp = p.Z + (size_t)j0 * p.ld;
-  const size_t ld = p.ld;
-  const int lane = threadIdx.x & 31, q = lane / RW;
-  const int kmin = ja >= 0 ? ja : jn;
-  const C fjn = (ja >= 0 && jn < jb) ? s_f[jn] : czero<C>();
-  // warp-uniform sweep (the __syncwarp below needs every lane), rows guarded
-  for (int r0 = (ja >= 0 ? ca : cn) + (threadIdx.x >> 5) * RW + rank * L::PR; r0 < p.W; r0 += L::PR * csize) {
-    const int r = r0 + lane % RW;
-    const bool act = r < p.W;
-    C v[HB];
-#pragma unroll
-    for (int k = 0; k < HB; ++k)
-      if (Q * k + Q > kmin && act && Q * k + q >= kmin && Q * k + q < jb) v[k] = Zp[r + (size_t)(Q * k + q) * ld];
-    const C x = (act && ja >= 0) ? Zp[r + (size_t)ja * ld] : czero<C>();
-    const C yold = (act && jn < jb) ? Zp[r + (size_t)jn * ld] : czero<C>();
-    __syncwarp();   // the threads of the row have read it before any of them writes it
-    if (!act) continue;
-    C vr = czero<C>();
-    if (ja >= 0) {
-      vr = (r == ca) ? mk((R)1, (R)0) : x * sc;
-      if (r > ca && q == ja % Q) Zp[r + (size_t)ja * ld] = vr;
-#pragma unroll
-      for (int k = 0; k < HB; ++k)
-        if (Q * k + Q - 1 > ja && Q * k + q > ja && Q * k + q < jb) {
-          cfms(v[k], s_f[Q * k + q], vr);
-          Zp[r + (size_t)(Q * k + q) * ld] = v[k];
-        }
-    }
-    if (jn < jb && r >= cn) {
-      C y = yold;
-      if (ja >= 0) cfms(y, fjn, vr);
-      if (q == 0) N += abs2(y);
-      if (r == cn) {
-#pragma unroll
-        for (int k = 0; k < HB; ++k) if (Q * k + q >= jn && Q * k + q < jb) s_row[Q * k + q] = v[k];
-      } else {
-#pragma unroll
-        for (int k = 0; k < HB; ++k)
-          if (Q * k + Q - 1 > jn && Q * k + q > jn && Q * k + q < jb) cfma_conj(S[k], y, v[k]);
-      }
-    }
-  }
-}
-
 __device__ __forceinline__ float2 shfl_xor_c(float2 v, int o) {
   return make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
 }
@@ -120,161 +62,292 @@ __device__ __forceinline__ longlong2 shfl_xor_c(longlong2 v, int o) {
   return make_longlong2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
 }
 
+// ---- complex64 panel ----------------------------------------------------------------
+// A panel of 32 columns in four sub-panels of SB = 8 on a cluster, each CTA
+// with a block of rows, a thread per row.  What bounded the plain right-looking
+// panel was the L2: every column's pass read and wrote all columns to its
+// right (16 of them on average) for one multiply-add per byte.  The 8 columns
+// of a sub-panel stay in shared memory (SM; in place, in L2, when a CTA has
+// more than SUB_ROWS rows) while their reflectors are found; the columns to
+// the right are then updated once per sub-panel, C -= V w with
+//   w_j = conj(tau_j) (v_j^H C - sum_{l<j} v_j^H v_l w_l),
+// and the products V^H [earlier V, V, C] of that update also give G = V^H V for
+// the compact-WY factor T (the sums over rows once per 256 products instead of
+// a separate pass).  Per column one cluster barrier: every CTA pushes its
+// partial sums to the others before it, and every warp forms the reflector
+// (LAPACK zlarfg phase) from them.
 // At most 112 registers: 512 x 112 leaves room on the SM for one CTA of the
 // operator assembly that may run beside the factorization.
-template <typename C>
-__global__ void __maxnreg__(112) k_qr_panel(const QrProb<C>* __restrict__ P, int j0) {
-  typedef typename real_of<C>::type R;
-  typedef PanelSplit<2> L;
-  constexpr int Q = L::Q, HB = L::HB, RW = L::RW;
+constexpr int SB = 8;
+constexpr int SUB_ROWS = 2560;                                    // x 64 bytes: 160 KB
+constexpr int YV = QR_NB * SB;                                    // products per sub-panel
+constexpr size_t PANEL_RED = (size_t)(PT / 32) * YV * sizeof(float2);   // every warp's
+template <bool SM>
+__global__ void __maxnreg__(112) k_qr_panel(const QrProb<float2>* __restrict__ P, int j0, int ldp) {
+  typedef float2 C;
   cg::cluster_group cluster = cg::this_cluster();
   const int csize = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const QrProb<C> p = P[blockIdx.x / csize];
   if (j0 >= p.n) return;   // the whole cluster (same matrix) leaves
-  const int jb = min(QR_NB, p.n - j0);
-  const int W = p.W;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q = lane / RW;
-  constexpr int NV = 4 * QR_NB + 1;   // S (re, im), N, row c' (re, im)
-  __shared__ R s_red[PT / 32][2 * QR_NB + 1];
-  __shared__ R s_part[2][NV];         // this CTA's partial sums, by pass parity
-  __shared__ R s_tot[NV];
-  __shared__ C s_f[QR_NB];
-  __shared__ C s_row[QR_NB];          // row c' entries held by this CTA (zero elsewhere)
+  const int jb = min(QR_NB, p.n - j0), W = p.W;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr int NS = 2 * SB + 1, NV = NS + 2 * SB;   // S (re, im), N; row c' (re, im)
+  extern __shared__ __align__(16) unsigned char qr_sm[];
+  C* s_yw = reinterpret_cast<C*>(qr_sm);                       // [PT / 32][YV]
+  C (*s_t)[QR_NB + 1] = reinterpret_cast<C (*)[QR_NB + 1]>(qr_sm);   // (after the last sub-panel)
+  __shared__ float s_red[PT / 32][NS];
+  __shared__ float s_in[2][8][NV];     // the CTAs' partial sums, by pass parity
+  __shared__ C s_row[SB];              // row c' (rank 0 has the pivot rows)
   __shared__ C s_tau[QR_NB];
-  __shared__ C s_sc;
-  __shared__ C s_v[RC][QR_NB + 1];
-  __shared__ C s_g[QR_NB][QR_NB + 1];
-  __shared__ C s_t[QR_NB][QR_NB + 1];
-  if (tid < QR_NB) s_row[tid] = czero<C>();
-  __syncthreads();
-  C sc = czero<C>();
+  __shared__ C s_y[YV], s_yt[YV];      // V^H [..]: this CTA's, the cluster's ([column][l])
+  __shared__ C s_w[QR_NB][SB];
+  __shared__ C s_g[QR_NB][QR_NB + 1];  // s_g[j][l] = v_j^H v_l, l <= j
+  // block of rows, a multiple of 32 (so rank 0 holds all pivot rows)
+  const int nr = ((W - j0 + csize - 1) / csize + 31) & ~31, rb = j0 + rank * nr, re = min(W, rb + nr);
+  const size_t ld = p.ld;
+  C* Zp = p.Z + (size_t)j0 * ld;       // panel column k at Zp + k ld
+  if (SM) {
+    C* X = reinterpret_cast<C*>(qr_sm + PANEL_RED);
+    for (int r = rb + tid; r < re; r += PT)
+#pragma unroll
+      for (int k = 0; k < SB; ++k)
+        if (k < jb) X[r - rb + k * ldp] = Zp[r + (size_t)k * ld];
+  }
+  if (tid < SB) s_row[tid] = make_float2(0.f, 0.f);
+  for (int e = tid; e < QR_NB * (QR_NB + 1); e += PT) (&s_g[0][0])[e] = make_float2(0.f, 0.f);
+  cluster.sync();   // no CTA writes to one that has not started
   int par = 0;
-  for (int ja = -1; ja < jb; ++ja, par ^= 1) {
-    R N = 0;
-    C S[HB];
+  for (int c0 = 0; c0 < jb; c0 += SB) {
+    const int nb = min(SB, jb - c0);
+    C* X = SM ? reinterpret_cast<C*>(qr_sm + PANEL_RED) - rb : Zp + (size_t)c0 * ld;   // row r of column k: X[r + k ldx]
+    const size_t ldx = SM ? (size_t)ldp : ld;
+    C f[SB], sc = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int k = 0; k < HB; ++k) S[k] = czero<C>();
-    panel_pass(p, j0, jb, ja, s_f, sc, s_row, N, S, rank, csize);
-    const int jn = ja + 1;
-    if (jn >= jb) break;
-    // CTA sums: N over all lanes; S over the RW lanes of each q, halving the
-    // columns with every exchange (lane i of a q ends with column slot i)
-    N = warp_sum(N);
+    for (int k = 0; k < SB; ++k) f[k] = make_float2(0.f, 0.f);
+    for (int ja = -1; ja < nb; ++ja, par ^= 1) {
+      // reflector ja applied (its column scaled into v); for step jn = ja + 1:
+      // N = sum_{r >= c'} |a_jn|^2, S_k = sum_{r > c'} conj(a_jn) a_k, k > jn
+      const int jn = ja + 1, ca = j0 + c0 + ja, cn = ca + 1;
+      float N = 0.f;
+      C S[SB];
 #pragma unroll
-    for (int o = RW / 2, cnt = HB / 2; o > 0; o >>= 1, cnt >>= 1) {
-      const bool up = (lane & o) != 0;
+      for (int k = 0; k < SB; ++k) S[k] = make_float2(0.f, 0.f);
+      for (int r = rb + tid; r < re; r += PT) {
+        if (r < (ja >= 0 ? ca : cn)) continue;
+        C a[SB];
 #pragma unroll
-      for (int k = 0; k < HB / 2; ++k)
-        if (k < cnt) {
-          const C send = up ? S[k] : S[k + cnt], keep = up ? S[k + cnt] : S[k];
-          S[k] = keep + shfl_xor_c(send, o);
+        for (int k = 0; k < SB; ++k) a[k] = (k > ja && k < nb) ? X[r + k * ldx] : make_float2(0.f, 0.f);
+        if (ja >= 0) {
+          C v = make_float2(1.f, 0.f);
+          if (r > ca) {
+            v = X[r + ja * ldx] * sc;
+            X[r + ja * ldx] = v;
+          }
+#pragma unroll
+          for (int k = 0; k < SB; ++k)
+            if (k > ja && k < nb) {
+              cfms(a[k], f[k], v);
+              X[r + k * ldx] = a[k];
+            }
         }
+        if (jn < nb && r >= cn) {
+          C y = a[0];
+#pragma unroll
+          for (int k = 1; k < SB; ++k)
+            if (k == jn) y = a[k];
+          N += abs2(y);
+          if (r == cn) {
+#pragma unroll
+            for (int k = 0; k < SB; ++k) s_row[k] = a[k];
+          } else {
+#pragma unroll
+            for (int k = 0; k < SB; ++k)
+              if (k > jn) cfma_conj(S[k], y, a[k]);
+          }
+        }
+      }
+      if (jn >= nb) break;
+      // warp sums, halving the columns with the first exchanges: column lane / 4
+      N = warp_sum(N);
+#pragma unroll
+      for (int o = 16, cnt = SB / 2; o >= 4; o >>= 1, cnt >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int k = 0; k < SB / 2; ++k)
+          if (k < cnt) {
+            const C send = up ? S[k] : S[k + cnt], keep = up ? S[k + cnt] : S[k];
+            S[k] = keep + shfl_xor_c(send, o);
+          }
+      }
+      S[0] = S[0] + shfl_xor_c(S[0], 2);
+      S[0] = S[0] + shfl_xor_c(S[0], 1);
+      if ((lane & 3) == 0) {
+        s_red[warp][lane >> 1] = S[0].x;
+        s_red[warp][(lane >> 1) + 1] = S[0].y;
+      }
+      if (lane == 0) s_red[warp][2 * SB] = N;
+      __syncthreads();
+      for (int t = tid; t < csize * NV; t += PT) {
+        const int dst = t / NV, i = t % NV;
+        float u = 0.f;
+        if (i < NS) {
+#pragma unroll
+          for (int w = 0; w < PT / 32; ++w) u += s_red[w][i];
+        } else {
+          u = reinterpret_cast<const float*>(s_row)[i - NS];
+        }
+        cluster.map_shared_rank(&s_in[par][rank][0], dst)[i] = u;
+      }
+      cluster.sync();   // every CTA's partials of this pass have arrived
+      // lanes 0 .. 15: S, 16 .. 31: row c'; N in all
+      float t = lane < 2 * SB ? 0.f : s_in[par][0][lane + 1];
+      N = 0.f;
+      for (int r = 0; r < csize; ++r) {   // rank order
+        if (lane < 2 * SB) t += s_in[par][r][lane];
+        N += s_in[par][r][2 * SB];
+      }
+      const C alpha = make_float2(__shfl_sync(0xffffffffu, t, 2 * SB + 2 * jn), __shfl_sync(0xffffffffu, t, 2 * SB + 2 * jn + 1));
+      const int kk = lane & (SB - 1);
+      const C Sk = make_float2(__shfl_sync(0xffffffffu, t, 2 * kk), __shfl_sync(0xffffffffu, t, 2 * kk + 1));
+      const C rowk = make_float2(__shfl_sync(0xffffffffu, t, 2 * SB + 2 * kk), __shfl_sync(0xffffffffu, t, 2 * SB + 2 * kk + 1));
+      const float xnorm = sqrtf(N);
+      C tau = make_float2(0.f, 0.f);
+      float beta = 0.f;
+      sc = tau;
+      if (xnorm > 0.f) {
+        beta = -copysignf(xnorm, alpha.x);
+        const C bm = make_float2(beta, 0.f);
+        tau = cdiv(bm - alpha, bm);
+        sc = cdiv(make_float2(1.f, 0.f), alpha - bm);
+      }
+      const C fk = conj(tau) * (rowk + conj(sc) * Sk);
+#pragma unroll
+      for (int k = 0; k < SB; ++k)
+        f[k] = make_float2(__shfl_sync(0xffffffffu, fk.x, k), __shfl_sync(0xffffffffu, fk.y, k));
+      if (rank == 0 && cn < re && tid == (cn - rb) % PT) X[cn + jn * ldx] = make_float2(beta, 0.f);   // (the row's thread)
+      if (tid == 0) s_tau[c0 + jn] = tau;
     }
-    {
-      const int col = Q * (lane % RW) + q;
-      s_red[warp][2 * col] = S[0].x;
-      s_red[warp][2 * col + 1] = S[0].y;
-      if (lane == 0) s_red[warp][2 * QR_NB] = N;
+    // V^H [earlier V, V, C], 4 columns at a time
+    auto masked = [&](C x, int r, int col) {
+      const int e = r - (j0 + col);
+      return e > 0 ? x : make_float2(e == 0 ? 1.f : 0.f, 0.f);
+    };
+    auto v_row = [&](int r, C* v) {
+#pragma unroll
+      for (int l = 0; l < SB; ++l) v[l] = l < nb ? X[r + l * ldx] : make_float2(0.f, 0.f);
+      if (r < j0 + QR_NB) {
+#pragma unroll
+        for (int l = 0; l < SB; ++l) v[l] = l < nb ? masked(v[l], r, c0 + l) : make_float2(0.f, 0.f);
+      }
+    };
+    for (int k0 = 0; k0 < QR_NB; k0 += 4) {
+      C acc[4 * SB];
+#pragma unroll
+      for (int i = 0; i < 4 * SB; ++i) acc[i] = make_float2(0.f, 0.f);
+      if (k0 < jb) {
+        const bool own = k0 >= c0 && k0 < c0 + SB;
+        const C* src = own ? X + (size_t)(k0 - c0) * ldx : Zp + (size_t)k0 * ld;
+        const size_t lds = own ? ldx : ld;
+        for (int r = rb + tid; r < re; r += PT) {
+          C v[SB], c[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) c[i] = k0 + i < jb ? src[r + i * lds] : make_float2(0.f, 0.f);
+          if (r < j0 + QR_NB && k0 < c0 + SB) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) c[i] = k0 + i < jb ? masked(c[i], r, k0 + i) : make_float2(0.f, 0.f);
+          }
+          v_row(r, v);
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int l = 0; l < SB; ++l) cfma_conj(acc[i * SB + l], v[l], c[i]);
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {   // lane i ends with product i
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int k = 0; k < 2 * SB; ++k)
+          if (k < o) {
+            const C send = up ? acc[k] : acc[k + o], keep = up ? acc[k + o] : acc[k];
+            acc[k] = keep + shfl_xor_c(send, o);
+          }
+      }
+      s_yw[warp * YV + k0 * SB + lane] = acc[0];
     }
     __syncthreads();
-    if (tid < 2 * QR_NB + 1) {
-      R t = 0;
+    {
+      float u = 0.f;
 #pragma unroll
-      for (int w = 0; w < PT / 32; ++w) t += s_red[w][tid];
-      s_part[par][tid] = t;
-    } else if (tid < NV) {
-      const int k = (tid - 2 * QR_NB - 1) >> 1;
-      s_part[par][tid] = ((tid - 2 * QR_NB - 1) & 1) ? s_row[k].y : s_row[k].x;
+      for (int w = 0; w < PT / 32; ++w) u += reinterpret_cast<const float*>(s_yw)[w * 2 * YV + tid];
+      reinterpret_cast<float*>(s_y)[tid] = u;
     }
-    cluster.sync();   // every CTA's partials of this pass are written
-    if (tid < NV) {
-      R t = 0;
-      for (int r = 0; r < csize; ++r) t += cluster.map_shared_rank(&s_part[par][0], r)[tid];   // rank order
-      s_tot[tid] = t;
+    cluster.sync();
+    {
+      float u = 0.f;
+      for (int r = 0; r < csize; ++r) u += reinterpret_cast<const float*>(cluster.map_shared_rank(&s_y[0], r))[tid];   // rank order
+      reinterpret_cast<float*>(s_yt)[tid] = u;
     }
-    if (tid < QR_NB) s_row[tid] = czero<C>();
     __syncthreads();
     if (warp == 0) {
-      // reflector of column jn (LAPACK zlarfg phase), factors of the next
-      // pass: lane k's column k (the scalars in every lane alike)
-      const int c = j0 + jn;
-      const C alpha = mk(s_tot[2 * QR_NB + 1 + 2 * jn], s_tot[2 * QR_NB + 2 + 2 * jn]);
-      const R xnorm = sqrt(s_tot[2 * QR_NB]);
-      C tau = czero<C>(), scn = czero<C>();
-      R beta = 0;
-      if (xnorm > 0) {
-        beta = -copysign(xnorm, alpha.x);
-        const C bm = mk(beta, (R)0);
-        tau = cdiv(bm - alpha, bm);
-        scn = cdiv(mk((R)1, (R)0), alpha - bm);
-      }
-      if (rank == 0 && lane == 0) p.Z[c + (size_t)c * p.ld] = mk(beta, (R)0);
-      if (lane == 0) {
-        s_tau[jn] = tau;
-        s_sc = scn;
-      }
-      const C ctau = conj(tau), cscn = conj(scn);
-      if (lane > jn && lane < jb) {
-        const C rowk = mk(s_tot[2 * QR_NB + 1 + 2 * lane], s_tot[2 * QR_NB + 2 + 2 * lane]);
-        s_f[lane] = ctau * (rowk + cscn * mk(s_tot[2 * lane], s_tot[2 * lane + 1]));
+      const int k = lane;
+      C w[SB];
+#pragma unroll
+      for (int j = 0; j < SB; ++j) {
+        C y = s_yt[k * SB + j];
+        if (j < nb && k <= c0 + j) s_g[c0 + j][k] = y;
+#pragma unroll
+        for (int l = 0; l < j; ++l) cfms(y, s_yt[(c0 + l) * SB + j], w[l]);
+        w[j] = j < nb ? conj(s_tau[c0 + j]) * y : make_float2(0.f, 0.f);
+        s_w[k][j] = w[j];
       }
     }
     __syncthreads();
-    sc = s_sc;
-  }
-  // the last pass stored its reflector in rows that other CTAs of the
-  // cluster read below (rows are dealt out differently there)
-  cluster.sync();
-  // G = V^H V over chunks of this CTA's rows staged in shared memory (V also
-  // written out), then summed over the cluster
-  {
-    const int gi = tid & 31, gj = tid >> 5;   // G[gi][gj] and G[gi][gj + 16]
-    C g0 = czero<C>(), g1 = czero<C>();
-    for (int r0 = j0 + rank * RC; r0 < W; r0 += RC * csize) {
-      for (int e = tid; e < RC * QR_NB; e += PT) {
-        const int i = e % RC, j = e / RC;
-        const C v = v_entry(p, j0, jb, r0 + i, j);
-        s_v[i][j] = v;
-        if (p.V && r0 + i < W) p.V[(r0 + i - j0) + (size_t)j * p.W] = v;
+    for (int r = rb + tid; r < re; r += PT) {
+      C v[SB];
+      if (SM) {
+#pragma unroll
+        for (int l = 0; l < SB; ++l)
+          if (l < nb) Zp[r + (size_t)(c0 + l) * ld] = X[r + l * ldx];
       }
-      __syncthreads();
-#pragma unroll 8
-      for (int i = 0; i < RC; ++i) {
-        const C a = s_v[i][gi];
-        cfma_conj(g0, a, s_v[i][gj]);
-        cfma_conj(g1, a, s_v[i][gj + 16]);
+      v_row(r, v);
+      if (p.V) {
+#pragma unroll
+        for (int l = 0; l < SB; ++l) p.V[(r - j0) + (size_t)(c0 + l) * W] = v[l];
       }
-      __syncthreads();
+#pragma unroll 4
+      for (int k = c0 + SB; k < jb; ++k) {
+        C c = Zp[r + (size_t)k * ld];
+#pragma unroll
+        for (int l = 0; l < SB; ++l) cfms(c, v[l], s_w[k][l]);
+        if (SM && k < c0 + 2 * SB) X[r + (k - c0 - SB) * ldx] = c;
+        else Zp[r + (size_t)k * ld] = c;
+      }
     }
-    s_t[gi][gj] = g0;   // s_t holds this CTA's partial G until T is built
-    s_t[gi][gj + 16] = g1;
-    cluster.sync();
-    C a0 = czero<C>(), a1 = czero<C>();
-    for (int q = 0; q < csize; ++q) {
-      const C* rt = &cluster.map_shared_rank(&s_t[0][0], q)[0];
-      a0 = a0 + rt[gi * (QR_NB + 1) + gj];
-      a1 = a1 + rt[gi * (QR_NB + 1) + gj + 16];
-    }
-    s_g[gi][gj] = a0;
-    s_g[gi][gj + 16] = a1;
-    cluster.sync();   // no CTA reuses s_t (or leaves) while another still reads it
   }
-  // T: T_jj = tau_j, T[0:j, j] = -tau_j T[0:j, 0:j] G[0:j, j]
-  for (int e = tid; e < QR_NB * QR_NB; e += PT) {
-    const int i = e % QR_NB, j = e / QR_NB;
-    s_t[i][j] = (i == j && i < jb) ? s_tau[i] : czero<C>();
-  }
-  __syncthreads();
-  for (int j = 1; j < jb; ++j) {
-    if (tid < j) {
-      C acc = czero<C>();
-      for (int l = tid; l < j; ++l) cfma(acc, s_t[tid][l], s_g[l][j]);
-      s_t[tid][j] = -(s_tau[j] * acc);
+  if (p.V)
+    for (int j = (jb + SB - 1) / SB * SB; j < QR_NB; ++j)
+      for (int r = rb + tid; r < re; r += PT) p.V[(r - j0) + (size_t)j * W] = make_float2(0.f, 0.f);
+  // T: T_jj = tau_j, T[0:j, j] = -tau_j T[0:j, 0:j] G[0:j, j]; 16 lanes per row
+  if (rank == 0) {
+    const int i = tid >> 4, part = tid & 15;
+    for (int e = tid; e < QR_NB * QR_NB; e += PT) {
+      const int a = e % QR_NB, b = e / QR_NB;
+      s_t[a][b] = (a == b && a < jb) ? s_tau[a] : make_float2(0.f, 0.f);
     }
     __syncthreads();
-  }
-  if (rank == 0)
+    for (int j = 1; j < jb; ++j) {
+      C acc = make_float2(0.f, 0.f);
+      if (i < j)
+        for (int l = i + part; l < j; l += 16) cfma(acc, s_t[i][l], conj(s_g[j][l]));
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) acc = acc + shfl_xor_c(acc, o);
+      if (i < j && part == 0) s_t[i][j] = -(s_tau[j] * acc);
+      __syncthreads();
+    }
     for (int e = tid; e < QR_NB * QR_NB; e += PT) p.T[e] = s_t[e % QR_NB][e / QR_NB];
+  }
+  cluster.sync();   // no CTA leaves while another may still read its sums
 }
 
 // ---- complex128 panel in 60-bit fixed point ----------------------------------------
@@ -970,7 +1043,21 @@ void qr_panel(const QrProb<C>* d_prob, int nprob, int j0, cudaStream_t st, int c
       cudaLaunchKernelEx(&cfg, k_qr_panel_fx<false>, d_prob, j0, 0);
     }
   } else {
-    cudaLaunchKernelEx(&cfg, k_qr_panel<C>, d_prob, j0);
+    auto rows = [&](int c) { return ((max_w - j0 + c - 1) / c + 31) & ~31; };
+    while (cs < 8 && rows(cs) > SUB_ROWS) cs *= 2;   // the sub-panels in shared memory
+    cfg.gridDim = dim3(nprob * cs);
+    attr[0].val.clusterDim.x = cs;
+    if (max_w > 0 && rows(cs) <= SUB_ROWS) {
+      cfg.dynamicSmemBytes = PANEL_RED + (size_t)rows(cs) * SB * sizeof(C);
+      // the same value every time: idempotent across threads and devices
+      cudaFuncSetAttribute(k_qr_panel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)(PANEL_RED + (size_t)SUB_ROWS * SB * sizeof(C)));
+      cudaLaunchKernelEx(&cfg, k_qr_panel<true>, d_prob, j0, rows(cs));
+    } else {
+      cfg.dynamicSmemBytes = PANEL_RED;
+      cudaFuncSetAttribute(k_qr_panel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PANEL_RED);
+      cudaLaunchKernelEx(&cfg, k_qr_panel<false>, d_prob, j0, 0);
+    }
   }
   pm_launch_count_add(1);
   KPROF_END(st, kname<C>("qr_panel", "qr_panel32"), 0.0);

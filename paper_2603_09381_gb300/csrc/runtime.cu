@@ -1398,7 +1398,7 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
             CK(cudaMemsetAsync(terr, 0, sizeof(int), st));
           }
           for (int j0 = 0; j0 < maxn; j0 += QR_NB) {
-            qr_panel<C>(dqp, nq, j0, st);
+            qr_panel<C>(dqp, nq, j0, st, 0, maxW);
             const int tiles = (maxn - j0 - QR_NB + 31) / 32;
             const int rbs = (maxW - j0 + QR_RB - 1) / QR_RB;
             if (tiles > 0)
@@ -1418,7 +1418,9 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
           // Y^H = C^H V, Y^H <- Y^H T, C -= V Y.  All panels' problem lists
           // are built and uploaded at once.
           std::vector<C*> yh(nq), y2h(nq);
+          int maxW = 0;
           for (int q = 0; q < nq; ++q) {
+            maxW = std::max(maxW, qp[q].W);
             qp[q].V = scr.get<C>((size_t)qp[q].W * QR_NB);
             yh[q] = scr.get<C>((size_t)qp[q].n * QR_NB);
             y2h[q] = scr.get<C>((size_t)qp[q].n * QR_NB);
@@ -1457,7 +1459,7 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
           auto* dqp = upload(scr, qp, st);
           int pi = 0;
           for (int j0 = 0; j0 < maxn; j0 += QR_NB, ++pi) {
-            qr_panel<C>(dqp, nq, j0, st);
+            qr_panel<C>(dqp, nq, j0, st, 0, maxW);
             const int s0 = pstart[pi], c = pcount[pi];
             if (c == 0) continue;
             for (int l = 0; l < 3; ++l) {
