@@ -390,17 +390,21 @@ __global__ void __launch_bounds__(PT, 1) k_qr_panel_fx(const QrProb<double2>* __
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q = lane / RW;
   const int rbeg = j0 + warp * RW + rank * L::PR, rstep = L::PR * csize;   // the warp's first row and stride
   const int xbeg = SM ? warp * RW + lane % RW : rbeg + lane % RW, xstep = SM ? L::PR : rstep;
-  constexpr int NV = 4 * QR_NB + 1;   // S (re, im), N, row c' (re, im)
-  __shared__ double s_red[PT / 32][2 * QR_NB + 1];
-  __shared__ double s_part[2][NV];    // this CTA's partial sums, by pass parity
-  __shared__ double s_tot[NV];
-  __shared__ longlong2 s_row[QR_NB];  // row c' entries held by this CTA (zero elsewhere)
+  constexpr int NS = 2 * QR_NB + 2;   // S (re, im), N (low, high)
+  __shared__ long long s_red[PT / 32][2 * QR_NB + 1];
+  __shared__ int s_ew[PT / 32];
+  __shared__ long long s_in[2][8][NS];      // the CTAs' partial sums, by pass parity,
+  __shared__ int s_m[2][8];                 // their shifts,
+  __shared__ longlong2 s_rowin[2][QR_NB];   // and row c'
+  __shared__ double s_nrm[PT / 32][QR_NB], s_n2[QR_NB];
+  __shared__ longlong2 s_row[QR_NB];  // row c' (rank 0 has the pivot rows)
   __shared__ int4 s_g[QR_NB];         // factors of the next pass: re, im as (h, l) ..
   __shared__ int2 s_gn[QR_NB];        // .. and -im
-  __shared__ double s_beta[QR_NB];
+  __shared__ long long s_beta[QR_NB]; // R's diagonal: 2^(s_bev - 60) in units of the column's scale
+  __shared__ int s_bev[QR_NB];
   __shared__ int s_exp[QR_NB];        // scale of column k: 2^s_exp
   __shared__ int s_bad;               // columns from here on are not finite, or follow one that is not
-  __shared__ double2 s_tau[QR_NB];
+  __shared__ longlong2 s_tau[QR_NB];  // tau / 2
   __shared__ longlong2 s_sc;
   __shared__ int s_ev;
   // column norms: the scale of column k is the power of two that brings its norm into (1/8, 1/4]
@@ -418,20 +422,19 @@ __global__ void __launch_bounds__(PT, 1) k_qr_panel_fx(const QrProb<double2>* __
       for (int o = RW / 2; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
     if (lane % RW == 0)
 #pragma unroll
-      for (int k = 0; k < HB; ++k) s_red[warp][Q * k + q] = acc[k];
-    if (tid < QR_NB) s_row[tid] = make_longlong2(0, 0);
+      for (int k = 0; k < HB; ++k) s_nrm[warp][Q * k + q] = acc[k];
     if (tid == 0) s_bad = QR_NB;
     __syncthreads();
     if (tid < QR_NB) {
       double t = 0;
 #pragma unroll
-      for (int w = 0; w < PT / 32; ++w) t += s_red[w][tid];
-      s_part[1][tid] = t;
+      for (int w = 0; w < PT / 32; ++w) t += s_nrm[w][tid];
+      s_n2[tid] = t;
     }
     cluster.sync();
     if (tid < jb) {
       double t = 0;
-      for (int r = 0; r < csize; ++r) t += cluster.map_shared_rank(&s_part[1][0], r)[tid];
+      for (int r = 0; r < csize; ++r) t += cluster.map_shared_rank(&s_n2[0], r)[tid];
       int e = 0;
       if (!isfinite(t)) atomicMin(&s_bad, tid);
       else if (t > 0) frexp(sqrt(t) * (1.0 + 1e-9), &e);
@@ -450,6 +453,9 @@ __global__ void __launch_bounds__(PT, 1) k_qr_panel_fx(const QrProb<double2>* __
     __syncwarp();
   }
   int par = 0;
+  // a row of y is below 2^55 (2^-5) after a warp's shift, less for very tall
+  // panels: |S| <= 2^-5 sqrt(2 W) / 4 stays below 2, a warp's N below 1
+  const int ytop = 54 - (33 - __clz(W >> 15)) / 2;
   for (int ja = -1; ja < jb; ++ja, par ^= 1) {
     const int jn = ja + 1, ca = j0 + ja, cn = j0 + jn;
     // column ja becomes v, column jn is brought up to date and measured
@@ -457,41 +463,39 @@ __global__ void __launch_bounds__(PT, 1) k_qr_panel_fx(const QrProb<double2>* __
     int ev = 0;
     if (ja >= 0) {
       const longlong2 sc = s_sc;
-      scr = fx(sc.x); sci = fx(sc.y); nsci = fx(-sc.y);
+      scr = fw(sc.x << 2); sci = fw(sc.y << 2); nsci = fw(-sc.y << 2);
       ev = s_ev;
     }
     unsigned long long any = 0;
-    for (int r0 = rbeg, xr = xbeg; r0 < W; r0 += rstep, xr += xstep) {   // the same steps for the whole warp
-      const int r = r0 + lane % RW;
-      const bool act = r < W && r >= (ja >= 0 ? ca : cn);
-      const longlong2 x = act && ja >= 0 ? Zx[xr + (size_t)ja * ldx] : make_longlong2(0, 0);
-      longlong2 y = act && jn < jb ? Zx[xr + (size_t)jn * ldx] : make_longlong2(0, 0);
-      __syncwarp();   // the row's threads have read both before one of them writes
-      if (!act) continue;
+    // (a thread per row here: the four threads of a row take four sweeps at a time)
+    for (int r = rbeg + lane % RW + q * rstep, xr = xbeg + q * xstep; r < W; r += Q * rstep, xr += Q * xstep) {
+      if (r < (ja >= 0 ? ca : cn)) continue;
+      longlong2 y = jn < jb ? Zx[xr + (size_t)jn * ldx] : make_longlong2(0, 0);
       if (ja >= 0) {
         longlong2 v;
         if (r == ca) {
           v = make_longlong2(1ll << 60, 0);
         } else {
-          v = fx_cfma(make_longlong2(0, 0), scr, sci, nsci, fx(x.x << ev), fx(x.y << ev));
+          const longlong2 x = Zx[xr + (size_t)ja * ldx];
+          v = fw_cfma(make_longlong2(0, 0), scr, sci, nsci, fw(x.x << (ev + 2)), fw(x.y << (ev + 2)));
           v.x <<= 1; v.y <<= 1;
-          if (q == 0) Zx[xr + (size_t)ja * ldx] = v;
+          Zx[xr + (size_t)ja * ldx] = v;
         }
         if (jn < jb) {
           const int4 g = s_g[jn];
           const int2 gn = s_gn[jn];
-          y = fx_cfma(y, Fx{g.x, g.y}, Fx{g.z, g.w}, Fx{gn.x, gn.y}, fx(v.x), fx(v.y));
-          if (q == 1) Zx[xr + (size_t)jn * ldx] = y;
+          y = fw_cfma(y, Fx{g.x, g.y}, Fx{g.z, g.w}, Fx{gn.x, gn.y}, fw(v.x << 2), fw(v.y << 2));
+          Zx[xr + (size_t)jn * ldx] = y;
         }
       }
       if (jn < jb && r >= cn) any |= (unsigned long long)(y.x ^ (y.x >> 63)) | (unsigned long long)(y.y ^ (y.y >> 63));
     }
     __syncwarp();
     if (jn >= jb) break;
-    // shift that brings this warp's rows of y just below 2^55
+    // shift that brings this warp's rows of y just below 2^(ytop + 1)
     const unsigned ah = __reduce_or_sync(0xffffffffu, (unsigned)(any >> 32)), al = __reduce_or_sync(0xffffffffu, (unsigned)any);
     const int top = ah ? 63 - __clz(ah) : (al ? 31 - __clz(al) : 0);
-    const int ew = 54 - top;   // top <= 58: may be negative
+    const int ew = ytop - top;   // top <= 58: may be negative
     long long N = 0;
     longlong2 S[HB];
 #pragma unroll
@@ -504,13 +508,14 @@ __global__ void __launch_bounds__(PT, 1) k_qr_panel_fx(const QrProb<double2>* __
         if (Q * k + Q - 1 > jn && Q * k + q > jn && Q * k + q < jb) a[k] = Zx[xr + (size_t)(Q * k + q) * ldx];
       const longlong2 v = ja < 0 ? make_longlong2(0, 0) : r == ca ? make_longlong2(1ll << 60, 0) : Zx[xr + (size_t)ja * ldx];
       const longlong2 y0 = Zx[xr + (size_t)jn * ldx];
-      const longlong2 y = ew >= 0 ? make_longlong2(y0.x << ew, y0.y << ew) : make_longlong2(y0.x >> -ew, y0.y >> -ew);
-      const Fx vr = fx(v.x), vi = fx(v.y), yr = fx(y.x), yi = fx(y.y), nyi = fx(-y.y);
-      if (r >= cn && q == 0) {
-        long long cr = FX_HALF;
+      // (ew >= -4: the products' 2^4 goes on top)
+      const longlong2 y = make_longlong2(y0.x << (ew + 4), y0.y << (ew + 4));
+      const Fx vr = fw(v.x << 2), vi = fw(v.y << 2), yr = fw(y.x), yi = fw(y.y), nyi = fw(-y.y);
+      if (r >= cn && q == 0) {   // N in 2^-64
+        long long cr = FW_HALF;
         fx_mac(N, cr, yr, yr);
         fx_mac(N, cr, yi, yi);
-        N += cr >> 30;
+        N += cr >> 32;
       }
       if (r == cn && q == jn % Q) s_row[jn] = y0;
 #pragma unroll
@@ -519,25 +524,25 @@ __global__ void __launch_bounds__(PT, 1) k_qr_panel_fx(const QrProb<double2>* __
           if (ja >= 0) {
             const int4 g = s_g[Q * k + q];
             const int2 gn = s_gn[Q * k + q];
-            a[k] = fx_cfma(a[k], Fx{g.x, g.y}, Fx{g.z, g.w}, Fx{gn.x, gn.y}, vr, vi);
+            a[k] = fw_cfma(a[k], Fx{g.x, g.y}, Fx{g.z, g.w}, Fx{gn.x, gn.y}, vr, vi);
             Zx[xr + (size_t)(Q * k + q) * ldx] = a[k];
           }
           if (r == cn) {
             s_row[Q * k + q] = a[k];
           } else if (r > cn) {
-            const Fx ar = fx(a[k].x), ai = fx(a[k].y);
-            long long cr = FX_HALF, ci = FX_HALF;
+            const Fx ar = fw(a[k].x), ai = fw(a[k].y);
+            long long cr = FW_HALF, ci = FW_HALF;
             fx_mac(S[k].x, cr, yr, ar);
             fx_mac(S[k].x, cr, yi, ai);
             fx_mac(S[k].y, ci, yr, ai);
             fx_mac(S[k].y, ci, nyi, ar);
-            S[k].x += cr >> 30;
-            S[k].y += ci >> 30;
+            S[k].x += cr >> 32;
+            S[k].y += ci >> 32;
           }
         }
     }
     __syncwarp();
-    // warp sums as in k_qr_panel, in integers, then FP64 with the warp's shift taken out
+    // warp sums as in k_qr_panel, in integers
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) N += __shfl_xor_sync(0xffffffffu, N, o);
 #pragma unroll
@@ -552,50 +557,71 @@ __global__ void __launch_bounds__(PT, 1) k_qr_panel_fx(const QrProb<double2>* __
     }
     {
       const int col = Q * (lane % RW) + q;
-      const double u = __longlong_as_double((long long)(1023 - 60 - ew) << 52);   // 2^(-60 - ew)
-      s_red[warp][2 * col] = (double)S[0].x * u;
-      s_red[warp][2 * col + 1] = (double)S[0].y * u;
-      if (lane == 0) s_red[warp][2 * QR_NB] = (double)N * u * __longlong_as_double((long long)(1023 - ew) << 52);
+      s_red[warp][2 * col] = S[0].x;
+      s_red[warp][2 * col + 1] = S[0].y;
+      if (lane == 0) { s_red[warp][2 * QR_NB] = N; s_ew[warp] = ew; }
     }
     __syncthreads();
+    // over warps, then over CTAs (rank order), each at the smallest shift among
+    // them; a CTA pushes its sums to all before the barrier
     if (tid < 2 * QR_NB + 1) {
-      double t = 0;
+      int m = s_ew[0];
 #pragma unroll
-      for (int w = 0; w < PT / 32; ++w) t += s_red[w][tid];
-      s_part[par][tid] = t;
-    } else if (tid < NV) {
-      const int k = (tid - 2 * QR_NB - 1) >> 1;
-      s_part[par][tid] = (double)(((tid - 2 * QR_NB - 1) & 1) ? s_row[k].y : s_row[k].x) * (1.0 / FX_ONE);
+      for (int w = 1; w < PT / 32; ++w) m = min(m, s_ew[w]);
+      if (tid < 2 * QR_NB) {
+        long long t = 0;
+#pragma unroll
+        for (int w = 0; w < PT / 32; ++w) t += fx_shr(s_red[w][tid], s_ew[w] - m);
+        for (int r = 0; r < csize; ++r) cluster.map_shared_rank(&s_in[par][rank][0], r)[tid] = t;
+      } else {
+        unsigned __int128 t = 0;
+#pragma unroll
+        for (int w = 0; w < PT / 32; ++w) t += fx_norm_shr((unsigned __int128)(unsigned long long)s_red[w][tid] << 40, s_ew[w] - m);
+        for (int r = 0; r < csize; ++r) {
+          long long* dst = cluster.map_shared_rank(&s_in[par][rank][0], r);
+          dst[tid] = (long long)t;
+          dst[tid + 1] = (long long)(t >> 64);
+          *cluster.map_shared_rank(&s_m[par][rank], r) = m;
+        }
+      }
+    } else if (rank == 0 && tid >= 4 * QR_NB && tid < 5 * QR_NB) {
+      const longlong2 u = s_row[tid - 4 * QR_NB];
+      for (int r = 0; r < csize; ++r) cluster.map_shared_rank(&s_rowin[par][0], r)[tid - 4 * QR_NB] = u;
     }
-    cluster.sync();   // every CTA's partials of this pass are written
-    if (tid < NV) {
-      double t = 0;
-      for (int r = 0; r < csize; ++r) t += cluster.map_shared_rank(&s_part[par][0], r)[tid];   // rank order
-      s_tot[tid] = t;
-    }
-    if (tid < QR_NB) s_row[tid] = make_longlong2(0, 0);
-    __syncthreads();
+    cluster.sync();   // every CTA's sums of this pass have arrived
     if (warp == 0) {
       // reflector of column jn, in units of its scale; lane k: the factor of column k
-      const double2 alpha = make_double2(s_tot[2 * QR_NB + 1 + 2 * jn], s_tot[2 * QR_NB + 2 + 2 * jn]);
-      double beta;
-      double2 tau, sc;
-      fx_reflector(alpha, s_tot[2 * QR_NB], beta, tau, sc);
-      if (lane == 0) {
-        // v = x sc = 2 (x 2^ev) (sc 2^-ev / 2) with x 2^ev below 1 and |sc| 2^-ev at most 2
-        const int ev = fx_shift(s_tot[2 * QR_NB], 0);
-        const double u = 0.5 * FX_ONE * __longlong_as_double((long long)(1023 - ev) << 52);
-        s_sc = make_longlong2(__double2ll_rn(sc.x * u), __double2ll_rn(sc.y * u));
+      int M = s_m[par][0];
+      for (int r = 1; r < csize; ++r) M = min(M, s_m[par][r]);
+      longlong2 Sk = make_longlong2(0, 0);
+      unsigned __int128 n2 = 0;
+      for (int r = 0; r < csize; ++r) {
+        const long long* in = s_in[par][r];
+        const int d = s_m[par][r] - M;
+        Sk.x += fx_shr(in[2 * lane], d);
+        Sk.y += fx_shr(in[2 * lane + 1], d);
+        n2 += fx_norm_shr(((unsigned __int128)(unsigned long long)in[2 * QR_NB + 1] << 64) | (unsigned long long)in[2 * QR_NB], d);
+      }
+      const longlong2 alpha = s_rowin[par][jn];
+      int ev;
+      longlong2 tau2, sc2;
+      long long beta;
+      fx_reflect(alpha.x, alpha.y, n2, 104 + 2 * M, ev, tau2, sc2, beta);
+      if (lane == 0) {   // v = x sc = 2 (x 2^ev) (sc 2^-ev / 2)
+        s_sc = sc2;
         s_ev = ev;
         s_beta[jn] = beta;
-        s_tau[jn] = jn < s_bad ? tau : make_double2(nan(""), 0.0);
+        s_bev[jn] = -ev;
+        s_tau[jn] = tau2;
       }
       if (lane > jn && lane < jb) {
-        const double2 ctau = conj(tau), csc = conj(sc);
-        const double2 rowk = make_double2(s_tot[2 * QR_NB + 1 + 2 * lane], s_tot[2 * QR_NB + 2 + 2 * lane]);
-        const double2 f = ctau * (rowk + csc * make_double2(s_tot[2 * lane], s_tot[2 * lane + 1]));
-        const Fx gr = fx(__double2ll_rn(-f.x * FX_ONE)), gi = fx(__double2ll_rn(-f.y * FX_ONE)),
-                 gn = fx(__double2ll_rn(f.y * FX_ONE));
+        // -conj(tau) (row_k + conj(sc) S_k) = -4 conj(tau/2) (row_k/2 + conj(sc 2^-ev/2) (S_k 2^ev))
+        auto scaled = [&](long long S) { return ev >= M ? S << (ev - M) : fx_shr(S, M - ev); };
+        const longlong2 row = s_rowin[par][lane];
+        longlong2 w = make_longlong2((row.x + 1) >> 1, (row.y + 1) >> 1);
+        w = fx_cfma(w, fx(sc2.x), fx(-sc2.y), fx(sc2.y), fx(scaled(Sk.x)), fx(scaled(Sk.y)));
+        const longlong2 f = fx_cfma(make_longlong2(0, 0), fx(tau2.x), fx(-tau2.y), fx(tau2.y), fx(w.x), fx(w.y));
+        const Fx gr = fw(-(f.x << 4)), gi = fw(-(f.y << 4)), gn = fw(f.y << 4);   // f 4, and the products' 2^2
         s_g[lane] = make_int4(gr.h, gr.l, gi.h, gi.l);
         s_gn[lane] = make_int2(gn.h, gn.l);
       }
@@ -611,11 +637,12 @@ __global__ void __launch_bounds__(PT, 1) k_qr_panel_fx(const QrProb<double2>* __
       const longlong2 a = Zx[x + (size_t)col * ldx];
       const int e2 = r > j0 + col ? 0 : s_exp[col];
       double2 z = make_double2(fx_to(a.x, e2), fx_to(a.y, e2));
-      if (r == j0 + col) z = make_double2(ldexp(s_beta[col], e2), 0.0);
+      if (r == j0 + col) z = make_double2(fx_to(s_beta[col], s_exp[col] + s_bev[col]), 0.0);
       if (col >= s_bad) z = make_double2(nan(""), nan(""));
       p.Z[r + (size_t)(j0 + col) * ld] = z;
     }
-  if (rank == 0 && tid < jb) p.T[tid] = s_tau[tid];
+  if (rank == 0 && tid < jb)
+    p.T[tid] = make_double2(tid < s_bad ? fx_to(s_tau[tid].x, 1) : nan(""), tid < s_bad ? fx_to(s_tau[tid].y, 1) : 0.0);
   cluster.sync();   // no CTA leaves while another may still read its partial sums
 }
 
