@@ -275,8 +275,8 @@ __device__ __forceinline__ C omit_entry(const PointsDev& P, int t, int s, double
   const double z = k * r;
   const double w = P.w[ps];
   // only the orders the entry needs (a warp's entries are mostly of one kind)
-  const bool near = (float)z < (float)HK_ZA;
-  const double q = hk_rsqrt(z), iz = q * q;
+  const bool near = hk_near(z);
+  const double q = fx_rsqrt(z), iz = q * q;
   double J0, Y0, J1, Y1;
   if (rg == 0 && cg == 0) {         // -eps+ S = -(i/4) H0 w
     if (near) { J0 = j0(z); Y0 = y0(z); } else hankel_asym(z, iz, q, J0, Y0, J1, Y1);

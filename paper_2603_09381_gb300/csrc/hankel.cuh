@@ -8,16 +8,15 @@
 //   P_nu, Q_nu, the reduction of z by pi/2, sine, cosine and their products are
 //   computed in 60-bit fixed point on the integer multipliers: every value is
 //   below 1.01 and within about 1e-17, a tenth of what the FP64 forms give.
-//   FP64 does 1/sqrt(z) from an FP32 estimate (6 operations) and the scaling:
-//   14 FP64 operations for one order of about 70 before.
+//   FP64 does 1/sqrt(z) from an FP32 estimate (5 operations) and the scaling:
+//   12 FP64 operations for one order of about 70 before.  Conversions take an
+//   FP64 operation's time each, so they go through the bit patterns as well.
 //   - P_nu and z Q_nu: polynomials in 1/z^2 on [8, 12), [12, 20), [20, 30),
 //     [30, 60), [60, inf) (hankel_fit.h, written by gen_hankel_fit.py from
 //     40-digit values).
 //   - sine and cosine of w_0 = z - pi/4 serve both orders (w_1 = w_0 - pi/2).
 //   A caller that uses one order pays for one: what it leaves unused is
 //   compiled away.
-// The interval of z is chosen on z rounded to FP32 (comparisons on the FP32
-// pipes): the fits hold a little beyond their ends.
 // z < 8: CUDA's j0 / y0 / j1 / y1.
 // Complex z (lossy interiors, self blocks): Miller's backward recurrence
 //   J_{n-1} = (2n/z) J_n - J_{n+1} from an even start M > |z| + 25 + 3 sqrt|z|,
@@ -31,27 +30,20 @@
 #include "fx.cuh"
 #include "hankel_fit.h"
 
-constexpr double HK_ZA = 8.0;    // modulus-phase form from here up
+// below 8: the modulus-phase form does not reach (z >= 0; comparisons of the
+// high words, an FP64 one takes a multiplication's time)
+__device__ __forceinline__ bool hk_near(double z) { return __double2hiint(z) < 0x40200000; }
 
-// 1/sqrt(z): Newton's iteration of third order on an FP32 estimate q (relative
-// error d below 2^-21): 1/sqrt(z) = q (1 - e)^(-1/2), e = 1 - z q^2, taken to
-// q (1 + e/2 + 3 e^2/8); q^2 is exact.
-__device__ __forceinline__ double hk_rsqrt(double z) {
-  const double q = (double)rsqrtf((float)z);
-  const double e = fma(-z, q * q, 1.0);
-  return fma(q * e, fma(0.375, e, 0.5), q);
-}
 // r = sqrt(r2) and ir = 1/r: one FP64 iteration on the estimate gives ir, and
 // a last one on r itself its rounding (z = k r is a phase, so that its error
 // counts as z times r's); FP32's range is left to sqrt and the division.
 __device__ __forceinline__ void hk_distance(double r2, double& r, double& ir) {
-  const float f = (float)r2;
-  if (!(f > 1e-30f && f < 1e30f)) {
+  if (!fx_f32_range(r2)) {
     r = sqrt(r2);
     ir = 1.0 / r;
     return;
   }
-  ir = hk_rsqrt(r2);
+  ir = fx_rsqrt(r2);
   r = r2 * ir;
   r = fma(fma(-r, r, r2), 0.5 * ir, r);
 }
@@ -62,7 +54,7 @@ __device__ __forceinline__ void hk_distance(double r2, double& r, double& ir) {
 // place of Cody and Waite's FP64 steps.  From z = 8192 up (to about 1e9) whole
 // turns are taken off in FP64 first.
 __device__ __forceinline__ void hk_sincos_shifted(double z, long long& sn, long long& cs) {
-  if (z >= 8192.0) {
+  if (__double2hiint(z) >= 0x40C00000) {
     const double n = rint(z * 0.15915494309189533577) - 4.0;   // leaves z in about [22, 29]
     z = fma(-n, 2.4492935982947064e-16, fma(-n, 6.2831853071795864769, z));
   }
@@ -91,7 +83,7 @@ __device__ __forceinline__ void hk_sincos_shifted(double z, long long& sn, long 
 // z >= 8, with iz = 1/z and q = 1/sqrt(z)
 __device__ __forceinline__ void hankel_asym(double z, double iz, double q, double& J0, double& Y0, double& J1,
                                             double& Y1) {
-  const float zf = (float)z;
+  const int zh = __double2hiint(z);
   const double v = iz * iz;
   const long long three = 0x4008000000000000ll;   // 3.0: 3 + x lies in [2, 4)
   long long P0, Q0, P1, Q1;
@@ -101,16 +93,16 @@ __device__ __forceinline__ void hankel_asym(double z, double iz, double q, doubl
     return fx(X << 9);
   };
   int x31;
-  if (zf >= 60.f) {
+  if (zh >= 0x404E0000) {   // z >= 60
     const Fx x = mapped(HK_IVH4, HK_SH4, x31);
     hankel_fit4(x, x31, P0, Q0, P1, Q1);
-  } else if (zf >= 30.f) {
+  } else if (zh >= 0x403E0000) {   // z >= 30
     const Fx x = mapped(HK_IVH3, HK_SH3, x31);
     hankel_fit3(x, x31, P0, Q0, P1, Q1);
-  } else if (zf >= 20.f) {
+  } else if (zh >= 0x40340000) {   // z >= 20
     const Fx x = mapped(HK_IVH2, HK_SH2, x31);
     hankel_fit2(x, x31, P0, Q0, P1, Q1);
-  } else if (zf >= 12.f) {
+  } else if (zh >= 0x40280000) {   // z >= 12
     const Fx x = mapped(HK_IVH1, HK_SH1, x31);
     hankel_fit1(x, x31, P0, Q0, P1, Q1);
   } else {
@@ -123,12 +115,12 @@ __device__ __forceinline__ void hankel_asym(double z, double iz, double q, doubl
   hk_sincos_shifted(z, sn, cs);
   const Fx s = fx(sn), c = fx(cs), ns = fx(-sn), nc = fx(-cs);
   const Fx p0 = fx(P0), q0 = fx(fx_mul(fx(Q0), izf)), p1 = fx(P1), q1 = fx(fx_mul(fx(Q1), izf));
-  const double amp = 6.9205453937208734e-19 * q;     // sqrt(2/pi) 2^-60 / sqrt(z)
+  const double amp = 0.79788456080286535588 * q;     // sqrt(2/pi) / sqrt(z)
   auto two = [&](Fx a0, Fx b0, Fx a1, Fx b1) {
     long long hh = 0, cr = FX_HALF;
     fx_mac(hh, cr, a0, b0);
     fx_mac(hh, cr, a1, b1);
-    return amp * (double)(hh + (cr >> 30));
+    return amp * fx_to(hh + (cr >> 30), 0);
   };
   J0 = two(p0, c, q0, ns);
   Y0 = two(p0, s, q0, c);
@@ -139,8 +131,8 @@ __device__ __forceinline__ void hankel_asym(double z, double iz, double q, doubl
 // The pair of orders at z (below 8 CUDA's j0/y0/j1/y1: ~1e-15 absolute,
 // measured against scipy on GB300).
 __device__ __forceinline__ void hankel01(double z, double& J0, double& Y0, double& J1, double& Y1) {
-  if ((float)z >= (float)HK_ZA) {
-    const double q = hk_rsqrt(z);
+  if (!hk_near(z)) {
+    const double q = fx_rsqrt(z);
     hankel_asym(z, q * q, q, J0, Y0, J1, Y1);
   } else { J0 = j0(z); Y0 = y0(z); J1 = j1(z); Y1 = y1(z); }
 }
