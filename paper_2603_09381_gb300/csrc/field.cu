@@ -2,10 +2,11 @@
 // evaluation point or direction sums the trapezoid rule over every node in a
 // fixed order (block-wide reduction), so results are reproducible.  The near
 // field's Hankel pair and the far field's sincos, which bound these kernels on
-// the FP64 pipe (about 100 of its instructions a node against 8 a right-hand
-// side), are formed once for up to NR right-hand sides: 8 x 8 stars, 4,096
-// points and 720 directions, 8 right-hand sides: 65 ms with one CTA per
-// right-hand side.
+// the FP64 pipe together with 8 (far: 6) fused multiply-adds a right-hand side,
+// are formed once for up to NR right-hand sides: 8 x 8 stars, 4,096 points and
+// 720 directions, 8 right-hand sides: 65 ms with one CTA per right-hand side,
+// 7.6 ms now.  Every fused operation is written out: left to the compiler, a
+// right-hand side took 12 and its last bits depended on NR (10.1 ms).
 #include "field.cuh"
 #include "hankel.cuh"
 #include "prof.cuh"
@@ -50,8 +51,8 @@ __global__ void __launch_bounds__(FT) k_far_field(const InclDev* __restrict__ in
   for (int c = 0; c < NR; ++c) acc[c] = make_double2(0, 0);
   for (int i = threadIdx.x; i < total; i += FT) {
     double s, co;
-    sincos(-k * (ca * nd.x[i] + sa * nd.y[i]), &s, &co);      // e^{-i k xhat.y}
-    const double kn = k * (ca * nd.nx[i] + sa * nd.ny[i]);
+    sincos(-k * fma(ca, nd.x[i], sa * nd.y[i]), &s, &co);     // e^{-i k xhat.y}
+    const double kn = k * fma(ca, nd.nx[i], sa * nd.ny[i]);
     const double w = nd.w[i];
     s *= w;
     co *= w;
@@ -60,9 +61,9 @@ __global__ void __launch_bounds__(FT) k_far_field(const InclDev* __restrict__ in
       double2 q, u;
       qu_of(inc, nd.incl, phi + (size_t)c * ldphi, i, q, u);
       // -i k (xhat.n) u - q  (eps+ = 1)
-      const double tx = kn * u.y - q.x, ty = -kn * u.x - q.y;
-      acc[c].x += co * tx - s * ty;
-      acc[c].y += co * ty + s * tx;
+      const double tx = fma(kn, u.y, -q.x), ty = fma(-kn, u.x, -q.y);
+      acc[c].x = fma(-s, ty, fma(co, tx, acc[c].x));
+      acc[c].y = fma(s, tx, fma(co, ty, acc[c].y));
     }
   }
 #pragma unroll
@@ -90,17 +91,17 @@ __global__ void __launch_bounds__(FT) k_scattered(const InclDev* __restrict__ in
   for (int i = threadIdx.x; i < total; i += FT) {
     const double dx = px - nd.x[i], dy = py - nd.y[i];
     double r, ir, J0, Y0, J1, Y1;
-    hk_distance(dx * dx + dy * dy, r, ir);
+    hk_distance(fma(dx, dx, dy * dy), r, ir);
     hankel01(k * r, J0, Y0, J1, Y1);
-    const double w = 0.25 * nd.w[i], b = k * w * ((nd.nx[i] * dx + nd.ny[i] * dy) * ir);
+    const double w = 0.25 * nd.w[i], b = k * w * (fma(nd.nx[i], dx, nd.ny[i] * dy) * ir);
     // G = (i/4) H0 = (-Y0 + i J0)/4;  dG/dn_y = (i k/4) H1 b = k b (-Y1 + i J1)/4
     const double gx = -w * Y0, gy = w * J0, ex = -b * Y1, ey = b * J1;
 #pragma unroll
     for (int c = 0; c < NR; ++c) {
       double2 q, u;
       qu_of(inc, nd.incl, phi + (size_t)c * ldphi, i, q, u);
-      acc[c].x += (ex * u.x - ey * u.y) - (gx * q.x - gy * q.y);
-      acc[c].y += (ex * u.y + ey * u.x) - (gx * q.y + gy * q.x);
+      acc[c].x = fma(gy, q.y, fma(-gx, q.x, fma(-ey, u.y, fma(ex, u.x, acc[c].x))));
+      acc[c].y = fma(-gy, q.x, fma(-gx, q.y, fma(ey, u.x, fma(ex, u.y, acc[c].y))));
     }
   }
 #pragma unroll
