@@ -771,11 +771,8 @@ int cpqr_resident_ctas(int n, int W) {
 }
 template <typename C>
 void cpqr_resident(const CpqrProb<C>* d_prob, const int* d_list, const int* h_n, const int* h_w, int count, int cs,
-                   cudaStream_t st) {
+                   int sms, cudaStream_t st) {
   if (count <= 0) return;
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int max_n = *std::max_element(h_n, h_n + count);
   while (cs < 8 && (long)count * cs * 2 <= sms && cs * 32 <= max_n) cs *= 2;   // spread a few matrices wider
   size_t bytes = 0;
@@ -849,8 +846,8 @@ void copy_batched(const CopyProb<S, D>* d_prob, int nprob, int max_elems, cudaSt
 template void cpqr_init_norms<double2>(const CpqrProb<double2>*, const CpqrChunk*, int, cudaStream_t);
 template int cpqr_resident_ctas<double2>(int, int);
 template int cpqr_resident_ctas<float2>(int, int);
-template void cpqr_resident<double2>(const CpqrProb<double2>*, const int*, const int*, const int*, int, int, cudaStream_t);
-template void cpqr_resident<float2>(const CpqrProb<float2>*, const int*, const int*, const int*, int, int, cudaStream_t);
+template void cpqr_resident<double2>(const CpqrProb<double2>*, const int*, const int*, const int*, int, int, int, cudaStream_t);
+template void cpqr_resident<float2>(const CpqrProb<float2>*, const int*, const int*, const int*, int, int, int, cudaStream_t);
 template void cpqr_start<double2>(const CpqrProb<double2>*, int, cudaStream_t);
 template void cpqr_start<float2>(const CpqrProb<float2>*, int, cudaStream_t);
 template void cpqr_step<double2>(const CpqrProb<double2>*, const CpqrChunk*, int, int, int*, cudaStream_t, bool);

@@ -110,13 +110,13 @@ void cpqr_step(const CpqrProb<C>* d_prob, const CpqrChunk* d_chunk, int nchunk, 
                cudaStream_t st, bool tall);
 // The whole phase of the `count` matrices listed in d_list (h_n, h_w: their
 // columns and rows), each in the shared memory of a cluster of at least cs
-// CTAs; cpqr_resident_ctas: the fewest CTAs that hold an n-column, W-row
+// CTAs (more while all of them fit on `sms` SMs); cpqr_resident_ctas: the fewest CTAs that hold an n-column, W-row
 // matrix, or 0.  Norms as cpqr_init_norms leaves them; no cpqr_start needed.
 template <typename C>
 int cpqr_resident_ctas(int n, int W);
 template <typename C>
 void cpqr_resident(const CpqrProb<C>* d_prob, const int* d_list, const int* h_n, const int* h_w, int count, int cs,
-                   cudaStream_t st);
+                   int sms, cudaStream_t st);
 // R11 (upper triangular, diagonal from rdiag) and R12 of every problem gathered
 // in pivot order into R11 and T (ldt = k), for a blocked triangular solve
 // T <- R11^{-1} T; max_elems = the largest k * n.

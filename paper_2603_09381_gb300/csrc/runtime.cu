@@ -227,6 +227,48 @@ T* upload(Arena& a, const std::vector<T>& v, cudaStream_t st) {
   return d;
 }
 
+// Streams forked off another one and joined to it again.  Left by an
+// exception, the destructor waits for their work: it uses the caller's memory.
+struct SideStreams {
+  std::vector<cudaStream_t> s;
+  std::vector<cudaEvent_t> e;   // the fork, then the end of each
+  size_t used = 0;
+  cudaEvent_t event(size_t i) {
+    while (e.size() <= i) {
+      cudaEvent_t v = nullptr;
+      CK(cudaEventCreateWithFlags(&v, cudaEventDisableTiming));
+      e.push_back(v);
+    }
+    return e[i];
+  }
+  // a stream whose work starts after what `from` holds at the first call since join()
+  cudaStream_t next(cudaStream_t from) {
+    if (used == 0) CK(cudaEventRecord(event(0), from));
+    if (s.size() == used) {
+      cudaStream_t v = nullptr;
+      CK(cudaStreamCreateWithFlags(&v, cudaStreamNonBlocking));
+      s.push_back(v);
+    }
+    CK(cudaStreamWaitEvent(s[used], e[0], 0));
+    return s[used++];
+  }
+  void join(cudaStream_t to) {
+    for (size_t i = 0; i < used; ++i) {
+      CK(cudaEventRecord(event(1 + i), s[i]));
+      CK(cudaStreamWaitEvent(to, e[1 + i], 0));
+    }
+    used = 0;
+  }
+  SideStreams() = default;
+  SideStreams(const SideStreams&) = delete;
+  SideStreams& operator=(const SideStreams&) = delete;
+  ~SideStreams() {
+    for (size_t i = 0; i < used; ++i) cudaStreamSynchronize(s[i]);
+    for (cudaEvent_t v : e) cudaEventDestroy(v);
+    for (cudaStream_t v : s) cudaStreamDestroy(v);
+  }
+};
+
 template <class C>
 __global__ void k_identity(C* A, int m, int ld) {
   int e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1523,14 +1565,32 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
       if (!rcs[i]) chunks.push_back(ch);
     }
   }
-  auto run_resident = [&](const CpqrProb<C>* d) {   // the phase of the resident matrices that have steps to do
-    for (int cs = 1; cs <= 8; cs *= 2) {
-      std::vector<int> list, hn, hw;
+  // The phase of the resident matrices that have steps to do, from the next
+  // point of st on: one launch per cluster size, each on a stream of its own,
+  // beside one another and beside the steps of the other matrices (each alone
+  // fills a part of the SMs); st waits for them at fork.join().  One after the
+  // other: batch of ellipses 90.7 ms, now 85.3; Burton-Miller 76.4, now 73.7.
+  SideStreams fork;
+  auto run_resident = [&](const CpqrProb<C>* d, bool beside) {
+    struct Group { int cs; const int* list; std::vector<int> n, w; };
+    std::vector<Group> groups;
+    long ctas = 0;
+    for (int cs = 8; cs >= 1; cs /= 2) {   // the largest matrices first
+      Group g{cs, nullptr, {}, {}};
+      std::vector<int> list;
       for (int i = 0; i < nid; ++i)
-        if (rcs[i] == cs && cp[i].target > cp[i].base) { list.push_back(i); hn.push_back(nn[i]); hw.push_back(We[i]); }
+        if (rcs[i] == cs && cp[i].target > cp[i].base) { list.push_back(i); g.n.push_back(nn[i]); g.w.push_back(We[i]); }
       if (list.empty()) continue;
-      const int* dl = upload(scr, list, st);
-      cpqr_resident<C>(d, dl, hn.data(), hw.data(), (int)list.size(), cs, st);
+      g.list = upload(scr, list, st);
+      ctas += (long)list.size() * cs;
+      groups.push_back(std::move(g));
+    }
+    for (size_t i = 0; i < groups.size(); ++i) {
+      const Group& g = groups[i];
+      const int count = (int)g.n.size();
+      cudaStream_t s = i == 0 && !beside ? st : fork.next(st);
+      // its share of the SMs
+      cpqr_resident<C>(d, g.list, g.n.data(), g.w.data(), count, g.cs, (int)(sms * ((long)count * g.cs) / ctas), s);
     }
     CK(cudaGetLastError());
   };
@@ -1545,7 +1605,7 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
   const int nch = (int)chunks.size();
   cpqr_init_norms<C>(dcp, upload(scr, init, st), (int)init.size(), st);
   if (nch > 0) cpqr_start<C>(dcp, nid, st);   // (also picks for the resident ones, before they move on)
-  run_resident(dcp);
+  run_resident(dcp, nch > 0);
   std::vector<int> hr(nid);
   // With predicted ranks, run the predicted number of steps (+1, where the stop
   // test of the last rank happens) before the first check; otherwise check
@@ -1578,6 +1638,7 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
     }
   }
   CK(cudaGetLastError());
+  fork.join(st);
   CK(cudaMemcpyAsync(hr.data(), rank, nid * sizeof(int), cudaMemcpyDeviceToHost, st));
   // an exactly zero ID input (no far field at all: the interior rows of the
   // simplified Burton-Miller system) gets a zero interpolation, not an
@@ -1610,8 +1671,9 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
   if (maxExt > 0 || resExt > 0) {
     dcp = upload(scr, cp, st);
     if (maxExt > 0) cpqr_start<C>(dcp, nid, st);
-    if (resExt > 0) run_resident(dcp);
+    if (resExt > 0) run_resident(dcp, maxExt > 0);
     for (int t = 0; t < maxExt; ++t) cpqr_step<C>(dcp, dch, nch, t, ctr + maxT + t, st, tall);
+    fork.join(st);
     for (const auto& J : jobs) J.F->stats.cpqr_launches += maxExt;
     CK(cudaGetLastError());
   }
