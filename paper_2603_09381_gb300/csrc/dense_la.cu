@@ -696,7 +696,66 @@ __global__ void __launch_bounds__(256) k_trsv_chain(const SolveProb<C>* __restri
   if (tid == 0) ts_store_release(&flags[b], 1);
 }
 
+// Products with at most GEMV_MAX_N columns (solves for one to three waves).
+// A 32 x 32 tile left 29 to 31 of its columns empty, FP64 operations and all;
+// here a CTA takes 32 rows, its 8 warps every eighth term of the sums, a lane
+// a row, so that A is read once, 512 bytes at a time, and only the products
+// themselves are formed.  The warps' sums meet in a fixed order.
+template <typename C, int N>
+__device__ __forceinline__ void gemv_rows(const GemmDesc<C>& g, int r0, C (*red)[32][GEMV_MAX_N]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, row = r0 + lane;
+  C acc[N];
+#pragma unroll
+  for (int j = 0; j < N; ++j) acc[j] = czero<C>();
+  if (row < g.m) {
+#pragma unroll 4
+    for (int l = warp; l < g.k; l += 8) {
+      const C a = g.A[row + (size_t)l * g.lda];
+#pragma unroll
+      for (int j = 0; j < N; ++j) cfma(acc[j], a, g.B[l + (size_t)j * g.ldb]);
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < N; ++j) red[warp][lane][j] = acc[j];
+  __syncthreads();
+  if (warp < N && row < g.m) {
+    C v = red[0][lane][warp];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) v = v + red[w][lane][warp];
+    C* p = g.Cm + row + (size_t)warp * g.ldc;
+    v = g.alpha * v;
+    if (!g.beta_zero) v = v + g.beta * (*p);
+    *p = v;
+  }
+}
+
+template <typename C>
+__global__ void __launch_bounds__(256) k_gemv_batched(const GemmDesc<C>* __restrict__ d,
+                                                      const int* __restrict__ tile_off, int nprob) {
+  __shared__ C red[8][32][GEMV_MAX_N];
+  const int t = blockIdx.x;
+  int lo = 0, hi = nprob;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (tile_off[mid] <= t) lo = mid; else hi = mid;
+  }
+  const GemmDesc<C> g = d[lo];
+  const int r0 = (t - tile_off[lo]) * 32;
+  if (g.n == 1) gemv_rows<C, 1>(g, r0, red);
+  else if (g.n == 2) gemv_rows<C, 2>(g, r0, red);
+  else gemv_rows<C, 3>(g, r0, red);
+}
+
 }  // namespace
+
+template <typename C>
+void la_gemv_batched(const GemmDesc<C>* d_desc, const int* d_tile_off, int nprob, int total_tiles, cudaStream_t st) {
+  if (nprob <= 0 || total_tiles <= 0) return;
+  KPROF_BEGIN(st);
+  k_gemv_batched<C><<<total_tiles, 256, 0, st>>>(d_desc, d_tile_off, nprob);
+  pm_launch_count_add(1);
+  KPROF_END(st, kname<C>("gemv_batched", "gemv_batched32"), 0.0);
+}
 
 template <typename C>
 void la_gemm_batched(const GemmDesc<C>* d_desc, const int* d_tile_off, int nprob, int total_tiles,
@@ -1004,6 +1063,8 @@ template void la_trsm_upper_batched<float2>(const SolveProb<float2>*, int, int, 
                                             cudaStream_t);
 template void la_gemm_batched_shape<double2>(int, const GemmDesc<double2>*, const int*, int, int, cudaStream_t);
 template void la_gemm_batched_shape<float2>(int, const GemmDesc<float2>*, const int*, int, int, cudaStream_t);
+template void la_gemv_batched<double2>(const GemmDesc<double2>*, const int*, int, int, cudaStream_t);
+template void la_gemv_batched<float2>(const GemmDesc<float2>*, const int*, int, int, cudaStream_t);
 template void la_gemm_batched<double2>(const GemmDesc<double2>*, const int*, int, int, cudaStream_t);
 template void la_gemm_batched<float2>(const GemmDesc<float2>*, const int*, int, int, cudaStream_t);
 template void la_getrf_batched<double2>(const LuProb<double2>*, int, int, const int*, cudaStream_t);

@@ -34,6 +34,12 @@ struct SolveProb {     // B (m x nrhs) <- A^{-1} B using the LU of A
 template <typename C>
 void la_gemm_batched(const GemmDesc<C>* d_desc, const int* d_tile_off, int nprob, int total_tiles,
                      cudaStream_t st);
+// The same for products of at most GEMV_MAX_N columns each; d_tile_off: prefix
+// sums of gemv_tiles(m).
+constexpr int GEMV_MAX_N = 3;
+inline int gemv_tiles(int m) { return (m + 31) / 32; }
+template <typename C>
+void la_gemv_batched(const GemmDesc<C>* d_desc, const int* d_tile_off, int nprob, int total_tiles, cudaStream_t st);
 // h_m: host copy of the matrix sizes (flop accounting for the optional profiler)
 template <typename C>
 void la_getrf_batched(const LuProb<C>* d_prob, int nprob, int maxm, const int* h_m, cudaStream_t st);

@@ -787,7 +787,28 @@ struct GemmBatch {
     }
     run_cuda_cores(scr, st);
   }
+  // The rest: products of a few columns row by row (per product, whatever the
+  // batch), the others in tiles.
   void run_cuda_cores(Arena& scr, cudaStream_t st) {
+    GemmBatch<C> tiled;
+    std::vector<GemmDesc<C>> v;
+    for (auto& x : d) {
+      if (x.n <= GEMV_MAX_N) v.push_back(x);
+      else { tiled.d.push_back(x); tiled.off.push_back(tiled.off.back() + gemm_tiles(x.m, x.n)); }
+    }
+    if (!v.empty()) {
+      std::vector<int> o{0};
+      double f = 0;
+      for (auto& x : v) { o.push_back(o.back() + gemv_tiles(x.m)); f += 8.0 * x.m * x.n * x.k; }
+      auto* dv = upload(scr, v, st);
+      int* dof = upload(scr, o, st);
+      la_gemv_batched<C>(dv, dof, (int)v.size(), o.back(), st);
+      if (g_kprof) g_kprof->add_flops(kname<C>("gemv_batched", "gemv_batched32"), f);
+      CK(cudaGetLastError());
+    }
+    tiled.run_tiles(scr, st);
+  }
+  void run_tiles(Arena& scr, cudaStream_t st) {
     if (d.empty()) return;
     auto* dd = upload(scr, d, st);
     int dev = 0;
