@@ -44,8 +44,8 @@ constexpr uint32_t SBO = (KR / 8) * 128;             // next 8 rows of an operan
 constexpr uint32_t A_BYTES = TM * KR * 2;            // one digit of A
 constexpr uint32_t B_BYTES = 2 * TN * KR * 2;        // one digit of B
 constexpr uint32_t OFF_B = NS * A_BYTES;
-constexpr uint32_t OFF_EXP = OFF_B + NS * B_BYTES;   // per k group: exponents of A's rows, then B's columns
-constexpr uint32_t OFF_BAR = OFF_EXP + 4 * (TM + TN) * 4;
+constexpr uint32_t OFF_EXP = OFF_B + NS * B_BYTES;   // per k group: exponents of A's rows, then B's columns; B's overall
+constexpr uint32_t OFF_BAR = OFF_EXP + (4 * (TM + TN) + TN) * 4;
 constexpr int SMEM = OFF_BAR + 32;
 constexpr int WAIT = 1 << 20;   // x ~1 us suspend hint: about a second
 
@@ -74,16 +74,12 @@ __device__ __forceinline__ int exponent(double x) { return (__double2hiint(x) >>
 // bias that turns its lower seven base-256 digits into unsigned bytes; neg: of
 // -x.  Subnormal x counts as zero.
 __device__ __forceinline__ uint64_t digits(double x, int E, bool neg) {
-  const uint64_t b = (uint64_t)__double_as_longlong(x);
-  const int e = (int)(b >> 52) & 0x7FF;
-  uint64_t q = 0;
-  const int d = E - e;
-  if (e != 0 && d < 63) {
-    q = ((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 9;
-    if (d > 0) q = (q + (1ull << (d - 1))) >> d;
-    if (((b >> 63) != 0) != neg) q = 0 - q;
-  }
-  return q + 0x0080808080808080ull;
+  const uint32_t h = (uint32_t)__double2hiint(x);
+  const int e = (int)(h >> 20) & 0x7FF, d = e ? min(E - e, 63) : 63;   // 63 leaves nothing
+  const uint64_t m = (uint64_t)((h & 0xFFFFFu) | 0x100000u) << 32 | (uint32_t)__double2loint(x);
+  const uint64_t q = ((m << 10 >> d) + 1) >> 1;                        // rounded
+  const int sg = ((int)h >> 31) ^ (neg ? -1 : 0);
+  return (q ^ (uint64_t)(int64_t)sg) + 0x0080808080808080ull + (uint32_t)(sg & 1);
 }
 
 // Digit i (0: the largest) of two numbers as a pair of fp16: bytes go
@@ -123,35 +119,34 @@ __device__ __forceinline__ void put8(unsigned char* p, uint32_t step, const uint
 }
 __device__ __forceinline__ uint32_t row_off(int row, int k) { return (uint32_t)(row >> 3) * SBO + (uint32_t)(k >> 3) * tcx::LBO + (uint32_t)(row & 7) * 16; }
 
-// The double nearest to (hi 2^32 + lo) 2^p2.
+// The double nearest to (hi 2^32 + lo) 2^p2, |hi| and |lo| below 2^62; in
+// 32-bit words, as 64-bit shifts by a variable take three instructions each and
+// a stage's epilogue is its largest part.
 __device__ __forceinline__ double join(int64_t hi, int64_t lo, int p2) {
   hi += lo >> 32;                       // = hi 2^32 + l, 0 <= l < 2^32
-  uint32_t l = (uint32_t)lo;
-  const uint64_t sign = (uint64_t)hi & 0x8000000000000000ull;
-  if (sign) {                           // magnitude
-    hi = ~hi + (l == 0 ? 1 : 0);
-    l = 0u - l;
-  }
-  uint64_t mag = (uint64_t)hi, rest = (uint64_t)l << 32;
+  const uint32_t sg = (uint32_t)((int32_t)(hi >> 32) >> 31);
+  uint32_t w2 = (uint32_t)(hi >> 32) ^ sg, w1 = (uint32_t)hi ^ sg, w0 = (uint32_t)lo ^ sg;   // magnitude
+  asm("add.cc.u32 %0, %0, %3;\n addc.cc.u32 %1, %1, 0;\n addc.u32 %2, %2, 0;" : "+r"(w0), "+r"(w1), "+r"(w2) : "r"(sg & 1));
   int e = 1023 + 95 + p2;
-  if (mag == 0) { mag = rest; rest = 0; e -= 64; }
-  const int lz = __clzll((long long)mag);   // not zero: bit 63 of the shifted magnitude is set
-  mag = (mag << (lz & 63)) | ((rest >> 1) >> (63 - (lz & 63)));
+  if (w2 == 0) { w2 = w1; w1 = w0; w0 = 0; e -= 32; }
+  if (w2 == 0) { w2 = w1; w1 = w0; e -= 32; }
+  const int lz = __clz((int)w2);
+  const uint32_t m1 = __funnelshift_l(w1, w2, lz), m0 = __funnelshift_l(w0, w1, lz);
   e -= lz;
-  mag = (mag + 1024) >> 11;             // 53 bits (a carry goes on into the exponent)
-  uint64_t r = sign | (((uint64_t)(uint32_t)(e - 1) << 52) + mag);
-  if (lz == 64 || e <= 0) r = 0;
-  if (e >= 2047) r = sign | 0x7FF0000000000000ull;
+  uint64_t r = ((uint64_t)m1 << 32 | m0) >> 11;
+  r += (m0 >> 10) & 1;                  // 53 bits (a carry goes on into the exponent)
+  r += (uint64_t)((uint32_t)(e - 1) << 20 | (sg & 0x80000000u)) << 32;
+  if (m1 == 0 || e <= 0) r = 0;
+  if (e >= 2047) r = (uint64_t)(sg & 0x80000000u | 0x7FF00000u) << 32;
   return __longlong_as_double((long long)r);
 }
 // The double nearest to V 2^(ex - 2112), V = sum_s v_s 2^(8 (7 - s)); ex: the
 // sum of the two exponents, or negative for a row or column that is not finite.
 __device__ __forceinline__ double join(const float* v, int ex) {
-  const int64_t hi = ((int64_t)__float2int_rn(v[0]) << 24) + ((int64_t)__float2int_rn(v[1]) << 16) +
-                     ((int64_t)__float2int_rn(v[2]) << 8) + __float2int_rn(v[3]);
-  const int64_t lo = ((int64_t)__float2int_rn(v[4]) << 24) + ((int64_t)__float2int_rn(v[5]) << 16) +
-                     ((int64_t)__float2int_rn(v[6]) << 8) + __float2int_rn(v[7]);
-  const double r = join(hi, lo, ex - 2112);
+  // |v_s| <= (s + 1) 2^20: pairs of sums fit 32 bits
+  const int p0 = __float2int_rn(v[0]) * 256 + __float2int_rn(v[1]), p1 = __float2int_rn(v[2]) * 256 + __float2int_rn(v[3]);
+  const int p2 = __float2int_rn(v[4]) * 256 + __float2int_rn(v[5]), p3 = __float2int_rn(v[6]) * 256 + __float2int_rn(v[7]);
+  const double r = join((int64_t)p0 * 65536 + p1, (int64_t)p2 * 65536 + p3, ex - 2112);
   return ex < 0 ? __longlong_as_double(0x7FF8000000000000ll) : r;
 }
 
@@ -197,6 +192,7 @@ __device__ __forceinline__ void stage(Cta& c, bool new_a, const FA& a, const FB&
   const int tid = threadIdx.x, warp = tid >> 5;
   int* ea = reinterpret_cast<int*>(c.sm + OFF_EXP);   // [k group][row]
   int* eb = ea + 4 * TM;                              // [k group][column]
+  int* ebm = eb + 4 * TN;                             // [column]: the largest, far below zero if not finite
   const int row = tid & (TM - 1), kg = tid >> 7;
   const int bn = tid & 31, bg = (tid >> 5) & 3, bpart = tid >> 7;   // B: threads 0 .. 255
   double2 va[8];
@@ -233,6 +229,7 @@ __device__ __forceinline__ void stage(Cta& c, bool new_a, const FA& a, const FB&
   }
   if (tid < 256) {
     const int E = max(max(eb[bn], eb[TN + bn]), max(eb[2 * TN + bn], eb[3 * TN + bn]));
+    if (tid < TN) ebm[bn] = E == 0x7FF ? -0x4000 : E;
     // real part: [row bn, k] and [row 32 + bn, 32 + k]; imaginary part: negated [row bn, 32 + k], [row 32 + bn, k]
     uint64_t q[8];
     unsigned char* B = c.sm + OFF_B;
@@ -266,7 +263,8 @@ __device__ __forceinline__ void stage(Cta& c, bool new_a, const FA& a, const FB&
   }
   // the exponents of this thread's outputs, while the MMAs run
   const int er = 32 * (warp & 3) + (tid & 31), cg = warp >> 2;
-  const int E = max(max(ea[er], ea[TM + er]), max(ea[2 * TM + er], ea[3 * TM + er]));
+  int E = max(max(ea[er], ea[TM + er]), max(ea[2 * TM + er], ea[3 * TM + er]));
+  if (E == 0x7FF) E = -0x4000;
   during();
   c.ok = c.ok && tcx::mbar_wait(bar, c.phase, WAIT);
   c.phase ^= 1;
@@ -275,6 +273,8 @@ __device__ __forceinline__ void stage(Cta& c, bool new_a, const FA& a, const FB&
     const uint32_t t0 = c.tmem + ((uint32_t)((warp & 3) * 32) << 16) + 8 * cg;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
+      const int4 F = *reinterpret_cast<const int4*>(ebm + 8 * cg + 4 * h);
+      const int ef[4] = {E + F.x, E + F.y, E + F.z, E + F.w};
 #pragma unroll
       for (int part = 0; part < 2; ++part) {
         float v[NS][4];
@@ -283,10 +283,8 @@ __device__ __forceinline__ void stage(Cta& c, bool new_a, const FA& a, const FB&
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const int n = 8 * cg + 4 * h + j;
-          const int F = max(max(eb[n], eb[TN + n]), max(eb[2 * TN + n], eb[3 * TN + n]));
           const float w[NS] = {v[0][j], v[1][j], v[2][j], v[3][j], v[4][j], v[5][j], v[6][j], v[7][j]};
-          const double d = join(w, E == 0x7FF || F == 0x7FF ? -1 : E + F);
+          const double d = join(w, ef[j]);
           emit(4 * h + j, part, d);
         }
       }
