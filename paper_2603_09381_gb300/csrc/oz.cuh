@@ -71,51 +71,44 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float* d) {
 __device__ __forceinline__ int exponent(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
 
 // x relative to the exponent E >= exponent(x) as a 62-bit integer, plus the
-// bias that turns its lower seven base-256 digits into unsigned bytes; neg: of
-// -x.  Subnormal x counts as zero.
+// bias that turns its base-256 digits into unsigned bytes; neg: of -x.
+// Subnormal x counts as zero.
+constexpr uint64_t BIAS = 0x8080808080808080ull;
 __device__ __forceinline__ uint64_t digits(double x, int E, bool neg) {
   const uint32_t h = (uint32_t)__double2hiint(x);
   const int e = (int)(h >> 20) & 0x7FF, d = e ? min(E - e, 63) : 63;   // 63 leaves nothing
   const uint64_t m = (uint64_t)((h & 0xFFFFFu) | 0x100000u) << 32 | (uint32_t)__double2loint(x);
   const uint64_t q = ((m << 10 >> d) + 1) >> 1;                        // rounded
   const int sg = ((int)h >> 31) ^ (neg ? -1 : 0);
-  return (q ^ (uint64_t)(int64_t)sg) + 0x0080808080808080ull + (uint32_t)(sg & 1);
+  return (q ^ (uint64_t)(int64_t)sg) + BIAS + (uint32_t)(sg & 1);
 }
 
-// Digit i (0: the largest) of two numbers as a pair of fp16: bytes go
-// through 1024 + byte (exact in fp16) to the signed digit.
+// Digits I and I + 1 (I even; 0: the largest) of two numbers as pairs of fp16:
+// bytes go through 1024 + byte (exact in fp16) to the signed digit.
 template <int I>
-__device__ __forceinline__ uint32_t digit_pair(uint64_t a, uint64_t b) {
-  uint32_t r;
-  if (I == 0) {   // the top digit is signed already, -64 .. 64: + 128 first
-    r = __byte_perm((uint32_t)(a >> 32), (uint32_t)(b >> 32), 0x0073) ^ 0x8080u;
-    r = __byte_perm(r, 0x64646464u, 0x4140);
-    asm("sub.f16x2 %0, %0, %1;" : "+r"(r) : "r"(0x64806480u));
-  } else {
-    constexpr int byte = 7 - I;
-    const uint32_t x = byte >= 4 ? (uint32_t)(a >> 32) : (uint32_t)a, y = byte >= 4 ? (uint32_t)(b >> 32) : (uint32_t)b;
-    constexpr uint32_t sel = (uint32_t)(byte & 3) | ((uint32_t)(4 + (byte & 3)) << 4);
-    r = __byte_perm(x, y, sel);                          // bytes 0 and 1
-    r = __byte_perm(r, 0x64646464u, 0x4140);             // 0x64 above each
-    asm("sub.f16x2 %0, %0, %1;" : "+r"(r) : "r"(0x64806480u));   // - 1152
-  }
+__device__ __forceinline__ uint2 digit_pairs(uint64_t a, uint64_t b) {
+  constexpr int byte = 7 - I;
+  const uint32_t x = byte >= 4 ? (uint32_t)(a >> 32) : (uint32_t)a, y = byte >= 4 ? (uint32_t)(b >> 32) : (uint32_t)b;
+  constexpr uint32_t hi = (uint32_t)(byte & 3), sel = hi | (4 + hi) << 4 | (hi - 1) << 8 | (3 + hi) << 12;
+  const uint32_t t = __byte_perm(x, y, sel);             // a's and b's byte of digit I, then of I + 1
+  uint2 r = make_uint2(__byte_perm(t, 0x64646464u, 0x4140), __byte_perm(t, 0x64646464u, 0x4342));   // 0x64 above each
+  asm("sub.f16x2 %0, %0, %1;" : "+r"(r.x) : "r"(0x64806480u));   // - 1152
+  asm("sub.f16x2 %0, %0, %1;" : "+r"(r.y) : "r"(0x64806480u));
   return r;
 }
 template <int I>
-__device__ __forceinline__ uint4 digit8(const uint64_t* q) {
-  return make_uint4(digit_pair<I>(q[0], q[1]), digit_pair<I>(q[2], q[3]), digit_pair<I>(q[4], q[5]),
-                    digit_pair<I>(q[6], q[7]));
+__device__ __forceinline__ void put2(unsigned char* p, uint32_t step, const uint64_t* q) {
+  const uint2 a = digit_pairs<I>(q[0], q[1]), b = digit_pairs<I>(q[2], q[3]), c = digit_pairs<I>(q[4], q[5]),
+              d = digit_pairs<I>(q[6], q[7]);
+  *reinterpret_cast<uint4*>(p + I * step) = make_uint4(a.x, b.x, c.x, d.x);
+  *reinterpret_cast<uint4*>(p + (I + 1) * step) = make_uint4(a.y, b.y, c.y, d.y);
 }
 // the eight digits of eight numbers into eight operands `step` bytes apart
 __device__ __forceinline__ void put8(unsigned char* p, uint32_t step, const uint64_t* q) {
-  *reinterpret_cast<uint4*>(p) = digit8<0>(q);
-  *reinterpret_cast<uint4*>(p + step) = digit8<1>(q);
-  *reinterpret_cast<uint4*>(p + 2 * step) = digit8<2>(q);
-  *reinterpret_cast<uint4*>(p + 3 * step) = digit8<3>(q);
-  *reinterpret_cast<uint4*>(p + 4 * step) = digit8<4>(q);
-  *reinterpret_cast<uint4*>(p + 5 * step) = digit8<5>(q);
-  *reinterpret_cast<uint4*>(p + 6 * step) = digit8<6>(q);
-  *reinterpret_cast<uint4*>(p + 7 * step) = digit8<7>(q);
+  put2<0>(p, step, q);
+  put2<2>(p, step, q);
+  put2<4>(p, step, q);
+  put2<6>(p, step, q);
 }
 __device__ __forceinline__ uint32_t row_off(int row, int k) { return (uint32_t)(row >> 3) * SBO + (uint32_t)(k >> 3) * tcx::LBO + (uint32_t)(row & 7) * 16; }
 
@@ -238,7 +231,7 @@ __device__ __forceinline__ void stage(Cta& c, bool new_a, const FA& a, const FB&
     put8(B + row_off(TN + bn, (bpart ? 0 : TKC) + 8 * bg), B_BYTES, q);
     if (bpart) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) q[i] = digits(vb[i], E, true);
+      for (int i = 0; i < 8; ++i) q[i] = 2 * BIAS - q[i];
     }
     put8(B + row_off(bn, (bpart ? TKC : 0) + 8 * bg), B_BYTES, q);
   }

@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(128) k_x_digits(const double2* __restrict__ X,
   for (int c = c0; c < c0 + fold && c * 128 < N; ++c) E = max(E, (int)xexp[c * 8 + q]);
   const double2 v = k < N && q < nrhs ? X[k + (size_t)q * ldx] : make_double2(0.0, 0.0);
   // 54 bits: oz::digits' 62 less the lowest byte
-  auto cut = [&](double x, bool neg) { return (uint64_t)((int64_t)(oz::digits(x, E, neg) - 0x0080808080808080ull + 128) >> 8) + BIAS; };
+  auto cut = [&](double x, bool neg) { return (uint64_t)((int64_t)(oz::digits(x, E, neg) - oz::BIAS + 128) >> 8) + BIAS; };
   const uint64_t r = cut(v.x, false), i = cut(v.y, false), ni = cut(v.y, true);
   unsigned char* o = out + (size_t)t * (NS * B_DIG);
   auto put = [&](uint64_t a, int row, int col) {
