@@ -170,6 +170,9 @@ __device__ __forceinline__ Cta begin(unsigned char* sm) {
 __device__ __forceinline__ void end(Cta& c, int* err) {
   asm volatile("tcgen05.fence::before_thread_sync;");
   const int all_ok = __syncthreads_and(c.ok ? 1 : 0);
+  // a wait ran out: once more, bounded, for what may be in flight
+  if (!all_ok && threadIdx.x == 0) tcx::mbar_wait(reinterpret_cast<uint64_t*>(c.sm + OFF_BAR), c.phase ^ 1, WAIT);
+  __syncwarp();
   asm volatile("tcgen05.fence::after_thread_sync;");
   if (threadIdx.x < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(c.tmem), "r"(512));
   if (!all_ok && threadIdx.x == 0) atomicExch(err, 1);

@@ -3,7 +3,9 @@
 // refinement.  The float-float products this replaces issued 12 FP32
 // operations per real multiply-add (58 ms at N = 65,536, 70 ms with their sums
 // folded into FP64); here an entry costs its cut into digits once, for all
-// columns of X, and the read of the operator bounds the kernel.
+// columns of X.  The cut's integer instructions bound the kernel (28 ms at N =
+// 65,536, 24 ms since hi and lo are cut together and two digits share a
+// permutation); the read of the operator would take 10 ms.
 //
 // Digits as in oz.cuh, seven per number: relative to the largest part of its
 // row within a fold of 128 or 512 columns (of X: of its column), each real is a
@@ -49,41 +51,52 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tcx::smem_u32(bar)) : "memory");
 }
 
-constexpr uint64_t BIAS = 0x0000808080808080ull;    // turns the lower six digits into unsigned bytes
+constexpr uint64_t BIAS = 0x0080808080808080ull;    // turns the seven digits into unsigned bytes
 
-// m 2^30 / 2^d with the sign of f, for f = +- m 2^(e - 150) and d = E - e >= 0
-__device__ __forceinline__ uint64_t part(float f, int E) {
-  const uint32_t b = __float_as_uint(f);
-  const int e = (int)(b >> 23) & 0xFF, d = min(E - e, 63);
-  const uint64_t q = e ? ((uint64_t)((b & 0x7FFFFFu) | 0x800000u) << 30) >> d : 0;
-  return (b >> 31) ? 0 - q : q;
+// hi + lo (lo of hi's sign and below hi's last place: SplitOp) relative to the
+// exponent E as a 54-bit integer, each part cut off, plus BIAS.
+__device__ __forceinline__ uint64_t cut(float hi, float lo, int E) {
+  const uint32_t H = __float_as_uint(hi), L = __float_as_uint(lo);
+  const int eh = (int)(H >> 23) & 0xFF, el = (int)(L >> 23) & 0xFF;
+  const uint32_t mh = eh ? H << 8 | 0x80000000u : 0, ml = el ? L << 8 | 0x80000000u : 0;
+  uint64_t q;
+  asm("shr.u64 %0, %1, %2;" : "=l"(q) : "l"((uint64_t)mh << 32), "r"(E - eh + 10));   // (shifts past the width give 0)
+  q += __funnelshift_rc(ml, 0u, (uint32_t)(E - el - 22));
+  const int sg = (int)H >> 31;
+  return (q ^ (uint64_t)(int64_t)sg) + BIAS + (uint32_t)(sg & 1);
 }
 
-// Digit I (0: the largest) of two biased 54-bit integers as a pair of fp16.
+// Digits I and I + 1 (I odd; 0: the largest) of two numbers as pairs of fp16
+// (oz::digit_pairs), and digit 0 of two.
 template <int I>
-__device__ __forceinline__ uint32_t digit_pair(uint64_t a, uint64_t b) {
+__device__ __forceinline__ uint2 digit_pairs(uint64_t a, uint64_t b) {
   constexpr int byte = 6 - I;
   const uint32_t x = byte >= 4 ? (uint32_t)(a >> 32) : (uint32_t)a, y = byte >= 4 ? (uint32_t)(b >> 32) : (uint32_t)b;
-  constexpr uint32_t sel = (uint32_t)(byte & 3) | ((uint32_t)(4 + (byte & 3)) << 4);
-  uint32_t r = __byte_perm(x, y, sel);
-  if (I == 0) r ^= 0x8080u;                            // the top digit is signed
-  r = __byte_perm(r, 0x64646464u, 0x4140);             // 1024 + byte
-  asm("sub.f16x2 %0, %0, %1;" : "+r"(r) : "r"(0x64806480u));   // - 1152
+  constexpr uint32_t hi = (uint32_t)(byte & 3), sel = hi | (4 + hi) << 4 | (hi - 1) << 8 | (3 + hi) << 12;
+  const uint32_t t = __byte_perm(x, y, sel);
+  uint2 r = make_uint2(__byte_perm(t, 0x64646464u, 0x4140), __byte_perm(t, 0x64646464u, 0x4342));   // 1024 + byte
+  asm("sub.f16x2 %0, %0, %1;" : "+r"(r.x) : "r"(0x64806480u));   // - 1152
+  asm("sub.f16x2 %0, %0, %1;" : "+r"(r.y) : "r"(0x64806480u));
+  return r;
+}
+__device__ __forceinline__ uint32_t digit0_pair(uint64_t a, uint64_t b) {
+  uint32_t r = __byte_perm(__byte_perm((uint32_t)(a >> 32), (uint32_t)(b >> 32), 0x0062), 0x64646464u, 0x4140);
+  asm("sub.f16x2 %0, %0, %1;" : "+r"(r) : "r"(0x64806480u));
   return r;
 }
 template <int I>
-__device__ __forceinline__ uint4 digit8(const uint64_t* q) {
-  return make_uint4(digit_pair<I>(q[0], q[1]), digit_pair<I>(q[2], q[3]), digit_pair<I>(q[4], q[5]),
-                    digit_pair<I>(q[6], q[7]));
+__device__ __forceinline__ void put2(unsigned char* p, const uint64_t* q) {
+  const uint2 a = digit_pairs<I>(q[0], q[1]), b = digit_pairs<I>(q[2], q[3]), c = digit_pairs<I>(q[4], q[5]),
+              d = digit_pairs<I>(q[6], q[7]);
+  *reinterpret_cast<uint4*>(p + I * A_DIG) = make_uint4(a.x, b.x, c.x, d.x);
+  *reinterpret_cast<uint4*>(p + (I + 1) * A_DIG) = make_uint4(a.y, b.y, c.y, d.y);
 }
 __device__ __forceinline__ void put8(unsigned char* p, const uint64_t* q) {
-  *reinterpret_cast<uint4*>(p) = digit8<0>(q);
-  *reinterpret_cast<uint4*>(p + A_DIG) = digit8<1>(q);
-  *reinterpret_cast<uint4*>(p + 2 * A_DIG) = digit8<2>(q);
-  *reinterpret_cast<uint4*>(p + 3 * A_DIG) = digit8<3>(q);
-  *reinterpret_cast<uint4*>(p + 4 * A_DIG) = digit8<4>(q);
-  *reinterpret_cast<uint4*>(p + 5 * A_DIG) = digit8<5>(q);
-  *reinterpret_cast<uint4*>(p + 6 * A_DIG) = digit8<6>(q);
+  *reinterpret_cast<uint4*>(p) = make_uint4(digit0_pair(q[0], q[1]), digit0_pair(q[2], q[3]), digit0_pair(q[4], q[5]),
+                                            digit0_pair(q[6], q[7]));
+  put2<1>(p, q);
+  put2<3>(p, q);
+  put2<5>(p, q);
 }
 
 // Exponent of the largest part of X's column q in every 128 columns of A (a warp each).
@@ -113,12 +126,12 @@ __global__ void __launch_bounds__(128) k_x_digits(const double2* __restrict__ X,
   for (int c = c0; c < c0 + fold && c * 128 < N; ++c) E = max(E, (int)xexp[c * 8 + q]);
   const double2 v = k < N && q < nrhs ? X[k + (size_t)q * ldx] : make_double2(0.0, 0.0);
   // 54 bits: oz::digits' 62 less the lowest byte
-  auto cut = [&](double x, bool neg) { return (uint64_t)((int64_t)(oz::digits(x, E, neg) - oz::BIAS + 128) >> 8) + BIAS; };
-  const uint64_t r = cut(v.x, false), i = cut(v.y, false), ni = cut(v.y, true);
+  auto cut_x = [&](double x, bool neg) { return (uint64_t)((int64_t)(oz::digits(x, E, neg) - oz::BIAS + 128) >> 8) + BIAS; };
+  const uint64_t r = cut_x(v.x, false), i = cut_x(v.y, false), ni = cut_x(v.y, true);
   unsigned char* o = out + (size_t)t * (NS * B_DIG);
   auto put = [&](uint64_t a, int row, int col) {
-    const uint32_t d[NS] = {digit_pair<0>(a, 0), digit_pair<1>(a, 0), digit_pair<2>(a, 0), digit_pair<3>(a, 0),
-                            digit_pair<4>(a, 0), digit_pair<5>(a, 0), digit_pair<6>(a, 0)};
+    const uint2 d1 = digit_pairs<1>(a, 0), d3 = digit_pairs<3>(a, 0), d5 = digit_pairs<5>(a, 0);
+    const uint32_t d[NS] = {digit0_pair(a, 0), d1.x, d1.y, d3.x, d3.y, d5.x, d5.y};
 #pragma unroll
     for (int s = 0; s < NS; ++s) *reinterpret_cast<unsigned short*>(o + s * B_DIG + off(row, col)) = (unsigned short)d[s];
   };
@@ -154,12 +167,14 @@ __global__ void __launch_bounds__(T, 1) k_dense_matvec_oz(const float2* __restri
   uint64_t* empty = full + NBUF;
   uint64_t* done = empty + NBUF;      // a fold's MMAs have finished
   uint64_t* drained = done + 1;       // its accumulators have been read
-  uint32_t* taddr = reinterpret_cast<uint32_t*>(drained + 1);
+  uint64_t* last = drained + 1;       // nothing is in flight any more
+  uint32_t* taddr = reinterpret_cast<uint32_t*>(last + 1);
   int* s_fail = reinterpret_cast<int*>(taddr + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     for (int i = 0; i < NBUF; ++i) { mbar_init(&full[i], 256); mbar_init(&empty[i], 1); }
     mbar_init(done, 1);
+    mbar_init(last, 1);
     mbar_init(drained, WORKERS);
     *s_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;");
@@ -198,6 +213,8 @@ __global__ void __launch_bounds__(T, 1) k_dense_matvec_oz(const float2* __restri
         tcx::mma_commit(&empty[b]);
         if (n % spf == spf - 1 || t == t1 - 1) tcx::mma_commit(done);
       }
+      tcx::mma_commit(last);   // also after a wait that ran out: TMEM is freed below
+      if (!tcx::mbar_wait(last, 0, WAIT)) *(volatile int*)s_fail = 1;
     }
     __syncwarp();
   } else {
@@ -234,10 +251,10 @@ __global__ void __launch_bounds__(T, 1) k_dense_matvec_oz(const float2* __restri
         unsigned char* A = sm + b * STAGE;
         uint64_t q[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) q[i] = part(h[i].x, E) + part(l[i].x, E) + BIAS;
+        for (int i = 0; i < 8; ++i) q[i] = cut(h[i].x, l[i].x, E);
         put8(A + off(r, 8 * kg), q);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) q[i] = part(h[i].y, E) + part(l[i].y, E) + BIAS;
+        for (int i = 0; i < 8; ++i) q[i] = cut(h[i].y, l[i].y, E);
         put8(A + off(r, KC + 8 * kg), q);
         if (u < XCHUNK / 2) {
           uint4* B = reinterpret_cast<uint4*>(A + NS * A_DIG);
