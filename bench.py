@@ -539,7 +539,7 @@ def run_ours(args):
             "vs_baseline": None, "dtype": "c64+c128" if precision == pm.PM_MIXED else "c128",
             "data": "synthetic",
             "config": _workload_config(WORKLOADS[args.workload], N, st["levels"], args.precision, ws, args.workload),
-            "refinement_confirm": "fp64" if args.fp64_confirm else "float-float folded into FP64 every 16 columns",
+            "refinement_confirm": "fp64" if args.fp64_confirm else "FP64-accurate product on the tensor cores",
             "solve_ms": solve, "factor_ms": ms - solve, "K": st["K"], "skeleton_per_level": st["skeleton"],
             "refinement": info,
             "rank_predictor": {"used": model_ptr is not None, "cpqr_launches": st["cpqr_launches"],
@@ -620,7 +620,7 @@ def main():
     ap.add_argument("--precision", default="mixed", choices=["mixed", "fp64"])
     ap.add_argument("--no-fp64-compare", action="store_true")
     ap.add_argument("--no-rank-model", action="store_true")
-    # the refinement ends on the FP64 product instead of the folded float-float one
+    # the refinement ends on the FP64 product instead of the tensor-core one
     ap.add_argument("--fp64-confirm", action="store_true")
     ap.add_argument("--no-oracle-error", action="store_true")
     # one factorization + solve only (ncu launch lists): no end-to-end pass, no

@@ -119,9 +119,9 @@ typedef struct pm_factor pm_factor;
  *      row count adds enough rounding error to raise the ranks at the
  *      complex64 threshold.
  *      Confirming residual (PM_MIXED with the dense operator): by default the
- *      residual that ends the refinement comes from a float-float product of
- *      the stored operator whose sums are folded into FP64 every 16 columns
- *      (worst-case error ~9e-13 of sum_j |a_ij| |x_j| per row, below that of
+ *      residual that ends the refinement comes from a product of the stored
+ *      operator on the tensor cores (digits of fp16, sums exact within 128 or
+ *      512 columns; error ~1e-15 of sum_j |a_ij| |x_j| per row, below that of
  *      a sequential FP64 sum); PM_FLAG_FP64_CONFIRM forms it with the FP64
  *      product instead.  PM_FLAG_FF_CONFIRM names the default and changes
  *      nothing.  PM_FLAG_NO_AUTOTUNE: the call tunes no batched-GEMM tile
@@ -134,9 +134,9 @@ typedef struct pm_factor pm_factor;
  *      every application eager.  Solves of one factor are serialised.
  * refine_tol: PM_MIXED: stop refining once every column's relative residual
  *      ||b - A x|| / ||b|| <= refine_tol (0 -> 1e-10).  Intermediate residuals
- *      may come from FP32 or float-float products of the stored operator;
- *      the residual that ends the refinement is formed by the folded
- *      float-float product (or, with PM_FLAG_FP64_CONFIRM, in complex128).
+ *      may come from FP32 products of the stored operator; the residual that
+ *      ends the refinement is formed at FP64 accuracy on the tensor cores
+ *      (or, with PM_FLAG_FP64_CONFIRM, in complex128).
  * max_refine: PM_MIXED: refinement steps at most (0 -> 10); not reaching
  *      refine_tol returns PM_ERR_NOT_CONVERGED.
  * low_tol: PM_MIXED: ID threshold of the complex64 levels (0 -> 5e-6).

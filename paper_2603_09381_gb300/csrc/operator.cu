@@ -142,11 +142,6 @@ __device__ __forceinline__ void store_split(const SplitOp& A, size_t idx, double
   A.lo[idx] = l;
 }
 
-__device__ __forceinline__ float4 split4(double re, double im) {
-  const float hr = (float)re, hi = (float)im;
-  return make_float4(hr, hi, (float)(re - (double)hr), (float)(im - (double)hi));
-}
-
 // Dense off-diagonal operator: thread = (node t, node s) with t < s; a block
 // covers 64 t by 4 s (s fastest), so that the writes of both halves fill
 // whole 32-byte sectors of each plane: the (t <- s) entries of 8 consecutive

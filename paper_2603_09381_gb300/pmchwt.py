@@ -297,7 +297,7 @@ class Factor:
         instead of complex64;
         operator_after: PM_MIXED assembles the dense operator after the factorization
         (PM_FLAG_OPERATOR_AFTER) instead of beside it;
-        ff_confirm: the refinement ends on the folded float-float product (default) or,
+        ff_confirm: the refinement ends on the tensor-core product at FP64 accuracy (default) or,
         with False, on the FP64 product (PM_FLAG_FP64_CONFIRM);
         debug_flags: PM_DEBUG_* fault injection for failure-path tests (0 in normal use)."""
         lib = load()

@@ -90,3 +90,18 @@ def test_tall_lu_panels(pm, n):
     A = dense.assemble(prob)
     # backward error: 2 n 2^-52 with a growth of ten, and entries that agree to 1e-12 of their block's size
     assert np.linalg.norm(A @ x - F) < 1e-11 * np.linalg.norm(A) * np.linalg.norm(x)
+
+
+@pytest.mark.parametrize("mixed", [False, True])
+@pytest.mark.parametrize("nrhs", [1, 2, 3, 4])
+def test_solutions_for_few_waves(pm, nrhs, mixed):
+    """One to three columns have a product kernel of their own, four do not;
+    98 nodes a star leave rows past its 32-row blocks."""
+    prob = wl.star_grid(2, 2, n=98, seed=6, k_out=4.0)
+    angs = list(np.linspace(0.2, 5.0, nrhs))
+    g = pm.Geometry(prob)
+    kw = {"precision": pm.PM_MIXED, "refine_tol": 1e-11} if mixed else {}
+    f = pm.Factor(g, 1e-12, **kw)
+    F, ref = g.plane_wave(angs), dense.solve(prob, angs)
+    assert _rel(f.solve(F), ref) < (1e-8 if mixed else 3e-11)
+    assert _rel(f.solve(F), ref) < (1e-8 if mixed else 3e-11)   # replayed from its graph
