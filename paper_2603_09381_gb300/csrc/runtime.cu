@@ -1126,11 +1126,22 @@ void sqnorm_batch(const std::vector<SqNormProb>& probs, Arena& scr, cudaStream_t
   CK(cudaGetLastError());
 }
 
-// complex128 ID inputs with at least this many candidates (and twice as many
-// rows) are reduced to their triangle first; a panel runs on a cluster of 8
-// CTAs above this many rows, else of 4.
+// One-launch pivoted QR (k_cpqr_resident) while its CTAs take at most this many
+// waves of the SMs.  None at all: two disks 6.05 -> 6.59 ms and 4 x 4 stars
+// 58.6 -> 59.9 in complex128; lossy disks 5.0 -> 5.6, 8 x 8 stars 66.7 -> 70.2
+// and a batch of ellipses 83.3 -> 88.9 in the mixed mode.  Between 2 and 64
+// waves nothing differs by more than 1% there; beyond, a CTA's serial steps
+// would queue behind one another.
 constexpr int RESIDENT_WAVES_64 = 4, RESIDENT_WAVES_32 = 8;
+// complex128 ID inputs with at least this many candidates (and twice as many
+// rows) are reduced to their triangle first.  From 64: two disks 6.05 -> 6.37
+// ms, 20 scattered ellipses 50.6 -> 49.6; from 160: 4 x 4 stars 58.6 -> 63.5,
+// 8 x 8 stars 319.5 -> 334.5, Burton-Miller 68.4 -> 74.0.
 constexpr int QR_FIRST_MIN_N64 = 80;
+// A panel runs on a cluster of 8 CTAs above this many rows, else of 4 (whose
+// shared memory holds as many).  Above 1,024: 8 x 8 stars 319.5 -> 326.3 ms,
+// 4 x 4 stars 58.6 -> 60.9; above 2,400: Fourier shapes 133.3 -> 140.7,
+// Burton-Miller 68.4 -> 72.0.
 constexpr int QR_CLUSTER8_W64 = 1536;
 
 // Held-out proxy check bound: an ID passes while ||H_J - H_S T|| <= PROXY_CHECK_BOUND tol ||H||.
