@@ -760,6 +760,10 @@ struct GemmBatch {
   }
   // complex128 products on the tensor cores (oz_gemm): all but those whose
   // 128 x 32 tile would be mostly padding.  Per product, whatever the batch.
+  // From 2 columns instead of 4 (two and three waves): Fourier shapes 133.6 ->
+  // 135.0 ms, Burton-Miller 68.6 -> 69.5; from 9 (four waves): two disks 6.28 ->
+  // 6.64, Fourier shapes 135.2 -> 139.1, (eight waves) 8 x 8 stars 320 -> 326.
+  // From 128 rows or 64 terms: within 1.5%, slower where anything changes.
   static bool on_tensor_cores(const GemmDesc<C>& x) { return x.m >= 32 && x.n >= 4 && x.k >= 16; }
   void run(Arena& scr, cudaStream_t st) {
     if (std::is_same<C, double2>::value && g_oz_err) {
