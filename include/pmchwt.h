@@ -192,9 +192,12 @@ typedef struct pm_factor pm_factor;
  *        with a short bound, on a barrier that nothing arrives at before
  *        they issue any work (-> PM_ERR_TIMEOUT);
  *      PM_DEBUG_SOLVE_NO_FLAG makes the chained top-level triangular solves
- *        (one launch per triangle, used for at most 8 right-hand sides) wait,
+ *        (one launch per triangle, used for at most 64 right-hand sides) wait,
  *        with a 1 ms bound, on a flag that nothing sets before any work
- *        (-> PM_ERR_TIMEOUT from pm_solve / pm_solve_ex). */
+ *        (-> PM_ERR_TIMEOUT from pm_solve / pm_solve_ex);
+ *      PM_DEBUG_OZ_NO_ARRIVE and PM_DEBUG_OZ_SOLVE_NO_ARRIVE do the same as
+ *        PM_DEBUG_TC_NO_ARRIVE for the FP64-accurate tensor-core products of
+ *        the factorization and of the solves (-> PM_ERR_TIMEOUT). */
 typedef struct {
   double tol;
   double proxy_factor;
@@ -223,7 +226,9 @@ enum {
   PM_DEBUG_SINGULAR_COMPRESSED = 2,
   PM_DEBUG_UNDERPREDICT = 4,
   PM_DEBUG_TC_NO_ARRIVE = 8,
-  PM_DEBUG_SOLVE_NO_FLAG = 16
+  PM_DEBUG_SOLVE_NO_FLAG = 16,
+  PM_DEBUG_OZ_NO_ARRIVE = 32,
+  PM_DEBUG_OZ_SOLVE_NO_ARRIVE = 64
 };
 
 /* Outcome of a refined solve (PM_MIXED): steps taken, the final largest

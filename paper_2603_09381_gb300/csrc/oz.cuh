@@ -151,15 +151,18 @@ struct Cta {
   unsigned char* sm;
   uint32_t tmem;
   uint32_t phase;
-  bool ok;
+  bool ok;   // no wait has run out: the same in every thread of the CTA
 };
 
 // All threads of the CTA; smem: oz::SMEM bytes of dynamic shared memory, 128-byte aligned.
-__device__ __forceinline__ Cta begin(unsigned char* sm) {
-  uint64_t* bar = reinterpret_cast<uint64_t*>(sm + OFF_BAR);
+// no_arrive (tests of the timeout path): the CTA first waits, with a bound of
+// about a millisecond, on a barrier that nothing arrives at.
+__device__ __forceinline__ Cta begin(unsigned char* sm, int no_arrive) {
+  uint64_t* bar = reinterpret_cast<uint64_t*>(sm + OFF_BAR);   // a stage's MMAs; then the drain's (end)
   uint32_t* taddr = reinterpret_cast<uint32_t*>(sm + OFF_BAR + 16);
   if (threadIdx.x == 0) {
     tcx::mbar_init(bar);
+    tcx::mbar_init(bar + 1);
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
   if (threadIdx.x < 32) {
@@ -169,17 +172,24 @@ __device__ __forceinline__ Cta begin(unsigned char* sm) {
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
-  return Cta{sm, *taddr, 0, true};
+  Cta c{sm, *taddr, 0, true};
+  if (no_arrive) c.ok = __syncthreads_and(tcx::mbar_wait(bar + 1, 0, 1 << 10) ? 1 : 0) != 0;
+  return c;
 }
+// After a wait that ran out nothing more was cut, issued or stored (stage); the
+// MMAs still in flight are waited for, with a limit, at a barrier of their own
+// (thread 0 issued them all), so that no earlier phase can stand in for theirs.
 __device__ __forceinline__ void end(Cta& c, int* err) {
+  if (!c.ok && threadIdx.x == 0) {
+    uint64_t* drain = reinterpret_cast<uint64_t*>(c.sm + OFF_BAR) + 1;
+    tcx::mma_commit(drain);
+    tcx::mbar_wait(drain, 0, WAIT);
+    atomicExch(err, 1);
+  }
   asm volatile("tcgen05.fence::before_thread_sync;");
-  const int all_ok = __syncthreads_and(c.ok ? 1 : 0);
-  // a wait ran out: once more, bounded, for what may be in flight
-  if (!all_ok && threadIdx.x == 0) tcx::mbar_wait(reinterpret_cast<uint64_t*>(c.sm + OFF_BAR), c.phase ^ 1, WAIT);
-  __syncwarp();
+  __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   if (threadIdx.x < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(c.tmem), "r"(512));
-  if (!all_ok && threadIdx.x == 0) atomicExch(err, 1);
 }
 
 // One stage: emit(j, part, d) receives the real (part 0) and imaginary parts
@@ -189,6 +199,7 @@ __device__ __forceinline__ void end(Cta& c, int* err) {
 // yet; during() runs while the MMAs do (loads for emit).  All 512 threads call it.
 template <class FA, class FB, class FE, class FD>
 __device__ __forceinline__ void stage(Cta& c, bool new_a, const FA& a, const FB& b, const FE& emit, const FD& during) {
+  if (!c.ok) return;   // a wait ran out before: the operands may still be read
   const int tid = threadIdx.x, warp = tid >> 5;
   int* ea = reinterpret_cast<int*>(c.sm + OFF_EXP);   // [k group][row]
   int* eb = ea + 4 * TM;                              // [k group][column]
@@ -266,10 +277,10 @@ __device__ __forceinline__ void stage(Cta& c, bool new_a, const FA& a, const FB&
   int E = max(max(ea[er], ea[TM + er]), max(ea[2 * TM + er], ea[3 * TM + er]));
   if (E == 0x7FF) E = -0x4000;
   during();
-  c.ok = c.ok && tcx::mbar_wait(bar, c.phase, WAIT);
+  const bool done = tcx::mbar_wait(bar, c.phase, WAIT);
   c.phase ^= 1;
   asm volatile("tcgen05.fence::after_thread_sync;");
-  if (__all_sync(0xffffffffu, c.ok ? 1 : 0)) {
+  if (__all_sync(0xffffffffu, done ? 1 : 0)) {
     const uint32_t t0 = c.tmem + ((uint32_t)((warp & 3) * 32) << 16) + 8 * cg;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -291,7 +302,7 @@ __device__ __forceinline__ void stage(Cta& c, bool new_a, const FA& a, const FB&
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
-  __syncthreads();   // the operands and accumulators may be overwritten
+  c.ok = __syncthreads_and(done ? 1 : 0) != 0;   // the operands and accumulators may be overwritten
   asm volatile("tcgen05.fence::after_thread_sync;");
 }
 

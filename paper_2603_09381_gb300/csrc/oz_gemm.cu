@@ -6,6 +6,7 @@
 #include <algorithm>
 
 thread_local int* g_oz_err = nullptr;
+thread_local int g_oz_no_arrive = 0;
 
 namespace {
 
@@ -55,7 +56,7 @@ __device__ __forceinline__ void oz_tiles_of(oz::Cta& cta, int m, int n, int k, c
 }
 
 __global__ void __launch_bounds__(oz::T) k_oz_gemm(const GemmDesc<double2>* __restrict__ d, const int* __restrict__ off,
-                                                   int nprob, int per, int* err) {
+                                                   int nprob, int per, int* err, int no_arrive) {
   extern __shared__ __align__(1024) unsigned char sm[];
   const int t = blockIdx.x;
   int lo = 0, hi = nprob;
@@ -66,7 +67,7 @@ __global__ void __launch_bounds__(oz::T) k_oz_gemm(const GemmDesc<double2>* __re
   const GemmDesc<double2> g = d[lo];
   const int local = t - off[lo], tm = (g.m + oz::TM - 1) / oz::TM, tn = (g.n + oz::TN - 1) / oz::TN;
   const int r0 = (local % tm) * oz::TM, t0 = (local / tm) * per;
-  oz::Cta cta = oz::begin(sm);
+  oz::Cta cta = oz::begin(sm, no_arrive);
   if (g.alpha.x == -1.0 && g.alpha.y == 0.0 && g.beta.x == 1.0 && g.beta.y == 0.0 && !g.beta_zero)
     oz_tiles_of<1>(cta, g.m, g.n, g.k, g.A, g.lda, g.B, g.ldb, g.Cm, g.ldc, r0, t0, min(tn, t0 + per), g.alpha, g.beta, 0);
   else
@@ -76,7 +77,7 @@ __global__ void __launch_bounds__(oz::T) k_oz_gemm(const GemmDesc<double2>* __re
 }
 
 __global__ void __launch_bounds__(oz::T) k_oz_lu_update(const LuProb<double2>* __restrict__ P, int p, int nb, int lo, int hi,
-                                                        int per, int* err) {
+                                                        int per, int* err, int no_arrive) {
   extern __shared__ __align__(1024) unsigned char sm[];
   const LuProb<double2> pr = P[blockIdx.z];
   if (p >= pr.m) return;
@@ -86,14 +87,14 @@ __global__ void __launch_bounds__(oz::T) k_oz_lu_update(const LuProb<double2>* _
   if (r0 >= mt || t0 >= tn) return;
   const size_t ld = pr.ld;
   const double2 z = make_double2(0.0, 0.0);
-  oz::Cta cta = oz::begin(sm);
+  oz::Cta cta = oz::begin(sm, no_arrive);
   oz_tiles_of<1>(cta, mt, n, jb, pr.A + (p + jb) + p * ld, ld, pr.A + p + c0 * ld, ld, pr.A + (p + jb) + c0 * ld, ld, r0, t0,
                  min(tn, t0 + per), z, z, 0);
   oz::end(cta, err);
 }
 
 __global__ void __launch_bounds__(oz::T) k_oz_getrs_update(const SolveProb<double2>* __restrict__ P, int p, int nb, int lower,
-                                                           int per, int* err) {
+                                                           int per, int* err, int no_arrive) {
   extern __shared__ __align__(1024) unsigned char sm[];
   const SolveProb<double2> pr = P[blockIdx.z];
   if (p >= pr.m) return;
@@ -102,7 +103,7 @@ __global__ void __launch_bounds__(oz::T) k_oz_getrs_update(const SolveProb<doubl
   const int r0 = blockIdx.x * oz::TM, t0 = blockIdx.y * per, tn = (pr.nrhs + oz::TN - 1) / oz::TN;
   if (r0 >= mt || t0 >= tn) return;
   const double2 z = make_double2(0.0, 0.0);
-  oz::Cta cta = oz::begin(sm);
+  oz::Cta cta = oz::begin(sm, no_arrive);
   oz_tiles_of<1>(cta, mt, pr.nrhs, jb, pr.A + b0 + p * (size_t)pr.ld, pr.ld, pr.B + p, pr.ldb, pr.B + b0, pr.ldb, r0, t0,
                  min(tn, t0 + per), z, z, 0);
   oz::end(cta, err);
@@ -118,7 +119,7 @@ void oz_gemm_batched(const GemmDesc<double2>* d_desc, const int* d_off, int npro
   KPROF_BEGIN(st);
   // the same value every time: idempotent across threads and devices
   cudaFuncSetAttribute(k_oz_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, oz::SMEM);
-  k_oz_gemm<<<total, oz::T, oz::SMEM, st>>>(d_desc, d_off, nprob, per, err);
+  k_oz_gemm<<<total, oz::T, oz::SMEM, st>>>(d_desc, d_off, nprob, per, err, g_oz_no_arrive);
   pm_launch_count_add(1);
   KPROF_END(st, "gemm_oz", 0.0);
 }
@@ -129,7 +130,8 @@ void oz_lu_update(const LuProb<double2>* d_prob, int nprob, int maxm, int p, int
   if (nprob <= 0 || mt <= 0 || n <= 0) return;
   const int tm = (mt + oz::TM - 1) / oz::TM, tn = (n + oz::TN - 1) / oz::TN, per = oz_per((long)tm * tn * nprob);
   cudaFuncSetAttribute(k_oz_lu_update, cudaFuncAttributeMaxDynamicSharedMemorySize, oz::SMEM);
-  k_oz_lu_update<<<dim3(tm, (tn + per - 1) / per, nprob), oz::T, oz::SMEM, st>>>(d_prob, p, nb, lo, hi, per, err);
+  k_oz_lu_update<<<dim3(tm, (tn + per - 1) / per, nprob), oz::T, oz::SMEM, st>>>(d_prob, p, nb, lo, hi, per, err,
+                                                                                 g_oz_no_arrive);
 }
 
 void oz_getrs_update(const SolveProb<double2>* d_prob, int nprob, int maxm, int maxrhs, int p, int nb, int lower, int* err,
@@ -138,5 +140,6 @@ void oz_getrs_update(const SolveProb<double2>* d_prob, int nprob, int maxm, int 
   if (nprob <= 0 || mt <= 0 || maxrhs <= 0) return;
   const int tm = (mt + oz::TM - 1) / oz::TM, tn = (maxrhs + oz::TN - 1) / oz::TN, per = oz_per((long)tm * tn * nprob);
   cudaFuncSetAttribute(k_oz_getrs_update, cudaFuncAttributeMaxDynamicSharedMemorySize, oz::SMEM);
-  k_oz_getrs_update<<<dim3(tm, (tn + per - 1) / per, nprob), oz::T, oz::SMEM, st>>>(d_prob, p, nb, lower, per, err);
+  k_oz_getrs_update<<<dim3(tm, (tn + per - 1) / per, nprob), oz::T, oz::SMEM, st>>>(d_prob, p, nb, lower, per, err,
+                                                                                    g_oz_no_arrive);
 }

@@ -5,11 +5,22 @@
 
 // Error word of the bounded tensor-core waits of the running call (device
 // int, set to 1 when a wait runs out): thread-local, set by OzErrScope.
+// no_arrive (tests of the timeout path): see oz::begin.
 extern thread_local int* g_oz_err;
+extern thread_local int g_oz_no_arrive;
 struct OzErrScope {
   int* prev;
-  explicit OzErrScope(int* e) : prev(g_oz_err) { g_oz_err = e; }
-  ~OzErrScope() { g_oz_err = prev; }
+  int prev_no_arrive;
+  explicit OzErrScope(int* e, bool no_arrive = false) : prev(g_oz_err), prev_no_arrive(g_oz_no_arrive) {
+    g_oz_err = e;
+    g_oz_no_arrive = no_arrive;
+  }
+  ~OzErrScope() {
+    g_oz_err = prev;
+    g_oz_no_arrive = prev_no_arrive;
+  }
+  OzErrScope(const OzErrScope&) = delete;
+  OzErrScope& operator=(const OzErrScope&) = delete;
 };
 
 // Tiles of an m x n product: rows in 128s, columns in groups of `per` tiles of 32.

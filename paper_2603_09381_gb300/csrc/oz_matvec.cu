@@ -20,6 +20,7 @@
 // fill up.  All waits are bounded; one that runs out sets *err.
 #include "operator.cuh"
 #include "oz.cuh"
+#include "oz_gemm.cuh"
 #include "prof.cuh"
 #include <algorithm>
 
@@ -161,20 +162,22 @@ __global__ void __launch_bounds__(T, 1) k_dense_matvec_oz(const float2* __restri
                                                           size_t lda, int N, const unsigned char* __restrict__ rexp,
                                                           const unsigned short* __restrict__ xexp,
                                                           const uint4* __restrict__ Xd, double2* __restrict__ Y, int ldy,
-                                                          int nrhs, int fold, int folds, int* err) {
+                                                          int nrhs, int fold, int folds, int* err, int no_arrive) {
   extern __shared__ __align__(1024) unsigned char sm[];
   uint64_t* full = reinterpret_cast<uint64_t*>(sm + OFF_BAR);
   uint64_t* empty = full + NBUF;
   uint64_t* done = empty + NBUF;      // a fold's MMAs have finished
   uint64_t* drained = done + 1;       // its accumulators have been read
   uint64_t* last = drained + 1;       // nothing is in flight any more
-  uint32_t* taddr = reinterpret_cast<uint32_t*>(last + 1);
+  uint64_t* never = last + 1;         // tests of the timeout path: nothing arrives at it
+  uint32_t* taddr = reinterpret_cast<uint32_t*>(never + 1);
   int* s_fail = reinterpret_cast<int*>(taddr + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     for (int i = 0; i < NBUF; ++i) { mbar_init(&full[i], 256); mbar_init(&empty[i], 1); }
     mbar_init(done, 1);
     mbar_init(last, 1);
+    mbar_init(never, 1);
     mbar_init(drained, WORKERS);
     *s_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;");
@@ -187,6 +190,10 @@ __global__ void __launch_bounds__(T, 1) k_dense_matvec_oz(const float2* __restri
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = *taddr;
+  if (no_arrive) {   // see oz::begin
+    if (!tcx::mbar_wait(never, 0, 1 << 10)) *(volatile int*)s_fail = 1;
+    __syncthreads();
+  }
   const int spf = 8 * fold;                                  // stages per fold
   const int t0 = (int)blockIdx.y * folds * spf, t1 = min((N + KC - 1) / KC, t0 + folds * spf);
   const int row0 = blockIdx.x * TM;
@@ -348,7 +355,8 @@ void dense_matvec_oz(SplitOp A, int N, const unsigned char* rexp, const double2*
     k_x_exponents<<<chunks, 256, 0, st>>>(X + (size_t)r0 * ldx, ldx, N, nr, xexp);
     k_x_digits<<<(N + KC - 1) / KC, 128, 0, st>>>(X + (size_t)r0 * ldx, ldx, N, nr, fold, xexp, xdig);
     k_dense_matvec_oz<<<dim3(rb, (nf + folds - 1) / folds), T, SMEM, st>>>(
-        A.hi, A.lo, A.ld, N, rexp, xexp, (const uint4*)xdig, Y + (size_t)r0 * ldy, ldy, nr, fold, folds, err);
+        A.hi, A.lo, A.ld, N, rexp, xexp, (const uint4*)xdig, Y + (size_t)r0 * ldy, ldy, nr, fold, folds, err,
+        g_oz_no_arrive);
     pm_launch_count_add(3);
   }
   KPROF_END(st, "dense_matvec_oz", 0.0);

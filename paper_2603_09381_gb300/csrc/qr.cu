@@ -924,7 +924,8 @@ __global__ void __maxnreg__(112) k_qr_apply_tc(const QrProb<float2>* __restrict_
 // columns from j0 on and row block), their sum with T^H applied, C -= V Y.
 
 // Partial (columns i, reflectors j): sum over the block's rows of conj(X_i) V_j, X the panel's V, then C.
-__global__ void __launch_bounds__(oz::T) k_qr_oz_ypart(const QrProb<double2>* __restrict__ P, int j0, int* err) {
+__global__ void __launch_bounds__(oz::T) k_qr_oz_ypart(const QrProb<double2>* __restrict__ P, int j0, int* err,
+                                                       int no_arrive) {
   extern __shared__ __align__(1024) unsigned char sm[];
   const QrProb<double2> p = P[blockIdx.z];
   const int c0 = j0 + (int)blockIdx.x * oz::TM, rbeg = j0 + (int)blockIdx.y * OZ_RB;
@@ -933,7 +934,7 @@ __global__ void __launch_bounds__(oz::T) k_qr_oz_ypart(const QrProb<double2>* __
   double2 acc[8];
 #pragma unroll
   for (int j = 0; j < 8; ++j) acc[j] = czero<double2>();
-  oz::Cta cta = oz::begin(sm);
+  oz::Cta cta = oz::begin(sm, no_arrive);
   for (int r0 = rbeg; r0 < rend; r0 += oz::TKC)
     oz::stage(cta, true,
                     [&](int i, int l) {
@@ -991,14 +992,15 @@ __global__ void __launch_bounds__(UT) k_qr_oz_yreduce(const QrProb<double2>* __r
   }
 }
 
-__global__ void __launch_bounds__(oz::T) k_qr_oz_apply(const QrProb<double2>* __restrict__ P, int j0, int per, int* err) {
+__global__ void __launch_bounds__(oz::T) k_qr_oz_apply(const QrProb<double2>* __restrict__ P, int j0, int per, int* err,
+                                                       int no_arrive) {
   extern __shared__ __align__(1024) unsigned char sm[];
   const QrProb<double2> p = P[blockIdx.z];
   const int cfirst = j0 + QR_NB, r0 = j0 + (int)blockIdx.x * oz::TM, t0 = (int)blockIdx.y * per;
   if (cfirst + t0 * oz::TN >= p.n || r0 >= p.W) return;
   const int t1 = min(t0 + per, (p.n - cfirst + oz::TN - 1) / oz::TN);
   const int warp = threadIdx.x >> 5, row = r0 + 32 * (warp & 3) + (threadIdx.x & 31), cgp = 8 * (warp >> 2);
-  oz::Cta cta = oz::begin(sm);
+  oz::Cta cta = oz::begin(sm, no_arrive);
   for (int t = t0; t < t1; ++t) {
     const int c0 = t * oz::TN;   // trailing column
     double2 z[8];   // C, minus the products
@@ -1120,9 +1122,11 @@ void qr_update_oz(const QrProb<double2>* d_prob, int nprob, int j0, int max_n, i
   const int rbs = (max_w - j0 + OZ_RB - 1) / OZ_RB, mt = (max_w - j0 + oz::TM - 1) / oz::TM;
   const int tiles = (nt + oz::TN - 1) / oz::TN, per = oz_per((long)mt * tiles * nprob);
   KPROF_BEGIN(st);
-  k_qr_oz_ypart<<<dim3((max_n - j0 + oz::TM - 1) / oz::TM, rbs, nprob), oz::T, oz::SMEM, st>>>(d_prob, j0, err);
+  k_qr_oz_ypart<<<dim3((max_n - j0 + oz::TM - 1) / oz::TM, rbs, nprob), oz::T, oz::SMEM, st>>>(d_prob, j0, err,
+                                                                                                   g_oz_no_arrive);
   k_qr_oz_yreduce<<<dim3(tiles, nprob), UT, 0, st>>>(d_prob, j0);
-  k_qr_oz_apply<<<dim3(mt, (tiles + per - 1) / per, nprob), oz::T, oz::SMEM, st>>>(d_prob, j0, per, err);
+  k_qr_oz_apply<<<dim3(mt, (tiles + per - 1) / per, nprob), oz::T, oz::SMEM, st>>>(d_prob, j0, per, err,
+                                                                                    g_oz_no_arrive);
   pm_launch_count_add(3);
   KPROF_END(st, "qr_update_oz", 0.0);
 }

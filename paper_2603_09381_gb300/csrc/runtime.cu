@@ -2727,13 +2727,23 @@ void factor_group_t(std::vector<pm_factor*>& Fs, double id_tol, Arena& scr, cuda
 void factor_group(std::vector<pm_factor*>& Fs, double id_tol, Arena& scr, cudaStream_t st) {
   if (Fs.empty()) return;
   int* err = Fs[0]->d_wait_err;
-  OzErrScope oz(err);
-  if (Fs[0]->precision == PM_FP64) factor_group_t<double2>(Fs, id_tol, scr, st);
-  else factor_group_t<float2>(Fs, id_tol, scr, st);
-  int werr = 0;
-  CK(cudaMemcpyAsync(&werr, err, sizeof(int), cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  if (werr) fail(PM_ERR_TIMEOUT, "a wait on the tensor cores ran out");
+  OzErrScope oz(err, (Fs[0]->opts.debug_flags & PM_DEBUG_OZ_NO_ARRIVE) != 0);
+  auto wait_ran_out = [&] {
+    int werr = 0;
+    CK(cudaMemcpyAsync(&werr, err, sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    return werr != 0;
+  };
+  const char* const msg = "a wait on the tensor cores ran out";
+  try {
+    if (Fs[0]->precision == PM_FP64) factor_group_t<double2>(Fs, id_tol, scr, st);
+    else factor_group_t<float2>(Fs, id_tol, scr, st);
+  } catch (const PmError&) {
+    // products that were not formed can show up as a singular block first
+    if (wait_ran_out()) fail(PM_ERR_TIMEOUT, msg);
+    throw;
+  }
+  if (wait_ran_out()) fail(PM_ERR_TIMEOUT, msg);
 }
 
 // Mixed mode, after the complex64 levels: the FP64 self blocks, index maps and
@@ -3037,7 +3047,7 @@ pm_status solve_impl(const pm_factor* Fc, const pm_c64* rhs, int32_t nrhs, pm_c6
       ~ProfScope() { g_kprof = nullptr; }
     } scope(F->profiling ? &F->prof : nullptr);
     std::lock_guard<std::mutex> plan_lock(F->plan_mu);   // solves of one factor share its graphs
-    OzErrScope oz(F->d_wait_err);
+    OzErrScope oz(F->d_wait_err, (F->opts.debug_flags & PM_DEBUG_OZ_SOLVE_NO_ARRIVE) != 0);
     if (F->precision == PM_FP64 && F->opts.formulation >= PM_FORM_BM) {
       // Burton-Miller: its own right-hand side, then its [u; q] unknowns reordered
       const pm_geometry* g = F->g;

@@ -90,6 +90,8 @@ PM_DEBUG_SINGULAR_COMPRESSED = 2
 PM_DEBUG_UNDERPREDICT = 4
 PM_DEBUG_TC_NO_ARRIVE = 8
 PM_DEBUG_SOLVE_NO_FLAG = 16
+PM_DEBUG_OZ_NO_ARRIVE = 32
+PM_DEBUG_OZ_SOLVE_NO_ARRIVE = 64
 _lib = None
 
 EXPORTS = {
