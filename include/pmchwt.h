@@ -34,7 +34,7 @@ typedef enum {
   PM_ERR_INVALID_ARG = 1,   /* bad pointer, size, shape or option */
   PM_ERR_OOM = 2,           /* device or host allocation failed */
   PM_ERR_CUDA = 3,          /* CUDA runtime error (message names the call) */
-  PM_ERR_SINGULAR = 4,      /* exactly singular pivot in an LU, or R A^{-1} L singular */
+  PM_ERR_SINGULAR = 4,      /* exactly singular pivot in an LU, R A^{-1} L singular, or an ID input not finite */
   PM_ERR_NOT_CONVERGED = 5, /* PM_MIXED: refinement stopped above refine_tol after max_refine steps */
   PM_ERR_TIMEOUT = 6,       /* a bounded device wait ran out (tensor-core completion, chained solve) */
   PM_ERR_GEOMETRY = 7,      /* inclusions not on a grid, two in one cell, ... */
@@ -197,7 +197,9 @@ typedef struct pm_factor pm_factor;
  *        (-> PM_ERR_TIMEOUT from pm_solve / pm_solve_ex);
  *      PM_DEBUG_OZ_NO_ARRIVE and PM_DEBUG_OZ_SOLVE_NO_ARRIVE do the same as
  *        PM_DEBUG_TC_NO_ARRIVE for the FP64-accurate tensor-core products of
- *        the factorization and of the solves (-> PM_ERR_TIMEOUT). */
+ *        the factorization and of the solves (-> PM_ERR_TIMEOUT);
+ *      PM_DEBUG_NONFINITE_ID writes a NaN into the first ID input of the leaf
+ *        level (PM_FP64 -> PM_ERR_SINGULAR, "not finite"). */
 typedef struct {
   double tol;
   double proxy_factor;
@@ -228,7 +230,8 @@ enum {
   PM_DEBUG_TC_NO_ARRIVE = 8,
   PM_DEBUG_SOLVE_NO_FLAG = 16,
   PM_DEBUG_OZ_NO_ARRIVE = 32,
-  PM_DEBUG_OZ_SOLVE_NO_ARRIVE = 64
+  PM_DEBUG_OZ_SOLVE_NO_ARRIVE = 64,
+  PM_DEBUG_NONFINITE_ID = 128
 };
 
 /* Outcome of a refined solve (PM_MIXED): steps taken, the final largest

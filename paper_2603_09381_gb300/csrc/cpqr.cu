@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(256) k_init_norms(const CpqrProb<C>* __restric
     acc = warp_sum(acc);
     if (lane == 0) p.norm2[c] = (double)acc;
     if constexpr (sizeof(C) == 16) {
-      // to fixed point, the norm brought into (1/8, 1/4] (a column that is not finite: zeros)
+      // to fixed point, the norm brought into (1/8, 1/4] (a column that is not finite: zeros, and *bad)
       int e = 0;
       const bool ok = isfinite(acc);
       if (ok && acc > 0) frexp(sqrt(acc) * (1.0 + 1e-9), &e);
@@ -52,7 +52,10 @@ __global__ void __launch_bounds__(256) k_init_norms(const CpqrProb<C>* __restric
         const double2 z = col[r];
         f[r] = make_longlong2(ok ? fx_from(z.x, e) : 0, ok ? fx_from(z.y, e) : 0);
       }
-      if (lane == 0) p.cexp[c] = e;
+      if (lane == 0) {
+        p.cexp[c] = e;
+        if (!ok) *p.bad = 1;
+      }
     }
   }
 }

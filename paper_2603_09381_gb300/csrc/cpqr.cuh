@@ -30,6 +30,7 @@ struct CpqrProb {
   CpqrPick<C>* pick;
   int* done;                     // chunks finished in the running step
   int* cexp;                     // complex128: column c holds integers of 2^(cexp[c] - 60)
+  int* bad;                      // complex128: set to 1 if a column is not finite
 };
 
 struct CpqrChunk { int id; int c0; int c1; int first; };
@@ -95,7 +96,8 @@ template <typename C>
 void qr_zero_lower(const QrProb<C>* d_prob, int nprob, int max_n, cudaStream_t st);
 
 void complete_perm(const PermFill* d_prob, int nprob, cudaStream_t st);
-// Initial norms; complex128 columns go to fixed point (cexp) here.
+// Initial norms; complex128 columns go to fixed point (cexp) here, which has no
+// NaN: *bad tells the host of columns that are not finite.
 template <typename C>
 void cpqr_init_norms(const CpqrProb<C>* d_prob, const CpqrChunk* d_chunk, int nchunk, cudaStream_t st);
 // Before the first step of a phase (mode, base, target set): its first pivot.

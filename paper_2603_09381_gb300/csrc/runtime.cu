@@ -1390,6 +1390,10 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
     }
   }
   gb.run(scr, P, 0.0, st);
+  if ((O.debug_flags & PM_DEBUG_NONFINITE_ID) && jobs[0].lev == jobs[0].F->L && jb0[0] == 0 && W[0] > 0 && nn[0] > 0) {
+    const C nan = mk((typename real_of<C>::type)NAN, (typename real_of<C>::type)0);   // injected
+    CK(cudaMemcpyAsync(Z[0], &nan, sizeof(C), cudaMemcpyHostToDevice, st));
+  }
   for (int i = 0; i < nid; ++i) jobs[job_of[i / 4]].F->stats.id_rows += W[i];
   const double ms_asm = t_asm.stop();
   for (const auto& J : jobs) J.F->stats.ms_assemble += ms_asm;
@@ -1571,6 +1575,8 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
   CpqrPick<C>* pick = scr.get<CpqrPick<C>>(nid);
   int* done = scr.get<int>(nid);
   int* cexp = scr.get<int>(std::max(total_n, 1));
+  int* bad = scr.get<int>(1);
+  CK(cudaMemsetAsync(bad, 0, sizeof(int), st));
   CK(cudaMemsetAsync(ref, 0, nid * sizeof(double), st));
   CK(cudaMemsetAsync(rank, 0xff, nid * sizeof(int), st));
   CK(cudaMemsetAsync(perm, 0, std::max(total_n, 1) * sizeof(int), st));
@@ -1593,7 +1599,7 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
     int tgt = std::min(We[i], nn[i]);
     cp[i] = CpqrProb<C>{Z[i], W[i], We[i], nn[i], tol, CPQR_FIND_RANK, 0, tgt,
                         norm2 + 2 * (size_t)noff[i], perm + noff[i], rdiag + noff[i], rank + i, ref + i, pick + i,
-                        done + i, cexp + noff[i]};
+                        done + i, cexp + noff[i], bad};
     if (!rcs[i]) maxT = std::max(maxT, tgt);
     for (int c0 = 0; c0 < nn[i]; c0 += CPQR_CB) {
       const CpqrChunk ch{i, c0, std::min(c0 + CPQR_CB, nn[i]), c0 == 0};
@@ -1680,8 +1686,11 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
   // simplified Burton-Miller system) gets a zero interpolation, not an
   // identity on arbitrary pivots
   std::vector<double> href(nid);
+  int hbad = 0;
   CK(cudaMemcpyAsync(href.data(), ref, nid * sizeof(double), cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
+  if (hbad) fail(PM_ERR_SINGULAR, "an ID input is not finite");
   std::vector<char> zero_in(nid);
   for (int i = 0; i < nid; ++i) zero_in[i] = nn[i] > 0 && !(href[i] > 0);
   std::vector<int> r(nid);
@@ -2738,9 +2747,9 @@ void factor_group(std::vector<pm_factor*>& Fs, double id_tol, Arena& scr, cudaSt
   try {
     if (Fs[0]->precision == PM_FP64) factor_group_t<double2>(Fs, id_tol, scr, st);
     else factor_group_t<float2>(Fs, id_tol, scr, st);
-  } catch (const PmError&) {
+  } catch (const PmError& e) {
     // products that were not formed can show up as a singular block first
-    if (wait_ran_out()) fail(PM_ERR_TIMEOUT, msg);
+    if (e.st == PM_ERR_SINGULAR && wait_ran_out()) fail(PM_ERR_TIMEOUT, msg);
     throw;
   }
   if (wait_ran_out()) fail(PM_ERR_TIMEOUT, msg);

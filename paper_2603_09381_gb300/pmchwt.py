@@ -92,6 +92,7 @@ PM_DEBUG_TC_NO_ARRIVE = 8
 PM_DEBUG_SOLVE_NO_FLAG = 16
 PM_DEBUG_OZ_NO_ARRIVE = 32
 PM_DEBUG_OZ_SOLVE_NO_ARRIVE = 64
+PM_DEBUG_NONFINITE_ID = 128
 _lib = None
 
 EXPORTS = {
