@@ -841,11 +841,11 @@ void lu_panel(const LuProb<C>* d_prob, int nprob, int maxm, int p, cudaStream_t 
 }
 
 // The trailing update of step p on trailing columns [lo, hi): complex128 on
-// the tensor cores (g_oz_err: their error word), complex64 on the FP32 pipe.
+// the tensor cores, complex64 on the FP32 pipe.
 template <typename C>
 void lu_update(const LuProb<C>* d_prob, int nprob, int maxm, int p, int lo, int hi, cudaStream_t st) {
   const int mt = maxm - p - LU_NB, n = std::min(hi, mt) - lo;
-  if constexpr (std::is_same<C, double2>::value) oz_lu_update(d_prob, nprob, maxm, p, LU_NB, lo, hi, g_oz_err, st);
+  if constexpr (std::is_same<C, double2>::value) oz_lu_update(d_prob, nprob, maxm, p, LU_NB, lo, hi, oz_err_word(), st);
   else k_lu_update<C><<<dim3(((mt + TB - 1) / TB) * ((n + TB - 1) / TB), nprob), 256, 0, st>>>(d_prob, p, LU_NB, lo, hi);
 }
 
@@ -854,7 +854,7 @@ template <typename C>
 void getrs_update(const SolveProb<C>* d_prob, int nprob, int maxm, int maxrhs, int p, int lower, cudaStream_t st) {
   const int mt = lower ? maxm - p - RS_NB : p;
   if constexpr (std::is_same<C, double2>::value)
-    oz_getrs_update(d_prob, nprob, maxm, maxrhs, p, RS_NB, lower, g_oz_err, st);
+    oz_getrs_update(d_prob, nprob, maxm, maxrhs, p, RS_NB, lower, oz_err_word(), st);
   else
     k_getrs_update<C><<<dim3(((mt + TB - 1) / TB) * ((maxrhs + TB - 1) / TB), nprob), 256, 0, st>>>(d_prob, p, RS_NB, lower);
 }

@@ -2,6 +2,7 @@
 // and the trailing updates of the FP64 LU and LU solves.
 #pragma once
 #include "dense_la.cuh"
+#include <stdexcept>
 
 // Error word of the bounded tensor-core waits of the running call (device
 // int, set to 1 when a wait runs out): thread-local, set by OzErrScope.
@@ -22,6 +23,10 @@ struct OzErrScope {
   OzErrScope(const OzErrScope&) = delete;
   OzErrScope& operator=(const OzErrScope&) = delete;
 };
+inline int* oz_err_word() {
+  if (!g_oz_err) throw std::logic_error("FP64 tensor-core product without an error word");
+  return g_oz_err;
+}
 
 // Tiles of an m x n product: rows in 128s, columns in groups of `per` tiles of 32.
 inline int oz_tiles(int m, int n, int per) { return ((m + 127) / 128) * ((n + 32 * per - 1) / (32 * per)); }

@@ -640,7 +640,7 @@ void assemble_self(const pm_geometry* g, const std::vector<int>& incl, const std
   // Maue: N-block += diag(1/|x'|) Dt (S0+/e+ + S0-/e-) Dt
   std::vector<GemmDesc<C>> d1(m), d2(m);
   std::vector<int> off1(m + 1, 0), off2(m + 1, 0);
-  const bool oz = std::is_same<C, double2>::value && g_oz_err;   // on the tensor cores (oz_gemm)
+  constexpr bool oz = std::is_same<C, double2>::value;   // on the tensor cores (oz_gemm)
   long tiles = 0;
   for (int i = 0; i < m; ++i) tiles += oz_tiles(sub[i].n, sub[i].n, 1);
   const int per = oz_per(tiles);
@@ -655,13 +655,8 @@ void assemble_self(const pm_geometry* g, const std::vector<int>& incl, const std
   auto run = [&](const std::vector<GemmDesc<C>>& d, const std::vector<int>& off) {
     auto* dd = upload(scr, d, st);
     auto* dof = upload(scr, off, st);
-    if constexpr (std::is_same<C, double2>::value) {
-      if (oz) {
-        oz_gemm_batched(dd, dof, m, off[m], per, g_oz_err, st);
-        return;
-      }
-    }
-    la_gemm_batched<C>(dd, dof, m, off[m], st);
+    if constexpr (oz) oz_gemm_batched(dd, dof, m, off[m], per, oz_err_word(), st);
+    else la_gemm_batched<C>(dd, dof, m, off[m], st);
   };
   run(d1, off1);
   run(d2, off2);
@@ -766,11 +761,11 @@ struct GemmBatch {
   // From 128 rows or 64 terms: within 1.5%, slower where anything changes.
   static bool on_tensor_cores(const GemmDesc<C>& x) { return x.m >= 32 && x.n >= 4 && x.k >= 16; }
   void run(Arena& scr, cudaStream_t st) {
-    if (std::is_same<C, double2>::value && g_oz_err) {
+    if constexpr (std::is_same<C, double2>::value) {
       GemmBatch<C> rest;
       std::vector<GemmDesc<double2>> t;
       for (auto& x : d) {
-        if (on_tensor_cores(x)) t.push_back(*(const GemmDesc<double2>*)&x);
+        if (on_tensor_cores(x)) t.push_back(x);
         else { rest.d.push_back(x); rest.off.push_back(rest.off.back() + gemm_tiles(x.m, x.n)); }
       }
       if (!t.empty()) {
@@ -782,7 +777,7 @@ struct GemmBatch {
         for (auto& x : t) { o.push_back(o.back() + oz_tiles(x.m, x.n, per)); f += 8.0 * x.m * x.n * x.k; }
         auto* dt = upload(scr, t, st);
         int* dof = upload(scr, o, st);
-        oz_gemm_batched(dt, dof, (int)t.size(), o.back(), per, g_oz_err, st);
+        oz_gemm_batched(dt, dof, (int)t.size(), o.back(), per, oz_err_word(), st);
         if (g_kprof) g_kprof->add_flops("gemm_oz", f);
         CK(cudaGetLastError());
         rest.run_cuda_cores(scr, st);
@@ -1412,7 +1407,7 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
     // complex128: the same reduction with the trailing updates on the tensor
     // cores (FP64-accurate products).  Each rule looks at one matrix alone, so
     // that a problem's bits do not depend on what shares its launches.
-    if (!(O.flags & PM_FLAG_NO_QR_FIRST) && g_oz_err) {
+    if (!(O.flags & PM_FLAG_NO_QR_FIRST)) {
       std::vector<QrProb<C>> qp[2];   // panels on 4 CTAs, on 8
       int maxn = 0;
       double fl = 0;
@@ -1438,7 +1433,7 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
         for (int j0 = 0; j0 < maxn; j0 += QR_NB) {
           qr_panel<C>(dqp, n4, j0, st, 4, std::min(maxW, QR_CLUSTER8_W64));
           qr_panel<C>(dqp + n4, (int)all.size() - n4, j0, st, 8, maxW);
-          qr_update_oz(dqp, (int)all.size(), j0, maxn, maxW, g_oz_err, st);
+          qr_update_oz(dqp, (int)all.size(), j0, maxn, maxW, oz_err_word(), st);
         }
         qr_zero_lower<C>(dqp, (int)all.size(), maxn, st);
         CK(cudaGetLastError());
@@ -2367,7 +2362,7 @@ void solve_refined(pm_factor* F, const double2* B, int nrhs, double2* X, Arena& 
       dense_row_exponents(F->dense_op, N, F->row_exp, st);
       F->row_exp_ready = true;
     }
-    dense_matvec_oz(F->dense_op, N, F->row_exp, scaled(x), N, Y, N, nrhs, xdig, xexp, g_oz_err, st);
+    dense_matvec_oz(F->dense_op, N, F->row_exp, scaled(x), N, Y, N, nrhs, xdig, xexp, oz_err_word(), st);
     CK(cudaGetLastError());
     return finish();
   };
@@ -2733,26 +2728,28 @@ void factor_group_t(std::vector<pm_factor*>& Fs, double id_tol, Arena& scr, cuda
   factor_tops<C>(Fs, scr, st);
 }
 
+// A wait of the tensor-core products on st ran out (their error word).
+bool oz_wait_ran_out(const int* err, cudaStream_t st) {
+  int werr = 0;
+  CK(cudaMemcpyAsync(&werr, err, sizeof(int), cudaMemcpyDeviceToHost, st));
+  CK(cudaStreamSynchronize(st));
+  return werr != 0;
+}
+const char* const OZ_TIMEOUT = "a wait on the tensor cores ran out";
+
 void factor_group(std::vector<pm_factor*>& Fs, double id_tol, Arena& scr, cudaStream_t st) {
   if (Fs.empty()) return;
   int* err = Fs[0]->d_wait_err;
   OzErrScope oz(err, (Fs[0]->opts.debug_flags & PM_DEBUG_OZ_NO_ARRIVE) != 0);
-  auto wait_ran_out = [&] {
-    int werr = 0;
-    CK(cudaMemcpyAsync(&werr, err, sizeof(int), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    return werr != 0;
-  };
-  const char* const msg = "a wait on the tensor cores ran out";
   try {
     if (Fs[0]->precision == PM_FP64) factor_group_t<double2>(Fs, id_tol, scr, st);
     else factor_group_t<float2>(Fs, id_tol, scr, st);
   } catch (const PmError& e) {
     // products that were not formed can show up as a singular block first
-    if (e.st == PM_ERR_SINGULAR && wait_ran_out()) fail(PM_ERR_TIMEOUT, msg);
+    if (e.st == PM_ERR_SINGULAR && oz_wait_ran_out(err, st)) fail(PM_ERR_TIMEOUT, OZ_TIMEOUT);
     throw;
   }
-  if (wait_ran_out()) fail(PM_ERR_TIMEOUT, msg);
+  if (oz_wait_ran_out(err, st)) fail(PM_ERR_TIMEOUT, OZ_TIMEOUT);
 }
 
 // Mixed mode, after the complex64 levels: the FP64 self blocks, index maps and
@@ -2870,7 +2867,11 @@ void finish_mixed(pm_factor* F) {
     F->self64[j] = F->arena.get<double2>((size_t)m2 * m2);
     incl.push_back(j); lda.push_back(m2); A64.push_back(F->self64[j]);
   }
-  if (!incl.empty()) assemble_self<double2>(g, incl, A64, lda, F->scratch, F->st);
+  if (!incl.empty()) {
+    OzErrScope oz(F->d_wait_err, (F->opts.debug_flags & PM_DEBUG_OZ_NO_ARRIVE) != 0);
+    assemble_self<double2>(g, incl, A64, lda, F->scratch, F->st);
+    if (oz_wait_ran_out(F->d_wait_err, F->st)) fail(PM_ERR_TIMEOUT, OZ_TIMEOUT);
+  }
   if (!F->op_started) start_mixed_operator(F, false);
   if (F->dense64) {
     if (F->op_done) CK(cudaStreamWaitEvent(F->st, F->op_done, 0));
@@ -3311,7 +3312,11 @@ pm_status pm_self_block(const pm_geometry* g, int32_t j, pm_c64* out) {
     cudaStream_t st = 0;
     int n = g->inc[j].n_nodes;
     Cd* d = ws.get<Cd>((size_t)4 * n * n);
+    int* err = ws.get<int>(1);
+    CK(cudaMemsetAsync(err, 0, sizeof(int), st));
+    OzErrScope oz(err);   // the products a factorization forms them with
     assemble_self<Cd>(g, {j}, {d}, {2 * n}, ws, st);
+    if (oz_wait_ran_out(err, st)) fail(PM_ERR_TIMEOUT, OZ_TIMEOUT);
     CK(cudaMemcpy(out, d, sizeof(Cd) * (size_t)4 * n * n, cudaMemcpyDeviceToHost));
   });
 }
