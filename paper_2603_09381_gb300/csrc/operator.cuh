@@ -54,7 +54,7 @@ void dense_matvec64(SplitOp A, int N, const double2* X, int ldx, double2* Y, int
                     cudaStream_t st);
 // The same product with the hi parts in FP32 arithmetic (~1e-7 relative to
 // |A| |X|): the first refinement residual only.  rexp (optional): receives the
-// row exponents of dense_row_exponents on the way.
+// row exponents of dense_row_exponents (without colexp) on the way.
 void dense_matvec32(SplitOp A, int N, const double2* X, int ldx, double2* Y, int ldy, int nrhs, unsigned char* rexp,
                     cudaStream_t st);
 // The product on the tensor cores at FP64 accuracy (oz_matvec.cu): the parts
@@ -62,11 +62,14 @@ void dense_matvec32(SplitOp A, int N, const double2* X, int ldx, double2* Y, int
 // exact products and sums.  rexp: the exponents of every row's largest part in
 // every 128 columns (ceil(N / 128) x N); xdig, xexp: workspace of
 // dense_matvec_oz_bytes(N) bytes and 8 ceil(N / 128) entries; *err is set if a
-// bounded wait runs out.
-void dense_row_exponents(SplitOp A, int N, unsigned char* rexp, cudaStream_t st);
+// bounded wait runs out.  colexp (or null: all zero): exponents, at most zero,
+// that the columns are weighted by before the largest is taken, padded to a
+// multiple of 128.
+void dense_row_exponents(SplitOp A, int N, const signed char* colexp, unsigned char* rexp, cudaStream_t st);
 size_t dense_matvec_oz_bytes(int N);
-void dense_matvec_oz(SplitOp A, int N, const unsigned char* rexp, const double2* X, int ldx, double2* Y, int ldy, int nrhs,
-                     unsigned char* xdig, unsigned short* xexp, int* err, cudaStream_t st);
+void dense_matvec_oz(SplitOp A, int N, const unsigned char* rexp, const signed char* colexp, const double2* X, int ldx,
+                     double2* Y, int ldy, int nrhs, unsigned char* xdig, unsigned short* xexp, int* err,
+                     cudaStream_t st);
 // R = B - Y, and norms2[2 r] += |R[:, r]|^2, norms2[2 r + 1] += |B[:, r]|^2 (norms2 zeroed by caller)
 void residual64(const double2* B, const double2* Y, double2* R, int N, int nrhs, double* norms2, cudaStream_t st);
 // dst[:, r] = scale[r] * src[:, r] (FP64 -> FP32)

@@ -390,6 +390,7 @@ struct pm_factor {
   size_t dense_bytes = 0;
   unsigned char* row_exp = nullptr;   // exponents of its rows per 128 columns (once row_exp_ready; under plan_mu)
   bool row_exp_ready = false;
+  signed char* col_exp = nullptr;     // exponents of its columns' weights, if they differ much (else null)
   // CUDA graphs of the compressed inverse (FP64) or the mixed preconditioner,
   // one per right-hand-side count; solves of one factor are serialised by plan_mu
   std::mutex plan_mu;
@@ -2359,10 +2360,10 @@ void solve_refined(pm_factor* F, const double2* B, int nrhs, double2* X, Arena& 
   };
   auto residual_oz = [&](const double2* x) {
     if (!F->row_exp_ready) {
-      dense_row_exponents(F->dense_op, N, F->row_exp, st);
+      dense_row_exponents(F->dense_op, N, F->col_exp, F->row_exp, st);
       F->row_exp_ready = true;
     }
-    dense_matvec_oz(F->dense_op, N, F->row_exp, scaled(x), N, Y, N, nrhs, xdig, xexp, oz_err_word(), st);
+    dense_matvec_oz(F->dense_op, N, F->row_exp, F->col_exp, scaled(x), N, Y, N, nrhs, xdig, xexp, oz_err_word(), st);
     CK(cudaGetLastError());
     return finish();
   };
@@ -2372,8 +2373,9 @@ void solve_refined(pm_factor* F, const double2* B, int nrhs, double2* X, Arena& 
     return finish();
   };
   auto product32 = [&](const double2* x) {
-    dense_matvec32(F->dense_op, N, scaled(x), N, Y, N, nrhs, F->row_exp_ready ? nullptr : F->row_exp, st);
-    F->row_exp_ready = true;
+    const bool record = !F->row_exp_ready && !F->col_exp;
+    dense_matvec32(F->dense_op, N, scaled(x), N, Y, N, nrhs, record ? F->row_exp : nullptr, st);
+    F->row_exp_ready = F->row_exp_ready || record;
     CK(cudaGetLastError());
   };
   auto residual_f32 = [&](const double2* x) {
@@ -2787,6 +2789,37 @@ double hankel_flops_per_pair(const pm_geometry* g) {
   return sum / n;
 }
 
+// Exponents of the weights that the columns of the stored operator are taken
+// with in its tensor-core product (oz_matvec.cu), relative to the largest; empty
+// if they differ by less than COL_EXP_SPREAD.  An entry of X (column-scaled) has
+// the size of its node's weight times k u, or w q with q of the size of
+// max(k, 1 / radius) u: A's columns times those weights hold the sizes of the
+// terms.  The product is exact to about 2^-49 of the largest weighted part times
+// X's; a spread of the weights comes off that.  With inclusions within a factor of
+// two in size and node spacing it stays below the line, at which the extra
+// millisecond of 24 begins.
+constexpr int COL_EXP_SPREAD = 4;
+std::vector<signed char> column_exponents(const pm_geometry* g) {
+  std::vector<int> e((size_t)g->N);
+  for (int j = 0; j < g->m; ++j) {
+    const int n = g->inc[j].n_nodes, r0 = g->row_off[j];
+    const double* w = &g->hw[g->node_off[j]];
+    double len = 0;
+    for (int l = 0; l < n; ++l) len += w[l];
+    const double kappa = std::max(g->k0, 2 * 3.141592653589793 / len);
+    for (int l = 0; l < n; ++l) {
+      e[r0 + l] = std::ilogb(kappa * w[l]);
+      e[r0 + n + l] = std::ilogb(g->k0 * w[l]);
+    }
+  }
+  const int hi = *std::max_element(e.begin(), e.end()), lo = *std::min_element(e.begin(), e.end());
+  std::vector<signed char> out;
+  if (hi - lo < COL_EXP_SPREAD) return out;
+  out.assign(((size_t)g->N + 127) / 128 * 128, 0);
+  for (size_t i = 0; i < e.size(); ++i) out[i] = (signed char)std::max(e[i] - hi, -64);
+  return out;
+}
+
 // Index maps, column scales and, when it fits, the dense FP64 operator of a
 // mixed factorization (its self blocks are copied in by finish_mixed).
 // beside: the assembly runs on a low-priority stream as the persistent
@@ -2829,6 +2862,8 @@ void start_mixed_operator(pm_factor* F, bool beside) {
   OpNodes nd{g->nodes.x, g->nodes.y, g->nodes.nx, g->nodes.ny, g->nodes.w, g->nodes.incl, F->d_iu, F->d_iq};
   F->d_colscale = F->arena.get<double>((size_t)g->N);
   F->row_exp = F->arena.get<unsigned char>((size_t)((g->N + 127) / 128) * g->N);
+  const std::vector<signed char> ce = column_exponents(g);
+  if (!ce.empty()) F->col_exp = upload(F->arena, ce, F->st);
   dense_colscale(g->nodes.w, F->d_iu, F->d_iq, g->total_nodes, g->k0, F->d_colscale, F->st);
   if (beside) {
     int pr_lo = 0, pr_hi = 0;
