@@ -88,7 +88,10 @@ typedef struct pm_factor pm_factor;
  * proxy_factor: proxy circle radius / cell radius (> 1; default 1.5).
  * proxy_points: points on every proxy circle; 0 selects
  *      p = max(32, 8 ceil((2 k^+ R_p + ceil(ln(1/tol)/ln(proxy_factor)))/8)).
- * precision: PM_FP64 (everything complex128), or PM_MIXED: the levels are
+ * precision: PM_FP64 (everything complex128; where the inclusions' mean radius
+ *      lies outside [2^-4, 2^4), the system is factored with all lengths scaled
+ *      by a power of two, and pm_solve scales the normal derivatives), or
+ *      PM_MIXED: the levels are
  *      factored in complex64 with ID threshold max(tol, low_tol) and serve as a
  *      preconditioner, and pm_solve refines the solution against the
  *      complex128 operator (no counterpart in the paper).  The top-level

@@ -8,6 +8,7 @@
 #include <cstring>
 #include <functional>
 #include <map>
+#include <memory>
 #include <tuple>
 #include <mutex>
 #include <thread>
@@ -317,6 +318,10 @@ struct pm_geometry {
   double ox = 0, oy = 0;
   bool general = false;   // spacing 0: an arbitrary arrangement, cells of the centres' bounding square
   std::vector<std::vector<Box>> levels;  // levels[l], l = 0..L
+  // the same scatterers with all lengths times `unit`, a power of two (see
+  // length_unit), where the unit of length is far from the inclusions' size
+  std::unique_ptr<pm_geometry> scaled;
+  double unit = 1;
 
   // global index -> packed point code (node * 2 + group)
   int code_of(int g) const {
@@ -398,6 +403,7 @@ struct pm_factor {
   int graph_launches = 0, graph_captures = 0;
   // set by a bounded wait of the chained top-level solve that ran out (checked after every solve)
   int* d_wait_err = nullptr;
+  double unit = 1;              // g is the caller's geometry with its lengths times unit
   ~pm_factor();
 };
 
@@ -2549,6 +2555,19 @@ __global__ void k_bm_order(const InclDev* __restrict__ inc, const int* __restric
   phi[o + d.n + l] = x[o + l];
 }
 
+// dst = src with the first (f1) and second (f2) halves of every inclusion's entries scaled.
+__global__ void k_scale_halves(const InclDev* __restrict__ inc, const int* __restrict__ incl, int total,
+                               const double2* src, double2* dst, int N, int nrhs, double f1, double f2) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= total) return;
+  const InclDev d = inc[incl[q]];
+  for (int c = blockIdx.y; c < nrhs; c += gridDim.y) {
+    const size_t o = (size_t)c * N + d.row_off + (q - d.node_off);
+    dst[o] = f1 * src[o];
+    dst[o + d.n] = f2 * src[o + d.n];
+  }
+}
+
 // Sets *flag when any of the n doubles at x is NaN or infinite.
 __global__ void k_flag_nonfinite(const double* __restrict__ x, size_t n, int* flag) {
   int bad = 0;
@@ -2608,6 +2627,9 @@ double setup_factor(pm_factor* F, const pm_geometry* g, const pm_factor_opts* op
       if (c.k_in.im != 0 || c.k_in.re != g->inc[0].k_in.re)
         fail(PM_ERR_UNSUPPORTED, "PMCHWT (All) and Burton-Miller need one real interior wavenumber for all inclusions");
   }
+  const bool rescaled = g->scaled && opts->precision == PM_FP64;
+  if (rescaled) F->unit = g->unit;
+  if (rescaled) g = g->scaled.get();
   F->g = g;
   F->opts = *opts;
   if (F->opts.proxy_factor == 0) F->opts.proxy_factor = 1.5;
@@ -2919,6 +2941,84 @@ void finish_mixed(pm_factor* F) {
   }
 }
 
+// Nodes, device arrays and tree of a checked problem.
+void fill_geometry(pm_geometry* g, const pm_problem* prob) {
+  CK(cudaGetDevice(&g->device));
+  g->m = prob->m; g->k0 = prob->k_out; g->spacing = prob->spacing;
+  g->general = prob->spacing == 0;
+  g->gnx = prob->grid_nx; g->gny = prob->grid_ny;
+  g->inc.assign(prob->inc, prob->inc + prob->m);
+  g->node_off.assign(g->m + 1, 0); g->row_off.assign(g->m + 1, 0);
+  for (int j = 0; j < g->m; ++j) {
+    g->node_off[j + 1] = g->node_off[j] + g->inc[j].n_nodes;
+    g->row_off[j + 1] = 2 * g->node_off[j + 1];
+    g->maxn = std::max(g->maxn, g->inc[j].n_nodes);
+  }
+  g->total_nodes = g->node_off[g->m];
+  g->N = 2 * g->total_nodes;
+  upload_inclusions(g);
+  cudaStream_t st = 0;
+  g->d_inc = upload(g->arena, g->hinc, st);
+  const size_t T = g->total_nodes;
+  NodesDev& nd = g->nodes;
+  nd.x = g->arena.get<double>(T); nd.y = g->arena.get<double>(T); nd.nx = g->arena.get<double>(T);
+  nd.ny = g->arena.get<double>(T); nd.speed = g->arena.get<double>(T); nd.w = g->arena.get<double>(T);
+  nd.curv = g->arena.get<double>(T); nd.kress = g->arena.get<double>(T);
+  std::vector<int> incl(T);
+  for (int j = 0; j < g->m; ++j) for (int q = g->node_off[j]; q < g->node_off[j + 1]; ++q) incl[q] = j;
+  nd.incl = upload(g->arena, incl, st);
+  geom_nodes(g->d_inc, nd, (int)T, g->hinc.data(), st);
+  CK(cudaGetLastError());
+  g->hx.resize(T); g->hy.resize(T); g->hnx.resize(T); g->hny.resize(T); g->hw.resize(T);
+  CK(cudaMemcpy(g->hx.data(), nd.x, T * 8, cudaMemcpyDeviceToHost));
+  CK(cudaMemcpy(g->hy.data(), nd.y, T * 8, cudaMemcpyDeviceToHost));
+  CK(cudaMemcpy(g->hnx.data(), nd.nx, T * 8, cudaMemcpyDeviceToHost));
+  CK(cudaMemcpy(g->hny.data(), nd.ny, T * 8, cudaMemcpyDeviceToHost));
+  CK(cudaMemcpy(g->hw.data(), nd.w, T * 8, cudaMemcpyDeviceToHost));
+  build_tree(g, nullptr);
+}
+
+// A power of two that brings the inclusions' mean radius (perimeter / 2 pi) into
+// [1/4, 1/2), for FP64 factorizations; 1 while it lies in [2^-4, 2^4).  In
+// another unit of length u and q, hence the rows and columns of the two
+// equations and unknowns, differ in size by as much, and
+//  - digits relative to the largest part of a row and a column (oz.cuh) lose
+//    what large entries that meet only small ones take up, wherever the 32 terms
+//    of a stage hold both kinds;
+//  - the IDs, accurate relative to a whole column, lose the smaller kind.
+// 3 x 3 stars of 90 nodes, tol 1e-12, error at radius 0.4, 4e-4, 4e-7, 400:
+// 2e-12, 1e-9, 7e-7, 1e-10 with FP64 products; 2e-12, 7e-8, 5e-2, 1e-10 with the
+// digits; scaled 2e-12, 2e-12, 1e-11, 2e-12.  Between radius 0.04 and 4 nothing differs.
+double length_unit(const pm_geometry* g) {
+  double len = 0;
+  for (double w : g->hw) len += w;
+  const double radius = len / (2 * 3.141592653589793 * g->m);
+  if (!std::isnormal(radius)) return 1;
+  const int e = std::ilogb(radius);
+  return e >= -4 && e < 4 ? 1.0 : std::ldexp(1.0, -2 - e);
+}
+
+// The problem with all lengths times unit; false where a number leaves FP64's range.
+bool scale_problem(const pm_problem* prob, double unit, std::vector<pm_inclusion>& inc, pm_problem& out) {
+  inc.assign(prob->inc, prob->inc + prob->m);
+  out = *prob;
+  out.inc = inc.data();
+  out.k_out /= unit;
+  out.spacing *= unit;
+  bool ok = std::isnormal(out.k_out) && std::isfinite(out.spacing);
+  for (pm_inclusion& c : inc) {
+    c.cx *= unit;
+    c.cy *= unit;
+    c.prm[0] *= unit;
+    if (c.shape == PM_ELLIPSE) c.prm[1] *= unit;
+    c.k_in.re /= unit;
+    c.k_in.im /= unit;
+    ok = ok && std::isfinite(c.cx) && std::isfinite(c.cy) && std::isnormal(c.prm[0]) && std::isnormal(c.k_in.re) &&
+         std::isfinite(c.k_in.im);
+  }
+  return ok;
+}
+
 }  // namespace
 
 extern "C" {
@@ -2952,39 +3052,16 @@ pm_status pm_build_geometry(const pm_problem* prob, pm_geometry** out) {
     }
     check_device();
     g = new pm_geometry();
-    CK(cudaGetDevice(&g->device));
-    g->m = prob->m; g->k0 = prob->k_out; g->spacing = prob->spacing;
-    g->general = prob->spacing == 0;
-    g->gnx = prob->grid_nx; g->gny = prob->grid_ny;
-    g->inc.assign(prob->inc, prob->inc + prob->m);
-    g->node_off.assign(g->m + 1, 0); g->row_off.assign(g->m + 1, 0);
-    for (int j = 0; j < g->m; ++j) {
-      g->node_off[j + 1] = g->node_off[j] + g->inc[j].n_nodes;
-      g->row_off[j + 1] = 2 * g->node_off[j + 1];
-      g->maxn = std::max(g->maxn, g->inc[j].n_nodes);
+    fill_geometry(g, prob);
+    g->unit = length_unit(g);
+    if (g->unit != 1) {
+      std::vector<pm_inclusion> inc;
+      pm_problem sp;
+      if (scale_problem(prob, g->unit, inc, sp)) {
+        g->scaled.reset(new pm_geometry());
+        fill_geometry(g->scaled.get(), &sp);
+      }
     }
-    g->total_nodes = g->node_off[g->m];
-    g->N = 2 * g->total_nodes;
-    upload_inclusions(g);
-    cudaStream_t st = 0;
-    g->d_inc = upload(g->arena, g->hinc, st);
-    const size_t T = g->total_nodes;
-    NodesDev& nd = g->nodes;
-    nd.x = g->arena.get<double>(T); nd.y = g->arena.get<double>(T); nd.nx = g->arena.get<double>(T);
-    nd.ny = g->arena.get<double>(T); nd.speed = g->arena.get<double>(T); nd.w = g->arena.get<double>(T);
-    nd.curv = g->arena.get<double>(T); nd.kress = g->arena.get<double>(T);
-    std::vector<int> incl(T);
-    for (int j = 0; j < g->m; ++j) for (int q = g->node_off[j]; q < g->node_off[j + 1]; ++q) incl[q] = j;
-    nd.incl = upload(g->arena, incl, st);
-    geom_nodes(g->d_inc, nd, (int)T, g->hinc.data(), st);
-    CK(cudaGetLastError());
-    g->hx.resize(T); g->hy.resize(T); g->hnx.resize(T); g->hny.resize(T); g->hw.resize(T);
-    CK(cudaMemcpy(g->hx.data(), nd.x, T * 8, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(g->hy.data(), nd.y, T * 8, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(g->hnx.data(), nd.nx, T * 8, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(g->hny.data(), nd.ny, T * 8, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(g->hw.data(), nd.w, T * 8, cudaMemcpyDeviceToHost));
-    build_tree(g, nullptr);
   });
   if (s != PM_OK) { delete g; return s; }
   *out = g;
@@ -3093,9 +3170,19 @@ pm_status solve_impl(const pm_factor* Fc, const pm_c64* rhs, int32_t nrhs, pm_c6
     } scope(F->profiling ? &F->prof : nullptr);
     std::lock_guard<std::mutex> plan_lock(F->plan_mu);   // solves of one factor share its graphs
     OzErrScope oz(F->d_wait_err, (F->opts.debug_flags & PM_DEBUG_OZ_SOLVE_NO_ARRIVE) != 0);
+    // normal derivatives (the q-equation rows and the unknowns q) in the factored geometry's unit of length
+    const pm_geometry* g = F->g;
+    const dim3 halves((g->total_nodes + 255) / 256, std::min(nrhs, 65535));
+    if (F->unit != 1) {
+      Cd* b = ws.get<Cd>((size_t)g->N * nrhs);
+      k_scale_halves<<<halves, 256, 0, st>>>(g->d_inc, g->nodes.incl, g->total_nodes, drhs, b, g->N, nrhs, 1.0,
+                                             1.0 / F->unit);
+      pm_launch_count_add(1);
+      CK(cudaGetLastError());
+      drhs = b;
+    }
     if (F->precision == PM_FP64 && F->opts.formulation >= PM_FORM_BM) {
       // Burton-Miller: its own right-hand side, then its [u; q] unknowns reordered
-      const pm_geometry* g = F->g;
       Cd* b = ws.get<Cd>((size_t)g->N * nrhs);
       Cd* x = ws.get<Cd>((size_t)g->N * nrhs);
       const dim3 grid((g->total_nodes + 255) / 256, nrhs);
@@ -3110,6 +3197,12 @@ pm_status solve_impl(const pm_factor* Fc, const pm_c64* rhs, int32_t nrhs, pm_c6
       run_planned(F, 0, drhs, nrhs, dphi, nullptr, st);
     } else {
       solve_refined(F, drhs, nrhs, dphi, ws, st, info);
+    }
+    if (F->unit != 1) {
+      k_scale_halves<<<halves, 256, 0, st>>>(g->d_inc, g->nodes.incl, g->total_nodes, dphi, dphi, g->N, nrhs, F->unit,
+                                             1.0);
+      pm_launch_count_add(1);
+      CK(cudaGetLastError());
     }
     if (!on_device) CK(cudaMemcpyAsync(phi, dphi, bytes, cudaMemcpyDeviceToHost, st));
     int werr = 0;
