@@ -239,10 +239,12 @@ def _pipe_busy_for(kernel):
     return ent.get("pipe_busy") if ent else None
 
 
-FLOP_KERNELS = {"cpqr_step", "lu_update", "lu_panel", "lu_swap_trsm", "getrs", "gemm_batched", "interp_solve",
+FLOP_KERNELS = {"lu_panel", "lu_swap_trsm", "getrs", "gemm_batched", "gemv_batched", "interp_solve",
                 "apply_offdiag64", "dense_matvec64", "dense_offdiag64"}        # FP64 flops
+OZ_FLOP_KERNELS = {"lu_update", "gemm_oz", "qr_update_oz"}     # FP64 flops as 36 fp16 products on the tensor cores
+INT_FLOP_KERNELS = {"cpqr_step"}     # FP64 flops in 60-bit integers (12 wide multiplications a complex multiply-add)
 FP32_FLOP_KERNELS = {"lu_update32", "lu_panel32", "lu_swap_trsm32", "getrs32", "gemm_batched32", "interp_solve32",
-                     "qr_update32", "qr_update_tc32", "tc_gemm32"}
+                     "qr_update32", "qr_update_tc32", "tc_gemm32", "gemv_batched32"}
 BYTE_KERNELS = {"cpqr_step32"}     # memory-bound FP32 CPQR: algorithmic bytes
 
 
@@ -302,7 +304,7 @@ def _kernel_table(prof_tot, steps):
     out = {}
     for k, v in sorted(prof_tot.items(), key=lambda kv: -kv[1]["ms"]):
         e = {"launches": v["launches"] // steps, "ms": round(v["ms"] / steps, 3)}
-        if v["ms"] > 0 and (k in FLOP_KERNELS or k in FP32_FLOP_KERNELS):
+        if v["ms"] > 0 and k in FLOP_KERNELS | OZ_FLOP_KERNELS | INT_FLOP_KERNELS | FP32_FLOP_KERNELS:
             e["tflops"] = round(v["work"] / (v["ms"] / 1e3) / 1e12, 4)
         if v["ms"] > 0 and k in BYTE_KERNELS:
             e["gbs"] = round(v["work"] / (v["ms"] / 1e3) / 1e9, 1)
@@ -347,6 +349,17 @@ def _alu_peak(kind, peaks):
         (FP32_DERIVED_TFLOPS, "FP32 FMA: 152 SMs x 128 lanes x 2 flops x 2.07 GHz")
 
 
+def _oz_peak():
+    """FP64-accurate products on the tensor cores: 36 exact fp16 products each."""
+    try:
+        d = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))
+        return float(d["bf16_tflops"]) / 36, "measured 16-bit tensor rate (MEASURED_PEAKS.json) / 36 digit products"
+    except (OSError, ValueError, KeyError):
+        return 1900.0 / 36, "fallback (recipe) 16-bit tensor rate / 36 digit products"
+
+
+INT_DERIVED_TFLOPS = 152 * 64 * 2.07e9 * 8 / 12 / 1e12   # 8 flops by 12 of 64 wide multiplications a clock and SM
+
 # Kernels whose event time is not on the step's critical path.
 ROOFLINE_NOTES = {
     "dense_offdiag64": "in the mixed factorization the operator is assembled beside the complex64 levels on a "
@@ -373,6 +386,12 @@ def _roofline(prof_tot, steps, peaks=None):
         peak, src = _alu_peak("fp32", peaks)
         roof.update({"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                      "frac": achieved / peak, "peak_source": src, "traffic": _traffic_for(name)})
+    elif name in OZ_FLOP_KERNELS | INT_FLOP_KERNELS and d["ms"] > 0:
+        achieved = d["work"] / (d["ms"] / 1e3) / 1e12
+        peak, src = _oz_peak() if name in OZ_FLOP_KERNELS else (
+            INT_DERIVED_TFLOPS, "integer multipliers: 152 SMs x 64 a clock x 2.07 GHz, 12 a complex multiply-add")
+        roof.update({"bound": "tensor" if name in OZ_FLOP_KERNELS else "alu", "achieved": achieved, "peak": peak,
+                     "unit": "TFLOP/s", "frac": achieved / peak, "peak_source": src, "traffic": _traffic_for(name)})
     elif name in BYTE_KERNELS and d["ms"] > 0:
         peak, src = _peaks()
         achieved = d["work"] / (d["ms"] / 1e3) / 1e9

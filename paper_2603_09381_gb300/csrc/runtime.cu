@@ -667,6 +667,11 @@ void assemble_self(const pm_geometry* g, const std::vector<int>& incl, const std
   };
   run(d1, off1);
   run(d2, off2);
+  if (oz && g_kprof) {
+    double f = 0;
+    for (auto& c : sub) f += 16.0 * c.n * c.n * (double)c.n;
+    g_kprof->add_flops("gemm_oz", f);
+  }
   CK(cudaGetLastError());
 }
 
@@ -1136,8 +1141,8 @@ void sqnorm_batch(const std::vector<SqNormProb>& probs, Arena& scr, cudaStream_t
 // waves of the SMs.  None at all: two disks 6.05 -> 6.59 ms and 4 x 4 stars
 // 58.6 -> 59.9 in complex128; lossy disks 5.0 -> 5.6, 8 x 8 stars 66.7 -> 70.2
 // and a batch of ellipses 83.3 -> 88.9 in the mixed mode.  Between 2 and 64
-// waves nothing differs by more than 1% there; beyond, a CTA's serial steps
-// would queue behind one another.
+// waves nothing differs by more than 1% there; the lines are put near the low
+// end of that range, as a CTA's serial steps queue behind one another in later waves.
 constexpr int RESIDENT_WAVES_64 = 4, RESIDENT_WAVES_32 = 8;
 // complex128 ID inputs with at least this many candidates (and twice as many
 // rows) are reduced to their triangle first.  From 64: two disks 6.05 -> 6.37
@@ -1610,10 +1615,11 @@ void process_levels(const std::vector<LevelJob>& jobs, Arena& scr, cudaStream_t 
     }
   }
   // The phase of the resident matrices that have steps to do, from the next
-  // point of st on: one launch per cluster size, each on a stream of its own,
-  // beside one another and beside the steps of the other matrices (each alone
-  // fills a part of the SMs); st waits for them at fork.join().  One after the
-  // other: batch of ellipses 90.7 ms, now 85.3; Burton-Miller 76.4, now 73.7.
+  // point of st on: one launch per cluster size, each on a stream of its own
+  // beside the steps of the other matrices (each alone fills a part of the SMs);
+  // st waits for them at fork.join().  Without other matrices the first group
+  // runs on st, and the others, forked after it, wait for it.  All one after
+  // the other: batch of ellipses 90.7 ms, now 85.3; Burton-Miller 76.4, now 73.7.
   SideStreams fork;
   auto run_resident = [&](const CpqrProb<C>* d, bool beside) {
     struct Group { int cs; const int* list; std::vector<int> n, w; };
@@ -2322,7 +2328,7 @@ void apply_operator64(pm_factor* F, const double2* X, int nrhs, double2* Y, Aren
     // complex multiply-adds); special functions not counted
     double pairs = (double)g->total_nodes * g->total_nodes;
     for (int j = 0; j < g->m; ++j) pairs -= (double)g->inc[j].n_nodes * g->inc[j].n_nodes;
-    g_kprof->add_flops("apply_offdiag64", pairs * (47.0 + hankel_flops_per_pair(g) + 32.0 * nrhs));
+    g_kprof->add_flops("apply_offdiag64", pairs * (59.0 + hankel_flops_per_pair(g) + 32.0 * nrhs));
   }
   CK(cudaGetLastError());
 }
@@ -2776,15 +2782,12 @@ void factor_group(std::vector<pm_factor*>& Fs, double id_tol, Arena& scr, cudaSt
   if (oz_wait_ran_out(err, st)) fail(PM_ERR_TIMEOUT, OZ_TIMEOUT);
 }
 
-// Mixed mode, after the complex64 levels: the FP64 self blocks, index maps and
-// (when it fits) the dense FP64 operator of the refinement residual.
-// Average algorithmic FP64 flops of one Hankel pair (H0, H1) over the node
-// pairs of a geometry (the square root, reciprocal square root, sincos and,
-// below z = 8, CUDA's Bessel functions not counted): 64 for the 12-term
-// expansion (z >= 60), 28 + 8 d for a degree-d fit (d = 5 on [20, 60), 7 on
-// [12, 20), 8 on [8, 12)), none below 8; averaged over 65,536 pairs of
-// nodes of different inclusions drawn with a fixed seed.  Used for the
-// profiler's counts of the operator kernels.
+// Average FP64 operations of one Hankel pair (H0, H1) over the node pairs of a
+// geometry: for z >= 8 18 (one reciprocal square root, 1/z, the polynomials'
+// variable and the scaling; the rest runs in integers), below that CUDA's Bessel
+// functions, not counted; averaged over 65,536 pairs of nodes of different
+// inclusions drawn with a fixed seed.  Used for the profiler's counts of the
+// operator kernels.
 double hankel_flops_per_pair(const pm_geometry* g) {
   const int T = g->total_nodes;
   if (T < 2 || g->m < 2) return 0.0;
@@ -2802,10 +2805,7 @@ double hankel_flops_per_pair(const pm_geometry* g) {
     const int t = next(), q = next();
     if (incl_of(t) == incl_of(q)) continue;
     const double z = g->k0 * std::hypot(g->hx[t] - g->hx[q], g->hy[t] - g->hy[q]);
-    if (z >= 60) sum += 64;
-    else if (z >= 20) sum += 28 + 8 * 5;
-    else if (z >= 12) sum += 28 + 8 * 7;
-    else if (z >= 8) sum += 28 + 8 * 8;
+    if (z >= 8) sum += 18;
     ++n;
   }
   return sum / n;
@@ -2903,13 +2903,15 @@ void start_mixed_operator(pm_factor* F, bool beside) {
   if (g_kprof) {
     double pairs = (double)g->total_nodes * g->total_nodes;
     for (int j = 0; j < g->m; ++j) pairs -= (double)g->inc[j].n_nodes * g->inc[j].n_nodes;
-    // per unordered pair: 40 for the geometry and the eight entries of both
-    // 2 x 2 blocks, plus the Hankel pair
-    g_kprof->add_flops("dense_offdiag64", 0.5 * pairs * (40.0 + hankel_flops_per_pair(g)));
+    // per unordered pair: 52 for the geometry (the distance's root included) and the
+    // eight entries of both 2 x 2 blocks, plus the Hankel pair
+    g_kprof->add_flops("dense_offdiag64", 0.5 * pairs * (52.0 + hankel_flops_per_pair(g)));
   }
   CK(cudaGetLastError());
 }
 
+// Mixed mode, after the complex64 levels: the FP64 self blocks, index maps and
+// (when it fits) the dense FP64 operator of the refinement residual.
 void finish_mixed(pm_factor* F) {
   const pm_geometry* g = F->g;
   // FP64 self blocks and index maps for the refinement residual
