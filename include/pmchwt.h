@@ -111,9 +111,11 @@ typedef struct pm_factor pm_factor;
  *      that each refinement step is one matrix product (else, or with
  *      PM_FLAG_NO_DENSE_OPERATOR, the operator is applied on the fly).  PM_MIXED reduces every complex64 ID
  *      input with at least twice as many rows as candidate columns to its
- *      triangular factor (unpivoted Householder QR) before the pivoted QR;
- *      PM_FLAG_NO_QR_FIRST pivots on the full input instead.  Each trailing
- *      update of that QR, Q^H C = C - V (T^H (V^H C)), forms V^H C per block
+ *      triangular factor (unpivoted Householder QR) before the pivoted QR, and
+ *      PM_FP64 every complex128 one that has 80 candidates and more besides;
+ *      PM_FLAG_NO_QR_FIRST pivots on the full input instead.  In PM_FP64 the
+ *      trailing updates run on the tensor cores at FP64 accuracy.  Each trailing
+ *      update of the complex64 QR, Q^H C = C - V (T^H (V^H C)), forms V^H C per block
  *      of 256 rows on the FP32 CUDA cores, sums the blocks in a fixed order,
  *      and applies C -= V Y on the tensor cores (3xTF32, FP32 accuracy; a
  *      64-term real accumulation per tile); PM_FLAG_QR_CUDA_CORES applies it
@@ -124,10 +126,11 @@ typedef struct pm_factor pm_factor;
  *      Confirming residual (PM_MIXED with the dense operator): by default the
  *      residual that ends the refinement comes from a product of the stored
  *      operator on the tensor cores (digits of fp16, sums exact within 128 or
- *      512 columns; error ~1e-15 of sum_j |a_ij| |x_j| per row, below that of
- *      a sequential FP64 sum); PM_FLAG_FP64_CONFIRM forms it with the FP64
- *      product instead.  PM_FLAG_FF_CONFIRM names the default and changes
- *      nothing.  PM_FLAG_NO_AUTOTUNE: the call tunes no batched-GEMM tile
+ *      512 columns; each real term is off by at most 2^-49 of the largest
+ *      |a_ij| times the largest |x_j| among them, both weighted by the columns'
+ *      scales where those differ by 16 and more); PM_FLAG_FP64_CONFIRM forms it
+ *      with the FP64 product instead.  PM_FLAG_FF_CONFIRM names the default and
+ *      changes nothing.  PM_FLAG_NO_AUTOTUNE: the call tunes no batched-GEMM tile
  *      shape (classes tuned before keep their choice; see pm_autotune_table).
  *      Solve graphs: the compressed inverse (PM_FP64) and the mixed
  *      preconditioner are launch sequences fixed by the factorization; the
@@ -291,7 +294,8 @@ pm_status pm_plane_wave_rhs(const pm_geometry* g, const double* angles, int32_t 
  * (paper Sec. 3): self blocks, proxy IDs per cell (exterior kernel only),
  * compressed blocks A~_i = (R_i A_ii^{-1} L_i)^{-1}, recursive merge, top LU.
  * Errors: PM_ERR_INVALID_ARG, PM_ERR_OOM, PM_ERR_CUDA, PM_ERR_SINGULAR,
- * PM_ERR_TIMEOUT (opt-in tensor-core path only), PM_ERR_UNSUPPORTED. */
+ * PM_ERR_TIMEOUT (a bounded wait on the tensor cores ran out),
+ * PM_ERR_UNSUPPORTED. */
 pm_status pm_factorize(const pm_geometry* g, const pm_factor_opts* opts, pm_factor** out);
 
 /* Solve A phi = rhs for nrhs right-hand sides (paper Sec. 3: eq. compressed and
@@ -301,9 +305,10 @@ pm_status pm_factorize(const pm_geometry* g, const pm_factor_opts* opts, pm_fact
  * pointers; they may alias.  A right-hand side with a NaN or infinite entry
  * -> PM_ERR_INVALID_ARG, phi untouched.  PM_MIXED factors refine the
  * solution (PM_ERR_NOT_CONVERGED if refine_tol is not reached).  With at
- * most 8 right-hand sides the top-level triangular solves run as one chained
- * launch per triangle whose cross-block waits are bounded: PM_ERR_TIMEOUT if
- * one ran out (phi then invalid; the factor stays usable). */
+ * most 64 right-hand sides the triangular solves run as one chained launch per
+ * triangle whose cross-block waits are bounded, as are those on the tensor
+ * cores: PM_ERR_TIMEOUT if one ran out (phi then invalid; the factor stays
+ * usable). */
 pm_status pm_solve(const pm_factor* f, const pm_c64* rhs, int32_t nrhs, pm_c64* phi, int32_t on_device);
 
 /* pm_solve that also reports the refinement outcome (info may be NULL). */
@@ -375,8 +380,9 @@ pm_status pm_scattered_field(const pm_geometry* g, const pm_c64* phi, int32_t nr
  * (no counterpart in the paper; measurement aid).  CUDA events bracket every
  * launch on the factorization's stream.  `work` is the algorithmic work of
  * all launches: real flops for cpqr_step, interp_solve, lu_*, getrs,
- * gemm_batched, qr_update32, dense_matvec64 and dense_offdiag64 (164 per node
- * pair); bytes for cpqr_step32 (one read and write of every trailing entry);
+ * gemm_batched, gemm_oz, gemv_batched, qr_update_oz, qr_update32,
+ * dense_matvec64 and dense_offdiag64 (its operations on the FP64 pipe, 52 to 70
+ * an unordered node pair); bytes for cpqr_step32 (one read and write of every trailing entry);
  * matrix entries for gather_entries; node pairs for self_pointwise.  Names
  * ending in 32 are the complex64 instances.  Writes up to cap entries, *count = number available. */
 typedef struct {

@@ -1,9 +1,10 @@
 // Batched complex GEMM / LU / LU-solve kernels.
 //
-// On GB300 the FP64 pipe (about 1.2 TFLOP/s) is the bound for all of these:
-// even a rank-1 update streamed from HBM needs only ~0.25 flop/byte, above
-// the chip's FP64:HBM balance (~0.18).  The kernels therefore favour simple
-// shared-memory tiling with enough resident warps to keep the DFMA pipe busy.
+// complex128 products and trailing updates run on the tensor cores (oz_gemm.cuh);
+// what is left to the FP64 pipe here (about 1.2 TFLOP/s: even a rank-1 update
+// streamed from HBM is bound by it) are panels, diagonal blocks, chained solves
+// and products of a few rows, columns or terms.  complex64 updates and products
+// run on the FP32 pipe, in shared-memory tiles.
 #include "dense_la.cuh"
 #include "oz_gemm.cuh"
 #include "prof.cuh"

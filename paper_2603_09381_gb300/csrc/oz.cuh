@@ -16,7 +16,11 @@
 // eight balanced base-256 digits, exact in fp16.  The products of digits i
 // and j of equal i + j = s <= 7 add up in one FP32 accumulator: at most
 // 64 x 8 products of at most 2^14, 2^23, hence exact.  What is left out
-// (s > 7) is below 2^-60 of the two maxima's product.  The eight sums are
+// (s > 7) is below 2^-57 of the product of the two maxima per real term: the
+// error is relative to those, not to each term, so that a row and a column
+// graded in opposite directions lose what their large parts do not share (the
+// callers' matrices are kept from that by their unit of length, length_unit in
+// runtime.cu).  The eight sums are
 // joined in a 75-bit integer, rounded once to a double and added in FP64.  A
 // stage's result depends only on its row of A and its column of B, so the
 // tiling changes no bit.
@@ -29,9 +33,11 @@
 // themselves.  K-major, no swizzle: the core matrices are written by
 // conflict-free 16-byte stores.  195 KB of shared memory: one CTA per SM.
 //
-// What bounds a stage is the issue of its integer instructions (44,000 a CTA
-// with the tensor pipe 12-18% busy before the join went to 32-bit words and two
-// digits to one permutation: 8 x 8 stars 336 -> 320 ms).
+// What bounds a stage is that its phases (load, cut, MMAs, join) come one after
+// the other on 16 warps an SM, behind barriers: ALU pipe 37-40% busy, FP64 15-23%,
+// tensor 16-18%, 32% of the issue slots.  The integer instructions are its largest
+// part: the join in 32-bit words and two digits to one permutation took 8 x 8 stars
+// from 336 to 320 ms.
 #pragma once
 #include "pm_common.cuh"
 #include "tc_common.cuh"

@@ -3,13 +3,14 @@
 // refinement.  The float-float products this replaces issued 12 FP32
 // operations per real multiply-add (58 ms at N = 65,536, 70 ms with their sums
 // folded into FP64); here an entry costs its cut into digits once, for all
-// columns of X.  The cut's integer instructions bound the kernel (28 ms at N =
-// 65,536, 24 ms since hi and lo are cut together and two digits share a
-// permutation); the read of the operator would take 10 ms.
+// columns of X.  The cut's integer instructions bound the kernel (ALU pipe 69% busy;
+// 28 ms at N = 65,536, 24 ms since hi and lo are cut together and two digits share
+// a permutation); the read of the operator would take 10 ms.
 //
 // Digits as in oz.cuh, seven per number: relative to the largest part of its
 // row within a fold of 128 or 512 columns (of X: of its column), each real is a
-// 54-bit integer.  Seven accumulators, one per digit i of A, take A_i times
+// 54-bit integer (both parts of an entry cut off).  What is left out (i + j > 6) is
+// below 2^-49 of the product of the two maxima per real term.  Seven accumulators, one per digit i of A, take A_i times
 // the digits 0 .. 6-i of X side by side (16 (7 - i) columns of TMEM each, 448 in
 // all), so A_i is read once; a fold's sums stay below 2^24 and are exact.  At
 // the end of a fold they are joined in integers and added in FP64.

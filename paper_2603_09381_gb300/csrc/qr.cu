@@ -364,7 +364,7 @@ __global__ void __maxnreg__(112) k_qr_panel(const QrProb<float2>* __restrict__ P
 //             far below its scale, and the reflector must be orthogonal to
 //             working precision, so each warp shifts its rows of y up to use
 //             all bits before the dot products; the shifts are taken out when
-//             the warps' sums meet in FP64.
+//             the warps' sums meet, in integers as well.
 // (fx.cuh holds the arithmetic.)
 // A matrix's panel on a cluster; rows go to warps 8 at a time and stay there
 // for the whole panel.  T receives the taus.  Same reflectors and order as
