@@ -42,44 +42,54 @@ __device__ __forceinline__ void qu_of(const InclDev* inc, const int* incl, const
 // an FMA into the running sum rounds at the sum's size, several times a node
 // (16,384 nodes, far field: rms error 3.33e-17 straight into the running sums,
 // 2.99e-17 with each node's finished term added, 2.13e-17 with runs of 8, which take
-// 2% of the case above).
+// 2% of the case above).  With one run a thread (LONG false, up to RUN * FT nodes)
+// the run is the total: the same bits without the totals, whose registers leave
+// three CTAs an SM for four (1,720 nodes, 6 right-hand sides, 600 points and 232
+// directions: 864 us with totals, 811 without).
 constexpr int RUN = 8;
-template <int NR>
+template <int NR, bool LONG>
 struct RunSums {
   double2 acc[NR];
   double2 (*tot)[FT];
   int nodes = 0;
   __device__ __forceinline__ explicit RunSums(double2 (*t)[FT]) : tot(t) {
 #pragma unroll
-    for (int c = 0; c < NR; ++c) acc[c] = tot[c][threadIdx.x] = make_double2(0, 0);
+    for (int c = 0; c < NR; ++c) {
+      acc[c] = make_double2(0, 0);
+      if constexpr (LONG) tot[c][threadIdx.x] = make_double2(0, 0);
+    }
   }
   __device__ __forceinline__ void flush() {
+    if constexpr (LONG) {
 #pragma unroll
-    for (int c = 0; c < NR; ++c) {
-      double2 t = tot[c][threadIdx.x];
-      t.x += acc[c].x;
-      t.y += acc[c].y;
-      tot[c][threadIdx.x] = t;
-      acc[c] = make_double2(0, 0);
+      for (int c = 0; c < NR; ++c) {
+        double2 t = tot[c][threadIdx.x];
+        t.x += acc[c].x;
+        t.y += acc[c].y;
+        tot[c][threadIdx.x] = t;
+        acc[c] = make_double2(0, 0);
+      }
     }
   }
   __device__ __forceinline__ void next() {
-    if ((++nodes & (RUN - 1)) == 0) flush();
+    if constexpr (LONG)
+      if ((++nodes & (RUN - 1)) == 0) flush();
   }
   __device__ __forceinline__ double2 total(int c) const {   // (after the last flush)
-    return tot[c][threadIdx.x];
+    if constexpr (LONG) return tot[c][threadIdx.x];
+    else return acc[c];
   }
 };
 
-template <int NR>
+template <int NR, bool LONG>
 __global__ void __launch_bounds__(FT) k_far_field(const InclDev* __restrict__ inc, NodesDev nd, int total, double k,
                                                   const double2* __restrict__ phi, int ldphi,
                                                   const double* __restrict__ ang, int ndir, double2* out) {
-  __shared__ double2 sh[FT / 32], tot[NR][FT];
+  __shared__ double2 sh[FT / 32], tot[LONG ? NR : 1][FT];
   const int dir = blockIdx.x;
   double sa, ca;
   sincos(ang[dir], &sa, &ca);
-  RunSums<NR> sum(tot);
+  RunSums<NR, LONG> sum(tot);
   for (int i = threadIdx.x; i < total; i += FT) {
     double s, co;
     sincos(-k * fma(ca, nd.x[i], sa * nd.y[i]), &s, &co);     // e^{-i k xhat.y}
@@ -112,14 +122,14 @@ __global__ void __launch_bounds__(FT) k_far_field(const InclDev* __restrict__ in
   }
 }
 
-template <int NR>
+template <int NR, bool LONG>
 __global__ void __launch_bounds__(FT) k_scattered(const InclDev* __restrict__ inc, NodesDev nd, int total, double k,
                                                   const double2* __restrict__ phi, int ldphi,
                                                   const double* __restrict__ xy, int npts, double2* out) {
-  __shared__ double2 sh[FT / 32], tot[NR][FT];
+  __shared__ double2 sh[FT / 32], tot[LONG ? NR : 1][FT];
   const int p = blockIdx.x;
   const double px = xy[2 * p], py = xy[2 * p + 1];
-  RunSums<NR> sum(tot);
+  RunSums<NR, LONG> sum(tot);
   for (int i = threadIdx.x; i < total; i += FT) {
     const double dx = px - nd.x[i], dy = py - nd.y[i];
     double r, ir, J0, Y0, J1, Y1;
@@ -147,15 +157,21 @@ __global__ void __launch_bounds__(FT) k_scattered(const InclDev* __restrict__ in
   }
 }
 
-// f(first right-hand side, group size as a constant) over groups of 8, 4, 2, 1
+// f(first right-hand side, group size as a constant, LONG as a constant) over
+// groups of 8, 4, 2, 1
 template <class F>
-void rhs_groups(int nrhs, F f) {
+void rhs_groups(int nrhs, int total, F f) {
   for (int c = 0; c < nrhs;) {
     const int left = nrhs - c;
-    if (left >= 8) { f(c, std::integral_constant<int, 8>()); c += 8; }
-    else if (left >= 4) { f(c, std::integral_constant<int, 4>()); c += 4; }
-    else if (left >= 2) { f(c, std::integral_constant<int, 2>()); c += 2; }
-    else { f(c, std::integral_constant<int, 1>()); c += 1; }
+    const auto with = [&](auto nr) {
+      if (total > RUN * FT) f(c, nr, std::true_type());
+      else f(c, nr, std::false_type());
+      c += nr;
+    };
+    if (left >= 8) with(std::integral_constant<int, 8>());
+    else if (left >= 4) with(std::integral_constant<int, 4>());
+    else if (left >= 2) with(std::integral_constant<int, 2>());
+    else with(std::integral_constant<int, 1>());
     pm_launch_count_add(1);
   }
 }
@@ -165,17 +181,17 @@ void rhs_groups(int nrhs, F f) {
 void far_field(const InclDev* d_inc, NodesDev nodes, int total, double k0, const double2* phi, int ldphi, int nrhs,
                const double* d_angles, int ndir, double2* out, cudaStream_t st) {
   if (ndir <= 0 || nrhs <= 0) return;
-  rhs_groups(nrhs, [&](int c, auto nr) {
-    k_far_field<decltype(nr)::value><<<ndir, FT, 0, st>>>(d_inc, nodes, total, k0, phi + (size_t)c * ldphi, ldphi,
-                                                          d_angles, ndir, out + (size_t)c * ndir);
+  rhs_groups(nrhs, total, [&](int c, auto nr, auto runs) {
+    k_far_field<decltype(nr)::value, decltype(runs)::value><<<ndir, FT, 0, st>>>(
+        d_inc, nodes, total, k0, phi + (size_t)c * ldphi, ldphi, d_angles, ndir, out + (size_t)c * ndir);
   });
 }
 
 void scattered_field(const InclDev* d_inc, NodesDev nodes, int total, double k0, const double2* phi, int ldphi,
                      int nrhs, const double* d_xy, int npts, double2* out, cudaStream_t st) {
   if (npts <= 0 || nrhs <= 0) return;
-  rhs_groups(nrhs, [&](int c, auto nr) {
-    k_scattered<decltype(nr)::value><<<npts, FT, 0, st>>>(d_inc, nodes, total, k0, phi + (size_t)c * ldphi, ldphi, d_xy,
-                                                          npts, out + (size_t)c * npts);
+  rhs_groups(nrhs, total, [&](int c, auto nr, auto runs) {
+    k_scattered<decltype(nr)::value, decltype(runs)::value><<<npts, FT, 0, st>>>(
+        d_inc, nodes, total, k0, phi + (size_t)c * ldphi, ldphi, d_xy, npts, out + (size_t)c * npts);
   });
 }
